@@ -324,6 +324,16 @@ int slim_quantize_minmax_sign1(const void* W, const uint8_t* bits_host, uint8_t*
 int slim_quantize_sqc(const void* W, const uint8_t* bits_host, uint8_t* codes, void* scales, void* zeros,
                       int* tau_index, int N, int K, int g, double lambda, int n, void* stream);
 
+/* A layer from its weight in one call: slim_group_salience, slim_allocate_bits (same avg_bits and p), slim_quantize_minmax
+ * and slim_pack_weights under that map, without the codes: packed, scales and zeros are what those calls give, byte for
+ * byte.  Since the bit-widths add up to avg_bits per group whatever the ranking, `packed` is N*K*avg_bits/8 bytes.
+ * bits_pinned_out[K/g] is PAGE-LOCKED host memory (SLIM_ERR_INVALID_ARG otherwise); the call returns when the bit map is
+ * there (a wait for the salience pass, so it cannot be captured in a graph), with the rest still running on `stream`.
+ * W fp16 [N][K], act_norm fp32 [K], scratch: device; scratch of slim_quantize_layer_scratch_bytes(). */
+int slim_quantize_layer_scratch_bytes(int K, int g, size_t* out_bytes);
+int slim_quantize_layer(const void* W, const float* act_norm, int avg_bits, int p, void* packed, void* scales, void* zeros,
+                        uint8_t* bits_pinned_out, int N, int K, int g, void* scratch, size_t scratch_bytes, void* stream);
+
 /* ---- Salience-Determined Bit Allocation (func SBA of Algorithm 2, Sec. 3.2.2, Eq. 4) --------- */
 
 /* y = x * W^T in full precision: x fp16 [M][K], W fp16 [N][K], y fp32 [M][N] (device), fp32

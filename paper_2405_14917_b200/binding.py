@@ -61,6 +61,8 @@ def lib():
             "slim_quantize_minmax": [vp, vp, vp, vp, vp, i, i, i, vp],
             "slim_quantize_minmax_sign1": [vp, vp, vp, vp, vp, i, i, i, vp],
             "slim_quantize_minmax_groups": [vp, vp, vp, vp, vp, i, i, i, vp, i, vp],
+            "slim_quantize_layer_scratch_bytes": [i, i, ctypes.POINTER(sz)],
+            "slim_quantize_layer": [vp, vp, i, i, vp, vp, vp, vp, i, i, i, vp, sz, vp],
             "slim_gemv_set_bytes": [vp, i, i, ctypes.POINTER(sz), ctypes.POINTER(sz)],
             "slim_gemv_set_plan": [vp, i, i, vp, sz, vp, vp],
             "slim_mpq_gemv_set": [vp, vp, vp, sz, vp],
@@ -435,12 +437,20 @@ class QuantLinear:
 
     @classmethod
     def from_weight(cls, W: torch.Tensor, act_norm: torch.Tensor, avg_bits: int, p: int = -1, g: int = GROUP) -> "QuantLinear":
-        """Salience -> bit allocation -> Eq. 1 quantizer -> packing, all on the device."""
+        """Salience -> bit allocation -> Eq. 1 quantizer -> packing, all on the device (slim_quantize_layer)."""
         N, K = W.shape
-        sal = group_salience(W, act_norm, g).cpu().numpy()
-        bits = allocate_bits(sal, avg_bits, p)
-        codes, scales, zeros = quantize_minmax(W, bits, g=g)
-        return cls(pack_weights(codes, bits, g=g), bits, scales, zeros, N, K, g)
+        need = ctypes.c_size_t(0)
+        _check("slim_quantize_layer_scratch_bytes", lib().slim_quantize_layer_scratch_bytes(K, g, ctypes.byref(need)))
+        G = K // g
+        scratch = torch.empty(need.value, dtype=torch.uint8, device=W.device)
+        packed = torch.empty(N * K * avg_bits // 8, dtype=torch.uint8, device=W.device)
+        scales = torch.empty((G, N), dtype=torch.float16, device=W.device)
+        zeros = torch.empty((G, N), dtype=torch.float16, device=W.device)
+        bits = torch.empty(G, dtype=torch.uint8, pin_memory=True)
+        _check("slim_quantize_layer", lib().slim_quantize_layer(
+            _dev(W, torch.float16, "W"), _dev(act_norm, torch.float32, "act_norm"), avg_bits, p, packed.data_ptr(), scales.data_ptr(),
+            zeros.data_ptr(), bits.data_ptr(), N, K, g, scratch.data_ptr(), need.value, _stream(W)))
+        return cls(packed, bits.numpy().copy(), scales, zeros, N, K, g)
 
     def workspace_bytes(self, M: int) -> int:
         return workspace_bytes(M, self.N, self.K, self.bits, self.g)

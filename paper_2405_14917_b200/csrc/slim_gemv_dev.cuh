@@ -5,7 +5,27 @@
 
 #include "slim_common.cuh"
 
+#include <cstring>
+
 namespace slim {
+
+// Launch configuration with programmatic stream serialization: the kernel may be set up while the one before it in
+// the stream is still running; it waits (griddepcontrol.wait) before it touches what that kernel reads or writes.
+struct PdlLaunch {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    PdlLaunch(unsigned grid, unsigned block, size_t smem, cudaStream_t stream, bool early = true) {
+        memset(&cfg, 0, sizeof cfg);
+        cfg.gridDim = dim3(grid, 1, 1);
+        cfg.blockDim = dim3(block, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = early ? 1 : 0;
+    }
+};
 
 // ------------------------------------------------------------------------------------------ PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }

@@ -848,24 +848,6 @@ static size_t set_plan_bytes(int n_layers, long long n_items) {
     return kSetPlanHeader + static_cast<size_t>(n_layers) * sizeof(SetLayer) + static_cast<size_t>(n_items) * sizeof(SetItem);
 }
 
-// Launch configuration with programmatic stream serialization: the kernel may be set up while the one before it in
-// the stream is still running; it waits (griddepcontrol.wait) before it touches what that kernel reads or writes.
-struct PdlLaunch {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[1];
-    PdlLaunch(unsigned grid, unsigned block, size_t smem, cudaStream_t stream, bool early = true) {
-        memset(&cfg, 0, sizeof cfg);
-        cfg.gridDim = dim3(grid, 1, 1);
-        cfg.blockDim = dim3(block, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = stream;
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = early ? 1 : 0;
-    }
-};
-
 template <int NT, bool ONE, int TPW>
 static cudaError_t launch_set(const SetParams& prm, int grid, size_t smem, cudaStream_t stream, bool early) {
     static std::atomic<bool> attr_set[64];    // zero-initialised; set-up is idempotent, so a race repeats it harmlessly
