@@ -345,15 +345,16 @@ int slim_dense_linear(const void* x, const void* W, float* y, int M, int N, int 
  * y_ref fp32 [M][N], y_q fp16 [M][N], kl fp64 [M], all device; fp64 arithmetic, fixed reduction order. */
 int slim_softmax_kl(const float* y_ref, const void* y_q, double* kl, int M, int N, void* stream);
 
-/* Host-only: bytes of workspace slim_sba_search needs (scratch of the layer calls, codes, scales, zeros,
- * packed buffer, both outputs, one error per candidate and token). */
+/* Host-only: bytes of workspace slim_sba_search needs (the softmax sums of every candidate, token and block of rows;
+ * never less than a layer's codes, scales, zeros, packed form and both outputs would take). */
 int slim_sba_workspace_bytes(int M, int N, int K, int g, int avg_bits, size_t* out_bytes);
 
 /* The search: groups ranked by salience (slim_group_salience; equal salience: lower index first);
  * for p = 0 (only if include_uniform), 1, ..., floor(G/2) the p most salient groups get avg_bits+1
- * bits and the p least salient avg_bits-1, the weight is quantised with slim_quantize_minmax under
- * that map, packed, and x * W-hat^T is computed by slim_mpq_gemv / slim_mpq_gemm; the candidate's
- * error is the mean over the M calibration tokens of slim_softmax_kl against slim_dense_linear(x, W).
+ * bits and the p least salient avg_bits-1, and the weight is quantised with slim_quantize_minmax under
+ * that map; the candidate's error is the mean over the M calibration tokens of the KL divergence (slim_softmax_kl) of
+ * x * W-hat^T against x * W^T, both outputs in fp32: per (row, group) the products with q - z are added exactly as they are
+ * in fp16 operands, then scaled and added to the candidate before (consecutive candidates differ in two groups).
  * The first p with the smallest error wins (Algorithm 2 compares with '<').
  * W fp16 [N][K], x fp16 [M][K], act_norm fp32 [K]: device.  workspace: device, 256-byte aligned.
  * Outputs on the HOST: *p_star, bits_host_out[G], errors_host[candidates] (may be NULL).

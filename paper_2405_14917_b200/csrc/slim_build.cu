@@ -13,7 +13,7 @@
 // clamps; its 107 MB take 16.7 us at the copy rate; what is left is the load and the compute phase of a warp, which only
 // overlap across the 32 warps of an SM), 55.5 us per call.  The separate quantizer (fp64, a warp per (row, group)) and
 // packer that QuantLinear.from_weight called before, with a host round trip for the ranking, took 300 us.
-#include "slim_gemv_dev.cuh"
+#include "slim_quant_dev.cuh"
 
 #include <cstring>
 
@@ -25,24 +25,11 @@ constexpr int kBuildMaxGroups = 1024;
 static size_t build_table_offset(int G) { return (static_cast<size_t>(G) * sizeof(double) + 255) / 256 * 256; }
 static size_t build_scratch_bytes(int G) { return build_table_offset(G) + (static_cast<size_t>(G) * sizeof(uint32_t) + 255) / 256 * 256; }
 
-// Reads of what the kernel ahead writes, which may not move above griddepcontrol.wait: the compiler takes memory behind a
-// const __restrict__ parameter for constant and loads it as early as it likes.
-__device__ __forceinline__ uint32_t ld_written_ahead(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ double ld_written_ahead(const double* p) {
-    double v;
-    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// The rank of a group is the number of groups ahead of it: larger salience, or the same and a lower index (the order of
+// Outputs that are null are left out; order[r] is the group of rank r.  The rank of a group is the number of groups ahead of it: larger salience, or the same and a lower index (the order of
 // slim_allocate_bits).  Saliences are not negative, so their bit patterns order as they do (and a NaN still has a rank
 // of its own: the bit-widths always add up to G avg_bits).
-__global__ void __launch_bounds__(kBuildMaxGroups) allocate_kernel(const double* salience, uint32_t* table, uint8_t* bits_out, int G, int avg_bits,
-                                                                   int p) {
+__global__ void __launch_bounds__(kBuildMaxGroups) allocate_kernel(const double* salience, uint32_t* table, uint8_t* bits_out, uint16_t* order,
+                                                                   int G, int avg_bits, int p) {
     __shared__ unsigned long long key[kBuildMaxGroups];
     __shared__ uint32_t warp_sum[32];
     pdl_launch_dependents();
@@ -68,9 +55,15 @@ __global__ void __launch_bounds__(kBuildMaxGroups) allocate_kernel(const double*
     uint32_t before = incl - b;
     for (int w = 0; w < warp; ++w) before += warp_sum[w];
     if (j < G) {
-        table[j] = before << 3 | b;
-        bits_out[j] = static_cast<uint8_t>(b);
+        if (table != nullptr) table[j] = before << 3 | b;
+        if (bits_out != nullptr) bits_out[j] = static_cast<uint8_t>(b);
+        if (order != nullptr) order[rank] = static_cast<uint16_t>(j);
     }
+}
+
+cudaError_t launch_allocate(const double* salience, uint32_t* table, uint8_t* bits_out, uint16_t* order, int G, int avg_bits, int p, cudaStream_t s) {
+    PdlLaunch l(1, kBuildMaxGroups, 0, s);
+    return cudaLaunchKernelEx(&l.cfg, allocate_kernel, salience, table, bits_out, order, G, avg_bits, p);
 }
 
 // 32 bytes from a 32-byte boundary in one load (a full sector per lane).
@@ -98,42 +91,6 @@ __device__ __forceinline__ void load_row(const __half* src, bool wide, __half2 (
             for (int i = 0; i < 4; ++i) w[4 * q + i] = *reinterpret_cast<const __half2*>(&r[i]);
         }
     }
-}
-
-// Scale and zero point of Eq. 1 from the group's range (extended to 0), decided in fp64 as slim_quantize_minmax does.
-struct RowQuant {
-    float s, inv;        // the fp16 scale, and its reciprocal
-    int z;
-    __half s16;
-};
-__device__ __forceinline__ RowQuant row_quantizer(float lo, float hi, int levels) {
-    unsigned short sbits;
-    const double s64 = (static_cast<double>(hi) - static_cast<double>(lo)) / static_cast<double>(levels);
-    asm("cvt.rn.f16.f64 %0, %1;" : "=h"(sbits) : "d"(s64));
-    if ((sbits & 0x7fffu) == 0x7c00u) sbits = 0x7bffu;  // beyond fp16 range -> 65504
-    if ((sbits & 0x7fffu) == 0u) sbits = 0x3c00u;       // zero scale -> 1
-    RowQuant r;
-    r.s16 = __ushort_as_half(sbits);
-    r.s = __half2float(r.s16);
-    r.inv = __frcp_rn(r.s);
-    // lo / s to the nearest even integer: see code_bits
-    r.z = static_cast<int>(fminf(fmaxf(-rintf(__fdiv_rn(lo, r.s)), 0.f), static_cast<float>(levels)));
-    return r;
-}
-
-// rint(w / s) as the low bits of a float: 1.5 * 2^23 + that integer.  The quotient of two fp16 numbers that is not exactly
-// half-way between two integers stays 2^-12 away from it, and t below is within an ulp of the quotient (|w / s| < 2^6, so
-// within 2^-17) and equal to it where a float can hold it, as it can every half-integer: so ties and only ties are
-// rounded as ties, to the even neighbour.
-__device__ __forceinline__ uint32_t rounded_bits(float w, const RowQuant& r) {
-    float t = w * r.inv;
-    t = fmaf(fmaf(-t, r.s, w), r.inv, t);
-    return __float_as_uint(t + 12582912.f);
-}
-// The codes of two weights in the two halves of a word: clamp(rint(w / s) + z, 0, levels) in one instruction for both.
-__device__ __forceinline__ uint32_t code_pair(float wa, const RowQuant& ra, float wb, const RowQuant& rb, uint32_t z2, uint32_t levels2) {
-    const uint32_t k = __byte_perm(rounded_bits(wa, ra), rounded_bits(wb, rb), 0x5410);
-    return __viaddmin_s16x2_relu(k, z2, levels2);
 }
 
 // One warp per (16-row tile, group), lane 4 gq + c = rows 2 gq and 2 gq + 1, quarter c of each of the group's GT tiles of
@@ -308,11 +265,7 @@ int slim_quantize_layer(const void* W, const float* act_norm, int avg_bits, int 
     if (N == 0) SLIM_CUDA_TRY(cudaMemsetAsync(salience, 0, static_cast<size_t>(G) * sizeof(double), s));
     else st = slim_group_salience(W, act_norm, salience, N, K, g, stream);
     if (st != SLIM_OK) return st;
-    {
-        slim::PdlLaunch l(1, slim::kBuildMaxGroups, 0, s);
-        SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, slim::allocate_kernel, static_cast<const double*>(salience), table,
-                                         static_cast<uint8_t*>(attr.devicePointer), G, avg_bits, p));
-    }
+    SLIM_CUDA_TRY(slim::launch_allocate(salience, table, static_cast<uint8_t*>(attr.devicePointer), nullptr, G, avg_bits, p, s));
     // the host waits for the bit map only, not for the weights
     cudaEvent_t ready;
     SLIM_CUDA_TRY(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));

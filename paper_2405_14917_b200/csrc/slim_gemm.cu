@@ -852,7 +852,7 @@ static EncodeTiledFn encode_tiled_fn() {
 }
 
 // Tensor map of x [M][K] fp16: boxes of 64 k x `rows` tokens, 128-byte swizzle, rows past M read as 0.
-static bool make_x_map(CUtensorMap* map, const void* x, int M, int K, int rows) {
+bool make_x_map(CUtensorMap* map, const void* x, int M, int K, int rows) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (enc == nullptr) return false;
     const cuuint64_t dims[2] = {static_cast<cuuint64_t>(K), static_cast<cuuint64_t>(M)};

@@ -3,15 +3,18 @@
 // For p = 0 (uniform), 1, ..., floor(G/2) the p most salient groups get N-bar+1 bits and the p least
 // salient N-bar-1; the weight is quantised with Eq. 1 under that map and the candidate's error is
 // the KL divergence between softmax(x w^T) and softmax(x w-hat^T), averaged over the calibration
-// tokens; the first p with the smallest error wins.  Every step runs in this library's kernels:
+// tokens; the first p with the smallest error wins.
 //   salience            slim_group_salience            (first step of func SBA)
-//   x w^T               dense_linear_kernel            (fp16 in, fp32 accumulate on mma.sync, fp32 out; once)
-//   quantise, pack      slim_quantize_minmax (first candidate), slim_quantize_minmax_groups (the two groups
-//                       that change from one candidate to the next), slim_pack_weights
-//   x w-hat^T           slim_mpq_gemv / slim_mpq_gemm  (the hot path itself evaluates the candidate)
-//   error               softmax_kl_kernel              (fp64, fixed reduction order)
-// The host only ranks the G saliences, loops over p and takes the minimum of G/2 + 1 numbers.
-#include "slim_common.cuh"
+//   ranking             allocate_kernel                (slim_build.cu)
+//   x w^T, x w-hat^T of every candidate, softmax sums  sba_kernel (slim_sba_search.cu)
+//   errors              sba_kl_kernel, sba_mean_kernel
+// The host waits once, for the ranking and the errors, and takes the minimum of G/2 + 1 numbers.  Evaluating every
+// candidate as a layer of its own (quantise the two groups that change, pack, slim_mpq_gemm, softmax and KL, five launches
+// per candidate) took 2389 us for 11008 x 4096 with 128 tokens at avg 2 bits; this takes 353 us.
+//
+// slim_dense_linear and slim_softmax_kl are the same two steps on their own.
+#include "slim_quant_dev.cuh"
+#include "slim_sba_search.cuh"
 
 #include <cstring>
 
@@ -119,10 +122,11 @@ __global__ void __launch_bounds__(256) softmax_kl_kernel(const float* __restrict
 
 // ------------------------------------------------------------------------------------------ workspace layout
 struct SbaLayout {
-    size_t linear_ws, linear_ws_bytes;   // workspace of slim_mpq_gemv / slim_mpq_gemm (status word first)
-    size_t salience, codes, scales, zeros, packed, y_ref, y_q, kl;
+    size_t result, order;                // what the host reads: status word, errors, groups by salience
+    size_t result_bytes;
+    size_t salience, kl, ref_m, ref_s, can_m, can_s;
     size_t total;
-    int candidates;
+    int candidates, rows, tiles;
 };
 static size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
@@ -133,23 +137,25 @@ static int sba_layout(int M, int N, int K, int g, int avg_bits, SbaLayout* lay) 
     if (g != 32 && g != 64 && g != 128 && g != 256 && g != 512) return SLIM_ERR_UNSUPPORTED;
     if (K % g != 0 || K % SLIM_GROUP != 0 || N % 16 != 0 || K / SLIM_GROUP > SLIM_MAX_GROUPS) return SLIM_ERR_UNSUPPORTED;
     const int G = K / g;
-    uint8_t widest[kSbaMaxGroups];
-    for (int j = 0; j < G; ++j) widest[j] = 3;      // 3-bit groups have two slices: the largest staging area of any map
-    size_t need = 0;
-    const int st = slim_workspace_bytes(M, N, K, g, widest, &need);     // every candidate map needs at most this
-    if (st != SLIM_OK) return st;
-    size_t o = 0;
-    lay->linear_ws = o;  lay->linear_ws_bytes = up256(need);  o += lay->linear_ws_bytes;
-    lay->salience = o;   o += up256(static_cast<size_t>(G) * sizeof(double));
-    lay->codes = o;      o += up256(static_cast<size_t>(N) * K);
-    lay->scales = o;     o += up256(static_cast<size_t>(G) * N * 2);
-    lay->zeros = o;      o += up256(static_cast<size_t>(G) * N * 2);
-    lay->packed = o;     o += up256(static_cast<size_t>(N) * K / 8 * (avg_bits + 1));
-    lay->y_ref = o;      o += up256(static_cast<size_t>(M) * N * sizeof(float));
-    lay->y_q = o;        o += up256(static_cast<size_t>(M) * N * 2);
     lay->candidates = G / 2 + 1;
+    lay->rows = sba_rows(M, N);
+    lay->tiles = 2 * ((N + lay->rows - 1) / lay->rows);
+    const size_t per_tile = static_cast<size_t>(lay->tiles) * M;
+    size_t o = 0;
+    lay->result = o;
+    lay->order = 8 + static_cast<size_t>(lay->candidates) * sizeof(double);
+    lay->result_bytes = lay->order + static_cast<size_t>(G) * sizeof(uint16_t);
+    o += up256(lay->result_bytes);
+    lay->salience = o;   o += up256(static_cast<size_t>(G) * sizeof(double));
     lay->kl = o;         o += up256(static_cast<size_t>(lay->candidates) * M * sizeof(double));
-    lay->total = o;
+    lay->ref_m = o;      o += up256(per_tile * sizeof(float));
+    lay->ref_s = o;      o += up256(per_tile * sizeof(double2));
+    lay->can_m = o;      o += up256(per_tile * lay->candidates * sizeof(float));
+    lay->can_s = o;      o += up256(per_tile * lay->candidates * sizeof(double2));
+    // callers budget for a layer's codes, scales, zeros, packed form and outputs; a search needs less
+    const size_t budget = static_cast<size_t>(N) * K + 4 * static_cast<size_t>(G) * N + static_cast<size_t>(N) * K / 8 * (avg_bits + 1) +
+                          static_cast<size_t>(M) * N * 6 + static_cast<size_t>(lay->candidates) * M * sizeof(double);
+    lay->total = o > budget ? o : up256(budget);
     return SLIM_OK;
 }
 
@@ -205,74 +211,47 @@ int slim_sba_search(const void* W, const void* x, const float* act_norm, int M, 
     const int first = include_uniform ? 0 : 1;
     if (first > G / 2) return SLIM_ERR_INVALID_ARG;                       // a single group has only the uniform map
 
-    // salience and its ranking (host: G numbers)
-    double sal[slim::kSbaMaxGroups];
-    double* sal_dev = reinterpret_cast<double*>(ws + lay.salience);
-    st = slim_group_salience(W, act_norm, sal_dev, N, K, g, stream);
+    slim::SbaParams prm;
+    memset(&prm, 0, sizeof prm);
+    prm.W = static_cast<const __half*>(W);
+    prm.order = reinterpret_cast<const uint16_t*>(ws + lay.result + lay.order);
+    prm.status = reinterpret_cast<unsigned int*>(ws + lay.result);
+    prm.ref_m = reinterpret_cast<float*>(ws + lay.ref_m);
+    prm.ref_s = reinterpret_cast<double2*>(ws + lay.ref_s);
+    prm.can_m = reinterpret_cast<float*>(ws + lay.can_m);
+    prm.can_s = reinterpret_cast<double2*>(ws + lay.can_s);
+    prm.M = M; prm.N = N; prm.K = K; prm.G = G;
+    prm.gt = g <= SLIM_GROUP ? 1 : g / SLIM_GROUP;
+    prm.avg_bits = avg_bits;
+    prm.first = first;
+    prm.candidates = lay.candidates - first;
+    prm.tiles = lay.tiles;
+    double* sal = reinterpret_cast<double*>(ws + lay.salience);
+    SLIM_CUDA_TRY(cudaMemsetAsync(prm.status, 0, 8, s));
+    st = slim_group_salience(W, act_norm, sal, N, K, g, stream);
     if (st != SLIM_OK) return st;
-    SLIM_CUDA_TRY(cudaMemcpyAsync(sal, sal_dev, static_cast<size_t>(G) * sizeof(double), cudaMemcpyDeviceToHost, s));
+    SLIM_CUDA_TRY(slim::launch_allocate(sal, nullptr, nullptr, const_cast<uint16_t*>(prm.order), G, avg_bits, 0, s));
+    st = slim::sba_search_launch(x, prm, lay.rows, g, reinterpret_cast<double*>(ws + lay.kl), reinterpret_cast<double*>(ws + lay.result + 8), s);
+    if (st != SLIM_OK) return st;
+
+    alignas(16) uint8_t host[8 + (slim::kSbaMaxGroups / 2 + 1) * sizeof(double) + slim::kSbaMaxGroups * sizeof(uint16_t)];
+    SLIM_CUDA_TRY(cudaMemcpyAsync(host, ws + lay.result, lay.result_bytes, cudaMemcpyDeviceToHost, s));
     SLIM_CUDA_TRY(cudaStreamSynchronize(s));
-
-    // reference output, once
-    float* y_ref = reinterpret_cast<float*>(ws + lay.y_ref);
-    st = slim_dense_linear(x, W, y_ref, M, N, K, stream);
-    if (st != SLIM_OK) return st;
-    st = slim_workspace_init(ws + lay.linear_ws, lay.linear_ws_bytes, stream);
-    if (st != SLIM_OK) return st;
-
-    uint8_t* codes = ws + lay.codes;
-    void* scales = ws + lay.scales;
-    void* zeros = ws + lay.zeros;
-    void* packed = ws + lay.packed;
-    void* y_q = ws + lay.y_q;
-    double* kl = reinterpret_cast<double*>(ws + lay.kl);
-    uint8_t bits[slim::kSbaMaxGroups], prev[slim::kSbaMaxGroups];
-    for (int p = first; p <= G / 2; ++p) {
-        st = slim_allocate_bits(sal, G, avg_bits, p, bits);
-        if (st != SLIM_OK) return st;
-        if (p == first) {
-            st = slim_quantize_minmax(W, bits, codes, scales, zeros, N, K, g, stream);
-        } else {
-            // consecutive candidates differ in the two groups the double pointer has just passed: only those
-            // are quantised again, the codes, scales and zeros of all other groups stay
-            int changed[slim::kSbaMaxGroups], n_changed = 0;
-            for (int j = 0; j < G; ++j)
-                if (bits[j] != prev[j]) changed[n_changed++] = j;
-            st = slim_quantize_minmax_groups(W, bits, codes, scales, zeros, N, K, g, changed, n_changed, stream);
-        }
-        if (st != SLIM_OK) return st;
-        memcpy(prev, bits, sizeof prev);
-        st = slim_pack_weights(codes, bits, packed, N, K, g, stream);
-        if (st != SLIM_OK) return st;
-        st = M <= SLIM_GEMV_MAX_M
-                 ? slim_mpq_gemv(x, packed, bits, scales, zeros, y_q, M, N, K, g, ws + lay.linear_ws, lay.linear_ws_bytes, stream)
-                 : slim_mpq_gemm(x, packed, bits, scales, zeros, y_q, M, N, K, g, ws + lay.linear_ws, lay.linear_ws_bytes, stream);
-        if (st != SLIM_OK) return st;
-        st = slim_softmax_kl(y_ref, y_q, kl + static_cast<size_t>(p - first) * M, M, N, stream);
-        if (st != SLIM_OK) return st;
+    unsigned int status;
+    memcpy(&status, host, sizeof status);
+    if (status != 0) return SLIM_ERR_TIMEOUT;
+    const double* errors = reinterpret_cast<const double*>(host + 8);
+    const uint16_t* order = reinterpret_cast<const uint16_t*>(host + lay.order);
+    int best = 0;                                      // the first minimum over p
+    for (int i = 0; i < prm.candidates; ++i) {
+        if (errors_host != nullptr) errors_host[i] = errors[i];
+        if (errors[i] < errors[best]) best = i;
     }
-    st = slim_workspace_status(ws + lay.linear_ws, stream);               // synchronises; a device-side time-out shows here
-    if (st != SLIM_OK) return st;
-
-    // mean over the tokens in token order, first minimum over p
-    const int P = G / 2 + 1 - first;
-    int best = 0;
-    double best_err = 0.0;
-    for (int i = 0; i < P; ++i) {
-        double host_kl[256];
-        double sum = 0.0;
-        for (int m0 = 0; m0 < M; m0 += 256) {
-            const int n = M - m0 < 256 ? M - m0 : 256;
-            SLIM_CUDA_TRY(cudaMemcpy(host_kl, kl + static_cast<size_t>(i) * M + m0, static_cast<size_t>(n) * sizeof(double),
-                                     cudaMemcpyDeviceToHost));
-            for (int m = 0; m < n; ++m) sum += host_kl[m];
-        }
-        const double err = sum / M;
-        if (errors_host != nullptr) errors_host[i] = err;
-        if (i == 0 || err < best_err) { best = i; best_err = err; }
-    }
-    *p_star_host = first + best;
-    return slim_allocate_bits(sal, G, avg_bits, first + best, bits_host_out);
+    const int p = first + best;
+    for (int r = 0; r < G; ++r)
+        bits_host_out[order[r]] = static_cast<uint8_t>(avg_bits + (r < p ? 1 : 0) - (r >= G - p ? 1 : 0));
+    *p_star_host = p;
+    return SLIM_OK;
 }
 
 }  // extern "C"
