@@ -7,9 +7,9 @@
 //                      bit map itself into the caller's page-locked memory
 //   quant_pack_kernel  reads W a second time, writes scales, zeros and packed slices
 //
-// Bound: two passes over the 2 N K bytes of W.  quant_pack_kernel issues about eight instructions per weight (convert,
-// three for the quotient, one to round, and for two weights together one to pair, one to clamp, one to place the
-// fields).  4096 x 11008 at avg 3 bits: salience 20 us (137 before), allocate 5 us, quant_pack 27 us (34 with scalar
+// Bound: two passes over the 2 N K bytes of W.  quant_pack_kernel issues about seven instructions per weight (convert,
+// two for the quotient, one to round, and for two weights together one to pair, one to clamp, one to place the
+// fields).  4096 x 11008 at avg 3 bits: salience 20 us (137 before), allocate 5 us, quant_pack 25 us (34 with scalar
 // clamps; its 107 MB take 16.7 us at the copy rate; what is left is the load and the compute phase of a warp, which only
 // overlap across the 32 warps of an SM), 55.5 us per call.  The separate quantizer (fp64, a warp per (row, group)) and
 // packer that QuantLinear.from_weight called before, with a host round trip for the ranking, took 300 us.

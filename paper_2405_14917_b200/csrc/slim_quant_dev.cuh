@@ -22,17 +22,16 @@ __device__ __forceinline__ double ld_written_ahead(const double* p) {
 // Scale and zero point of Eq. 1 from the group's range (extended to 0), the values slim_quantize_minmax decides in
 // fp64.
 struct RowQuant {
-    float s, inv;        // the fp16 scale, and its reciprocal
+    float s, inv, inv_lo;    // the fp16 scale, and its reciprocal as a sum of two floats
     int z;
     __half s16;
 };
 // rint(w / s) as the low bits of a float: 1.5 * 2^23 + that integer.  The quotient of two fp16 numbers that is not exactly
-// half-way between two integers stays 2^-12 away from it, and t below is within an ulp of the quotient (|w / s| < 2^6, so
-// within 2^-17) and equal to it where a float can hold it, as it can every half-integer: so ties and only ties are
-// rounded as ties, to the even neighbour.
+// half-way between two integers stays 2^-12 away from it; t below is the quotient, 2^-46 off at most, rounded to a float
+// (|w / s| < 2^6, so within 2^-18 of it), and equal to it where a float can hold it, as it can every half-integer: so
+// ties and only ties are rounded as ties, to the even neighbour.
 __device__ __forceinline__ uint32_t rounded_bits(float w, const RowQuant& r) {
-    float t = w * r.inv;
-    t = fmaf(fmaf(-t, r.s, w), r.inv, t);
+    const float t = fmaf(w, r.inv, w * r.inv_lo);
     return __float_as_uint(t + 12582912.f);
 }
 __device__ __forceinline__ RowQuant row_quantizer(float lo, float hi, int levels) {
@@ -53,6 +52,7 @@ __device__ __forceinline__ RowQuant row_quantizer(float lo, float hi, int levels
     r.s16 = __ushort_as_half(sbits);
     r.s = __half2float(r.s16);
     r.inv = __frcp_rn(r.s);
+    r.inv_lo = fmaf(-r.inv, r.s, 1.f) * r.inv;
     r.z = min(max(static_cast<int>(0x4B400000u - rounded_bits(lo, r)), 0), levels);
     return r;
 }

@@ -25,9 +25,13 @@ namespace slim {
 // small integer, exact in fp16, and the scale is applied in fp32, so no weight is rounded.
 //
 // Warps: 0 brings x (TMA), 1 issues the MMAs (M = 128 tokens, N = R rows, operands in shared memory, accumulators in tensor
-// memory), 2 to 9 read W, quantise and write the second operand, 10 to 17 fold and reduce (thread = token; four warps take
+// memory), 2 to 11 read W, quantise and write the second operand, 12 to 19 fold and reduce (thread = token; four warps take
 // the first half of the rows, four the second).
-constexpr int kSbaQuant = 8, kSbaFold = 8;
+//
+// Bound: instructions, most of them the quantising warps' (about 12 per weight and width, its bytes would take 14 us a pass):
+// 11008 x 4096, 128 tokens, avg 2 bits: 163 us (240 with eight quantising warps and every lane working out its row's scale,
+// 187 before the quotient went from three operations to two and the scales were passed on instead of divided again).
+constexpr int kSbaQuant = 10, kSbaFold = 8;
 constexpr int kSbaFirstQuant = 2, kSbaFirstFold = kSbaFirstQuant + kSbaQuant;
 constexpr int kSbaWarps = kSbaFirstFold + kSbaFold;
 constexpr int kSbaTokens = 128;
@@ -41,8 +45,7 @@ template <int R, int CW> struct SbaCfg {
     static constexpr int STAGE = XBYTES + 2 * BBYTES;
     static constexpr int STAGES = 3;
     static constexpr int OFF_SCALE = STAGES * STAGE;
-    static constexpr int OFF_ZERO = OFF_SCALE + kSbaScaleSlots * 2 * R * 4;
-    static constexpr int OFF_ORDER = OFF_ZERO + 2 * R * 4;
+    static constexpr int OFF_ORDER = OFF_SCALE + kSbaScaleSlots * 2 * R * 4;
     static constexpr int OFF_BAR = OFF_ORDER + 2 * 1024;
     static constexpr int NBAR = 3 * STAGES + 4 + 3;
     static constexpr int OFF_MISC = OFF_BAR + 8 * NBAR;
@@ -174,13 +177,46 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
                 mx = __hmax2(mx, h);
             }
         };
-        auto row_range = [&](const __half2& mn, const __half2& mx, float& lo, float& hi) {
-            __half2 a = __hmin2(mn, __lowhigh2highlow(mn)), b = __hmax2(mx, __lowhigh2highlow(mx));
-            __half2 v = __halves2half2(__low2half(a), __hneg(__low2half(b)));              // (lo, -hi): both by minimum
+        // (lo, -hi) of the row, in all its lanes
+        auto row_range = [&](const __half2& mn, const __half2& mx) {
+            const __half2 a = __hmin2(mn, __lowhigh2highlow(mn)), b = __hmax2(mx, __lowhigh2highlow(mx));
+            __half2 v = __halves2half2(__low2half(a), __hneg(__low2half(b)));              // both by minimum
 #pragma unroll
             for (int o = 1; o < LPR; o <<= 1) v = __hmin2(v, __shfl_xor_sync(0xffffffffu, v, o));
-            lo = __low2float(v);
-            hi = -__high2float(v);
+            return *reinterpret_cast<const uint32_t*>(&v);
+        };
+        // A row's constants cost about 60 instructions, so a lane works them out for one (row of the warp, width): lane i < IT RPW
+        // for row i under the old width, lane 16 + i under the new one (in two rounds if there are more than 16 rows).
+        constexpr int ROWS = IT * RPW, ROUNDS = (ROWS + 15) / 16;
+        struct Consts { float s[ROUNDS], inv[ROUNDS], inv_lo[ROUNDS]; int z[ROUNDS]; };
+        auto row_constants = [&](const uint32_t (&range)[IT], int l_old, int l_new) {
+            Consts c;
+#pragma unroll
+            for (int k = 0; k < ROUNDS; ++k) {
+                const int row = 16 * k + (lane & 15);                  // = it * RPW + (row of the step)
+                uint32_t v = range[0];                                 // lanes without a row repeat one
+#pragma unroll
+                for (int it = 0; it < IT; ++it) {
+                    const uint32_t w = __shfl_sync(0xffffffffu, range[it], (row % RPW) * LPR);
+                    if (row / RPW == it) v = w;
+                }
+                const __half2 h = *reinterpret_cast<const __half2*>(&v);
+                const RowQuant q = row_quantizer(__low2float(h), -__high2float(h), lane < 16 ? l_old : l_new);
+                c.s[k] = q.s;
+                c.inv[k] = q.inv;
+                c.inv_lo[k] = q.inv_lo;
+                c.z[k] = q.z;
+            }
+            return c;
+        };
+        // the constants of my row of step `it` (width 0: old, 1: new)
+        auto my_constants = [&](const Consts& c, int it, int width) {
+            const int k = it * RPW / 16, from = ((it * RPW + lane / LPR) & 15) + 16 * width;
+            RowQuant q;
+            q.inv = __shfl_sync(0xffffffffu, c.inv[k], from);
+            q.inv_lo = __shfl_sync(0xffffffffu, c.inv_lo[k], from);
+            q.z = __shfl_sync(0xffffffffu, c.z[k], from);
+            return q;
         };
         // eight weights -> eight q - z in fp16
         auto operand = [&](const uint4& v, const RowQuant& rq, int levels) {
@@ -222,7 +258,7 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
             const int b_old = p.avg_bits, b_new = ((u - G) & 1) ? p.avg_bits - 1 : p.avg_bits + 1;
             const int l_old = (1 << b_old) - 1, l_new = (1 << b_new) - 1;
             float* sc = scale_ring + (u & (kSbaScaleSlots - 1)) * 2 * R;
-            int* zc = reinterpret_cast<int*>(smem + C::OFF_ZERO);
+            Consts consts;
             if (!MULTI) {
 #pragma unroll
                 for (int it = 0; it < IT; ++it) raw[it] = nxt[it];
@@ -236,52 +272,33 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
                 if (!tc::warp_wait(empty(s), ph ^ 1u, abort)) { ok = false; break; }
                 uint8_t* b0 = smem + s * C::STAGE + C::XBYTES;
                 uint8_t* b1 = b0 + C::BBYTES;
-                if (MULTI) {
-                    if (ch == 0) {
-                        // range over the whole group; scales and zero points of my rows go through shared memory
+                if (ch == 0) {
+                    uint32_t range[IT];
 #pragma unroll
-                        for (int it = 0; it < IT; ++it) {
-                            __half2 mn = __float2half2_rn(0.f), mx = mn;
+                    for (int it = 0; it < IT; ++it) {
+                        __half2 mn = __float2half2_rn(0.f), mx = mn;
+                        if (MULTI)
                             for (int c = 0; c < gt; ++c) range_of(load(it, j, c), mn, mx);
-                            float lo, hi;
-                            row_range(mn, mx, lo, hi);
-                            const int r = r0 + it * STEP;
-                            if (sub == 0 && r < R) {
-                                const RowQuant q = row_quantizer(lo, hi, l_old);
-                                sc[r] = q.s;
-                                zc[r] = q.z;
-                                if (second) {
-                                    const RowQuant q2 = row_quantizer(lo, hi, l_new);
-                                    sc[R + r] = q2.s;
-                                    zc[R + r] = q2.z;
-                                }
-                            }
-                        }
-                        __syncwarp();
+                        else
+                            range_of(raw[it], mn, mx);
+                        range[it] = row_range(mn, mx);
                     }
+                    consts = row_constants(range, l_old, l_new);
+                    // row i of the warp is row (i / RPW) STEP + qw RPW + i % RPW of the CTA
+#pragma unroll
+                    for (int k = 0; k < ROUNDS; ++k) {
+                        const int i = 16 * k + (lane & 15), r = (i / RPW) * STEP + qw * RPW + i % RPW;
+                        if (i < ROWS && r < R) sc[(lane < 16 ? 0 : R) + r] = consts.s[k];
+                    }
+                }
+                if (MULTI)
 #pragma unroll
                     for (int it = 0; it < IT; ++it) raw[it] = load(it, j, ch);
-                }
 #pragma unroll
                 for (int it = 0; it < IT; ++it) {
                     const int r = r0 + it * STEP;
-                    RowQuant q, q2;
-                    if (MULTI) {
-                        const int rc = min(r, R - 1);
-                        q.s = sc[rc]; q.inv = __frcp_rn(q.s); q.z = zc[rc];
-                        if (second) { q2.s = sc[R + rc]; q2.inv = __frcp_rn(q2.s); q2.z = zc[R + rc]; }
-                    } else {
-                        __half2 mn = __float2half2_rn(0.f), mx = mn;
-                        range_of(raw[it], mn, mx);
-                        float lo, hi;
-                        row_range(mn, mx, lo, hi);
-                        q = row_quantizer(lo, hi, l_old);
-                        if (second) q2 = row_quantizer(lo, hi, l_new);
-                        if (sub == 0 && r < R) {
-                            sc[r] = q.s;
-                            if (second) sc[R + r] = q2.s;
-                        }
-                    }
+                    const RowQuant q = my_constants(consts, it, 0);
+                    const RowQuant q2 = second ? my_constants(consts, it, 1) : q;
                     if (r < R) {
                         const int at = (sub >> 3) * R * 128 + r * 128 + (((sub & 7) ^ (r & 7)) << 4);
                         *reinterpret_cast<uint4*>(b0 + at) = operand(raw[it], q, l_old);
@@ -306,17 +323,24 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
         for (int i = 0; i < C::RH; ++i) y[i] = 0.f;
         // y += (or -=) scale * D
         auto fold = [&](uint32_t d, const float* sc, float sign) {
-            uint32_t v[C::RH];
+            constexpr int kBatch = 24;                     // columns on their way at a time (registers)
 #pragma unroll
-            for (int c = 0; c < C::RH / 8; ++c) tc::ld8(d + t_lane + h * C::RH + 8 * c, v + 8 * c);
-            tc::wait_ld();
+            for (int c0 = 0; c0 < C::RH; c0 += kBatch) {
+                uint32_t v[kBatch];
 #pragma unroll
-            for (int i = 0; i < C::RH; i += 4) {
-                const float4 f = *reinterpret_cast<const float4*>(sc + h * C::RH + i);
-                y[i] = fmaf(sign * f.x, __uint_as_float(v[i]), y[i]);
-                y[i + 1] = fmaf(sign * f.y, __uint_as_float(v[i + 1]), y[i + 1]);
-                y[i + 2] = fmaf(sign * f.z, __uint_as_float(v[i + 2]), y[i + 2]);
-                y[i + 3] = fmaf(sign * f.w, __uint_as_float(v[i + 3]), y[i + 3]);
+                for (int c = 0; c < kBatch; c += 8)
+                    if (c0 + c < C::RH) tc::ld8(d + t_lane + h * C::RH + c0 + c, v + c);
+                tc::wait_ld();
+#pragma unroll
+                for (int c = 0; c < kBatch; c += 4) {
+                    if (c0 + c >= C::RH) break;
+                    const int i = c0 + c;
+                    const float4 f = *reinterpret_cast<const float4*>(sc + h * C::RH + i);
+                    y[i] = fmaf(sign * f.x, __uint_as_float(v[c]), y[i]);
+                    y[i + 1] = fmaf(sign * f.y, __uint_as_float(v[c + 1]), y[i + 1]);
+                    y[i + 2] = fmaf(sign * f.z, __uint_as_float(v[c + 2]), y[i + 2]);
+                    y[i + 3] = fmaf(sign * f.w, __uint_as_float(v[c + 3]), y[i + 3]);
+                }
             }
         };
         float mr = -INFINITY;
@@ -417,46 +441,64 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
 }
 
 // ------------------------------------------------------------------------------------------ errors
-// Sums relative to exp(-m), merged by rescaling to the larger m; empty: m = -inf, s = a = 0.
-struct SbaMerge { double m, s, a; };
-__device__ __forceinline__ void sba_merge(SbaMerge& t, double m, double s, double a) {
-    if (m > t.m) {
-        const double f = exp(t.m - m);
-        t.s = t.s * f + s;
-        t.a = t.a * f + a;
-        t.m = m;
-    } else if (m > -INFINITY) {
-        const double f = exp(m - t.m);
-        t.s += s * f;
-        t.a += a * f;
-    }
-}
-
 // kl[c][t] = sum_n p_n (log p_n - log q_n), p the softmax of the reference and q that of candidate c, in fp64 from the tiles'
-// sums.  A block takes 32 tokens of one candidate; its warps take every eighth tile, and their sums are merged in
-// warp order.
-__global__ void __launch_bounds__(256) sba_kl_kernel(SbaParams p, double* kl) {
-    __shared__ SbaMerge ref_part[8][32], can_part[8][32];
+// sums.  A block takes 16 tokens of one candidate; its 64 half warps take every 64th tile: the largest outputs first, then
+// the sums relative to them (one exp per sum), added over the half warps by a fixed tree.
+constexpr int kKlTokens = 16, kKlSlices = 64;
+__global__ void __launch_bounds__(kKlTokens * kKlSlices) sba_kl_kernel(SbaParams p, double* kl) {
+    __shared__ float top[2][kKlSlices][kKlTokens + 1];
+    __shared__ double part[3][kKlSlices][kKlTokens + 1];
     pdl_wait();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.y, m = blockIdx.x * 32 + lane;
-    SbaMerge ref{-INFINITY, 0.0, 0.0}, can = ref;
+    const int tok = threadIdx.x % kKlTokens, slice = threadIdx.x / kKlTokens, c = blockIdx.y, m = blockIdx.x * kKlTokens + tok;
+    const float* ref_m = p.ref_m + m;
+    const float* can_m = p.can_m + static_cast<size_t>(c) * p.tiles * p.M + m;
+    const double2* ref_s = p.ref_s + m;
+    const double2* can_s = p.can_s + static_cast<size_t>(c) * p.tiles * p.M + m;
+    float mr = -INFINITY, mq = -INFINITY;
     if (m < p.M)
-        for (int k = warp; k < p.tiles; k += 8) {
-            const size_t r = static_cast<size_t>(k) * p.M + m, q = (static_cast<size_t>(c) * p.tiles + k) * p.M + m;
-            const double2 rs = __ldcg(p.ref_s + r), qs = __ldcg(p.can_s + q);
-            sba_merge(ref, __ldcg(p.ref_m + r), rs.x, rs.y - qs.y);
-            sba_merge(can, __ldcg(p.can_m + q), qs.x, 0.0);
+        for (int k = slice; k < p.tiles; k += kKlSlices) {
+            mr = fmaxf(mr, __ldcg(ref_m + static_cast<size_t>(k) * p.M));
+            mq = fmaxf(mq, __ldcg(can_m + static_cast<size_t>(k) * p.M));
         }
-    ref_part[warp][lane] = ref;
-    can_part[warp][lane] = can;
+    top[0][slice][tok] = mr;
+    top[1][slice][tok] = mq;
     __syncthreads();
-    if (warp != 0 || m >= p.M) return;
-    for (int w = 1; w < 8; ++w) {
-        sba_merge(ref, ref_part[w][lane].m, ref_part[w][lane].s, ref_part[w][lane].a);
-        sba_merge(can, can_part[w][lane].m, can_part[w][lane].s, 0.0);
+#pragma unroll 8
+    for (int w = 0; w < kKlSlices; ++w) {
+        mr = fmaxf(mr, top[0][w][tok]);
+        mq = fmaxf(mq, top[1][w][tok]);
+    }
+    double v[3] = {0.0, 0.0, 0.0};                 // sum e, sum e (y - y_q), sum e_q
+    if (m < p.M)
+        for (int k = slice; k < p.tiles; k += kKlSlices) {
+            const size_t at = static_cast<size_t>(k) * p.M;
+            const double2 r = __ldcg(ref_s + at), q = __ldcg(can_s + at);
+            const double fr = exp(static_cast<double>(__ldcg(ref_m + at)) - static_cast<double>(mr));
+            const double fq = exp(static_cast<double>(__ldcg(can_m + at)) - static_cast<double>(mq));
+            v[0] = fma(r.x, fr, v[0]);
+            v[1] = fma(r.y - q.y, fr, v[1]);
+            v[2] = fma(q.x, fq, v[2]);
+        }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) part[i][slice][tok] = v[i];
+    __syncthreads();
+    // warp w < 16 adds the parts of token w
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = blockIdx.x * kKlTokens + warp;
+    if (warp >= kKlTokens || t >= p.M) return;
+    mr = fmaxf(top[0][lane][warp], top[0][lane + 32][warp]);
+    mq = fmaxf(top[1][lane][warp], top[1][lane + 32][warp]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v[i] = part[i][lane][warp] + part[i][lane + 32][warp];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
+        mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
     }
     // sum p (y - y_q) - log sum exp y + log sum exp y_q
-    kl[static_cast<size_t>(c) * p.M + m] = ref.a / ref.s - (ref.m + log(ref.s)) + (can.m + log(can.s));
+    if (lane == 0)
+        kl[static_cast<size_t>(c) * p.M + t] = v[1] / v[0] - (static_cast<double>(mr) + log(v[0])) + (static_cast<double>(mq) + log(v[2]));
 }
 
 // Mean over the tokens, one warp per candidate, in a fixed order.
@@ -517,7 +559,7 @@ int sba_search_launch(const void* x, const SbaParams& p, int rows, int g, double
                   : rows == 48 ? launch_search_for<48>(g, map, p, s)
                   : rows == 64 ? launch_search_for<64>(g, map, p, s)
                                : launch_search_for<80>(g, map, p, s));
-    PdlLaunch k(static_cast<unsigned>((p.M + 31) / 32), 256, 0, s);
+    PdlLaunch k(static_cast<unsigned>((p.M + kKlTokens - 1) / kKlTokens), kKlTokens * kKlSlices, 0, s);
     k.cfg.gridDim.y = static_cast<unsigned>(p.candidates);
     SLIM_CUDA_TRY(cudaLaunchKernelEx(&k.cfg, sba_kl_kernel, p, kl));
     PdlLaunch e(static_cast<unsigned>(p.candidates), 32, 0, s);
