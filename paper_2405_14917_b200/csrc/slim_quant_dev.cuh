@@ -57,6 +57,11 @@ __device__ __forceinline__ RowQuant row_quantizer(float lo, float hi, int levels
     return r;
 }
 
+// clamp(rint(w / s) + z, 0, levels) for any quotient.
+__device__ __forceinline__ int clamped_code(float w, const RowQuant& r, float z, float levels) {
+    const float t = fminf(fmaxf(fmaf(w, r.inv, w * r.inv_lo), -z), levels - z);
+    return static_cast<int>(__float_as_uint(t + 12582912.f) - 0x4B400000u) + static_cast<int>(z);
+}
 // The codes of two weights in the two halves of a word: clamp(rint(w / s) + z, 0, levels) in one instruction for both.
 __device__ __forceinline__ uint32_t code_pair(float wa, const RowQuant& ra, float wb, const RowQuant& rb, uint32_t z2, uint32_t levels2) {
     const uint32_t k = __byte_perm(rounded_bits(wa, ra), rounded_bits(wb, rb), 0x5410);

@@ -2,7 +2,7 @@
 // asymmetric min-max quantizer of Eq. 1.  fp64 arithmetic from fp16 weights, fixed summation
 // order, so the outputs are reproducible bit for bit.  Every kernel is a template over the group
 // size GS (32, 64, 128, 256, 512 columns: the sizes of the paper's group-size ablation).
-#include "slim_common.cuh"
+#include "slim_sqc_dev.cuh"
 
 #include <cstring>
 
@@ -30,44 +30,6 @@ static int make_group_bits(int N, int K, int g, const uint8_t* bits_host, GroupB
         out->w[j >> 4] |= static_cast<uint32_t>(b - 1) << (2 * (j & 15));
     }
     return SLIM_OK;
-}
-
-// The CPL = GS / 32 consecutive weights of a lane, and its codes (one byte each).
-template <int CPL>
-__device__ __forceinline__ void load_weights(const __half* src, float (&w)[CPL]) {
-    if constexpr (CPL == 1) {
-        w[0] = __half2float(*src);
-    } else if constexpr (CPL == 2) {
-        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(src));
-        w[0] = f.x; w[1] = f.y;
-    } else if constexpr (CPL == 4) {
-        const uint2 raw = *reinterpret_cast<const uint2*>(src);
-        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&raw.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
-        w[0] = a.x; w[1] = a.y; w[2] = b.x; w[3] = b.y;
-    } else {
-#pragma unroll
-        for (int q = 0; q < CPL / 8; ++q) {
-            const uint4 raw = reinterpret_cast<const uint4*>(src)[q];
-            const uint32_t r[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&r[i]));
-                w[8 * q + 2 * i] = v.x; w[8 * q + 2 * i + 1] = v.y;
-            }
-        }
-    }
-}
-template <int CPL>
-__device__ __forceinline__ void store_codes(uint8_t* dst, const uint8_t (&q)[CPL]) {
-    if constexpr (CPL == 1) {
-        dst[0] = q[0];
-    } else if constexpr (CPL == 2) {
-        *reinterpret_cast<uint16_t*>(dst) = static_cast<uint16_t>(q[0] | (q[1] << 8));
-    } else {
-#pragma unroll
-        for (int v = 0; v < CPL / 4; ++v)
-            reinterpret_cast<uint32_t*>(dst)[v] = q[4 * v] | (q[4 * v + 1] << 8) | (q[4 * v + 2] << 16) | (static_cast<uint32_t>(q[4 * v + 3]) << 24);
-    }
 }
 
 // One cluster of kSalCluster blocks per group; block r of the cluster owns the r-th slice of the rows.  A thread owns
@@ -321,19 +283,12 @@ int slim_quantize_minmax_sign1(const void* W, const uint8_t* bits_host, uint8_t*
 }  // extern "C"
 
 // ------------------------------------------------------------------------------------------ SQC
-// Salience-Weighted Quantizer Calibration (Sec. 3.3, Eq. 5; function SQC of Algorithm 2).
-// One warp per (row, group): the group's weights sit in shared memory as fp64, every lane evaluates
-// the candidates tau_i with i = lane, lane + 32, ... one after another, walking the columns in
-// order, so that every loss is the same fp64 sum a sequential program would form.  Every fp64
-// operation is an explicit round-to-nearest intrinsic: nothing may be contracted into an FMA.
+// One warp per (row, group); the search is in slim_sqc_dev.cuh.  Bound: fp32 and min/max instructions, four issue slots per
+// weight and candidate.  A 7B block (202 M weights) took 39.3 ms
+// with every candidate in fp64; a 11008-row group of 128 columns takes 43 to 102 us in the loop of slim_gptq.cu (314 before).
 namespace slim {
 
-constexpr int kSqcWarps = 4;
-
-struct SqcBest {
-    double loss;
-    int idx;
-};
+constexpr int kSqcWarps = 8;
 
 template <int GS>
 __global__ void __launch_bounds__(kSqcWarps * 32) quantize_sqc_kernel(const __half* __restrict__ W, uint8_t* __restrict__ codes,
@@ -341,98 +296,21 @@ __global__ void __launch_bounds__(kSqcWarps * 32) quantize_sqc_kernel(const __ha
                                                                        int* __restrict__ tau_index, int N, int K, double lambda,
                                                                        int n_half, GroupBits gb) {
     constexpr int CPL = GS / 32;
-    __shared__ double sw[kSqcWarps][GS];
+    __shared__ __align__(16) float sw[kSqcWarps][GS];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const long long pair = static_cast<long long>(blockIdx.x) * kSqcWarps + wl;
     const int G = gb.G;
     if (pair >= static_cast<long long>(N) * G) return;
     const int n = static_cast<int>(pair / G), j = static_cast<int>(pair % G);
     const size_t off = static_cast<size_t>(n) * K + GS * j + CPL * lane;
-    float w4[CPL];
-    load_weights<CPL>(W + off, w4);
-    float lo = w4[0], hi = w4[0];
-#pragma unroll
-    for (int i = 1; i < CPL; ++i) { lo = fminf(lo, w4[i]); hi = fmaxf(hi, w4[i]); }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    const double dlo = static_cast<double>(fminf(lo, 0.0f)), dhi = static_cast<double>(fmaxf(hi, 0.0f));
-#pragma unroll
-    for (int i = 0; i < CPL; ++i) sw[wl][CPL * lane + i] = static_cast<double>(w4[i]);
-    __syncwarp();
-    const double* w = sw[wl];
-
-    // 3-sigma mask: mean and population standard deviation, both sums in column order
-    double tot = 0.0;
-#pragma unroll 4
-    for (int k = 0; k < GS; ++k) tot = __dadd_rn(tot, w[k]);
-    const double mu = __ddiv_rn(tot, static_cast<double>(GS));
-    double var = 0.0;
-#pragma unroll 4
-    for (int k = 0; k < GS; ++k) {
-        const double d = __dsub_rn(w[k], mu);
-        var = __dadd_rn(var, __dmul_rn(d, d));
-    }
-    const double sd = __dsqrt_rn(__ddiv_rn(var, static_cast<double>(GS)));
-    const double t_lo = __dsub_rn(mu, __dmul_rn(3.0, sd)), t_hi = __dadd_rn(mu, __dmul_rn(3.0, sd));
-
-    const int b = gb.at(j);
-    const double levels = static_cast<double>((1 << b) - 1);
-    const double tau0 = __dsub_rn(1.0, lambda), step = __ddiv_rn(lambda, static_cast<double>(n_half));
-    const double range = __dsub_rn(dhi, dlo);
-
-    // scale (fp16 bits) and zero point of candidate i
-    auto candidate = [&](int i, double* s_out, double* z_out) -> unsigned short {
-        const double tau = __dadd_rn(tau0, __dmul_rn(static_cast<double>(i), step));
-        unsigned short sbits = double_to_half_bits_rn(__ddiv_rn(__dmul_rn(tau, range), levels));
-        if ((sbits & 0x7fffu) == 0x7c00u) sbits = 0x7bffu;  // beyond fp16 range -> 65504
-        if ((sbits & 0x7fffu) == 0u) sbits = 0x3c00u;       // zero scale -> 1
-        const double s = static_cast<double>(__half2float(__ushort_as_half(sbits)));
-        *s_out = s;
-        *z_out = fmin(fmax(-rint(__ddiv_rn(__dmul_rn(tau, dlo), s)), 0.0), levels) + 0.0;
-        return sbits;
-    };
-
-    SqcBest best{__longlong_as_double(0x7ff0000000000000ll), 0x7fffffff};
-    for (int i = lane; i < 2 * n_half; i += 32) {
-        double s, z;
-        (void)candidate(i, &s, &z);
-        const double inv_s = __ddiv_rn(1.0, s);           // |w / s| < 2^6 here too: see rint_quotient
-        double Ls = 0.0, Lus = 0.0;
-#pragma unroll 2
-        for (int k = 0; k < GS; ++k) {
-            const double wk = w[k];
-            const double q = fmin(fmax(__dadd_rn(rint_quotient(wk, inv_s), z), 0.0), levels);
-            const double e = __dsub_rn(wk, __dmul_rn(s, __dsub_rn(q, z)));
-            const double sq = __dmul_rn(e, e);
-            if (wk < t_lo || wk > t_hi) Ls = __dadd_rn(Ls, sq);
-            else Lus = __dadd_rn(Lus, sq);
-        }
-        const double total = __dadd_rn(Ls, Lus);
-        if (total < best.loss) { best.loss = total; best.idx = i; }   // strict: the first candidate wins ties
-    }
-    // smallest loss over the warp, smallest index among equals
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double ol = __shfl_xor_sync(0xffffffffu, best.loss, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, best.idx, o);
-        if (ol < best.loss || (ol == best.loss && oi < best.idx)) { best.loss = ol; best.idx = oi; }
-    }
-    double s, z;
-    const unsigned short sbits = candidate(best.idx, &s, &z);
-    uint8_t q8[CPL];
-#pragma unroll
-    for (int i = 0; i < CPL; ++i) {
-        const double q = fmin(fmax(__dadd_rn(rint(__ddiv_rn(static_cast<double>(w4[i]), s)), z), 0.0), levels);
-        q8[i] = static_cast<uint8_t>(static_cast<int>(q));
-    }
-    store_codes<CPL>(codes + off, q8);
+    float w[CPL];
+    load_weights<CPL>(W + off, w);
+    const SqcResult<CPL> r = sqc_quantize<GS>(w, sw[wl], gb.at(j), lambda, n_half, lane);
+    store_codes<CPL>(codes + off, r.codes);
     if (lane == 0) {
-        scales[static_cast<size_t>(j) * N + n] = __ushort_as_half(sbits);
-        zeros[static_cast<size_t>(j) * N + n] = __float2half_rn(static_cast<float>(z));
-        if (tau_index != nullptr) tau_index[static_cast<size_t>(j) * N + n] = best.idx;
+        scales[static_cast<size_t>(j) * N + n] = r.s16;
+        zeros[static_cast<size_t>(j) * N + n] = __float2half_rn(r.z);
+        if (tau_index != nullptr) tau_index[static_cast<size_t>(j) * N + n] = r.index;
     }
 }
 
