@@ -12,6 +12,17 @@ namespace slim {
 bool make_x_map(CUtensorMap_st* map, const void* x, int M, int K, int rows);
 
 namespace tc {
+// One lane of a converged warp.  An MMA is issued by a whole warp that runs the same way, with the instruction inside
+// `if (elect())`: its operands then stay in uniform registers and the warp issues one every 9 cycles (N = 16; from N = 32 on the
+// tensor pipe's N / 2 cycles show).  From code that a single lane runs, each operand is moved there first, 48 to 77 cycles.
+__device__ __forceinline__ bool elect() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+    return p != 0;
+}
+// A value that is the same in all lanes, in a uniform register (the reduction instruction writes one): what an issuing warp reads
+// from memory goes through this, or the compiler has to take everything that depends on it for different per lane.
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __reduce_or_sync(0xffffffffu, v); }
 // One warp executes these together.
 __device__ __forceinline__ void alloc(uint32_t smem_dst, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
