@@ -2,23 +2,28 @@
 
 Argument marshalling only: every function checks dtypes/devices, takes raw device
 pointers from torch tensors and the current CUDA stream, and calls the entry point
-of the same name.  There is no fallback: if the CUDA library has not been built
-the first call raises.
+of the same name; for the linear layers and the layer sets, which a decode loop calls
+per layer, the host module (csrc/slim_host.cpp) does that without the interpreter.
+There is no fallback: if the CUDA library has not been built the first call raises.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import numpy as np
 import torch
 
-from .build import LIB_PATH
+from .build import HOST_PATH, LIB_PATH
 
 GROUP = 128
 GEMV_MAX_M = 16
 
 _lib = None
+_host = None             # the host module, and the addresses of the entry points that it calls
+_entry = {}
 
 
 class SlimError(RuntimeError):
@@ -80,6 +85,22 @@ def lib():
             fn.argtypes = args
         _lib = L
     return _lib
+
+
+def host():
+    """Loads lib/slim_host.so (built with the CUDA library)."""
+    global _host
+    if _host is None:
+        L = lib()
+        if not os.path.exists(HOST_PATH):
+            raise RuntimeError(f"host module not built: {HOST_PATH} is missing; run `python -m paper_2405_14917_b200.build`")
+        loader = importlib.machinery.ExtensionFileLoader("slim_host", HOST_PATH)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("slim_host", loader))
+        loader.exec_module(module)
+        for name in ("slim_mpq_gemv", "slim_mpq_gemm", "slim_mpq_gemv_set"):
+            _entry[name] = ctypes.cast(getattr(L, name), ctypes.c_void_p).value
+        _host = module
+    return _host
 
 
 def _check(fn: str, status: int):
@@ -180,6 +201,12 @@ def dequant(packed: torch.Tensor, bits, scales: torch.Tensor, zeros: torch.Tenso
 
 
 def _linear(fn_name: str, x, packed, bits, scales, zeros, N, workspace, out, g: int = GROUP):
+    y = (_host or host()).linear(_entry[fn_name], x, packed, bits, scales, zeros, N, workspace, out, g)
+    if y is not None:
+        if type(y) is int:
+            _check(fn_name, y)
+        return y
+    # not the plain call: convert what can be converted, raise for the rest
     b = _bits(bits)
     M, K = x.shape
     if out is None:
@@ -422,8 +449,12 @@ class LayerSet:
 
     def run(self) -> None:
         """Enqueues the set on the current stream: y of every entry is overwritten."""
-        _check("slim_mpq_gemv_set", lib().slim_mpq_gemv_set(ctypes.addressof(self._info), self.plan.data_ptr(), self.workspace.data_ptr(),
-                                                          self.workspace.numel(), _stream(self.plan)))
+        status = (_host or host()).run_set(_entry["slim_mpq_gemv_set"], ctypes.addressof(self._info), self.plan, self.workspace)
+        if status is None:                                 # a caller's own buffers in place of the set's
+            status = lib().slim_mpq_gemv_set(ctypes.addressof(self._info), self.plan.data_ptr(), self.workspace.data_ptr(),
+                                             self.workspace.numel(), _stream(self.plan))
+        if status:
+            _check("slim_mpq_gemv_set", status)
 
     def check(self) -> None:
         workspace_status(self.workspace)

@@ -1,16 +1,19 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (no JIT, no torch extension)."""
+"""Builds the CUDA library (nvcc, sm_100a) and the binding's host module (g++, torch headers) in-tree; no JIT."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB_DIR = os.path.join(_HERE, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libslim_b200.so")
+HOST_SRC = os.path.join(CSRC, "slim_host.cpp")
+HOST_PATH = os.path.join(LIB_DIR, "slim_host.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xptxas=-v"]
@@ -28,8 +31,28 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_host(force: bool = False, verbose: bool = False) -> str:
+    """Compile the host module of the binding (csrc/slim_host.cpp) into lib/slim_host.so.  Returns its path."""
+    if not force and os.path.exists(HOST_PATH) and os.path.getmtime(HOST_PATH) >= os.path.getmtime(HOST_SRC):
+        return HOST_PATH
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    os.makedirs(LIB_DIR, exist_ok=True)
+    torch_lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += [f"-isystem{d}" for d in include_paths(device_type="cuda")] + ["-I" + sysconfig.get_paths()["include"], HOST_SRC, "-o", HOST_PATH]
+    cmd += ["-L" + torch_lib, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath," + torch_lib]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode != 0:
+        sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+    if r.returncode != 0:
+        raise RuntimeError(f"{cmd[0]} failed on {HOST_SRC}")
+    return HOST_PATH
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into lib/libslim_b200.so.  Returns the library path."""
+    """Compile every .cu under csrc/ into lib/libslim_b200.so, and the host module.  Returns the library path."""
+    build_host(force, verbose)
     if not force and not _stale():
         return LIB_PATH
     os.makedirs(LIB_DIR, exist_ok=True)
