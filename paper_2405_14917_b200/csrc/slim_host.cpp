@@ -4,7 +4,7 @@
 // One token through a 4096 x 4096 layer takes 5.7 us on the device.  Checked and marshalled in Python (six tensors, a
 // numpy bit map, the stream, an output, a ctypes call of thirteen arguments) the call took 15 us of the host, so the
 // device waited for it; here the tensors are read without the interpreter, and the calls of a loop follow each other every
-6.0 us (10.2 instead of 16.4 at a group size of 64).  A layer's very first call: 37 -> 24 us.
+// 6.0 us (10.2 instead of 16.4 at a group size of 64).  A layer's very first call: 37 -> 24 us.
 //
 // Nothing is decided here.  A call that is not the plain one (another dtype or layout, a tensor subclass, a bit map that
 // is not a one-dimensional uint8 buffer, ...) returns None before anything has been enqueued and binding.py takes its
