@@ -250,7 +250,7 @@ typedef struct slim_gemv_set_info {
     int resident_pairs;    /* > 0: a small single-token set that runs as ONE launch with every CTA resident at once (the
                               whole K of 2 x resident_pairs row tiles per CTA, no ring, no staging kernel); the ring
                               fields above are then unused.  0: the persistent ring */
-    int resident_cluster;  /* CTAs that share the staging of x in that launch (8 or 4) */
+    int resident_cluster;  /* the CTAs of each layer in that launch are padded to a multiple of this */
     size_t plan_bytes;
     size_t workspace_bytes;
     size_t resident_smem;  /* dynamic shared memory of that launch */

@@ -10,14 +10,18 @@
 //  * warp w owns the groups w, w + 16, ... of the CTA's tiles: it brings their slices with one cp.async.bulk per
 //    group onto a barrier of its own, their scales and zeros with 16-byte cp.async, multiplies and folds.  Warps
 //    meet at the end to add their sixteen partial sums per row in warp order (deterministic).
-//  * the digit form of x is the same for every CTA and costs a warp about as much as a group's products, so the
-//    CTAs of a cluster of eight share it: CTA r stages the groups r, r + 8, ... (one per warp) and writes each
-//    record into the shared memory of all eight through distributed shared memory; one cluster barrier follows.
+//  * every CTA makes the digit form of all of x itself, four K-tiles per warp and pass (stage_groups_i8): about 1900 of the
+//    5000 cycles between the release of a CTA by the kernel ahead and its end at K = 4096.  Eight CTAs of a cluster that
+//    each staged a share for the others took 4600 cycles to the same point: the stores into the other CTAs and the cluster
+//    barrier cost more than the work they saved, and whole clusters left up to 12 SMs idle.  One token, device time per
+//    layer of a chain: 4096 x 4096 5.65 -> 4.57 us, q/k/v 7.2 -> 5.75, gate/up 14.8 -> 8.5, 4096 x 11008 9.1 -> 7.1; four
+//    LLaMA-7B blocks in decoder order 155 -> 113.  (Cutting K over the CTAs of a cluster, which divides the staging,
+//    measured 5.5 at 4096 x 4096: the exchange of the sums costs 3000 cycles.)
 //  * everything that does not depend on x (the slices, scales, zeros) is requested BEFORE griddepcontrol.wait, and
 //    the dependents are released right after, so with programmatic dependent launch the loads of layer l + 1 are in
 //    flight while layer l computes.
 //  * a set of a few single-token layers (q/k/v, gate/up) whose CTAs are all resident at once is ONE launch of the
-//    same body: every layer owns whole clusters, a CTA reads its layer's descriptor from the plan buffer first.
+//    same body: every layer owns a range of CTAs, a CTA reads its layer's descriptor from the plan buffer first.
 //
 // Every wait on a barrier in memory is bounded and reports through the workspace status word.
 #include "slim_common.cuh"
@@ -31,11 +35,12 @@ namespace slim {
 
 constexpr int kOneWarps = 16;
 constexpr int kOneThreads = 32 * kOneWarps;
-constexpr int kOneCluster = 8;                          // CTAs that share the staging of x (4 where eight do not all fit)
-constexpr int kOneMaxPairs = 4;                         // tile pairs per CTA
+constexpr int kOneSetPad = 4;                           // the CTAs of a layer of a set are a multiple of this
+constexpr int kOneMaxPairs = 5;                         // tile pairs per CTA
 constexpr uint32_t kOneOffAbort = 8 * kOneWarps;        // after the warps' barriers
-constexpr uint32_t kOneOffXs = 256;                     // per warp: 128 ints of scratch for the digit staging, later its partial sums
-constexpr uint32_t kOneOffDesc = kOneOffXs + kOneWarps * 512;   // the layer's descriptor, when it comes from the plan buffer of a set
+constexpr uint32_t kOneOffSums = 256;                   // per warp: its partial sums
+constexpr uint32_t kOneSumsWarp = 2 * kOneMaxPairs * 64;
+constexpr uint32_t kOneOffDesc = kOneOffSums + kOneWarps * kOneSumsWarp;   // the layer's descriptor, when it comes from the plan buffer of a set
 constexpr uint32_t kOneOffS = kOneOffDesc + 1408;
 
 struct OneParams {
@@ -54,12 +59,6 @@ struct OneParams {
 };
 static_assert(sizeof(OneParams) % 16 == 0 && sizeof(OneParams) <= kOneOffS - kOneOffDesc, "descriptors are copied in 16-byte pieces");
 
-__device__ __forceinline__ void st_cluster_u32x4(uint32_t local_addr, uint32_t rank, uint4 v) {
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_addr), "r"(rank));
-    asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(remote), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
 // One K-tile of B bits for the PAIRS tile pairs of the CTA: integer MMAs on byte-masked words, then the fold
 // acc += s (D 2^(-S-Pc) - z sum_x) per (row, K-tile); lane pair c >> 1 folds tile c >> 1 of every pair.
 template <int B, int PAIRS>
@@ -74,7 +73,7 @@ __device__ __forceinline__ void one_group(const OneParams& p, uint32_t wj, uint3
     const uint2 tkw = lds64(rec);
     const float sum_x = __uint_as_float(tkw.x), e = __uint_as_float(tkw.y);
     const float ka = ma * e, kb = mb * e;
-    const uint32_t xs_lane = rec + 128 + ((gq & 3) * 4 + c) * 8;
+    const uint32_t xs_lane = rec + staged_header_bytes(2) + ((gq & 3) * 4 + c) * 8;
 #pragma unroll
     for (int tp = 0; tp < PAIRS; ++tp) {
         const uint32_t item0 = wj + 8u * lane + static_cast<uint32_t>(2 * tp) * (256u * B);
@@ -133,6 +132,16 @@ __device__ __forceinline__ void one_group(const OneParams& p, uint32_t wj, uint3
     }
 }
 
+// Barriers and the abort flag; a __syncthreads follows before one_body.
+__device__ __forceinline__ void one_init(uint8_t* smem) {
+    if ((threadIdx.x & 31) == 0) {
+        sb::init(smem_u32(smem) + 8u * (threadIdx.x >> 5), 1);
+        if (threadIdx.x == 0) *reinterpret_cast<volatile int*>(smem + kOneOffAbort) = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+}
+
 // The work of CTA `bid` of layer p (see the head of the file).
 template <int PAIRS>
 __device__ __forceinline__ void one_body(const OneParams& p, int bid, uint8_t* status, uint8_t* smem) {
@@ -142,20 +151,11 @@ __device__ __forceinline__ void one_body(const OneParams& p, int bid, uint8_t* s
     volatile int* abort = reinterpret_cast<volatile int*>(smem + kOneOffAbort);
     const uint32_t bar = sbase + 8u * warp;
     const int tile0 = TPC * bid;
-    const int tiles_here = max(min(TPC, (p.N >> 4) - tile0), 0);  // 0: a CTA that only fills up its cluster
+    const int tiles_here = max(min(TPC, (p.N >> 4) - tile0), 0);  // 0: a CTA that only fills up its layer's range
     const int ng = (p.G - warp + kOneWarps - 1) / kOneWarps;      // this warp's K-tiles: warp, warp + 16, ...
-    const uint32_t rank = cluster_ctarank();
-    uint32_t nrank;                                        // CTAs of the cluster: 8 or 4
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nrank));
+    if (tiles_here == 0) return;
 
     // ---- requests that do not depend on x
-    if (lane == 0) {
-        sb::init(bar, 1);
-        if (warp == 0) *abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();                                       // the abort flag is clear before any warp can poll it
     {
         const int j = warp + kOneWarps * lane;             // lane i brings the slices of the warp's i-th K-tile
         const uint32_t b = lane < ng ? p.bits[j] : 0u;
@@ -167,39 +167,32 @@ __device__ __forceinline__ void one_body(const OneParams& p, int bid, uint8_t* s
             sb::bulk_g2s(sbase + p.off_w + static_cast<uint32_t>(TPC) * 256u * p.prefix[j],
                          p.packed + 16ull * p.N * p.prefix[j] + static_cast<size_t>(tile0) * 256 * b, bytes, bar);
         // scales and zeros of the warp's K-tiles, 16 bytes (8 rows) at a time
-        const int chunks = 2 * tiles_here;
-        for (int i = lane; i < ng * chunks * 2; i += 32) {
-            const int which = i & 1, q = i >> 1, gi = q / chunks, ch = q - gi * chunks;
+        constexpr int kChunks = 4 * TPC;                   // per K-tile: 2 TPC of the scales, 2 TPC of the zeros
+        for (int i = lane; i < ng * kChunks; i += 32) {
+            const int gi = i / kChunks, r = i - gi * kChunks, which = r & 1, ch = r >> 1;
             const int jj = warp + kOneWarps * gi;
             const __half* src = (which ? p.zeros : p.scales) + static_cast<size_t>(jj >> p.gshift) * p.N + 16 * tile0 + 8 * ch;
-            cp_async16(sbase + (which ? p.off_z : kOneOffS) + static_cast<uint32_t>(jj) * (32u * TPC) + 16u * ch, src);
+            if (ch < 2 * tiles_here) cp_async16(sbase + (which ? p.off_z : kOneOffS) + static_cast<uint32_t>(jj) * (32u * TPC) + 16u * ch, src);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
     pdl_launch_dependents();
     pdl_wait();                                            // x may be the output of the kernel before
 
-    // ---- the activations as digits: this CTA's share of the K-tiles, written into every CTA of the cluster
-    int* Xs = reinterpret_cast<int*>(smem + kOneOffXs + 512 * warp);
-    for (int j = static_cast<int>(rank + nrank * warp); j < p.G; j += static_cast<int>(nrank) * kOneWarps) {
-        const uint32_t off = p.off_x + static_cast<uint32_t>(staged_group_offset(j, p.pre3[j], 2));
-        stage_group_i8(p.x + SLIM_GROUP * j, smem + off, p.bits[j], lane, Xs);
-        __syncwarp();
-        const int pieces = (128 + 512 * slice_count(p.bits[j])) / 16;
-        for (int i = lane; i < pieces; i += 32) {
-            const uint4 v = lds128(sbase + off + 16u * i);
-            for (uint32_t r = 0; r < nrank; ++r)
-                if (r != rank) st_cluster_u32x4(sbase + off + 16u * i, r, v);
-        }
+    // ---- the activations as digits, eight lanes per K-tile
+    for (int q = 4 * warp; q < p.G; q += 4 * kOneWarps) {
+        const int j = q + (lane >> 3), jj = min(j, p.G - 1);
+        const uint32_t off = p.off_x + static_cast<uint32_t>(staged_group_offset(jj, p.pre3[jj], 2));
+        stage_groups_i8(p.x + SLIM_GROUP * jj, j < p.G ? smem + off : nullptr, p.bits[jj], lane);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    __syncthreads();
 
     float acc[PAIRS][2];
 #pragma unroll
     for (int tp = 0; tp < PAIRS; ++tp) acc[tp][0] = acc[tp][1] = 0.f;
     const bool ok = __all_sync(0xffffffffu, sb::wait(bar, 0, abort));
-    if (ok && tiles_here > 0) {
+    if (ok) {
         for (int gi = 0; gi < ng; ++gi) {
             const int j = warp + kOneWarps * gi;
             const uint32_t wj = sbase + p.off_w + static_cast<uint32_t>(TPC) * 256u * p.prefix[j];
@@ -216,7 +209,7 @@ __device__ __forceinline__ void one_body(const OneParams& p, int bid, uint8_t* s
     }
     // ---- the warps' partial sums, added in warp order
     __syncwarp();
-    float* mine = reinterpret_cast<float*>(smem + kOneOffXs + 512 * warp);      // [TPC * 16] floats, the scratch is free now
+    float* mine = reinterpret_cast<float*>(smem + kOneOffSums + kOneSumsWarp * warp);      // [TPC * 16] floats
     {
         const int gq = lane >> 2, c = lane & 3;
         if ((c & 1) == 0) {
@@ -231,11 +224,11 @@ __device__ __forceinline__ void one_body(const OneParams& p, int bid, uint8_t* s
         return;
     }
     if (tid < 8 * tiles_here) {                            // a pair of rows per thread
-        const float* all = reinterpret_cast<const float*>(smem + kOneOffXs);
+        const float* all = reinterpret_cast<const float*>(smem + kOneOffSums);
         float2 sum = *reinterpret_cast<const float2*>(all + 2 * tid);
 #pragma unroll
         for (int w = 1; w < kOneWarps; ++w) {
-            const float2 v = *reinterpret_cast<const float2*>(all + 128 * w + 2 * tid);
+            const float2 v = *reinterpret_cast<const float2*>(all + kOneSumsWarp / 4 * w + 2 * tid);
             sum.x += v.x;
             sum.y += v.y;
         }
@@ -246,6 +239,8 @@ __device__ __forceinline__ void one_body(const OneParams& p, int bid, uint8_t* s
 template <int PAIRS>
 __global__ void __launch_bounds__(kOneThreads, PAIRS == 1 ? 2 : 1) gemv_one_kernel(const __grid_constant__ OneParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
+    one_init(smem);
+    __syncthreads();
     one_body<PAIRS>(p, static_cast<int>(blockIdx.x), p.ws, smem);
 }
 
@@ -256,8 +251,12 @@ __global__ void __launch_bounds__(kOneThreads, PAIRS == 1 ? 2 : 1) gemv_one_set_
                                                                                      const int* __restrict__ cta0, int n_layers,
                                                                                      uint8_t* status) {
     extern __shared__ __align__(128) uint8_t smem[];
-    int l = 0;
-    while (l + 1 < n_layers && cta0[l + 1] <= static_cast<int>(blockIdx.x)) ++l;
+    one_init(smem);
+    // The layers that begin at or below this CTA, counted by the whole warp: one round of loads, not one per layer.
+    const int lane = threadIdx.x & 31;
+    int l = -1;
+    for (int k = 0; k < n_layers; k += 32)
+        l += __popc(__ballot_sync(0xffffffffu, k + lane < n_layers && cta0[k + lane] <= static_cast<int>(blockIdx.x)));
     const uint4* src = reinterpret_cast<const uint4*>(layers + l);
     uint4* dst = reinterpret_cast<uint4*>(smem + kOneOffDesc);
     for (int i = threadIdx.x; i < static_cast<int>(sizeof(OneParams) / 16); i += kOneThreads) dst[i] = src[i];
@@ -266,7 +265,7 @@ __global__ void __launch_bounds__(kOneThreads, PAIRS == 1 ? 2 : 1) gemv_one_set_
 }
 
 template <int PAIRS>
-static cudaError_t launch_one(const OneParams& prm, int grid, int cluster, size_t smem, cudaStream_t stream) {
+static cudaError_t launch_one(const OneParams& prm, int grid, size_t smem, cudaStream_t stream) {
     static std::atomic<bool> attr_set[64];    // zero-initialised; set-up is idempotent, so a race repeats it harmlessly
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -276,58 +275,36 @@ static cudaError_t launch_one(const OneParams& prm, int grid, int cluster, size_
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(static_cast<unsigned>(grid), 1, 1);
-    cfg.blockDim = dim3(kOneThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemv_one_kernel<PAIRS>, prm);
+    PdlLaunch l(static_cast<unsigned>(grid), kOneThreads, smem, stream);
+    return cudaLaunchKernelEx(&l.cfg, gemv_one_kernel<PAIRS>, prm);
 }
 
-// Clusters of the kernel that can be resident at once with `smem` bytes of dynamic shared memory (0 on failure).
+// CTAs of the kernel that can be resident at once with `smem` bytes of dynamic shared memory (0 on failure).
 template <int PAIRS>
-static int one_max_clusters(size_t smem, int cluster) {
-    if (cudaFuncSetAttribute(gemv_one_kernel<PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024) != cudaSuccess) return 0;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(static_cast<unsigned>(cluster), 1, 1);
-    cfg.blockDim = dim3(kOneThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(cluster);
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+static int one_max_resident(size_t smem, int sms) {
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemv_one_kernel<PAIRS>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
-    return n;
+    if (cudaFuncSetAttribute(gemv_one_kernel<PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gemv_one_kernel<PAIRS>, kOneThreads, smem) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return n * sms;
 }
 
 // The same, asked once per device for the two sizes that matter: a CTA small enough for two per SM, and the largest.
 constexpr size_t kOneHalfSm = 112 * 1024;
-static int one_clusters_cached(int pairs, size_t smem, int cluster) {
-    static std::atomic<int> cache[64][kOneMaxPairs][2][2];  // 0: not asked yet; idempotent, so a race repeats the query
-    int dev = 0;
+static int one_resident_cached(int pairs, size_t smem) {
+    static std::atomic<int> cache[64][kOneMaxPairs][2];     // 0: not asked yet; idempotent, so a race repeats the query
+    int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    const int cls = smem <= kOneHalfSm ? 0 : 1, ci = cluster == kOneCluster ? 0 : 1;
-    int v = cache[dev][pairs - 1][cls][ci].load();
+    const int cls = smem <= kOneHalfSm ? 0 : 1;
+    int v = cache[dev][pairs - 1][cls].load();
     if (v == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
         const size_t ask = cls == 0 ? kOneHalfSm : 224 * 1024;
-        v = pairs == 1 ? one_max_clusters<1>(ask, cluster) : pairs == 2 ? one_max_clusters<2>(ask, cluster)
-          : pairs == 3 ? one_max_clusters<3>(ask, cluster) : one_max_clusters<4>(ask, cluster);
-        cache[dev][pairs - 1][cls][ci].store(v > 0 ? v : -1);
+        v = pairs == 1 ? one_max_resident<1>(ask, sms) : pairs == 2 ? one_max_resident<2>(ask, sms)
+          : pairs == 3 ? one_max_resident<3>(ask, sms) : pairs == 4 ? one_max_resident<4>(ask, sms) : one_max_resident<5>(ask, sms);
+        cache[dev][pairs - 1][cls].store(v > 0 ? v : -1);
     }
     return v > 0 ? v : 0;
 }
@@ -378,27 +355,25 @@ int gemv_one(const void* x, const void* packed, const GroupTable& gt, const void
     (void)K;
     if (M != 1 || N <= 0 || gt.G < 1) return 1;
     const int tiles = N >> 4;
-    int pairs = 0, cluster = 0, best_waves = 1 << 30;
+    int pairs = 0, best_waves = 1 << 30;
     OneShape shape;
-    for (int pr = 1; pr <= kOneMaxPairs; ++pr) {
+    for (int pr = 1; pr <= kOneMaxPairs && best_waves > 1; ++pr) {
         OneShape sh;
         if (!one_shape(gt, pr, &sh)) break;
-        for (int cs = kOneCluster; cs >= 4; cs /= 2) {                         // eight CTAs share the staging, or four
-            const int grid = pad_to((tiles + 2 * pr - 1) / (2 * pr), cs), resident = one_clusters_cached(pr, sh.smem, cs) * cs;
-            if (resident <= 0) continue;
-            const int waves = (grid + resident - 1) / resident;
-            if (waves < best_waves) { best_waves = waves; pairs = pr; cluster = cs; shape = sh; }
-        }
-        if (best_waves == 1) break;
+        const int grid = (tiles + 2 * pr - 1) / (2 * pr), resident = one_resident_cached(pr, sh.smem);
+        if (resident <= 0) continue;
+        const int waves = (grid + resident - 1) / resident;
+        if (waves < best_waves) { best_waves = waves; pairs = pr; shape = sh; }
     }
     if (pairs == 0) return 1;
     OneParams prm;
     one_fill(&prm, x, packed, scales, zeros, y, workspace, N, gt, shape);
-    const int grid = pad_to((tiles + 2 * pairs - 1) / (2 * pairs), cluster);
-    const cudaError_t e = pairs == 1 ? launch_one<1>(prm, grid, cluster, shape.smem, stream)
-                        : pairs == 2 ? launch_one<2>(prm, grid, cluster, shape.smem, stream)
-                        : pairs == 3 ? launch_one<3>(prm, grid, cluster, shape.smem, stream)
-                                     : launch_one<4>(prm, grid, cluster, shape.smem, stream);
+    const int grid = (tiles + 2 * pairs - 1) / (2 * pairs);
+    const cudaError_t e = pairs == 1 ? launch_one<1>(prm, grid, shape.smem, stream)
+                        : pairs == 2 ? launch_one<2>(prm, grid, shape.smem, stream)
+                        : pairs == 3 ? launch_one<3>(prm, grid, shape.smem, stream)
+                        : pairs == 4 ? launch_one<4>(prm, grid, shape.smem, stream)
+                                     : launch_one<5>(prm, grid, shape.smem, stream);
     SLIM_CUDA_TRY(e);
     return SLIM_OK;
 }
@@ -419,23 +394,9 @@ static cudaError_t launch_one_set(const OneSetPlan& pl, const void* plan, int n_
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(static_cast<unsigned>(pl.grid), 1, 1);
-    cfg.blockDim = dim3(kOneThreads, 1, 1);
-    cfg.dynamicSmemBytes = pl.smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = static_cast<unsigned>(pl.cluster);
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    PdlLaunch launch(static_cast<unsigned>(pl.grid), kOneThreads, pl.smem, stream);
     const uint8_t* base = static_cast<const uint8_t*>(plan);
-    return cudaLaunchKernelEx(&cfg, gemv_one_set_kernel<PAIRS>, reinterpret_cast<const OneParams*>(base + kOneSetPlanHeader),
+    return cudaLaunchKernelEx(&launch.cfg, gemv_one_set_kernel<PAIRS>, reinterpret_cast<const OneParams*>(base + kOneSetPlanHeader),
                               reinterpret_cast<const int*>(base), n_layers, static_cast<uint8_t*>(workspace));
 }
 
@@ -461,33 +422,32 @@ int one_set_plan(const slim_layer* layers, int n_layers, int g, void* plan, size
             smem = smem > sh[l].smem ? smem : sh[l].smem;
         }
         if (!fits) { if (waves == 1) break; else continue; }
-        for (int cs = kOneCluster; cs >= 4; cs /= 2) {
-            int cta0[kOneSetMaxLayers + 1];
-            cta0[0] = 0;
-            for (int l = 0; l < n_layers; ++l) cta0[l + 1] = cta0[l] + pad_to(((layers[l].N >> 4) + 2 * pr - 1) / (2 * pr), cs);
-            if (cta0[n_layers] > waves * one_clusters_cached(pr, smem, cs) * cs) continue;
-            // taken: descriptors and CTA ranges into the plan buffer (pageable sources are staged before the copies return)
-            std::vector<OneParams> prm(static_cast<size_t>(n_layers));
-            for (int l = 0; l < n_layers; ++l)
-                one_fill(&prm[l], layers[l].x, layers[l].packed, layers[l].scales, layers[l].zeros, layers[l].y, nullptr, layers[l].N, gt[l], sh[l]);
-            uint8_t* base = static_cast<uint8_t*>(plan);
-            SLIM_CUDA_TRY(cudaMemcpyAsync(base, cta0, static_cast<size_t>(n_layers + 1) * sizeof(int), cudaMemcpyHostToDevice, stream));
-            SLIM_CUDA_TRY(cudaMemcpyAsync(base + kOneSetPlanHeader, prm.data(), static_cast<size_t>(n_layers) * sizeof(OneParams), cudaMemcpyHostToDevice, stream));
-            out->pairs = pr; out->cluster = cs; out->grid = cta0[n_layers]; out->smem = smem;
-            return SLIM_OK;
-        }
+        int cta0[kOneSetMaxLayers + 1];
+        cta0[0] = 0;
+        for (int l = 0; l < n_layers; ++l) cta0[l + 1] = cta0[l] + pad_to(((layers[l].N >> 4) + 2 * pr - 1) / (2 * pr), kOneSetPad);
+        if (cta0[n_layers] > waves * one_resident_cached(pr, smem)) continue;
+        // taken: descriptors and CTA ranges into the plan buffer (pageable sources are staged before the copies return)
+        std::vector<OneParams> prm(static_cast<size_t>(n_layers));
+        for (int l = 0; l < n_layers; ++l)
+            one_fill(&prm[l], layers[l].x, layers[l].packed, layers[l].scales, layers[l].zeros, layers[l].y, nullptr, layers[l].N, gt[l], sh[l]);
+        uint8_t* base = static_cast<uint8_t*>(plan);
+        SLIM_CUDA_TRY(cudaMemcpyAsync(base, cta0, static_cast<size_t>(n_layers + 1) * sizeof(int), cudaMemcpyHostToDevice, stream));
+        SLIM_CUDA_TRY(cudaMemcpyAsync(base + kOneSetPlanHeader, prm.data(), static_cast<size_t>(n_layers) * sizeof(OneParams), cudaMemcpyHostToDevice, stream));
+        out->pairs = pr; out->cluster = kOneSetPad; out->grid = cta0[n_layers]; out->smem = smem;
+        return SLIM_OK;
     }
     return 1;
 }
 
 int one_set_launch(const OneSetPlan& pl, const void* plan, int n_layers, void* workspace, cudaStream_t stream) {
-    if (pl.pairs < 1 || pl.pairs > kOneMaxPairs || (pl.cluster != 4 && pl.cluster != kOneCluster) || pl.grid < pl.cluster ||
+    if (pl.pairs < 1 || pl.pairs > kOneMaxPairs || pl.cluster != kOneSetPad || pl.grid < pl.cluster ||
         pl.grid % pl.cluster != 0 || pl.smem > 224 * 1024 || n_layers < 1 || n_layers > kOneSetMaxLayers)
         return SLIM_ERR_INVALID_ARG;
     const cudaError_t e = pl.pairs == 1 ? launch_one_set<1>(pl, plan, n_layers, workspace, stream)
                         : pl.pairs == 2 ? launch_one_set<2>(pl, plan, n_layers, workspace, stream)
                         : pl.pairs == 3 ? launch_one_set<3>(pl, plan, n_layers, workspace, stream)
-                                        : launch_one_set<4>(pl, plan, n_layers, workspace, stream);
+                        : pl.pairs == 4 ? launch_one_set<4>(pl, plan, n_layers, workspace, stream)
+                                        : launch_one_set<5>(pl, plan, n_layers, workspace, stream);
     SLIM_CUDA_TRY(e);
     return SLIM_OK;
 }

@@ -50,7 +50,7 @@ constexpr int kSetMaxTokens = 64;                      // tokens of a layer in a
 constexpr int kSlotOffS = 16;
 __host__ __device__ constexpr int slot_off_z(int tpi) { return kSlotOffS + 32 * tpi; }
 __host__ __device__ constexpr int slot_off_e(int tpi) { return kSlotOffS + 64 * tpi; }
-__host__ __device__ constexpr int slot_off_x(int tpi, int mp) { return slot_off_e(tpi) + (mp > 16 ? 8 * mp : 128); }
+__host__ __device__ constexpr int slot_off_x(int tpi, int mp) { return slot_off_e(tpi) + staged_header_bytes(mp); }
 __host__ __device__ constexpr int slot_off_w(int tpi, int mp) { return slot_off_x(tpi, mp) + 2 * 256 * mp; }
 
 // Device-side description of one layer (lives in the plan buffer).
@@ -68,7 +68,7 @@ struct SetLayer {
     int task0;             // first (token, group) staging task of the layer
     int MP;                // 256-byte pieces per slice in the staged layout: 8 or 16 = tokens of the f16 fragments for the
                            // whole set (absent tokens are staged as zeros, so the kernel reads without a test); 2 if every
-                           // layer of the set has one token: the 8-bit digit form (stage_group_i8)
+                           // layer of the set has one token: the 8-bit digit form (stage_groups_i8)
     uint16_t prefix[SLIM_MAX_GROUPS + 1];
     uint16_t pre3[SLIM_MAX_GROUPS + 1];   // 3-bit groups (two slices) before group j
     uint8_t bits[SLIM_MAX_GROUPS];
@@ -115,15 +115,17 @@ __device__ __forceinline__ void stage_clear_counters(uint8_t* ws, int n_counters
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_counters; i += gridDim.x * blockDim.x) cnt[i] = 0u;
 }
 
-// Staging task `pi` of layer L (one warp): token pi / G, group pi % G.
+// Staging tasks of a single-token set: task `pi` (a group) of layer L by the eight lanes that have it; all lanes of the
+// warp call it together, those without a task with `live` false and any other task.
+__device__ __forceinline__ void stage_task_one(const SetLayer& L, uint8_t* ws, int pi, int lane, bool live) {
+    uint8_t* grp = ws + L.x_off + staged_group_offset(pi, L.pre3[pi], 2);
+    stage_groups_i8(L.x + pi * SLIM_GROUP, live ? grp : nullptr, L.bits[pi], lane);
+}
+
+// Staging task `pi` of layer L (one warp) of any other set: token pi / G, group pi % G.
 __device__ __forceinline__ void stage_task(const SetLayer& L, uint8_t* ws, int pi, int lane) {
     const int m = pi / L.G, j = pi - m * L.G;        // m < MP
     uint8_t* grp = ws + L.x_off + staged_group_offset(j, L.pre3[j], L.MP);
-    if (L.MP == 2) {                                     // single-token set: the 8-bit form, one task per group
-        __shared__ int Xs[8][SLIM_GROUP];
-        stage_group_i8(L.x + j * SLIM_GROUP, grp, L.bits[j], lane, Xs[threadIdx.x >> 5]);
-        return;
-    }
     float2* sxe = reinterpret_cast<float2*>(grp);
     if (m < L.M) {
         const float2 r = stage_group(L.x + static_cast<size_t>(m) * L.K + j * SLIM_GROUP, grp + staged_header_bytes(L.MP), L.bits[j], m, L.MP, lane);
@@ -139,14 +141,16 @@ __device__ __forceinline__ void stage_task(const SetLayer& L, uint8_t* ws, int p
             if (t >= L.M) sxe[t] = make_float2(0.f, 1.f);                          // absent tokens read 0
 }
 
-// One warp per (layer, token, group): fragments and sums of the whole set, once.
+// One warp per (layer, token, group), or eight lanes per (layer, group) if every layer has ONE token: fragments and sums
+// of the whole set, once.
+template <bool ONE>
 __global__ void __launch_bounds__(256) gemv_set_stage_kernel(const SetLayer* __restrict__ layers, uint8_t* ws, int n_layers, int n_tasks,
                                                              int n_counters) {
     pdl_wait();                       // x may be the output of the kernel before; the workspace may still be read by it
     pdl_launch_dependents();
     stage_clear_counters(ws, n_counters);
     const int lane = threadIdx.x & 31;
-    const int task = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int task = ONE ? blockIdx.x * 32 + (threadIdx.x >> 3) : blockIdx.x * 8 + (threadIdx.x >> 5);
     // The layer of a task is the last one whose first task is not above it.  A search through the descriptors is a
     // chain of dependent loads from global memory (eight for the 224 layers of a 7B sweep, most of this kernel's time),
     // so a set of up to kStageTable layers first puts their first tasks into shared memory, all loads in flight at once.
@@ -157,13 +161,19 @@ __global__ void __launch_bounds__(256) gemv_set_stage_kernel(const SetLayer* __r
         for (int l = threadIdx.x; l < n_layers; l += blockDim.x) first_task[l] = layers[l].task0;
         __syncthreads();
     }
-    if (task >= n_tasks) return;
+    if (!ONE && task >= n_tasks) return;
     int lo = 0, hi = n_layers - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if ((table ? first_task[mid] : layers[mid].task0) <= task) lo = mid; else hi = mid - 1;
     }
-    stage_task(layers[lo], ws, task - (table ? first_task[lo] : layers[lo].task0), lane);
+    const int pi = task - (table ? first_task[lo] : layers[lo].task0);
+    if constexpr (ONE) {
+        __syncwarp();
+        stage_task_one(layers[lo], ws, task < n_tasks ? pi : 0, lane, task < n_tasks);
+    } else {
+        stage_task(layers[lo], ws, pi, lane);
+    }
 }
 
 // D = A * B with a zero accumulator input: starts an accumulation chain without clearing registers first.
@@ -213,7 +223,7 @@ __device__ __noinline__ bool wait_full_slow(uint32_t bar, uint32_t parity, volat
     return __all_sync(0xffffffffu, sb::wait(bar, parity, abort));
 }
 
-// Consumer warp of a single-token set: integer MMAs on byte-masked words (see stage_group_i8), then the fold
+// Consumer warp of a single-token set: integer MMAs on byte-masked words (see stage_groups_i8), then the fold
 // acc += s (D 2^(-S-Pc) - z sum_x) per (row, group).  The loop is bound by instruction dispatch, above all by the
 // half-rate integer/logic pipe, so everything that is not a mask runs on the multiply-add pipe: the two
 // accumulation chains of a tile are added, and the tile of this lane pair is selected, by integer multiply-adds
@@ -664,6 +674,11 @@ __global__ void __launch_bounds__(256) set_single_stage_kernel(const __grid_cons
             items[c * q + min(c, r) + t] = it;
         }
     }
+    if (d.MP == 2) {                                             // one token
+        const int task = blockIdx.x * 32 + (threadIdx.x >> 3);
+        stage_task_one(d, ws, min(task, n_tasks - 1), threadIdx.x & 31, task < n_tasks);
+        return;
+    }
     const int task = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (task < n_tasks) stage_task(d, ws, task, threadIdx.x & 31);
 }
@@ -988,7 +1003,8 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
     // blocks are many and early launches measured 1 to 4 % slower, so those keep plain stream order.
     const bool early = M == 1;
     {
-        PdlLaunch l(static_cast<unsigned>((info.stage_tasks + 7) / 8), 256, 0, stream, early);
+        const int per_block = M == 1 ? 32 : 8;
+        PdlLaunch l(static_cast<unsigned>((info.stage_tasks + per_block - 1) / per_block), 256, 0, stream, early);
         SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, set_single_stage_kernel, d, plan, prm.ws, grid, r.n_rb, r.sp, info.stage_tasks, info.n_counters));
     }
     return launch_set_for(&info, prm, smem, stream, early);
@@ -1194,8 +1210,10 @@ int slim_mpq_gemv_set(const slim_gemv_set_info* info, const void* plan, void* wo
     if (st != SLIM_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     {
-        slim::PdlLaunch l(static_cast<unsigned>((info->stage_tasks + 7) / 8), 256, 0, s, false);
-        SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, slim::gemv_set_stage_kernel, prm.layers, prm.ws, info->n_layers, info->stage_tasks, info->n_counters));
+        const bool one = info->max_tokens == 1;
+        const int per_block = one ? 32 : 8;
+        slim::PdlLaunch l(static_cast<unsigned>((info->stage_tasks + per_block - 1) / per_block), 256, 0, s, false);
+        SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, one ? slim::gemv_set_stage_kernel<true> : slim::gemv_set_stage_kernel<false>, prm.layers, prm.ws, info->n_layers, info->stage_tasks, info->n_counters));
     }
     return slim::launch_set_for(info, prm, smem, s, false);
 }
