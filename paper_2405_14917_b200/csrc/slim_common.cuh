@@ -39,6 +39,11 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
 int gemv_one(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y,
              int M, int N, int K, void* workspace, cudaStream_t stream);
 
+// ... and layers of a few tokens, or of one that does not fit there, to one that cuts them over the whole GPU
+// (slim_gemv_few.cu): as above.
+int gemv_few(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y,
+             int M, int N, int K, void* workspace, cudaStream_t stream);
+
 // A set of single-token layers as one resident launch of that kernel (small sets: q/k/v, gate/up).  one_set_plan decides
 // (SLIM_OK: taken, descriptors written into the plan buffer; 1: not taken; negative: error), one_set_launch runs it.
 struct OneSetPlan {

@@ -587,6 +587,12 @@ int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host, c
         const int taken = slim::gemv_one(x, packed, gt, scales, zeros, y, M, N, K, workspace, s);
         if (taken <= 0) return taken;
     }
+    // More tokens, or one whose layer does not fit that kernel: the layer cut over the whole GPU in one launch.  What is
+    // left for the kernel of this file are more than 8 tokens on a K whose fragments do not fit (about 28000 columns).
+    {
+        const int taken = slim::gemv_few(x, packed, gt, scales, zeros, y, M, N, K, workspace, s);
+        if (taken <= 0) return taken;
+    }
     // From kPreStageMinM tokens on, a small kernel puts x into fragment order once, in the
     // workspace; with a workspace too small for that every CTA stages its own part of x.
     const bool pre = M >= slim::kPreStageMinM && workspace_bytes >= slim::prestage_bytes(M, gt);

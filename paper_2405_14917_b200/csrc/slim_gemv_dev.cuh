@@ -142,4 +142,75 @@ __device__ __forceinline__ float2 stage_group(const __half* xg, uint8_t* xs_slot
     return make_float2(sum, __int_as_float((127 + 24 - S) << 23));
 }
 
+// The same for up to four tokens of one group of b bits by one warp, with a quarter of the instructions per token: eight
+// lanes per token (bits 2 and 3 of the lane), lane (c, h) of the eight reads the 16 columns 32 c + 16 h .. + 15 once and
+// writes the fragments of lane column c for four MMAs of every slice.  x: the group's first column of token 0, K halves
+// from token to token; tokens m0 .. m0 + 3 below M are staged; xs: first fragment slot of the group, MP tokens to a row;
+// sums: (sum_k x, 2^(24-S)) per token.  All lanes call it together.  With h in the top bit of the lane the 16 lanes that
+// a shared-memory store serves at once write 128 bytes in a row.
+__device__ __forceinline__ void stage_tokens(const __half* x, size_t K, int b, int m0, int M, int MP, uint8_t* xs, float2* sums, int lane) {
+    const int c = lane & 3, m = m0 + ((lane >> 2) & 3), h = lane >> 4;
+    const bool live = m < M;
+    uint32_t W[8];                                          // columns 2i, 2i + 1 of the lane's 16
+    {
+        const __half* xl = x + static_cast<size_t>(live ? m : m0) * K + 32 * c + 16 * h;
+        const uint4 lo = *reinterpret_cast<const uint4*>(xl), hi = *reinterpret_cast<const uint4*>(xl + 8);
+        W[0] = lo.x; W[1] = lo.y; W[2] = lo.z; W[3] = lo.w; W[4] = hi.x; W[5] = hi.y; W[6] = hi.z; W[7] = hi.w;
+    }
+    uint32_t mx = 0;
+    float sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        mx = __vmaxu2(mx, W[i] & 0x7fff7fffu);
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&W[i]));
+        sum += f.x + f.y;
+    }
+    mx = max(mx & 0xffffu, mx >> 16);
+    auto across = [&](int o) {
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    };
+    across(1);
+    across(2);
+    across(16);
+    // 2^S lifts the group's largest |x| into [2^13, 2^14) (Inf/NaN: the top binade)
+    const int S = mx == 0 ? 0 : 28 - max(static_cast<int>(mx >> 10), 1);
+    if (live && c == 0 && h == 0) sums[m] = make_float2(sum, __int_as_float((127 + 24 - S) << 23));
+    // MMA 4 h + i of a slice of width WD: words A and B hold columns 2 ii, 2 ii + 1 of the first and of the second half of
+    // its unit's fields (ii: the MMA's place in the unit)
+    auto put = [&](auto wtag, int lo, int i, uint32_t A, uint32_t B, int ii, uint8_t* slot) {
+        constexpr int WD = decltype(wtag)::value;
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&A)), g = __half22float2(*reinterpret_cast<const __half2*>(&B));
+        const float sc0 = __int_as_float((127 + S + lo - pair_pos(WD, 2 * ii)) << 23), sc1 = __int_as_float((127 + S + lo - pair_pos(WD, 2 * ii + 1)) << 23);
+        const __half2 b0 = __floats2half2_rn(f.x * sc0, g.x * sc0), b1 = __floats2half2_rn(f.y * sc1, g.y * sc1);
+        if (live) *reinterpret_cast<uint2*>(slot + ((static_cast<size_t>(4 * h + i) * MP + m) * 4 + c) * 8) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&b0), *reinterpret_cast<const uint32_t*>(&b1));
+    };
+    if (b == 2 || b == 3) {                                 // unit h: fields 16 h .. 16 h + 15
+#pragma unroll
+        for (int i = 0; i < 4; ++i) put(W2{}, 0, i, W[i], W[i + 4], i, xs);
+    }
+    if (b == 4) {                                           // units 2 h and 2 h + 1 of eight fields
+#pragma unroll
+        for (int i = 0; i < 4; ++i) put(W4{}, 0, i, W[4 * (i >> 1) + (i & 1)], W[4 * (i >> 1) + (i & 1) + 2], i & 1, xs);
+    }
+    if (b == 1 || b == 3) {                                 // one unit of 32 fields: MMAs 4 h .. take columns 8 h .. + 7 of both halves
+        uint8_t* slot = xs + (b == 3 ? static_cast<size_t>(8) * MP * 32 : 0);
+        const int lo = b == 3 ? 2 : 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t got = __shfl_xor_sync(0xffffffffu, h == 0 ? W[4 + i] : W[i], 16);
+            const uint32_t A = h == 0 ? W[i] : got, B = h == 0 ? got : W[4 + i];
+            // ii = 4 h + i: the field position depends on the lane
+            const int p0 = 2 * (4 * h + i);
+            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&A)), g = __half22float2(*reinterpret_cast<const __half2*>(&B));
+            const int pos0 = pair_direct(1, p0) ? p0 : p0 - pair_shift(1), pos1 = pair_direct(1, p0 + 1) ? p0 + 1 : p0 + 1 - pair_shift(1);
+            const float sc0 = __int_as_float((127 + S + lo - pos0) << 23), sc1 = __int_as_float((127 + S + lo - pos1) << 23);
+            const __half2 b0 = __floats2half2_rn(f.x * sc0, g.x * sc0), b1 = __floats2half2_rn(f.y * sc1, g.y * sc1);
+            if (live) *reinterpret_cast<uint2*>(slot + ((static_cast<size_t>(4 * h + i) * MP + m) * 4 + c) * 8) =
+                make_uint2(*reinterpret_cast<const uint32_t*>(&b0), *reinterpret_cast<const uint32_t*>(&b1));
+        }
+    }
+}
+
 }  // namespace slim
