@@ -49,13 +49,14 @@ constexpr int kWarpPacked = kWarpEpi + 4;   // producer of packed slices
 constexpr int kGemmThreads = 32 * (kWarpPacked + 1);
 constexpr int kRowsPerCta = 128;
 constexpr int kRowsPerPair = 2 * kRowsPerCta;
-constexpr int kGPS = 2;                     // groups per pipeline stage: one round of barriers serves this many
+constexpr int kGPS = 1;                     // groups per pipeline stage
 constexpr int kNS = 4 / kGPS;               // pipeline stages: a shared-memory slot of x + 64 tensor-memory columns of A per group
 constexpr int kPStageBytes = 8192 + 512;    // 128 rows x 128 k x 4 bits, + scales + zeros
 constexpr int kTmemCols = 512;
 constexpr int kEpiCols = 16;                // accumulator columns (tokens) the epilogue handles at a time
 constexpr int kYBox = 32;                   // tokens, and rows, of one output store
 constexpr int kYBoxBytes = kYBox * kYBox * 2;
+constexpr int kUnitCost = 16;
 constexpr int kTmemAcol = 256;              // A stages start here; D occupies [0, TOK)
 constexpr unsigned long long kGemmWaitNs = 2000000000ull;
 constexpr unsigned int kGemmTryNs = 1000000u;     // suspend-time hint of one mbarrier.try_wait
@@ -70,7 +71,9 @@ struct GemmParams {
     float* partials;         // [grid][4 epilogue warps][TOK][32 rows] fp32 (stream-K only)
     int M, N, K;
     int row_blocks, tok_tiles;   // 256-row blocks, TOK-token tiles
+    uint32_t magic;          // kMagic1024, as a value the compiler cannot fold into an immediate (see DqRow)
     int stream_k;            // 1: clusters take equal shares of (tile, group) units; 0: whole tiles
+    int last_cost;           // stream-K: cost of a unit of the last token tile where kUnitCost is that of the others
     GroupTable gt;
 };
 
@@ -286,6 +289,7 @@ __device__ __forceinline__ __half2 pow2_h2(int e) { return as_half2(0x00010001u 
 struct DqRow {
     __half2 s;        // (s, s)
     __half2 add[4];   // -(constant of position i + z), see the decoders
+    uint32_t magic;   // kMagic1024 in a register: a three-input logic instruction takes one immediate, and that is the mask
 };
 __device__ __forceinline__ uint32_t lo_halves(uint32_t a, uint32_t b) { return g::prmt(a, b, 0x5410u); }
 __device__ __forceinline__ uint32_t hi_halves(uint32_t a, uint32_t b) { return g::prmt(a, b, 0x7632u); }
@@ -325,11 +329,11 @@ __device__ __forceinline__ void decode_word(uint32_t word, uint32_t X, const DqR
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
             const int f = PER * c + i, pos = 6 + W * i;
-            const uint32_t v = (copy & (kField << pos)) | kMagic1024;
+            const uint32_t v = (copy & (kField << pos)) | r.magic;
             __half2 t = __hfma2(as_half2(v), pow2_h2(-pos), r.add[HIGH ? (f & 3) : i]);
             if (HIGH) {
                 const int xpos = 6 + (f & 3);
-                const uint32_t vb = (shift_to(X, 6 - 4 * (f >> 2)) & (0x00010001u << xpos)) | kMagic1024;
+                const uint32_t vb = (shift_to(X, 6 - 4 * (f >> 2)) & (0x00010001u << xpos)) | r.magic;
                 t = __hfma2(as_half2(vb), pow2_h2(2 - xpos), t);
             }
             H[f] = as_u32(__hmul2(t, r.s));
@@ -391,6 +395,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = static_cast<int>(g::cluster_ctarank());     // 0 = leader of the pair
+    // The next kernel's CTAs may be set up as this one's leave; in turn the roles that touch x, y or the workspace wait for
+    // the kernel ahead (warp 0, the epilogue), the others only read the layer and start at once.
+    pdl_launch_dependents();
     const uint32_t bar0 = sbase + C::OFF_BAR;
     // Barriers of this CTA.  Stage s is ready for the MMA when `full(s)` of the LEADER completes:
     // 16 dequant warps of the pair have written A, the leader's half of x has landed (its TMA
@@ -433,13 +440,22 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
     // This pair's contiguous range [u0, u1) of (tile, group) units, unit = tile * G + group,
     // tile = token tile * row_blocks + 256-row block.  Without stream-K the range is whole tiles.
     auto range_begin = [&](int c) -> long long {
-        return p.stream_k ? (static_cast<long long>(c) * total_tiles * G) / ncl
-                          : ((static_cast<long long>(c) * total_tiles) / ncl) * G;
+        if (!p.stream_k) return ((static_cast<long long>(c) * total_tiles) / ncl) * G;
+        if (p.last_cost == kUnitCost) return (static_cast<long long>(c) * total_tiles * G) / ncl;
+        // equal shares of the cost: the units of the last token tile come last and are cheaper
+        const long long per = static_cast<long long>(p.row_blocks) * G, whole = per * (p.tok_tiles - 1);
+        const long long at = (static_cast<long long>(c) * (whole * kUnitCost + per * p.last_cost)) / ncl;
+        return at <= whole * kUnitCost ? at / kUnitCost : whole + (at - whole * kUnitCost) / p.last_cost;
     };
+    // Tokens of token tile mt that exist, and the MMA's N: those rounded up to the instruction's step.  Rank 0 brings the
+    // first N / 2 of them, rank 1 the rest.
+    auto tile_tokens = [&](int mt) { return min(TOK, p.M - mt * TOK); };
+    auto tile_n = [&](int mt) { return (tile_tokens(mt) + 31) & ~31; };
     const long long u0 = range_begin(cl), u1 = range_begin(cl + 1);
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer of activations
+        pdl_wait();
         if (lane == 0) {
             int sx = 0;
             uint32_t phx = 0;
@@ -448,7 +464,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                 const int tile = static_cast<int>(u / G), gb = static_cast<int>(u - static_cast<long long>(tile) * G);
                 const int ge = static_cast<int>(min(static_cast<long long>(G), gb + (u1 - u)));
                 u += ge - gb;
-                const int m0 = (tile / p.row_blocks) * TOK + rank * C::HALF;     // my half of the token tile
+                const int mt = tile / p.row_blocks, m0 = mt * TOK + rank * (tile_n(mt) / 2);     // my half of the token tile
                 for (int j = gb; j < ge; j += kGPS) {
                     const int ng = min(kGPS, ge - j);                            // groups of this stage
                     if (!g::mbar_wait(empty(sx), phx ^ 1u, abort)) { ok = false; break; }
@@ -512,7 +528,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
             // -------------------------------------------------------------- MMA issuer (leader)
             // The whole warp runs this loop and one elected lane issues: the operands then stay in uniform registers.
             // (Code that a single lane runs moves every operand there first, 48 to 77 cycles per MMA instead of 10.)
-            constexpr uint32_t idesc = (1u << 4) | (static_cast<uint32_t>(TOK >> 3) << 17) | (static_cast<uint32_t>(kRowsPerPair >> 4) << 24);
             const uint32_t tmem_u = tc::uniform(tmem);
             int st = 0;
             uint32_t ph = 0, phd = 0;
@@ -521,6 +536,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                 const int tile = static_cast<int>(u / G), gb = static_cast<int>(u - static_cast<long long>(tile) * G);
                 const int ge = static_cast<int>(min(static_cast<long long>(G), gb + (u1 - u)));
                 u += ge - gb;
+                const uint32_t idesc = tc::uniform((1u << 4) | (static_cast<uint32_t>(tile_n(tile / p.row_blocks) >> 3) << 17) | (static_cast<uint32_t>(kRowsPerPair >> 4) << 24));
                 if (!g::mbar_wait_warp(d_empty, phd ^ 1u, abort)) { ok = false; break; }   // both epilogues have drained D
                 g::tc_fence_after();
                 for (int j = gb; j < ge; j += kGPS) {
@@ -570,6 +586,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
         const int t = r >> 4, gq = (r & 15) >> 1, half = r & 1;
         bool ok = true;
         const uint32_t full_leader = g::map_to_cta(full(0), 0);
+        const uint32_t magic = p.magic;
         int si = 0, gi = 0;                                     // running numbers of the stage and of the group in this CTA's range
         for (long long u = u0; u < u1 && ok;) {
             const int tile = static_cast<int>(u / G), gb = static_cast<int>(u - static_cast<long long>(tile) * G);
@@ -598,9 +615,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
                             if (u < b) {
-                                const uint4 v = g::lds128(stage + t * 256 * b + 256 * u + 8 * (4 * gq + 2 * kh));
-                                w0[u] = half ? v.y : v.x;
-                                w1[u] = half ? v.w : v.z;
+                                const uint32_t at = stage + t * 256 * b + 256 * u + 8 * (4 * gq + 2 * kh) + 4 * half;
+                                w0[u] = lds32(at);
+                                w1[u] = lds32(at + 8);
                             }
                         }
                         sc = *reinterpret_cast<const __half*>(smem + C::OFF_P + sp * kPStageBytes + 8192 + 2 * r);
@@ -612,6 +629,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                     const uint32_t a_t = tmem + (static_cast<uint32_t>(32 * q) << 16) + kTmemAcol + 64 * (kGPS * sa + i) + 32 * kh;
                     uint32_t cols[16];
                     DqRow row;
+                    row.magic = magic;
                     // first 32 k of my half, then (the stage's columns are free by now) the other 32
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -645,6 +663,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
         // segment last, the others reach theirs first) waits for those flags, adds the partials in
         // pair order and stores the tile.  Each CTA deals with the CTAs of the same rank, which
         // hold the same 128 rows.
+        pdl_wait();
         const int q = warp & 3;
         const int et = tid - 32 * kWarpEpi;                     // 0..127 among the epilogue threads
         uint32_t phd = 0;
@@ -664,7 +683,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
             const int ge = static_cast<int>(min(static_cast<long long>(G), gb + (u1 - u)));
             u += ge - gb;
             const int rb = 2 * (tile % p.row_blocks) + rank, mt = tile / p.row_blocks;
-            const int n = kRowsPerCta * rb + 32 * q + lane;
+            const int chunks = tile_n(mt) / kYBox;               // pieces of 32 tokens that hold any
             const bool is_partial = gb > 0;
             // peers: the pairs after this one, up to the one that ends the tile (pairs with an empty
             // range take no part); peer k is CTA blockIdx.x + 2k
@@ -707,7 +726,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                 // whole tile: 32 tokens at a time through shared memory, one tensor store per chunk; the
                 // store of a chunk reads its buffer while the next chunk is written into the other one
 #pragma unroll 1
-                for (int cc = 0; cc < TOK / kYBox; ++cc) {
+                for (int cc = 0; cc < chunks; ++cc) {
                     const uint32_t buf = stg + (cc & 1) * kYBoxBytes;
                     if (lane == 0) g::bulk_wait_read<1>();
                     __syncwarp();
@@ -730,7 +749,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                 }
             } else if (is_partial) {
 #pragma unroll 1
-                for (int cc = 0; cc < TOK / kEpiCols; ++cc) {
+                for (int cc = 0; cc < 2 * chunks; ++cc) {
                     uint32_t v[kEpiCols];
                     g::tmem_ld16(tmem + (static_cast<uint32_t>(32 * q) << 16) + kEpiCols * cc, v);
                     g::tc_wait_ld();
@@ -746,7 +765,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                 constexpr int S = C::NPEERBAR;
                 static_assert((S & (S - 1)) == 0 && S * 2048 * 4 <= C::OFF_P, "ring of the peers' partials");
                 const int np_act = __popcll(act);
-                const int J = S * np_act;
+                const int n_pieces = 2 * chunks, J = n_pieces * np_act;
                 // the active peer after peer k, going round
                 auto next_peer = [&](int k) {
                     const unsigned long long above = k < 64 ? act >> k : 0ull;
@@ -769,7 +788,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                 g::fence_proxy_async_all();                      // the flags were seen through ordinary loads
                 while (j_iss < min(S, J)) issue_next();
 #pragma unroll 1
-                for (int cc = 0; cc < S && !bad; ++cc) {
+                for (int cc = 0; cc < n_pieces && !bad; ++cc) {
                     float t[kEpiCols];
 #pragma unroll
                     for (int i = 0; i < kEpiCols; ++i) t[i] = 0.f;
@@ -918,7 +937,7 @@ static int max_resident_pairs() {
 // (tile, group) units per CTA pair, partial tiles combined through the workspace) is used when it
 // is predicted to beat whole tiles, whose last wave may leave most SMs idle.
 struct GemmPlan {
-    int tok, row_blocks, tok_tiles, grid, stream_k;
+    int tok, row_blocks, tok_tiles, grid, stream_k, last_cost;
     size_t workspace_bytes;
 };
 static GemmPlan plan_gemm(int M, int N, int G) {
@@ -936,6 +955,7 @@ static GemmPlan plan_gemm(int M, int N, int G) {
     const int waves = (tiles + pairs - 1) / pairs;
     pl.grid = 2 * npairs;
     pl.stream_k = 0;
+    pl.last_cost = kUnitCost;
     // Time in units of one group.  Whole tiles take waves * G.  Equal shares of the (tile, group) units over P
     // pairs take units / P plus the hand-over of the cut tiles: a dozen groups' worth when a tile has one peer
     // (drains, flags, one partial tile brought in and added), with more peers seven more per peer at 256 tokens
@@ -974,8 +994,8 @@ static cudaError_t launch_gemm(const CUtensorMap& map, const CUtensorMap& ymap, 
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    gemm_kernel<TOK><<<grid, kGemmThreads, GemmCfg<TOK>::SMEM, stream>>>(map, ymap, prm);   // clusters of 2: see the kernel
-    return cudaGetLastError();
+    PdlLaunch l(static_cast<unsigned>(grid), kGemmThreads, GemmCfg<TOK>::SMEM, stream);      // clusters of 2: see the kernel
+    return cudaLaunchKernelEx(&l.cfg, gemm_kernel<TOK>, map, ymap, prm);
 }
 
 }  // namespace slim
@@ -1029,6 +1049,8 @@ extern "C" int slim_mpq_gemm(const void* x, const void* packed, const uint8_t* b
     prm.row_blocks = pl.row_blocks;
     prm.tok_tiles = pl.tok_tiles;
     prm.stream_k = pl.stream_k;
+    prm.last_cost = pl.last_cost;
+    prm.magic = slim::kMagic1024;
     prm.gt = gt;
     const cudaError_t e = tok == 128 ? slim::launch_gemm<128>(map, ymap, prm, pl.grid, s) : slim::launch_gemm<256>(map, ymap, prm, pl.grid, s);
     SLIM_CUDA_TRY(e);
