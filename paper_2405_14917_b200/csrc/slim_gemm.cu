@@ -56,7 +56,7 @@ constexpr int kTmemCols = 512;
 constexpr int kEpiCols = 16;                // accumulator columns (tokens) the epilogue handles at a time
 constexpr int kYBox = 32;                   // tokens, and rows, of one output store
 constexpr int kYBoxBytes = kYBox * kYBox * 2;
-constexpr int kUnitCost = 16;
+constexpr int kMaxEven = 16;                // most pairs that share a tile evenly (a bit each in a flag word)
 constexpr int kTmemAcol = 256;              // A stages start here; D occupies [0, TOK)
 constexpr unsigned long long kGemmWaitNs = 2000000000ull;
 constexpr unsigned int kGemmTryNs = 1000000u;     // suspend-time hint of one mbarrier.try_wait
@@ -67,13 +67,14 @@ struct GemmParams {
     const __half* zeros;
     __half* y;
     unsigned int* status;
-    unsigned int* flags;     // [grid]: "partial of this CTA is ready" (stream-K only; zero between launches)
+    unsigned int* flags;     // [grid], stream-K only, zero between launches: "partial of this CTA is ready", or with `even` one bit per
+                             // pair of the tile whose partial is ready for this CTA
     float* partials;         // [grid][4 epilogue warps][TOK][32 rows] fp32 (stream-K only)
     int M, N, K;
     int row_blocks, tok_tiles;   // 256-row blocks, TOK-token tiles
     uint32_t magic;          // kMagic1024, as a value the compiler cannot fold into an immediate (see DqRow)
     int stream_k;            // 1: clusters take equal shares of (tile, group) units; 0: whole tiles
-    int last_cost;           // stream-K: cost of a unit of the last token tile where kUnitCost is that of the others
+    int even;                // > 1: stream-K with this many pairs per tile, each of which finishes a share of its tokens
     GroupTable gt;
 };
 
@@ -440,12 +441,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
     // This pair's contiguous range [u0, u1) of (tile, group) units, unit = tile * G + group,
     // tile = token tile * row_blocks + 256-row block.  Without stream-K the range is whole tiles.
     auto range_begin = [&](int c) -> long long {
-        if (!p.stream_k) return ((static_cast<long long>(c) * total_tiles) / ncl) * G;
-        if (p.last_cost == kUnitCost) return (static_cast<long long>(c) * total_tiles * G) / ncl;
-        // equal shares of the cost: the units of the last token tile come last and are cheaper
-        const long long per = static_cast<long long>(p.row_blocks) * G, whole = per * (p.tok_tiles - 1);
-        const long long at = (static_cast<long long>(c) * (whole * kUnitCost + per * p.last_cost)) / ncl;
-        return at <= whole * kUnitCost ? at / kUnitCost : whole + (at - whole * kUnitCost) / p.last_cost;
+        return p.stream_k ? (static_cast<long long>(c) * total_tiles * G) / ncl
+                          : ((static_cast<long long>(c) * total_tiles) / ncl) * G;
     };
     // Tokens of token tile mt that exist, and the MMA's N: those rounded up to the instruction's step.  Rank 0 brings the
     // first N / 2 of them, rank 1 the rest.
@@ -657,7 +654,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
         }
     } else if (warp < kWarpPacked) {
         // ------------------------------------------------------------------ epilogue warps
-        // A segment that covers its whole tile is stored as fp16.  With stream-K a tile may be cut:
+        // A segment that covers its whole tile is stored as fp16.  With `even` every tile is cut into as many segments as it
+        // has pairs, and they share its end (below).  With plain stream-K a tile may be cut anywhere:
         // a pair whose segment does not start the tile leaves its fp32 partials in its CTAs'
         // workspace slots and raises their flags; the pair that starts the tile (it reaches that
         // segment last, the others reach theirs first) waits for those flags, adds the partials in
@@ -685,6 +683,91 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
             const int rb = 2 * (tile % p.row_blocks) + rank, mt = tile / p.row_blocks;
             const int chunks = tile_n(mt) / kYBox;               // pieces of 32 tokens that hold any
             const bool is_partial = gb > 0;
+            if (p.even > 1) {
+                // ---- the pairs of a tile end together, so each of them finishes every k-th 32-token piece: it leaves the others'
+                // pieces in its slot, tells each pair that has pieces, and adds what those left for it, in the order of the pairs
+                const int k = p.even, seg = cl % k, base = static_cast<int>(blockIdx.x) - 2 * seg;
+                const bool gave_up = epi_any(!g::mbar_wait_long(d_full, phd, abort));
+                if (gave_up) { ok = false; break; }
+                g::tc_fence_after();
+                const uint32_t acc_t = tmem + (static_cast<uint32_t>(32 * q) << 16);
+                float* slot = p.partials + static_cast<size_t>(blockIdx.x) * (TOK * kRowsPerCta) + q * (TOK * 32) + lane;
+#pragma unroll 1
+                for (int cc = 0; cc < 2 * chunks; ++cc) {
+                    if ((cc >> 1) % k == seg) continue;
+                    uint32_t v[kEpiCols];
+                    g::tmem_ld16(acc_t + kEpiCols * cc, v);
+                    g::tc_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < kEpiCols; ++i) slot[(kEpiCols * cc + i) * 32] = __uint_as_float(v[i]);
+                }
+                __threadfence();
+                epi_sync();
+                if (et < k && et != seg && et < chunks) {
+                    __threadfence();
+                    atomicOr(p.flags + base + 2 * et, 1u << seg);
+                }
+                if (seg < chunks) {
+                    bool late = false;
+                    if (et == 0) {
+                        volatile unsigned int* f = p.flags + blockIdx.x;
+                        const unsigned int all = ((1u << k) - 1u) & ~(1u << seg);
+                        const unsigned long long t0 = g::global_timer_ns();
+                        while (*f != all) {
+                            if (*abort != 0 || g::global_timer_ns() - t0 > kGemmWaitNs) { *abort = 1; late = true; break; }
+                        }
+                        __threadfence();
+                        *f = 0u;                                 // ready for the next launch
+                    }
+                    if (epi_any(late)) { ok = false; break; }
+                    const uint32_t stg = sbase + C::OFF_STAGE + q * 2 * kYBoxBytes + 2 * lane;
+                    const int n0 = kRowsPerCta * rb + 32 * q;
+#pragma unroll 1
+                    for (int c32 = seg, nth = 0; c32 < chunks; c32 += k, ++nth) {
+                        const uint32_t buf = stg + (nth & 1) * kYBoxBytes;
+                        if (lane == 0) g::bulk_wait_read<1>();
+                        __syncwarp();
+#pragma unroll 1
+                        for (int hf = 0; hf < 2; ++hf) {
+                            const int cc = 2 * c32 + hf;
+                            uint32_t v[kEpiCols];
+                            g::tmem_ld16(acc_t + kEpiCols * cc, v);
+                            g::tc_wait_ld();
+                            float t[kEpiCols];
+#pragma unroll
+                            for (int i = 0; i < kEpiCols; ++i) t[i] = 0.f;
+                            for (int o = 0; o < k; ++o) {
+                                const float* from = p.partials + static_cast<size_t>(base + 2 * o) * (TOK * kRowsPerCta) + q * (TOK * 32) + lane + cc * (kEpiCols * 32);
+                                if (o == seg) {
+#pragma unroll
+                                    for (int i = 0; i < kEpiCols; ++i) t[i] += __uint_as_float(v[i]);
+                                } else {
+                                    float w[kEpiCols];
+#pragma unroll
+                                    for (int i = 0; i < kEpiCols; ++i) w[i] = __ldcg(from + i * 32);
+#pragma unroll
+                                    for (int i = 0; i < kEpiCols; ++i) t[i] += w[i];
+                                }
+                            }
+#pragma unroll
+                            for (int i = 0; i < kEpiCols; ++i)
+                                g::sts_u16(buf + (kEpiCols * hf + i) * 2 * kYBox, __half_as_ushort(__float2half_rn(t[i])));
+                        }
+                        g::fence_proxy_async();
+                        __syncwarp();
+                        const int m0 = mt * TOK + kYBox * c32;
+                        if (lane == 0 && n0 < N && m0 < p.M) {
+                            g::tma_store_2d(&y_map, n0, m0, buf - 2 * lane);
+                            g::bulk_commit();
+                        }
+                    }
+                }
+                g::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) g::mbar_arrive_cluster(d_empty_leader);
+                phd ^= 1u;
+                continue;
+            }
             // peers: the pairs after this one, up to the one that ends the tile (pairs with an empty
             // range take no part); peer k is CTA blockIdx.x + 2k
             int npeer = 0;
@@ -937,7 +1020,7 @@ static int max_resident_pairs() {
 // (tile, group) units per CTA pair, partial tiles combined through the workspace) is used when it
 // is predicted to beat whole tiles, whose last wave may leave most SMs idle.
 struct GemmPlan {
-    int tok, row_blocks, tok_tiles, grid, stream_k, last_cost;
+    int tok, row_blocks, tok_tiles, grid, stream_k, even;
     size_t workspace_bytes;
 };
 static GemmPlan plan_gemm(int M, int N, int G) {
@@ -955,27 +1038,36 @@ static GemmPlan plan_gemm(int M, int N, int G) {
     const int waves = (tiles + pairs - 1) / pairs;
     pl.grid = 2 * npairs;
     pl.stream_k = 0;
-    pl.last_cost = kUnitCost;
-    // Time in units of one group.  Whole tiles take waves * G.  Equal shares of the (tile, group) units over P
-    // pairs take units / P plus the hand-over of the cut tiles: a dozen groups' worth when a tile has one peer
-    // (drains, flags, one partial tile brought in and added), with more peers seven more per peer at 256 tokens
-    // and three and a half at 128 (measured: graph-replayed timings of nine layer shapes at M = 32 ... 2048 with
-    // either schedule).  P is every resident pair, or, for a layer with few tiles, two, three or four pairs per
-    // tile: the cuts then fall on the same groups in every tile and a tile has one, two or three peers, where
-    // equal shares over all pairs would give it more.
+    pl.even = 0;
+    // Time in units of one group.  Whole tiles take waves * G.  Equal shares of the (tile, group) units over all resident
+    // pairs take units / P plus the hand-over of the cut tiles: a dozen groups' worth when a tile has one peer (drains,
+    // flags, one partial tile brought in and added), with more peers seven more per peer at 256 tokens and three and a
+    // half at 128 (measured: graph-replayed timings of nine layer shapes at M = 32 ... 2048 with either schedule).
+    // With few tiles, k pairs per tile: the cuts fall on the same groups in every tile, the pairs of a tile end together
+    // and each finishes its share of the tile's 32-token pieces, which costs what writing the others' pieces takes and
+    // then (k - 1) reads of each own piece.  (Measured at 40 and 256 tokens with k = 2 ... 8, us: 512 x 4096 13.8 / 11.9 / 12.5
+    // / - / 13.4 / - / 14.8 for k = 2, 3, 4, 6, 8 against 18.2 whole; 1024 x 28672 at 256 tokens 76.6 / 57.5 / 47.5 / 42.6 / 33.9
+    // against 130.5.  One pair that gathered the others' whole tiles took 8 us at 40 tokens where this takes 4.)
     const long long units = static_cast<long long>(tiles) * G;
     const double per_peer = pl.tok == 256 ? 7.0 : 3.5;
+    const int chunks = ((M < pl.tok ? M : pl.tok) + kYBox - 1) / kYBox;
     double best = 0.95 * static_cast<double>(waves) * G;
-    for (int k = 1; k <= 4 && resident > 0; ++k) {
+    for (int k = 1; k <= kMaxEven && resident > 0; ++k) {
         const int P = k == 1 ? pairs : k * tiles;
-        if (P > pairs || units < 8ll * P) continue;
+        if (P > pairs || units < (k == 1 ? 8ll : 4ll) * P) continue;
         const double share = static_cast<double>(units) / P;
-        const double peers = k == 1 ? ceil(static_cast<double>(G) / share) : static_cast<double>(k - 1);
-        const double cost = share + 12.0 + (peers > 1.0 ? per_peer * peers : 0.0);
+        double cost = share;
+        if (k == 1) {
+            const double peers = ceil(static_cast<double>(G) / share);
+            cost += 12.0 + (peers > 1.0 ? per_peer * peers : 0.0);
+        } else {
+            cost += 4.0 + chunks + 2.0 * ((chunks + k - 1) / k) * (k - 1);
+        }
         if (cost < best) {
             best = cost;
             pl.stream_k = 1;
             pl.grid = 2 * P;
+            pl.even = k == 1 ? 0 : k;
         }
     }
     pl.workspace_bytes = pl.stream_k ? kGemmWsPartials + static_cast<size_t>(pl.grid) * pl.tok * kRowsPerCta * sizeof(float) : 256;
@@ -1049,7 +1141,7 @@ extern "C" int slim_mpq_gemm(const void* x, const void* packed, const uint8_t* b
     prm.row_blocks = pl.row_blocks;
     prm.tok_tiles = pl.tok_tiles;
     prm.stream_k = pl.stream_k;
-    prm.last_cost = pl.last_cost;
+    prm.even = pl.stream_k ? pl.even : 0;
     prm.magic = slim::kMagic1024;
     prm.gt = gt;
     const cudaError_t e = tok == 128 ? slim::launch_gemm<128>(map, ymap, prm, pl.grid, s) : slim::launch_gemm<256>(map, ymap, prm, pl.grid, s);
