@@ -71,7 +71,8 @@ struct GemmParams {
                              // pair of the tile whose partial is ready for this CTA
     float* partials;         // [grid][4 epilogue warps][TOK][32 rows] fp32 (stream-K only)
     int M, N, K;
-    int row_blocks, tok_tiles;   // 256-row blocks, TOK-token tiles
+    int row_blocks, tok_tiles;   // 256-row blocks, token tiles
+    int step;                    // tokens of a token tile (a multiple of 32, at most TOK; the last tile may have fewer)
     uint32_t magic;          // kMagic1024, as a value the compiler cannot fold into an immediate (see DqRow)
     int stream_k;            // 1: clusters take equal shares of (tile, group) units; 0: whole tiles
     int even;                // > 1: stream-K with this many pairs per tile, each of which finishes a share of its tokens
@@ -446,7 +447,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
     };
     // Tokens of token tile mt that exist, and the MMA's N: those rounded up to the instruction's step.  Rank 0 brings the
     // first N / 2 of them, rank 1 the rest.
-    auto tile_tokens = [&](int mt) { return min(TOK, p.M - mt * TOK); };
+    auto tile_tokens = [&](int mt) { return min(p.step, p.M - mt * p.step); };
     auto tile_n = [&](int mt) { return (tile_tokens(mt) + 31) & ~31; };
     const long long u0 = range_begin(cl), u1 = range_begin(cl + 1);
 
@@ -461,7 +462,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                 const int tile = static_cast<int>(u / G), gb = static_cast<int>(u - static_cast<long long>(tile) * G);
                 const int ge = static_cast<int>(min(static_cast<long long>(G), gb + (u1 - u)));
                 u += ge - gb;
-                const int mt = tile / p.row_blocks, m0 = mt * TOK + rank * (tile_n(mt) / 2);     // my half of the token tile
+                const int mt = tile / p.row_blocks, m0 = mt * p.step + rank * (tile_n(mt) / 2);     // my half of the token tile
                 for (int j = gb; j < ge; j += kGPS) {
                     const int ng = min(kGPS, ge - j);                            // groups of this stage
                     if (!g::mbar_wait(empty(sx), phx ^ 1u, abort)) { ok = false; break; }
@@ -755,7 +756,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                         }
                         g::fence_proxy_async();
                         __syncwarp();
-                        const int m0 = mt * TOK + kYBox * c32;
+                        const int m0 = mt * p.step + kYBox * c32;
                         if (lane == 0 && n0 < N && m0 < p.M) {
                             g::tma_store_2d(&y_map, n0, m0, buf - 2 * lane);
                             g::bulk_commit();
@@ -824,7 +825,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                     }
                     g::fence_proxy_async();
                     __syncwarp();
-                    const int m0 = mt * TOK + kYBox * cc;
+                    const int m0 = mt * p.step + kYBox * cc;
                     if (lane == 0 && n0 < N && m0 < p.M) {
                         g::tma_store_2d(&y_map, n0, m0, buf - 2 * lane);
                         g::bulk_commit();
@@ -902,7 +903,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                     if (cc & 1) {
                         g::fence_proxy_async();
                         __syncwarp();
-                        const int m0 = mt * TOK + kEpiCols * (cc - 1);
+                        const int m0 = mt * p.step + kEpiCols * (cc - 1);
                         if (lane == 0 && n0 < N && m0 < p.M) {
                             g::tma_store_2d(&y_map, n0, m0, stg - 2 * lane + ((cc >> 1) & 1) * kYBoxBytes);
                             g::bulk_commit();
@@ -1020,54 +1021,54 @@ static int max_resident_pairs() {
 // (tile, group) units per CTA pair, partial tiles combined through the workspace) is used when it
 // is predicted to beat whole tiles, whose last wave may leave most SMs idle.
 struct GemmPlan {
-    int tok, row_blocks, tok_tiles, grid, stream_k, even;
+    int tok, step, row_blocks, tok_tiles, grid, stream_k, even;
     size_t workspace_bytes;
 };
 static GemmPlan plan_gemm(int M, int N, int G) {
     GemmPlan pl;
     pl.tok = M <= 128 ? 128 : 256;
     pl.row_blocks = (N + kRowsPerPair - 1) / kRowsPerPair;
-    pl.tok_tiles = (M + pl.tok - 1) / pl.tok;
-    const int tiles = pl.row_blocks * pl.tok_tiles;
     int pairs = gemm_sm_count() / 2;
     const int resident = pl.tok == 128 ? max_resident_pairs<128>() : max_resident_pairs<256>();
     if (resident > 0 && pairs > resident) pairs = resident;
     if (pairs > kGemmMaxGrid / 2) pairs = kGemmMaxGrid / 2;
     if (pairs < 1) pairs = 1;
-    const int npairs = tiles < pairs ? tiles : pairs;
-    const int waves = (tiles + pairs - 1) / pairs;
-    pl.grid = 2 * npairs;
-    pl.stream_k = 0;
-    pl.even = 0;
-    // Time in units of one group.  Whole tiles take waves * G.  Equal shares of the (tile, group) units over all resident
-    // pairs take units / P plus the hand-over of the cut tiles: a dozen groups' worth when a tile has one peer (drains,
-    // flags, one partial tile brought in and added), with more peers seven more per peer at 256 tokens and three and a
-    // half at 128 (measured: graph-replayed timings of nine layer shapes at M = 32 ... 2048 with either schedule).
+    // Time in units of one group of a full tile.  Whole tiles take waves * G.  Equal shares of the (tile, group) units
+    // over all resident pairs take units / P plus the hand-over of the cut tiles: a dozen groups' worth when a tile has one
+    // peer (drains, flags, one partial tile brought in and added), with more peers seven more per peer at 256 tokens and
+    // three and a half at 128 (measured: graph-replayed timings of nine layer shapes at M = 32 ... 2048 with either schedule).
     // With few tiles, k pairs per tile: the cuts fall on the same groups in every tile, the pairs of a tile end together
     // and each finishes its share of the tile's 32-token pieces, which costs what writing the others' pieces takes and
     // then (k - 1) reads of each own piece.  (Measured at 40 and 256 tokens with k = 2 ... 8, us: 512 x 4096 13.8 / 11.9 / 12.5
     // / - / 13.4 / - / 14.8 for k = 2, 3, 4, 6, 8 against 18.2 whole; 1024 x 28672 at 256 tokens 76.6 / 57.5 / 47.5 / 42.6 / 33.9
     // against 130.5.  One pair that gathered the others' whole tiles took 8 us at 40 tokens where this takes 4.)
-    const long long units = static_cast<long long>(tiles) * G;
-    const double per_peer = pl.tok == 256 ? 7.0 : 3.5;
-    const int chunks = ((M < pl.tok ? M : pl.tok) + kYBox - 1) / kYBox;
-    double best = 0.95 * static_cast<double>(waves) * G;
-    for (int k = 1; k <= kMaxEven && resident > 0; ++k) {
-        const int P = k == 1 ? pairs : k * tiles;
-        if (P > pairs || units < (k == 1 ? 8ll : 4ll) * P) continue;
-        const double share = static_cast<double>(units) / P;
-        double cost = share;
-        if (k == 1) {
-            const double peers = ceil(static_cast<double>(G) / share);
-            cost += 12.0 + (peers > 1.0 ? per_peer * peers : 0.0);
-        } else {
-            cost += 4.0 + chunks + 2.0 * ((chunks + k - 1) / k) * (k - 1);
-        }
-        if (cost < best) {
+    // The tokens may also be cut into up to two tiles more than they need, of equal width.  Narrower tiles cost more per
+    // token (bound by the dequantisation, a unit of 128 tokens takes 85 % of one of 256) but fill the pairs better, and a
+    // last tile of a few tokens goes away: 5120 x 5120 at 512 tokens, 60 tiles of 192 for 40 of 256 on 74 pairs, 32.2 -> 30.4
+    // us; 512 x 4096 at 256 tokens 18.6 -> 13.4; 13824 x 5120 at 300 tokens, two tiles of 160 for 256 and 44, 55.3 -> 48.3.
+    double best = 1e30;
+    const int tt_min = (M + pl.tok - 1) / pl.tok;
+    for (int tt = tt_min; tt <= tt_min + 2; ++tt) {
+        const int step = ((M + tt - 1) / tt + 31) / 32 * 32, tok_tiles = (M + step - 1) / step;
+        if (tt > tt_min && (pl.tok == 128 || tok_tiles != tt || step < 128)) break;
+        const int tiles = pl.row_blocks * tok_tiles, waves = (tiles + pairs - 1) / pairs;
+        const long long units = static_cast<long long>(tiles) * G;
+        const double unit = pl.tok == 128 ? 1.0 : step <= 128 ? 0.85 : 0.7 + 0.3 / 256 * step;
+        const double per_peer = pl.tok == 256 ? 7.0 : 3.5;
+        const int chunks = step / kYBox;
+        auto take = [&](double cost, int pairs_used, int stream_k, int even) {
+            if (cost >= best) return;
             best = cost;
-            pl.stream_k = 1;
-            pl.grid = 2 * P;
-            pl.even = k == 1 ? 0 : k;
+            pl.step = step; pl.tok_tiles = tok_tiles;
+            pl.grid = 2 * pairs_used; pl.stream_k = stream_k; pl.even = even;
+        };
+        take(0.95 * unit * waves * G, tiles < pairs ? tiles : pairs, 0, 0);
+        for (int k = 1; k <= kMaxEven && resident > 0; ++k) {
+            const int P = k == 1 ? pairs : k * tiles;
+            if (P > pairs || units < (k == 1 ? 8ll : 4ll) * P) continue;
+            const double share = static_cast<double>(units) / P, peers = ceil(static_cast<double>(G) / share);
+            if (k == 1) take(unit * share + 12.0 + (peers > 1.0 ? per_peer * peers : 0.0), P, 1, 0);
+            else take(unit * share + 3.0 + 2.0 * ((chunks + k - 1) / k) * (k - 1), P, 1, k);
         }
     }
     pl.workspace_bytes = pl.stream_k ? kGemmWsPartials + static_cast<size_t>(pl.grid) * pl.tok * kRowsPerCta * sizeof(float) : 256;
@@ -1140,6 +1141,7 @@ extern "C" int slim_mpq_gemm(const void* x, const void* packed, const uint8_t* b
     prm.partials = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + slim::kGemmWsPartials);
     prm.row_blocks = pl.row_blocks;
     prm.tok_tiles = pl.tok_tiles;
+    prm.step = pl.step;
     prm.stream_k = pl.stream_k;
     prm.even = pl.stream_k ? pl.even : 0;
     prm.magic = slim::kMagic1024;

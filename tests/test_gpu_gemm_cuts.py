@@ -16,6 +16,8 @@ pytestmark = pytest.mark.gpu
     (512, 8192, 200),     # seven pieces in a tile of 256 tokens
     (256, 2048, 300),     # a second token tile with two pieces, the last one of 12 tokens
     (80, 16384, 128),     # the most pairs
+    (1024, 1024, 330),    # tiles narrower than they could be, a last one of fewer tokens
+    (1296, 512, 700),     # whole tiles of equal width
 ])
 def test_pieces_and_pairs(N, K, M):
     L = oracle_layer(N, K, 3, M, seed_name="gemm-cuts")
