@@ -33,7 +33,7 @@
  * (slim_quantize_minmax, _groups, _sign1, _sqc; these also take a K that is any multiple of g), the SBA search and
  * the GPTQ loop take every g; the layer-set launch and slim_mpq_gemm_static take 128, 256 and 512
  * (SLIM_ERR_UNSUPPORTED otherwise).  Groups of 256 and 512 columns run on the tensor-core kernels of the 128-column tiles (a group is 2 or 4
- * tiles that share a row of scales and zeros); groups of 32 and 64 columns run on plain CUDA-core kernels, and the
+ * tiles that share a row of scales and zeros); groups of 32 and 64 columns run on a kernel of their own, and the
  * batched entry point then wants room for the fp16 weights in its workspace (slim_workspace_bytes says how much).
  *
  * Packed format ("sliced bit planes", version SLIM_FORMAT_VERSION).  K is cut into K-tiles of T = min(g, 128)

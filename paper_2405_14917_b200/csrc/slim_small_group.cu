@@ -6,13 +6,12 @@
 // fields.  This is the 128-column layout with every 32 replaced by T/4, so the decode below is the same bit
 // shuffling on 8- and 16-bit items.
 //
-// These group sizes trade a fifth to a half more scale and zero-point bytes for accuracy; they are served by plain
-// CUDA-core kernels (one FMA per weight and token), not by the tensor-core kernels of the 128-column tiles:
+// These group sizes trade a fifth to a half more scale and zero-point bytes for accuracy.
 //   pack_small_kernel, dequant_small_kernel   one thread per item / per 8 outputs, bit-exact
-//   gemv_small_kernel (1 <= M <= 16)          a block per 16-row tile, the groups dealt to its 16 warps, fp32 accumulation
-//   M > 16                                    the weights are materialised as fp16 in the workspace (dequant_small_kernel)
-//                                             and multiplied by dense_f16_kernel (mma.sync, fp32 accumulation)
+//   linear_small_kernel                       y = x W-hat^T for any number of tokens: mma.sync on the codes, which are
+//                                             exact as fp16, fp32 accumulation, scale and zero point per group in fp32
 #include "slim_common.cuh"
+#include "slim_gemv_dev.cuh"
 
 #include <cstring>
 
@@ -114,33 +113,37 @@ __global__ void __launch_bounds__(256) dequant_small_kernel(const uint8_t* __res
     *reinterpret_cast<uint4*>(W + static_cast<size_t>(row) * K + k0) = *reinterpret_cast<const uint4*>(out);
 }
 
-// ------------------------------------------------------------------------------------------ decode path, 1 <= M <= 16
-// A block of 16 warps per 16-row tile; warp w takes the groups w, w + 16, ...; lane 4*gq + c holds the items of rows
-// 2gq, 2gq + 1 for the column range c of the group, decodes its T/4 codes per row and multiplies them with the
-// tokens' activations (fp32 FMAs); per (row, group) acc += s * (sum_k q x - z * sum_k x).  The four lanes of a row
-// pair are added by shuffles, the sixteen warps through shared memory, in a fixed order.
-// The kernel is a chain of small loads, so a group's bytes (its b units, both rows of a lane in one load, and the
-// scale and zero-point pairs) are requested one group ahead of their use.
-constexpr int kSmallWarps = 16;
-
+// ------------------------------------------------------------------------------------------ the linear layer
+// A block takes 16 R rows and 8 NT tokens, its warps cut K: warp w takes the groups w, w + WARPS, ...  Lane 4*gq + c holds
+// the items of rows 2gq, 2gq + 1 of a tile for the column range c of a group, which is an A fragment of the MMA when its
+// rows gq and gq + 8 stand for tile rows 2gq and 2gq + 1 and its k slots for the lane's own columns: slot pair f of a lane
+// is columns (f, f + T/8) of its T/4, because those two fields sit in the halves of a word after one byte permutation,
+// whatever the width.  One logic instruction and one HFMA2 make the two codes of a register, exactly, as fp16.  The B
+// fragment of token gq is the lane's T/4 columns of x, 32 (T = 64) or 16 bytes in a row, with the same pairing.
+// sum_k x, which the zero points need, comes from one more MMA per step with all-ones rows.  Per (row, token, group)
+// acc += s * (sum_k q x - z * sum_k x); the warps' sums are added through shared memory in warp order.
+// A group's codes, scales and zero points are requested one group ahead, the first ones before the kernel ahead is done.
+//
+// Measured (us, 4096 x 4096 at 2 bits, tokens 1 / 8 / 16 / 40 / 128): group size 64 5.9 / 5.9 / 9.0 / 21 / 42, 32 8.2 / 8.1 / 10 /
+// 22 / 42.  An FMA per weight and token took 8.4 / 22 / 43 and 9.5 / 29 / 58 for up to 16 tokens, the weights written out as
+// fp16 and a product that read its fragments from global memory 280 beyond.  One token is a chain of loads of a few
+// bytes per lane; from 32 tokens on the codes are decoded again for every token tile, and x comes from L2 for every 32 rows.
 template <int T>
 struct SmallRaw {
     uint32_t unit[4];      // the lane's items of rows 2gq (low part) and 2gq + 1 of up to four units
     uint32_t s2, z2;       // scales and zero points of the two rows (half2)
-    int b;
 };
 template <int T>
-__device__ __forceinline__ SmallRaw<T> small_load(const uint8_t* __restrict__ packed, const __half* __restrict__ scales,
-                                                  const __half* __restrict__ zeros, int N, const SmallTable& st, int j, int t, int lane,
-                                                  int row0) {
+__device__ __forceinline__ SmallRaw<T> small_load(const uint8_t* packed, const __half* scales, const __half* zeros, int N,
+                                                  const SmallTable& st, int j, int t, int lane) {
     typedef typename SmallItem<T>::type item_t;
     SmallRaw<T> r;
-    r.b = st.bits[j];
+    const int b = st.bits[j], row0 = 16 * t + 2 * (lane >> 2);
     const uint8_t* base = packed + small_item_offset<T>(N, st, j, t, 0, lane, 0);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         r.unit[u] = 0u;
-        if (u < r.b) {
+        if (u < b) {
             if (sizeof(item_t) == 1) r.unit[u] = *reinterpret_cast<const uint16_t*>(base + 2 * T * u);
             else r.unit[u] = *reinterpret_cast<const uint32_t*>(base + 2 * T * u);
         }
@@ -149,141 +152,160 @@ __device__ __forceinline__ SmallRaw<T> small_load(const uint8_t* __restrict__ pa
     r.z2 = *reinterpret_cast<const uint32_t*>(zeros + static_cast<size_t>(j) * N + row0);
     return r;
 }
-// The codes of one lane (rows 2gq, 2gq + 1, its T/4 columns) from the W units of a width-W slice that start at unit `u0`.
-template <int T, int W>
-__device__ __forceinline__ void small_decode(const SmallRaw<T>& raw, int u0, int lo, uint32_t (&q)[2][T / 4]) {
-    typedef typename SmallItem<T>::type item_t;
-    constexpr int NF = T / 4 / W, IB = 8 * sizeof(item_t);
-    constexpr uint32_t kMask = (1u << W) - 1u;
+__device__ __forceinline__ __half2 small_h2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
+__device__ __forceinline__ uint32_t small_u32(__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); }
+// Items of two units of one row (half 0: row 2gq, 1: row 2gq + 1) in the low bits of the two halves of a word.
+template <int T>
+__device__ __forceinline__ uint32_t small_pair(uint32_t ua, uint32_t ub, int half) {
+    return T == 64 ? __byte_perm(ua, ub, half ? 0x7632 : 0x5410) : __byte_perm(ua, ub, half ? 0x2521 : 0x2420);
+}
+// The lower and the upper half of one item of one row, likewise.
+template <int T>
+__device__ __forceinline__ uint32_t small_split(uint32_t u, int half) {
+    if (T == 64) return __byte_perm(u, 0u, half ? 0x4342 : 0x4140);
+    const uint32_t v = __byte_perm(u, 0u, half ? 0x4441 : 0x4440);
+    return v | (v << 12);
+}
+// The codes of one row of a lane as T/8 fp16 pairs (columns f and f + T/8).  one: half2(1024, 1024) in a register.
+template <int T>
+__device__ __forceinline__ void small_codes(const SmallRaw<T>& raw, int b, int half, uint32_t one, uint32_t (&q)[T / 8]) {
+    constexpr int F = T / 8;
+    // field f of width W at bit W f of both halves: (1024 + v 2^pos) 2^-pos - 2^(10 - pos) = v; fields above bit 9 are shifted down
+    auto field = [&](uint32_t word, int W, int f) {
+        const int bit = W * f, down = bit + W > 10 ? 8 : 0, pos = bit - down;
+        const uint32_t v = ((down ? word >> 8 : word) & ((0x00010001u * ((1u << W) - 1u)) << pos)) | one;
+        return __hfma2(small_h2(v), __float2half2_rn(1.f / static_cast<float>(1 << pos)), __float2half2_rn(-static_cast<float>(1 << (10 - pos))));
+    };
+    if (b == 1) {
+        const uint32_t w = small_split<T>(raw.unit[0], half);
 #pragma unroll
-    for (int u = 0; u < W; ++u) {
-        const uint32_t i0 = raw.unit[u0 + u] & ((1u << IB) - 1u), i1 = raw.unit[u0 + u] >> IB;
+        for (int f = 0; f < F; ++f) q[f] = small_u32(field(w, 1, f));
+    } else if (b == 4) {
+        const uint32_t wa = small_pair<T>(raw.unit[0], raw.unit[2], half), wb = small_pair<T>(raw.unit[1], raw.unit[3], half);
 #pragma unroll
-        for (int f = 0; f < NF; ++f) {
-            q[0][NF * u + f] |= ((i0 >> (W * f)) & kMask) << lo;
-            q[1][NF * u + f] |= ((i1 >> (W * f)) & kMask) << lo;
+        for (int f = 0; f < F / 2; ++f) { q[f] = small_u32(field(wa, 4, f)); q[F / 2 + f] = small_u32(field(wb, 4, f)); }
+    } else {
+        const uint32_t w = small_pair<T>(raw.unit[0], raw.unit[1], half);
+#pragma unroll
+        for (int f = 0; f < F; ++f) q[f] = small_u32(field(w, 2, f));
+        if (b == 3) {
+            const uint32_t h = small_split<T>(raw.unit[2], half);
+#pragma unroll
+            for (int f = 0; f < F; ++f) q[f] = small_u32(__hfma2(field(h, 1, f), __float2half2_rn(4.f), small_h2(q[f])));
         }
     }
 }
 
-template <int T, int MT>     // MT: tokens handled per pass (the block loops over the token tiles)
-__global__ void __launch_bounds__(32 * kSmallWarps, MT == 1 ? 2 : 1) gemv_small_kernel(const __half* __restrict__ x, const uint8_t* __restrict__ packed,
-                                                                      const __half* __restrict__ scales, const __half* __restrict__ zeros,
-                                                                      __half* __restrict__ y, int M, int N, int K,
-                                                                      const __grid_constant__ SmallTable st) {
-    constexpr int C = T / 4;                               // columns per lane
-    __shared__ float red[kSmallWarps][MT][16];
+template <int T, int NT, int R, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) linear_small_kernel(const __half* x, const uint8_t* packed, const __half* scales, const __half* zeros,
+                                                                  __half* __restrict__ y, int M, int N, int K, uint32_t one,
+                                                                  const __grid_constant__ SmallTable st) {
+    constexpr int STEPS = T / 16, F = T / 8;
+    __shared__ float red[WARPS][8 * NT][16 * R];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gq = lane >> 2, c = lane & 3;
-    const int t = blockIdx.x;
-    const int row0 = 16 * t + 2 * gq;
-    for (int m0 = 0; m0 < M; m0 += MT) {
-        float acc[MT][2];
+    const int t0 = R * blockIdx.x, m0 = 8 * NT * blockIdx.y, tiles = N >> 4;
+    SmallRaw<T> next[R];
+    auto load = [&](int j) {
 #pragma unroll
-        for (int m = 0; m < MT; ++m) acc[m][0] = acc[m][1] = 0.f;
-        SmallRaw<T> next;
-        if (warp < st.G) next = small_load<T>(packed, scales, zeros, N, st, warp, t, lane, row0);
-        for (int j = warp; j < st.G; j += kSmallWarps) {
-            const SmallRaw<T> raw = next;
-            if (j + kSmallWarps < st.G) next = small_load<T>(packed, scales, zeros, N, st, j + kSmallWarps, t, lane, row0);
-            uint32_t q[2][C];
+        for (int r = 0; r < R; ++r) next[r] = small_load<T>(packed, scales, zeros, N, st, j, min(t0 + r, tiles - 1), lane);
+    };
+    if (warp < st.G) load(warp);
+    pdl_launch_dependents();
+    pdl_wait();                                            // x may be the output of the kernel before
+    const __half* xp[NT];                                  // this lane's columns of its token of every token tile
 #pragma unroll
-            for (int i = 0; i < C; ++i) q[0][i] = q[1][i] = 0u;
-            switch (raw.b) {
-                case 1: small_decode<T, 1>(raw, 0, 0, q); break;
-                case 2: small_decode<T, 2>(raw, 0, 0, q); break;
-                case 3: small_decode<T, 2>(raw, 0, 0, q); small_decode<T, 1>(raw, 2, 2, q); break;
-                default: small_decode<T, 4>(raw, 0, 0, q); break;
+    for (int n = 0; n < NT; ++n) xp[n] = x + static_cast<size_t>(min(m0 + 8 * n + gq, M - 1)) * K + (T / 4) * c;
+    float acc[R][NT][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[r][n][i] = 0.f;
+    constexpr uint32_t kOnes = 0x3C003C00u;                // half2(1, 1)
+    for (int j = warp; j < st.G; j += WARPS) {
+        uint32_t W[NT][F];                                 // columns 2i, 2i + 1
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int v = 0; v < F / 4; ++v) {
+                const uint4 q4 = *reinterpret_cast<const uint4*>(xp[n] + static_cast<size_t>(T) * j + 8 * v);
+                W[n][4 * v] = q4.x; W[n][4 * v + 1] = q4.y; W[n][4 * v + 2] = q4.z; W[n][4 * v + 3] = q4.w;
             }
-            const float2 sf = __half22float2(*reinterpret_cast<const __half2*>(&raw.s2));
-            const float2 zf = __half22float2(*reinterpret_cast<const __half2*>(&raw.z2));
+        SmallRaw<T> raw[R];
 #pragma unroll
-            for (int m = 0; m < MT; ++m) {
-                if (m0 + m >= M) break;
-                const uint4* xp = reinterpret_cast<const uint4*>(x + static_cast<size_t>(m0 + m) * K + T * j + C * c);
-                float d0 = 0.f, d1 = 0.f, sx = 0.f;
+        for (int r = 0; r < R; ++r) raw[r] = next[r];
+        const int b = st.bits[j];
+        if (j + WARPS < st.G) load(j + WARPS);
+        uint2 bf[NT][STEPS];                               // (f, f + T/8) for f = 2 step and 2 step + 1
 #pragma unroll
-                for (int v = 0; v < C / 8; ++v) {
-                    const uint4 xv4 = xp[v];
-                    const uint32_t w4[4] = {xv4.x, xv4.y, xv4.z, xv4.w};
+        for (int n = 0; n < NT; ++n)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float2 xv = __half22float2(*reinterpret_cast<const __half2*>(&w4[i]));
-                        d0 = fmaf(static_cast<float>(q[0][8 * v + 2 * i]), xv.x, d0);
-                        d1 = fmaf(static_cast<float>(q[1][8 * v + 2 * i]), xv.x, d1);
-                        d0 = fmaf(static_cast<float>(q[0][8 * v + 2 * i + 1]), xv.y, d0);
-                        d1 = fmaf(static_cast<float>(q[1][8 * v + 2 * i + 1]), xv.y, d1);
-                        sx += xv.x;
-                        sx += xv.y;
-                    }
-                }
-                acc[m][0] = fmaf(sf.x, fmaf(-zf.x, sx, d0), acc[m][0]);
-                acc[m][1] = fmaf(sf.y, fmaf(-zf.y, sx, d1), acc[m][1]);
-            }
+            for (int i = 0; i < STEPS; ++i)
+                bf[n][i] = make_uint2(__byte_perm(W[n][i], W[n][F / 2 + i], 0x5410), __byte_perm(W[n][i], W[n][F / 2 + i], 0x7632));
+        float sx[NT][4];
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            sx[n][0] = sx[n][1] = sx[n][2] = sx[n][3] = 0.f;
+#pragma unroll
+            for (int i = 0; i < STEPS; ++i) mma_f16(sx[n], kOnes, kOnes, kOnes, kOnes, bf[n][i]);
         }
 #pragma unroll
-        for (int m = 0; m < MT; ++m) {
+        for (int r = 0; r < R; ++r) {
+            uint32_t q0[F], q1[F];
+            small_codes<T>(raw[r], b, 0, one, q0);
+            small_codes<T>(raw[r], b, 1, one, q1);
+            const float2 sf = __half22float2(small_h2(raw[r].s2)), zf = __half22float2(small_h2(raw[r].z2));
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float v = acc[m][h];
-                v += __shfl_xor_sync(0xffffffffu, v, 1);
-                v += __shfl_xor_sync(0xffffffffu, v, 2);
-                if (c == 0) red[warp][m][2 * gq + h] = v;
+            for (int n = 0; n < NT; ++n) {
+                float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int i = 0; i < STEPS; ++i) mma_f16(d, q0[2 * i], q1[2 * i], q0[2 * i + 1], q1[2 * i + 1], bf[n][i]);
+                acc[r][n][0] = fmaf(sf.x, fmaf(-zf.x, sx[n][0], d[0]), acc[r][n][0]);
+                acc[r][n][1] = fmaf(sf.x, fmaf(-zf.x, sx[n][1], d[1]), acc[r][n][1]);
+                acc[r][n][2] = fmaf(sf.y, fmaf(-zf.y, sx[n][0], d[2]), acc[r][n][2]);
+                acc[r][n][3] = fmaf(sf.y, fmaf(-zf.y, sx[n][1], d[3]), acc[r][n][3]);
             }
         }
-        __syncthreads();
-        for (int e = threadIdx.x; e < MT * 16; e += blockDim.x) {
-            const int m = e >> 4, r = e & 15;
-            if (m0 + m < M) {
-                float v = 0.f;
+    }
 #pragma unroll
-                for (int k = 0; k < kSmallWarps; ++k) v += red[k][m][r];
-                y[static_cast<size_t>(m0 + m) * N + 16 * t + r] = __float2half_rn(v);
-            }
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)                    // token 2c + h of the tile, rows 2gq and 2gq + 1
+                *reinterpret_cast<float2*>(&red[warp][8 * n + 2 * c + h][16 * r + 2 * gq]) = make_float2(acc[r][n][h], acc[r][n][2 + h]);
+    __syncthreads();
+    for (int e = threadIdx.x; e < 8 * NT * 8 * R; e += 32 * WARPS) {
+        const int m = e / (8 * R), r2 = 2 * (e - m * 8 * R);
+        if (m0 + m >= M || 16 * t0 + r2 >= N) continue;
+        float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < WARPS; ++k) {
+            const float2 p = *reinterpret_cast<const float2*>(&red[k][m][r2]);
+            v.x += p.x;
+            v.y += p.y;
         }
-        __syncthreads();
+        *reinterpret_cast<__half2*>(y + static_cast<size_t>(m0 + m) * N + 16 * t0 + r2) = __floats2half2_rn(v.x, v.y);
     }
 }
 
-// ------------------------------------------------------------------------------------------ dense product with fp16 output
-// y[m][n] = sum_k x[m][k] * W[n][k]: fp16 operands, fp32 accumulation on mma.sync m16n8k16, fp16 output.  A block of
-// four warps takes 64 tokens x 64 rows, warp w the tokens 16w .. 16w+15; fragments are read from global memory.
-__global__ void __launch_bounds__(128) dense_f16_kernel(const __half* __restrict__ x, const __half* __restrict__ W, __half* __restrict__ y,
-                                                        int M, int N, int K) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int gq = lane >> 2, c = lane & 3;
-    const int m0 = blockIdx.y * 64 + 16 * warp, n0 = blockIdx.x * 64;
-    const int ma = min(m0 + gq, M - 1), mb = min(m0 + gq + 8, M - 1);          // clamped for the loads, masked at the store
-    const uint32_t* xa = reinterpret_cast<const uint32_t*>(x + static_cast<size_t>(ma) * K) + c;
-    const uint32_t* xb = reinterpret_cast<const uint32_t*>(x + static_cast<size_t>(mb) * K) + c;
-    const uint32_t* wr[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) wr[t] = reinterpret_cast<const uint32_t*>(W + static_cast<size_t>(min(n0 + 8 * t + gq, N - 1)) * K) + c;
-    float acc[8][4];
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-#pragma unroll
-        for (int r = 0; r < 4; ++r) acc[t][r] = 0.f;
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        const int o = k0 >> 1;
-        const uint32_t a0 = __ldg(xa + o), a1 = __ldg(xb + o), a2 = __ldg(xa + o + 4), a3 = __ldg(xb + o + 4);
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            const uint32_t b0 = __ldg(wr[t] + o), b1 = __ldg(wr[t] + o + 4);
-            asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                         : "+f"(acc[t][0]), "+f"(acc[t][1]), "+f"(acc[t][2]), "+f"(acc[t][3])
-                         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-        }
-    }
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        const int n = n0 + 8 * t + 2 * c;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int m = m0 + gq + 8 * h;
-            if (m < M && n < N) *reinterpret_cast<__half2*>(y + static_cast<size_t>(m) * N + n) = __floats2half2_rn(acc[t][2 * h], acc[t][2 * h + 1]);
-        }
-    }
+template <int T, int NT, int R, int WARPS>
+static cudaError_t launch_small(const __half* x, const uint8_t* packed, const __half* scales, const __half* zeros, __half* y, int M, int N, int K,
+                                const SmallTable& st, cudaStream_t s) {
+    PdlLaunch l(static_cast<unsigned>(((N >> 4) + R - 1) / R), 32 * WARPS, 0, s);
+    l.cfg.gridDim.y = static_cast<unsigned>((M + 8 * NT - 1) / (8 * NT));
+    return cudaLaunchKernelEx(&l.cfg, linear_small_kernel<T, NT, R, WARPS>, x, packed, scales, zeros, y, M, N, K, 0x64006400u, st);
+}
+// 16 rows and 16 warps per block up to 16 tokens (blocks are few and the chain of a warp is what counts), 32 rows and 8 warps
+// for more: the loads of x and the ones MMAs serve two row tiles.
+template <int T>
+static cudaError_t launch_small_for(const __half* x, const uint8_t* packed, const __half* scales, const __half* zeros, __half* y, int M, int N,
+                                    int K, const SmallTable& st, cudaStream_t s) {
+    if (M <= 8) return launch_small<T, 1, 1, 16>(x, packed, scales, zeros, y, M, N, K, st, s);
+    if (M <= 16) return launch_small<T, 2, 1, 16>(x, packed, scales, zeros, y, M, N, K, st, s);
+    return launch_small<T, 4, 2, 8>(x, packed, scales, zeros, y, M, N, K, st, s);
 }
 
 // ------------------------------------------------------------------------------------------ host side
@@ -299,8 +321,8 @@ int small_workspace_bytes(int M, int N, int K, int g, const uint8_t* bits_host, 
     SmallTable st;
     const int rc = make_small_table(N, K, g, bits_host, &st);
     if (rc != SLIM_OK) return rc;
-    // the batched path materialises the fp16 weights behind the status header
-    *out_bytes = M > SLIM_GEMV_MAX_M ? 256 + static_cast<size_t>(N) * K * sizeof(__half) : 256;
+    (void)M;
+    *out_bytes = 256;                                      // the status header
     return SLIM_OK;
 }
 
@@ -363,27 +385,7 @@ int small_linear(const void* x, const void* packed, const uint8_t* bits_host, co
     const __half* sc = static_cast<const __half*>(scales);
     const __half* zp = static_cast<const __half*>(zeros);
     __half* yh = static_cast<__half*>(y);
-    if (M <= SLIM_GEMV_MAX_M) {
-        const unsigned grid = static_cast<unsigned>(N / 16);
-        if (g == 32) {
-            if (M == 1) gemv_small_kernel<32, 1><<<grid, 32 * kSmallWarps, 0, s>>>(xh, pk, sc, zp, yh, M, N, K, st);
-            else if (M <= 4) gemv_small_kernel<32, 4><<<grid, 32 * kSmallWarps, 0, s>>>(xh, pk, sc, zp, yh, M, N, K, st);
-            else gemv_small_kernel<32, 8><<<grid, 32 * kSmallWarps, 0, s>>>(xh, pk, sc, zp, yh, M, N, K, st);
-        } else {
-            if (M == 1) gemv_small_kernel<64, 1><<<grid, 32 * kSmallWarps, 0, s>>>(xh, pk, sc, zp, yh, M, N, K, st);
-            else if (M <= 4) gemv_small_kernel<64, 4><<<grid, 32 * kSmallWarps, 0, s>>>(xh, pk, sc, zp, yh, M, N, K, st);
-            else gemv_small_kernel<64, 8><<<grid, 32 * kSmallWarps, 0, s>>>(xh, pk, sc, zp, yh, M, N, K, st);
-        }
-        SLIM_CUDA_TRY(cudaGetLastError());
-        return SLIM_OK;
-    }
-    if (workspace_bytes < 256 + static_cast<size_t>(N) * K * sizeof(__half)) return SLIM_ERR_WORKSPACE;
-    __half* Wd = reinterpret_cast<__half*>(static_cast<uint8_t*>(workspace) + 256);
-    const int rd = small_dequant_into(packed, st, scales, zeros, Wd, N, K, s);
-    if (rd != SLIM_OK) return rd;
-    const dim3 grid((N + 63) / 64, (M + 63) / 64);
-    dense_f16_kernel<<<grid, 128, 0, s>>>(xh, Wd, yh, M, N, K);
-    SLIM_CUDA_TRY(cudaGetLastError());
+    SLIM_CUDA_TRY(g == 32 ? launch_small_for<32>(xh, pk, sc, zp, yh, M, N, K, st, s) : launch_small_for<64>(xh, pk, sc, zp, yh, M, N, K, st, s));
     return SLIM_OK;
 }
 
