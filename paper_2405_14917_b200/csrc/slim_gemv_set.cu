@@ -122,27 +122,17 @@ __device__ __forceinline__ void stage_task_one(const SetLayer& L, uint8_t* ws, i
     stage_groups_i8(L.x + pi * SLIM_GROUP, live ? grp : nullptr, L.bits[pi], lane);
 }
 
-// Staging task `pi` of layer L (one warp) of any other set: token pi / G, group pi % G.
+// Staging task `pi` of layer L (one warp) of any other set: four tokens from 4 (pi / G) on, group pi % G.  What the workspace
+// holds for tokens that the layer does not have is multiplied like the rest and never stored.
 __device__ __forceinline__ void stage_task(const SetLayer& L, uint8_t* ws, int pi, int lane) {
-    const int m = pi / L.G, j = pi - m * L.G;        // m < MP
+    const int q = pi / L.G, j = pi - q * L.G;
+    if (4 * q >= L.M) return;
     uint8_t* grp = ws + L.x_off + staged_group_offset(j, L.pre3[j], L.MP);
-    float2* sxe = reinterpret_cast<float2*>(grp);
-    if (m < L.M) {
-        const float2 r = stage_group(L.x + static_cast<size_t>(m) * L.K + j * SLIM_GROUP, grp + staged_header_bytes(L.MP), L.bits[j], m, L.MP, lane);
-        if (lane == 0) sxe[m] = r;
-    } else {
-        // a token the layer does not have: zero fragments in every slice of the group
-        const int cc = lane & 3, mi = lane >> 2;
-        for (int sl = 0; sl < slice_count(L.bits[j]); ++sl)
-            *reinterpret_cast<uint2*>(grp + staged_header_bytes(L.MP) + (((static_cast<size_t>(sl) * 8 + mi) * L.MP + m) * 4 + cc) * 8) = make_uint2(0u, 0u);
-    }
-    if (m == 0)
-        for (int t = lane; t < max(L.MP, 16); t += 32)
-            if (t >= L.M) sxe[t] = make_float2(0.f, 1.f);                          // absent tokens read 0
+    stage_tokens(L.x + j * SLIM_GROUP, L.K, L.bits[j], 4 * q, L.M, L.MP, grp + staged_header_bytes(L.MP), reinterpret_cast<float2*>(grp), lane);
 }
 
-// One warp per (layer, token, group), or eight lanes per (layer, group) if every layer has ONE token: fragments and sums
-// of the whole set, once.
+// One warp per (layer, four tokens, group), or eight lanes per (layer, group) if every layer has ONE token: fragments and
+// sums of the whole set, once.  n_tasks and a layer's first task count (token, group) pairs.
 template <bool ONE>
 __global__ void __launch_bounds__(256) gemv_set_stage_kernel(const SetLayer* __restrict__ layers, uint8_t* ws, int n_layers, int n_tasks,
                                                              int n_counters) {
@@ -150,7 +140,7 @@ __global__ void __launch_bounds__(256) gemv_set_stage_kernel(const SetLayer* __r
     pdl_launch_dependents();
     stage_clear_counters(ws, n_counters);
     const int lane = threadIdx.x & 31;
-    const int task = ONE ? blockIdx.x * 32 + (threadIdx.x >> 3) : blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int task = ONE ? blockIdx.x * 32 + (threadIdx.x >> 3) : 4 * (blockIdx.x * 8 + (threadIdx.x >> 5));
     // The layer of a task is the last one whose first task is not above it.  A search through the descriptors is a
     // chain of dependent loads from global memory (eight for the 224 layers of a 7B sweep, most of this kernel's time),
     // so a set of up to kStageTable layers first puts their first tasks into shared memory, all loads in flight at once.
@@ -172,7 +162,7 @@ __global__ void __launch_bounds__(256) gemv_set_stage_kernel(const SetLayer* __r
         __syncwarp();
         stage_task_one(layers[lo], ws, task < n_tasks ? pi : 0, lane, task < n_tasks);
     } else {
-        stage_task(layers[lo], ws, pi, lane);
+        stage_task(layers[lo], ws, pi >> 2, lane);
     }
 }
 
@@ -680,7 +670,7 @@ __global__ void __launch_bounds__(256) set_single_stage_kernel(const __grid_cons
         return;
     }
     const int task = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (task < n_tasks) stage_task(d, ws, task, threadIdx.x & 31);
+    if (4 * task < n_tasks) stage_task(d, ws, task, threadIdx.x & 31);
 }
 
 // ------------------------------------------------------------------------------------------ self-test of the bounded wait
@@ -1003,7 +993,7 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
     // blocks are many and early launches measured 1 to 4 % slower, so those keep plain stream order.
     const bool early = M == 1;
     {
-        const int per_block = M == 1 ? 32 : 8;
+        constexpr int per_block = 32;                    // tasks
         PdlLaunch l(static_cast<unsigned>((info.stage_tasks + per_block - 1) / per_block), 256, 0, stream, early);
         SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, set_single_stage_kernel, d, plan, prm.ws, grid, r.n_rb, r.sp, info.stage_tasks, info.n_counters));
     }
@@ -1211,7 +1201,7 @@ int slim_mpq_gemv_set(const slim_gemv_set_info* info, const void* plan, void* wo
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     {
         const bool one = info->max_tokens == 1;
-        const int per_block = one ? 32 : 8;
+        constexpr int per_block = 32;                // tasks
         slim::PdlLaunch l(static_cast<unsigned>((info->stage_tasks + per_block - 1) / per_block), 256, 0, s, false);
         SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, one ? slim::gemv_set_stage_kernel<true> : slim::gemv_set_stage_kernel<false>, prm.layers, prm.ws, info->n_layers, info->stage_tasks, info->n_counters));
     }
