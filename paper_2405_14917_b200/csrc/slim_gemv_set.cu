@@ -179,6 +179,7 @@ __device__ __forceinline__ void mma_f16_first(float (&d)[4], uint32_t a0, uint32
 // counts itself on the row block's counter of this warp.  The warp that counts last sees the other parts and adds all
 // parts in part order, so the result does not depend on which part came last: y = fp16 of that sum.  Out of line: it
 // runs once per item.
+template <int Q>
 __device__ __noinline__ void finish_parts(const SetParams& p, int layer, int rb, int warp, int lane, int tile0, int n_act, int M, int N) {
     const SetLayer* L = p.layers + layer;
     __threadfence();                                    // this lane's partial sums before the count
@@ -193,18 +194,33 @@ __device__ __noinline__ void finish_parts(const SetParams& p, int layer, int rb,
     const float* part = reinterpret_cast<const float*>(p.ws + L->part_off);
     const size_t MN = static_cast<size_t>(M) * N;
     __half* y = L->y;
-    // 16 * n_act rows x M tokens as pairs of rows: pair i of token m
-    const int pairs = 8 * n_act;
-    for (int i = lane; i < pairs * M; i += 32) {
-        const int m = i / pairs, r = i - m * pairs;
-        const size_t at = static_cast<size_t>(m) * N + 16 * tile0 + 2 * r;
-        float2 sum = __ldcg(reinterpret_cast<const float2*>(part + at));
-        for (int k = 1; k < S; ++k) {
-            const float2 v = __ldcg(reinterpret_cast<const float2*>(part + k * MN + at));
-            sum.x += v.x;
-            sum.y += v.y;
+    // 16 * n_act rows x M tokens as pairs of rows: pair i of token m.  Q pairs of a lane at a time, so that their loads are in
+    // flight together: the warp holds up the ring's slots meanwhile (one 70B block of 16 tokens as a set: 199 us with one pair
+    // at a time, 159 with two).  What is live here costs registers in the loop that calls it, so four only where one CTA has
+    // the SM: with four in the two-CTA forms their loops spilled, 7B sweep of one token 89 -> 93 us.
+    const int pairs = 8 * n_act, total = pairs * M;
+    for (int i0 = lane; i0 < total; i0 += 32 * Q) {
+        float2 sum[Q];
+        unsigned int at[Q];                             // below 64 * N
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int i = min(i0 + 32 * q, total - 1), m = i / pairs;
+            at[q] = static_cast<unsigned int>(m * N + 16 * tile0 + 2 * (i - m * pairs));
+            sum[q] = __ldcg(reinterpret_cast<const float2*>(part + at[q]));
         }
-        *reinterpret_cast<__half2*>(y + at) = __floats2half2_rn(sum.x, sum.y);
+        const float* next = part;
+        for (int k = 1; k < S; ++k) {
+            next += MN;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const float2 v = __ldcg(reinterpret_cast<const float2*>(next + at[q]));
+                sum[q].x += v.x;
+                sum[q].y += v.y;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if (i0 + 32 * q < total) *reinterpret_cast<__half2*>(y + at[q]) = __floats2half2_rn(sum[q].x, sum[q].y);
     }
 }
 
@@ -358,7 +374,7 @@ __device__ __forceinline__ void consume_one(const SetParams& p, const uint32_t s
                     else *reinterpret_cast<__half2*>(reinterpret_cast<__half*>(yword) + row) = __floats2half2_rn(acc0, acc2);
                 }
             }
-            if (counts & kItemPartial) finish_parts(p, layer, rb, warp, lane, tile0, n_act, 1, N);
+            if (counts & kItemPartial) finish_parts<1>(p, layer, rb, warp, lane, tile0, n_act, 1, N);
         }
     }
 }
@@ -517,7 +533,7 @@ __device__ __forceinline__ void consume_f16(const SetParams& p, const uint32_t s
                     }
                 }
             }
-            if (partial) finish_parts(p, layer, rb, warp, lane, tile0, n_act, M, N);
+            if (partial) finish_parts<NT <= 2 ? 2 : 4>(p, layer, rb, warp, lane, tile0, n_act, M, N);
         }
     }
 }
@@ -527,12 +543,12 @@ constexpr uint32_t kSetOffAbort = 16 * kSetMaxSlots;          // after the full 
 constexpr uint32_t kSetOffDesc = 1024;                        // the producer's copy of its layer's descriptor
 constexpr uint32_t kSetOffRing = (kSetOffDesc + kSetProducers * sizeof(SetLayer) + 127) / 128 * 128;
 
-// NT: 8-token MMA tiles, 1 (every M <= 8) or 2.  ONE: every layer has a single token; then only
+// NT: 8-token MMA tiles, as many as the widest layer needs.  ONE: every layer has a single token; then only
 // column 0 of the MMA results is ever used, so every lane feeds token 0's fragment and folds token 0.
 // TPW: 16-row tiles per consumer warp (an item is 8 * TPW tiles; always 2 today); two tiles share the fragment
 // loads and the per-group bookkeeping.
 template <int NT, bool ONE, int TPW>
-__global__ void __launch_bounds__(kSetThreads, NT >= 4 ? 1 : kSetCtasPerSm) gemv_set_kernel(const __grid_constant__ SetParams p) {
+__global__ void __launch_bounds__(kSetThreads, NT >= 3 ? 1 : kSetCtasPerSm) gemv_set_kernel(const __grid_constant__ SetParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -696,6 +712,7 @@ __global__ void __launch_bounds__(32) wait_selftest_kernel(uint8_t* ws, unsigned
 // What the whole set fixes: token tiles, slot geometry, ring depth, grid, sizes.
 struct SetGeometry {
     int nt, bmax, mmax, tpw, mpad;     // tpw: tiles per consumer warp; mpad: tokens in the staged layout
+    int mres;                          // tokens that the workspace has room for: 2 (digit form), 8, 16, 32 or 64
     int slot_bytes;
     int n_slots, grid, ctas_per_sm;
     int split;                         // parts the groups of every row block are cut into (fewer for layers with few groups)
@@ -714,11 +731,12 @@ static int layer_split(int split, int G) {
 }
 
 static size_t align_to(size_t v, size_t a) { return (v + a - 1) / a * a; }
-// Workspace of one layer: per group the sums and the fragments of its slices.
+// Workspace set aside for one layer: per group the sums and the fragments of its slices, for the reserved number of tokens
+// (the staged layout takes no more).
 static size_t layer_ws_bytes(int M, const GroupTable& gt) {
     int slots = gt.G;
     for (int j = 0; j < gt.G; ++j) slots += gt.bits[j] == 3 ? 1 : 0;
-    return align_to(static_cast<size_t>(gt.G) * staged_header_bytes(M) + static_cast<size_t>(slots) * 256 * M, 128);
+    return align_to(static_cast<size_t>(gt.G) * (M == 2 ? 128 : staged_header_bytes(M)) + static_cast<size_t>(slots) * 256 * M, 128);
 }
 // Work of an item for the deal.  The kernel is bound by the instructions it issues, so a (tile, group)
 // weighs what a consumer warp issues for it: about 70 / 73 / 120 / 80 instructions at 1 / 2 / 3 / 4 bits
@@ -745,8 +763,12 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
     sg->ws_bytes = 256;
     for (int l = 0; l < n_layers; ++l) sg->mmax = sg->mmax > layers[l].M ? sg->mmax : layers[l].M;
     sg->tpw = 2;
-    // one token: the 8-bit digit form, 512 bytes per slice; else the tokens of the widest layer rounded up to 8, 16, 32, 64
-    sg->mpad = sg->mmax <= 1 ? 2 : (sg->mmax <= 8 ? 8 : (sg->mmax <= 16 ? 16 : (sg->mmax <= 32 ? 32 : 64)));
+    // one token: the 8-bit digit form, 512 bytes per slice; else the tokens of the widest layer rounded up to 8: the kernel is
+    // bound by its MMAs, and with 8, 16, 32 or 64 alone 40 tokens paid for 64 (four LLaMA-7B blocks
+    // at 3 bits, 17 / 40 / 56 tokens: 227 / 425 / 428 us -> 181 / 267 / 368; from 17 tokens on one CTA per SM, whose registers
+    // hold the accumulators: two gave 197 at 17)
+    sg->mpad = sg->mmax <= 1 ? 2 : (sg->mmax + 7) / 8 * 8;
+    sg->mres = sg->mmax <= 1 ? 2 : (sg->mmax <= 8 ? 8 : (sg->mmax <= 16 ? 16 : (sg->mmax <= 32 ? 32 : 64)));
     const int tpi = kSetConsumers * sg->tpw;          // tiles per item
     for (int l = 0; l < n_layers; ++l) {
         const slim_layer& L = layers[l];
@@ -759,13 +781,13 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
         const int items = ((L.N >> 4) + tpi - 1) / tpi;
         sg->n_items += items;
         sg->n_tasks += static_cast<long long>(sg->mpad == 2 ? 1 : sg->mpad) * gt.G;   // staging tasks: (token, group)
-        sg->ws_bytes += layer_ws_bytes(sg->mpad, gt);
+        sg->ws_bytes += layer_ws_bytes(sg->mres, gt);
     }
     if (sg->n_items > 0x3fffffff || sg->n_tasks > 0x3fffffff) return SLIM_ERR_UNSUPPORTED;
     sg->nt = sg->mmax <= 1 ? 1 : sg->mpad / 8;
     // A set with fewer row blocks than persistent CTAs cuts the groups of every row block into parts (items of their
     // own, fp32 partial outputs in the workspace, added in part order by the consumer warp whose part lands last).
-    const long long want = static_cast<long long>(set_sm_count()) * (sg->nt >= 4 ? 1 : kSetCtasPerSm);
+    const long long want = static_cast<long long>(set_sm_count()) * (sg->nt >= 3 ? 1 : kSetCtasPerSm);
     sg->split = 1;
     if (sg->n_items < 2 * want) {
         // the number of parts that fills the last wave of CTAs best (the smallest one within 2 % of the best)
@@ -804,7 +826,7 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
     // as many CTAs per SM (kSetCtasPerSm at most) as still leaves each a ring of 4 slots
     const size_t per_sm = 224 * 1024;
     size_t budget = 0;
-    for (sg->ctas_per_sm = sg->nt >= 4 ? 1 : kSetCtasPerSm; sg->ctas_per_sm >= 1; --sg->ctas_per_sm) {
+    for (sg->ctas_per_sm = sg->nt >= 3 ? 1 : kSetCtasPerSm; sg->ctas_per_sm >= 1; --sg->ctas_per_sm) {
         budget = per_sm / sg->ctas_per_sm - 1024 - kSetOffRing;   // 1 KB per CTA is reserved by the system
         if (budget / sg->slot_bytes >= 4 || sg->ctas_per_sm == 1) break;
     }
@@ -895,7 +917,7 @@ static bool route_layout(int M, int N, int K, int g, const uint8_t* bits_host, c
     r->plan_off = kSetOffCounters + r->sg.cnt_bytes;
     r->plan_bytes = set_plan_bytes(1, static_cast<long long>(r->n_rb) * r->sp);
     r->x_off = r->plan_off + align_to(r->plan_bytes, 256);
-    r->part_off = r->x_off + layer_ws_bytes(r->sg.mpad, gt);
+    r->part_off = r->x_off + layer_ws_bytes(r->sg.mres, gt);
     r->total = r->part_off + (r->sp > 1 ? align_to(static_cast<size_t>(r->sp) * M * N * sizeof(float), 128) : 0);
     return true;
 }
@@ -914,7 +936,7 @@ static int set_params(const slim_gemv_set_info* info, const void* plan, void* wo
     if (info == nullptr || plan == nullptr) return SLIM_ERR_INVALID_ARG;
     if (info->n_layers < 1 || info->grid < 1 || info->grid > kSetMaxGrid || info->n_slots < 2 ||
         info->n_slots > kSetMaxSlots || info->slot_bytes < 128 || info->slot_bytes % 128 != 0 ||
-        (info->token_tiles != 1 && info->token_tiles != 2 && info->token_tiles != 4 && info->token_tiles != 8) ||
+        info->token_tiles < 1 || info->token_tiles > 8 ||
         info->max_tokens < 1 || info->max_tokens > 8 * info->token_tiles ||
         info->tiles_per_warp != 2 ||
         info->max_bits < 1 || info->max_bits > 4 || info->stage_tasks < 1 || info->split < 1 || info->split > kSetMaxSplit ||
@@ -946,11 +968,10 @@ static int set_params(const slim_gemv_set_info* info, const void* plan, void* wo
 
 // The persistent kernel of the set in the form its token count asks for.
 static int launch_set_for(const slim_gemv_set_info* info, const SetParams& prm, size_t smem, cudaStream_t s, bool early) {
-    const cudaError_t e = info->max_tokens == 1 ? launch_set<1, true, 2>(prm, info->grid, smem, s, early)
-                        : info->token_tiles == 8 ? launch_set<8, false, 2>(prm, info->grid, smem, s, early)
-                        : info->token_tiles == 4 ? launch_set<4, false, 2>(prm, info->grid, smem, s, early)
-                        : info->token_tiles == 1 ? launch_set<1, false, 2>(prm, info->grid, smem, s, early)
-                                                 : launch_set<2, false, 2>(prm, info->grid, smem, s, early);
+    using Launch = cudaError_t (*)(const SetParams&, int, size_t, cudaStream_t, bool);
+    static const Launch forms[8] = {launch_set<1, false, 2>, launch_set<2, false, 2>, launch_set<3, false, 2>, launch_set<4, false, 2>,
+                                    launch_set<5, false, 2>, launch_set<6, false, 2>, launch_set<7, false, 2>, launch_set<8, false, 2>};
+    const cudaError_t e = info->max_tokens == 1 ? launch_set<1, true, 2>(prm, info->grid, smem, s, early) : forms[info->token_tiles - 1](prm, info->grid, smem, s, early);
     SLIM_CUDA_TRY(e);
     return SLIM_OK;
 }
@@ -1075,7 +1096,7 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
         for (int l = 0; l < n_layers; ++l) {
             slim::GroupTable gt;
             slim::make_group_table(layers_host[l].N, layers_host[l].K, g, layers_host[l].bits_host, &gt);
-            off += slim::layer_ws_bytes(sg.mpad, gt);
+            off += slim::layer_ws_bytes(sg.mres, gt);
         }
         for (int l = 0; l < n_layers; ++l) {
             const slim_layer& L = layers_host[l];
@@ -1099,7 +1120,7 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
         }
         x_off[l] = same >= 0 ? x_off[same] : ws_off;
         slim::fill_descriptor(L, gt, sg.mpad, task, x_off[l], sp, part_off[l], cnt0, &d);
-        ws_off += slim::layer_ws_bytes(sg.mpad, gt);
+        ws_off += slim::layer_ws_bytes(sg.mres, gt);
         SLIM_CUDA_TRY(cudaMemcpyAsync(plan_dev + slim::kSetPlanHeader + static_cast<size_t>(l) * sizeof d, &d, sizeof d,
                                       cudaMemcpyHostToDevice, s));
         const int n_rb = ((L.N >> 4) + tpi - 1) / tpi;

@@ -62,3 +62,21 @@ def test_wider_groups(g):
     y = _run(L["x"], L["codes"], L["bits"][::step].copy(), scales.copy(), zeros.copy(), g=g)
     ref = orc.linear_f64(L["x"], L["codes"], np.repeat(scales, step, axis=0), np.repeat(zeros, step, axis=0))
     check_output(y, ref, f"g={g}")
+
+
+@pytest.mark.parametrize("M", [20, 24, 33, 41, 49, 57])
+def test_sets_of_every_number_of_token_tiles(M):
+    """Layer sets whose widest layer needs three, five, six, seven or eight MMA tiles, next to layers of fewer tokens; few
+    row blocks, so that these are cut into parts."""
+    layers = [oracle_layer(304, 1152, 3, M, seed_name="set-tiles", block=0), oracle_layer(512, 1024, 2, 3, seed_name="set-tiles", block=1)]
+    entries = []
+    for L in layers:
+        layer = slim.QuantLinear(torch.from_numpy(orc.pack(L["codes"], L["bits"])).cuda(), L["bits"], torch.from_numpy(L["scales"]).cuda(),
+                                 torch.from_numpy(L["zeros"]).cuda(), L["N"], L["K"])
+        entries.append((layer, torch.from_numpy(L["x"]).cuda(), torch.full((L["M"], L["N"]), float("nan"), dtype=torch.float16, device="cuda")))
+    s = slim.LayerSet(entries)
+    assert s.info["token_tiles"] == (M + 7) // 8
+    s.run()
+    s.check()
+    for L, (_, _, y) in zip(layers, entries):
+        check_output(y.cpu().numpy(), orc.linear_f64(L["x"], L["codes"], L["scales"], L["zeros"]), f"M={L['M']}")
