@@ -869,7 +869,7 @@ def group_size_entries(device, timer):
         achieved = alg / (ms * 1e-3) / 1e9
         out.append({"name": f"single-4096x4096-avg2-m1-g{g}", "metric": f"one 4096 x 4096 layer per launch, avg 2-bit, M = 1, group size {g} (slim_mpq_gemv, 64 rotating copies)",
                     "value": achieved, "unit": UNIT, "ms_per_step": ms, "timing": tm,
-                    "kernel": "gemv_small_kernel (CUDA cores)" if g < 128 else "gemv_one_kernel (tensor cores)",
+                    "kernel": "linear_small_kernel (tensor cores)" if g < 128 else "gemv_one_kernel (tensor cores)",
                     "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_kind": peak_kind,
                                  "avg_launch_us": 1e3 * ms / copies, "algorithmic_bytes_per_launch": alg / copies},
                     "config": {"workload": f"single-4096x4096-avg2-m1-g{g}", "g": g, "layers": copies, "algorithmic_bytes_per_step": alg,
