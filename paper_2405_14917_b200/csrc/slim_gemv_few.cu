@@ -1,4 +1,5 @@
-// slim_mpq_gemv for 2 to 16 tokens in one launch, sm_100a: one layer cut over the whole GPU.
+// slim_mpq_gemv for 2 to 16 tokens (slim_mpq_gemm: small layers, up to 32) in one launch, sm_100a: one layer cut over the whole
+// GPU.
 //
 // A layer of a few tens of megabytes is over in 5 to 20 us, so what counts is that every byte is requested at once, that
 // no CTA waits for a second wave, and the length of the chain launch - x - products - sums.  A cluster of CS CTAs owns
@@ -34,9 +35,11 @@ constexpr int kFewWarps = 16;                           // 128 registers a threa
 constexpr int kFewThreads = 32 * kFewWarps;
 constexpr int kFewMaxSlots = 64;
 constexpr int kFewMaxPw = 4;                            // tile pairs per warp
+constexpr int kFewMaxNt = 4;                            // 8-token MMA tiles
 constexpr int kFewMaxKw = 8;                            // warps that share a set of tile pairs
 constexpr uint32_t kFewOffAbort = 16 * kFewMaxSlots;    // after the full and empty barriers
-constexpr uint32_t kFewOffE = kFewOffAbort + 128;       // (sum_k x, 2^(24-S)) of 16 tokens per K-tile of the CTA, then the fragments, then the ring
+constexpr uint32_t kFewOffE = kFewOffAbort + 128;       // (sum_k x, 2^(24-S)) per token and K-tile of the CTA, then the fragments, then the ring
+__host__ __device__ constexpr uint32_t few_sums(int nt) { return nt <= 2 ? 128 : 256; }     // bytes per K-tile
 constexpr size_t kFewMaxSmem = 226 * 1024;
 
 struct FewParams {
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) gemv_few_kernel(const __grid_c
     for (int t = warp; t < gc * ((M + 3) >> 2); t += kFewWarps) {
         const int q = t / gc, i = t - q * gc, j = j0 + i;
         stage_tokens(p.x + j * SLIM_GROUP, p.K, p.bits[j], 4 * q, M, MP, smem + p.off_x + static_cast<size_t>(i + p.pre3[j] - before3) * 8 * MP * 32,
-                     reinterpret_cast<float2*>(smem + kFewOffE + 128 * i), lane);
+                     reinterpret_cast<float2*>(smem + kFewOffE + few_sums(NT) * i), lane);
     }
     __syncthreads();
 
@@ -204,7 +207,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) gemv_few_kernel(const __grid_c
             const uint32_t w = slot + 8u * lane + static_cast<uint32_t>(2 * PW * set) * 256u * b;
             const uint32_t xs = sbase + p.off_x + static_cast<uint32_t>(i + p.pre3[j] - before3) * (8 * MP * 32) + (gq * 4 + c) * 8;
             const uint32_t sz = slot + p.sz_off + static_cast<uint32_t>(2 * PW * set) * 32u + gq * 4;
-            const uint32_t e = sbase + kFewOffE + 128u * i + 16u * c;
+            const uint32_t e = sbase + kFewOffE + few_sums(NT) * i + 16u * c;
             const uint32_t zo = 64u * np;
             switch (b) {
                 case 1: few_group<1, NT, PW>(w, xs, sz, zo, e, acc); break;
@@ -300,11 +303,15 @@ struct FewLaunch {
 
 using FewKernel = void (*)(const FewParams, int);
 static FewKernel few_kernel(int nt, int pw) {
-    static const FewKernel table[2][kFewMaxPw] = {
+    static const FewKernel table[kFewMaxNt][kFewMaxPw] = {
         {gemv_few_kernel<1, 1>, gemv_few_kernel<1, 2>, gemv_few_kernel<1, 3>, gemv_few_kernel<1, 4>},
-        {gemv_few_kernel<2, 1>, gemv_few_kernel<2, 2>, gemv_few_kernel<2, 3>, gemv_few_kernel<2, 4>}};
+        {gemv_few_kernel<2, 1>, gemv_few_kernel<2, 2>, gemv_few_kernel<2, 3>, gemv_few_kernel<2, 4>},
+        {gemv_few_kernel<3, 1>, gemv_few_kernel<3, 2>, nullptr, nullptr},
+        {gemv_few_kernel<4, 1>, gemv_few_kernel<4, 2>, nullptr, nullptr}};
     return table[nt - 1][pw - 1];
 }
+// Tile pairs per warp that leave the accumulators in registers.
+static int few_max_pw(int nt) { return nt <= 2 ? kFewMaxPw : 2; }
 
 // Clusters of 1 << log_cs CTAs that are resident at once (one CTA per SM), asked once per device; the first question also
 // lets the kernels have their shared memory there.
@@ -315,8 +322,8 @@ static int few_clusters(int log_cs) {
     int v = cache[dev][log_cs].load();
     if (v == 0) {
         bool ok = true;
-        for (int nt = 1; nt <= 2; ++nt)
-            for (int pw = 1; pw <= kFewMaxPw; ++pw)
+        for (int nt = 1; nt <= kFewMaxNt; ++nt)
+            for (int pw = 1; pw <= few_max_pw(nt); ++pw)
                 ok = ok && cudaFuncSetAttribute(reinterpret_cast<const void*>(few_kernel(nt, pw)), cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kFewMaxSmem)) == cudaSuccess;
         FewLaunch l(1 << log_cs, 1 << log_cs, kFewMaxSmem, nullptr);
         l.cfg.numAttrs = 1;
@@ -336,7 +343,7 @@ struct FewPlan {
 
 // How a layer is cut; false if it does not fit the kernel.
 static bool few_plan(int M, int N, const GroupTable& gt, int log_cs, FewPlan* pl) {
-    const int cs = 1 << log_cs, clusters = few_clusters(log_cs), P = (N + 31) / 32, nt = M > 8 ? 2 : 1;
+    const int cs = 1 << log_cs, clusters = few_clusters(log_cs), P = (N + 31) / 32, nt = (M + 7) / 8;
     if (clusters <= 0) return false;
     pl->log_cs = log_cs;
     pl->np = (P + clusters - 1) / clusters;
@@ -348,13 +355,13 @@ static bool few_plan(int M, int N, const GroupTable& gt, int log_cs, FewPlan* pl
         gc = gc > b - a ? gc : b - a;
         slices = slices > sl ? slices : sl;
     }
-    pl->off_x = kFewOffE + 128u * static_cast<uint32_t>(gc);
+    pl->off_x = kFewOffE + few_sums(nt) * static_cast<uint32_t>(gc);
     pl->off_ring = pl->off_x + static_cast<uint32_t>(slices) * (8 * 8 * nt * 32);
     pl->sz_off = 2 * pl->np * 256 * bmax;
     pl->slot_bytes = (pl->sz_off + 128 * pl->np + 127) / 128 * 128;
     // pairs per warp and warps per set: the least work of the busiest scheduler among those that fit
     int best = 1 << 30;
-    for (int pw = 1; pw <= kFewMaxPw; ++pw) {
+    for (int pw = 1; pw <= few_max_pw(nt); ++pw) {
         const int npw = (pl->np + pw - 1) / pw;
         if (npw > kFewWarps) continue;
         // a warp of the last set reads (and does not use) up to PW - 1 pairs past the slot's slices, scales and zeros: its slot, or the next
@@ -382,7 +389,7 @@ static bool few_plan(int M, int N, const GroupTable& gt, int log_cs, FewPlan* pl
 // Enqueues the layer and returns SLIM_OK, a negative status on failure, or 1 if this shape is not for this kernel.
 int gemv_few(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y,
              int M, int N, int K, void* workspace, cudaStream_t stream) {
-    if (M < 1 || M > 16 || N <= 0 || gt.G < 1) return 1;
+    if (M < 1 || M > 8 * kFewMaxNt || N <= 0 || gt.G < 1) return 1;
     // CTAs per cluster.  More of them stage less of x each and have more rows, i.e. longer copies and more of the warps on
     // different rows; fewer leave shorter sums to exchange.  Measured with 2, 4 and 8 at 6 tokens: 16384 x 1024 (8 K-tiles)
     // 5.7 / 5.9 / 6.7 us, 4096 x 4096 (32) 7.6 / 6.4 / 7.0, 8192 x 8192 (64) 15.1 / 12.8 / 12.5, 4096 x 11008 (86) 15.5 /
@@ -413,7 +420,7 @@ int gemv_few(const void* x, const void* packed, const GroupTable& gt, const void
         prm.pre3[j + 1] = static_cast<uint16_t>(prm.pre3[j] + (j < gt.G && gt.bits[j] == 3 ? 1 : 0));
     const int cs = 1 << pl.log_cs, grid = ((N + 31) / 32 + pl.np - 1) / pl.np * cs;
     FewLaunch l(grid, cs, pl.smem, stream);
-    SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, few_kernel(M > 8 ? 2 : 1, pl.pw), prm, cs));
+    SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, few_kernel((M + 7) / 8, pl.pw), prm, cs));
     return SLIM_OK;
 }
 

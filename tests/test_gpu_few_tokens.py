@@ -33,6 +33,18 @@ def test_remainders(N, K, avg, M):
     check_output(y, orc.linear_f64(L["x"], L["codes"], L["scales"], L["zeros"]), f"{N}x{K} M={M}")
 
 
+@pytest.mark.parametrize("M", [17, 24, 25, 32])
+@pytest.mark.parametrize("N,K,avg", [(528, 2048, 3), (1040, 8192, 2), (48, 2176, 3)])
+def test_three_and_four_token_tiles(N, K, avg, M):
+    """The batched entry point sends its fewest tokens here."""
+    L = oracle_layer(N, K, avg, M, seed_name="few-batched")
+    ws = slim.new_workspace(M, N, K, L["bits"])
+    y = slim.mpq_gemm(torch.from_numpy(L["x"]).cuda(), torch.from_numpy(orc.pack(L["codes"], L["bits"])).cuda(), L["bits"],
+                      torch.from_numpy(L["scales"]).cuda(), torch.from_numpy(L["zeros"]).cuda(), N, ws)
+    slim.workspace_status(ws)
+    check_output(y.cpu().numpy(), orc.linear_f64(L["x"], L["codes"], L["scales"], L["zeros"]), f"{N}x{K} M={M}")
+
+
 @pytest.mark.parametrize("N,K,M", [(8192, 8192, 8), (4096, 16384, 16), (13824, 2560, 12), (640, 32768, 1), (640, 32768, 16)])
 def test_more_bytes_than_the_ring_holds(N, K, M):
     """K-tiles that take the slot of an earlier one, every width among them; 32768 columns, where one token does not fit
