@@ -334,7 +334,7 @@ def run_sba(args):
                     "h2d_bytes_per_step": int(sum(2 * W.numel() + 2 * x.numel() for W, x, *_ in layers)),
                     "d2h_bytes_per_step": int(sum(8 * (W.shape[1] // 128) + 8 * (W.shape[1] // 256 + 1) * (M + 1) for W, *_ in layers)),
                     "steps": e2e_steps, "ms_per_step": ms_e2e / e2e_steps},
-            "gpu_launches": steps * (candidates * 4 + 2 * len(layers)), "clocks": clocks}
+            "gpu_launches": steps * 5 * len(layers), "clocks": clocks}   # salience, allocation, search, losses, their mean
     print(json.dumps(line), flush=True)
 
 
@@ -484,7 +484,8 @@ def run_gptq(args):
     achieved = flops * steps / (ms * 1e-3) / 1e12
     peak = 148 * 64 * 2 * 1.965e9 / 1e12
     levels = (nb - 1).bit_length()
-    launches = 2 + nb + 2 * (nb - 1) + 2 * levels + 1 + 1 + 4 * G - 1
+    # Hessian, damping, last diagonal block; panel and trailing update per block; inverse; coefficients, start; quantise and update
+    launches = 3 + 2 * (nb - 1) + 2 * levels + 2 + 2 * G - 1
     line = {"metric": "GPTQ error compensation with SQC (Algorithm 1): weights quantised per second (LLaMA-7B 4096x4096 layer, avg 2-bit, g=128)",
             "value": value, "unit": "Mweight/s", "n_gpus": 1, "steps": steps, "warmup": warmup, "ms_per_step": ms / steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
@@ -598,6 +599,11 @@ def decode_buffers(layers, M, device, seed):
     return x_host, y_host, x_dev, y_dev, xs, ys
 
 
+def _layer_launches(layer):
+    """Kernels of one slim_mpq_gemv call: layers of 32 MB or more go through the layer-set kernels (staging and ring)."""
+    return 2 if layer.packed.numel() >= 32 << 20 else 1
+
+
 def decode_sweep(layers, M, device, launch, seed=1234):
     """One pass over `layers` at M tokens as a CUDA graph.  launch: 'set' (one layer-set launch for everything),
     'per-layer' (slim_mpq_gemv per layer) or 'decoder-order' (what a decoder can issue: per block the q/k/v
@@ -618,7 +624,7 @@ def decode_sweep(layers, M, device, launch, seed=1234):
         def run():
             for L, x, y in zip(layers, xs, ys):
                 L.forward(x, ws, out=y)
-        checks, n_dom, n_kern = [], len(layers), len(layers) * (2 if M >= 4 else 1)
+        checks, n_dom, n_kern = [], len(layers), sum(_layer_launches(L) for L in layers)
     else:
         assert len(layers) % 7 == 0
         calls, checks, n_kern = [], [], 0
@@ -630,8 +636,7 @@ def decode_sweep(layers, M, device, launch, seed=1234):
             checks += [qkv.check, gu.check]
             calls += [qkv.run, (lambda i=o: layers[i].forward(xs[i], ws, out=ys[i])), gu.run,
                       (lambda i=down: layers[i].forward(xs[i], ws, out=ys[i]))]
-            one = 1 if M < 4 else 2                                  # slim_mpq_gemv: from four tokens on a kernel stages x first
-            n_kern += sum(1 if st.info["resident_pairs"] > 0 else 2 for st in (qkv, gu)) + 2 * one
+            n_kern += sum(1 if st.info["resident_pairs"] > 0 else 2 for st in (qkv, gu)) + _layer_launches(layers[o]) + _layer_launches(layers[down])
 
         def run():
             for c in calls:
