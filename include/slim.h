@@ -353,8 +353,8 @@ int slim_sba_workspace_bytes(int M, int N, int K, int g, int avg_bits, size_t* o
  * for p = 0 (only if include_uniform), 1, ..., floor(G/2) the p most salient groups get avg_bits+1
  * bits and the p least salient avg_bits-1, and the weight is quantised with slim_quantize_minmax under
  * that map; the candidate's error is the mean over the M calibration tokens of the KL divergence (slim_softmax_kl) of
- * x * W-hat^T against x * W^T, both outputs in fp32: per (row, group) the products with q - z are added exactly as they are
- * in fp16 operands, then scaled and added to the candidate before (consecutive candidates differ in two groups).
+ * x * W-hat^T against x * W^T.  The first is the output of the layer that the map gives: fp16, from the exact weights up to 16
+ * tokens (as slim_mpq_gemv) and from weights rounded to fp16 beyond (as slim_mpq_gemm decodes them); the second is fp32.
  * The first p with the smallest error wins (Algorithm 2 compares with '<').
  * W fp16 [N][K], x fp16 [M][K], act_norm fp32 [K]: device.  workspace: device, 256-byte aligned.
  * Outputs on the HOST: *p_star, bits_host_out[G], errors_host[candidates] (may be NULL).

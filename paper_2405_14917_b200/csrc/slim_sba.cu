@@ -226,6 +226,7 @@ int slim_sba_search(const void* W, const void* x, const float* act_norm, int M, 
     prm.first = first;
     prm.candidates = lay.candidates - first;
     prm.tiles = lay.tiles;
+    prm.half_weights = M > SLIM_GEMV_MAX_M ? 1 : 0;
     double* sal = reinterpret_cast<double*>(ws + lay.salience);
     SLIM_CUDA_TRY(cudaMemsetAsync(prm.status, 0, 8, s));
     st = slim_group_salience(W, act_norm, sal, N, K, g, stream);

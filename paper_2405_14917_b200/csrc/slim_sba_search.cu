@@ -21,8 +21,11 @@ namespace slim {
 //                the new one; y += s_new D_new - s_old D_old.
 //   after every candidate: the CTA's share of the softmax sums of its tokens.
 //
-// Two passes over W and four products in all, where evaluating every candidate on its own takes G / 2 + 1 layers; q - z is a
-// small integer, exact in fp16, and the scale is applied in fp32, so no weight is rounded.
+// Two passes over W and four products in all, where evaluating every candidate on its own takes G / 2 + 1 layers.
+//
+// A candidate's outputs are those of the layer it would become: rounded to fp16, from exact weights up to 16 tokens
+// (q - z is a small integer, exact in fp16, and the scale is applied in fp32) and from weights rounded to fp16 beyond, as
+// the batched path forms them (s (q - z) is the operand and the fold adds it as it is).
 //
 // Warps: 0 brings x (TMA), 1 issues the MMAs (M = 128 tokens, N = R rows, operands in shared memory, accumulators in tensor
 // memory), 2 to 11 read W, quantise and write the second operand, 12 to 19 fold and reduce (thread = token; four warps take
@@ -209,17 +212,19 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
             }
             return c;
         };
+        struct RowOperand : RowQuant { __half2 s2; };
         // the constants of my row of step `it` (width 0: old, 1: new)
         auto my_constants = [&](const Consts& c, int it, int width) {
             const int k = it * RPW / 16, from = ((it * RPW + lane / LPR) & 15) + 16 * width;
-            RowQuant q;
+            RowOperand q;
+            q.s2 = __float2half2_rn(p.half_weights ? __shfl_sync(0xffffffffu, c.s[k], from) : 1.f);
             q.inv = __shfl_sync(0xffffffffu, c.inv[k], from);
             q.inv_lo = __shfl_sync(0xffffffffu, c.inv_lo[k], from);
             q.z = __shfl_sync(0xffffffffu, c.z[k], from);
             return q;
         };
-        // eight weights -> eight q - z in fp16
-        auto operand = [&](const uint4& v, const RowQuant& rq, int levels) {
+        // eight weights -> eight q - z in fp16, times s (rounded) or 1
+        auto operand = [&](const uint4& v, const RowOperand& rq, int levels) {
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
             const uint32_t z2 = static_cast<uint32_t>(rq.z) * 0x00010001u, l2 = static_cast<uint32_t>(levels) * 0x00010001u;
             const __half2 off = __half2half2(__ushort_as_half(static_cast<unsigned short>(0x6400 + rq.z)));      // 1024 + z
@@ -228,7 +233,7 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
             for (int i = 0; i < 4; ++i) {
                 const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
                 const uint32_t q = code_pair(f.x, rq, f.y, rq, z2, l2) | 0x64006400u;       // 1024 + q
-                const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&q), off);
+                const __half2 h = __hmul2(__hsub2(*reinterpret_cast<const __half2*>(&q), off), rq.s2);
                 o[i] = *reinterpret_cast<const uint32_t*>(&h);
             }
             return make_uint4(o[0], o[1], o[2], o[3]);
@@ -288,7 +293,7 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
 #pragma unroll
                     for (int k = 0; k < ROUNDS; ++k) {
                         const int i = 16 * k + (lane & 15), r = (i / RPW) * STEP + qw * RPW + i % RPW;
-                        if (i < ROWS && r < R) sc[(lane < 16 ? 0 : R) + r] = consts.s[k];
+                        if (i < ROWS && r < R) sc[(lane < 16 ? 0 : R) + r] = p.half_weights ? 1.f : consts.s[k];
                     }
                 }
                 if (MULTI)
@@ -297,8 +302,8 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
 #pragma unroll
                 for (int it = 0; it < IT; ++it) {
                     const int r = r0 + it * STEP;
-                    const RowQuant q = my_constants(consts, it, 0);
-                    const RowQuant q2 = second ? my_constants(consts, it, 1) : q;
+                    const RowOperand q = my_constants(consts, it, 0);
+                    const RowOperand q2 = second ? my_constants(consts, it, 1) : q;
                     if (r < R) {
                         const int at = (sub >> 3) * R * 128 + r * 128 + (((sub & 7) ^ (r & 7)) << 4);
                         *reinterpret_cast<uint4*>(b0 + at) = operand(raw[it], q, l_old);
@@ -343,13 +348,14 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
                 }
             }
         };
+        auto fp16_of = [](float v) { return __half2float(__float2half_rn(v)); };
         float mr = -INFINITY;
         // sums of candidate c: partial sums of eight outputs in fp32, the rest in fp64
         auto evaluate = [&](int c) {
             float mq = -INFINITY;
 #pragma unroll
             for (int i = 0; i < C::RH; ++i)
-                if (i < nv) mq = fmaxf(mq, y[i]);
+                if (i < nv) mq = fmaxf(mq, fp16_of(y[i]));
             double sum = 0.0, cross = 0.0;
 #pragma unroll
             for (int k = 0; k < C::RH / 8; ++k) {
@@ -360,8 +366,9 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
                 float a = 0.f, b = 0.f;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    a += expf(y[8 * k + i] - mq);
-                    b = fmaf(__uint_as_float(e[i]), y[8 * k + i] - mr, b);
+                    const float yq = fp16_of(y[8 * k + i]);
+                    a += expf(yq - mq);
+                    b = fmaf(__uint_as_float(e[i]), yq - mr, b);
                 }
                 sum += static_cast<double>(a);
                 cross += static_cast<double>(b);

@@ -16,6 +16,7 @@ struct SbaParams {
     int M, N, K, G;
     int gt;                      // chunks of CW columns in a group
     int avg_bits, first, candidates, tiles;
+    int half_weights;            // the candidates' weights are rounded to fp16
 };
 
 // Weight rows per CTA for M tokens and N rows; tiles = 2 ceil(N / rows).

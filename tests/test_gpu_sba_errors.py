@@ -1,0 +1,58 @@
+"""GPU: the errors that the SBA search returns, against the same quantities in fp64 from torch on the device."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2405_14917_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+# norm of the difference of two error curves over the norm of the curve.  What is left between the device and fp64 are the
+# fp32 sums of a product (a few 1e-6 of the error at 11008 columns) and the outputs, a few in a thousand, that those sums put
+# on the other side of an fp16 rounding; leaving out the fp16 rounding of the outputs moves the curves below by 7e-5 to 1.5e-4
+CURVE_RTOL = 4e-5
+
+
+def _slim():
+    from paper_2405_14917_b200 import binding
+    return binding
+
+
+def _kl(y, y_q):
+    log_p = torch.log_softmax(y, dim=1)
+    return (log_p.exp() * (log_p - torch.log_softmax(y_q, dim=1))).sum(dim=1).mean().item()
+
+
+def _errors(W, x, a, avg, g):
+    """Every candidate as the layer it would become: fp16 outputs, and from 17 tokens on fp16 weights."""
+    slim = _slim()
+    N, K = W.shape
+    M, G = x.shape[0], K // g
+    sal = slim.group_salience(W, a, g).cpu().numpy()
+    xd = x.double()
+    y = xd @ W.double().t()
+    out = []
+    for p in range(G // 2 + 1):
+        codes, s, z = slim.quantize_minmax(W, slim.allocate_bits(sal, avg, p), g=g)
+        w = (s.t().double().unsqueeze(2) * (codes.view(N, G, g).double() - z.t().double().unsqueeze(2))).reshape(N, K)
+        if M > slim.GEMV_MAX_M:
+            w = w.half().double()
+        out.append(_kl(y, (xd @ w.t()).half().double()))
+    return np.array(out)
+
+
+def _inputs(N, K, M, seed, scale=1.0):
+    W, a = wl.make_weight_and_norms_device((seed, 5, 0), N, K, "cuda")
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    x = (scale * torch.randn((M, K), generator=gen, device="cuda")).half()
+    return W, a, x
+
+
+@pytest.mark.parametrize("N,K,M,g,avg", [(2048, 4096, 36, 128, 3), (2048, 11008, 24, 128, 2), (2048, 8192, 12, 64, 2), (512, 8192, 16, 256, 3),
+                                         (1024, 8192, 17, 512, 2)])
+def test_a_candidate_is_the_layer_it_would_become(N, K, M, g, avg):
+    W, a, x = _inputs(N, K, M, seed=N + K + M)
+    _, _, got = _slim().sba_search(W, x, a, avg, g=g)
+    want = _errors(W, x, a, avg, g)
+    assert np.linalg.norm(got - want) <= CURVE_RTOL * np.linalg.norm(want), (np.linalg.norm(got - want) / np.linalg.norm(want))
