@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256) softmax_kl_kernel(const float* __restrict
 struct SbaLayout {
     size_t result, order;                // what the host reads: status word, errors, groups by salience
     size_t result_bytes;
-    size_t salience, kl, ref_m, ref_s, can_m, can_s;
+    size_t salience, kl, ref_m, ref_s, can;
     size_t total;
     int candidates, rows, tiles;
 };
@@ -149,9 +149,8 @@ static int sba_layout(int M, int N, int K, int g, int avg_bits, SbaLayout* lay) 
     lay->salience = o;   o += up256(static_cast<size_t>(G) * sizeof(double));
     lay->kl = o;         o += up256(static_cast<size_t>(lay->candidates) * M * sizeof(double));
     lay->ref_m = o;      o += up256(per_tile * sizeof(float));
-    lay->ref_s = o;      o += up256(per_tile * sizeof(double2));
-    lay->can_m = o;      o += up256(per_tile * lay->candidates * sizeof(float));
-    lay->can_s = o;      o += up256(per_tile * lay->candidates * sizeof(double2));
+    lay->ref_s = o;      o += up256(per_tile * sizeof(double));
+    lay->can = o;        o += up256(per_tile * lay->candidates * sizeof(double2));
     // callers budget for a layer's codes, scales, zeros, packed form and outputs; a search needs less
     const size_t budget = static_cast<size_t>(N) * K + 4 * static_cast<size_t>(G) * N + static_cast<size_t>(N) * K / 8 * (avg_bits + 1) +
                           static_cast<size_t>(M) * N * 6 + static_cast<size_t>(lay->candidates) * M * sizeof(double);
@@ -217,9 +216,8 @@ int slim_sba_search(const void* W, const void* x, const float* act_norm, int M, 
     prm.order = reinterpret_cast<const uint16_t*>(ws + lay.result + lay.order);
     prm.status = reinterpret_cast<unsigned int*>(ws + lay.result);
     prm.ref_m = reinterpret_cast<float*>(ws + lay.ref_m);
-    prm.ref_s = reinterpret_cast<double2*>(ws + lay.ref_s);
-    prm.can_m = reinterpret_cast<float*>(ws + lay.can_m);
-    prm.can_s = reinterpret_cast<double2*>(ws + lay.can_s);
+    prm.ref_s = reinterpret_cast<double*>(ws + lay.ref_s);
+    prm.can = reinterpret_cast<double2*>(ws + lay.can);
     prm.M = M; prm.N = N; prm.K = K; prm.G = G;
     prm.gt = g <= SLIM_GROUP ? 1 : g / SLIM_GROUP;
     prm.avg_bits = avg_bits;

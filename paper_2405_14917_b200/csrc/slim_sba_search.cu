@@ -40,6 +40,29 @@ constexpr int kSbaWarps = kSbaFirstFold + kSbaFold;
 constexpr int kSbaTokens = 128;
 constexpr int kSbaScaleSlots = 8;
 
+// A KL divergence of two outputs that are close together is second order in their difference d = y_q - y, so it must not be
+// a difference of first-order sums.  With e = exp(y - m), A = sum e, b = sum e d / A and f = sum e (exp(d) - 1 - d) / A,
+//   KL = log(sum exp(y_q) / sum exp(y)) - sum p d = log1p(b + f) - b = f - (c - log1p(c)),  c = b + f,
+// where f has no negative terms and c - log1p(c) is of the order of c^2.  (With sums of exp(y_q), e y and e y_q, 8 terms at a time
+// in fp32, the KL of outputs of standard deviation 1e-3 was up to 26 % off.)
+// exp(d) - 1 - d: by its series up to |d| = 0.35 (next term 8e-8 of it), where the difference would cancel; beyond, the difference
+// is off by 4e-6 of itself at most, either way.
+__device__ __forceinline__ float exp_second_order(float d) {
+    float t = fmaf(d, 1.f / 5040.f, 1.f / 720.f);
+    t = fmaf(d, t, 1.f / 120.f);
+    t = fmaf(d, t, 1.f / 24.f);
+    t = fmaf(d, t, 1.f / 6.f);
+    t = fmaf(d, t, 0.5f) * (d * d);
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(d * 1.4426950408889634f));
+    return fabsf(d) <= 0.35f ? t : (e - 1.f) - d;
+}
+// A tile hands over L = log sum exp(y_q) in place of f, lowered below zero by kSbaFarMark so that it can be told from it, where
+// e exp(d) may be beyond fp32 (|d| > 40) or its A + sum e d + sum e (exp(d) - 1 - d), which is sum exp(y_q - m), would be left over
+// from much larger terms (below 2 % of A times the largest |d|).  Its share of the divergence is large then, and L says it.
+constexpr float kSbaFar = 40.f, kSbaLeftOver = 0.02f;
+constexpr double kSbaFarMark = 1e6;
+
 template <int R, int CW> struct SbaCfg {
     static constexpr int RH = R / 2;                               // rows of a fold thread
     static constexpr int XW = CW < 64 ? 64 : CW;                   // columns brought of x
@@ -53,7 +76,7 @@ template <int R, int CW> struct SbaCfg {
     static constexpr int NBAR = 3 * STAGES + 4 + 3;
     static constexpr int OFF_MISC = OFF_BAR + 8 * NBAR;
     static constexpr int SMEM = OFF_MISC + 16 + 1024;
-    static_assert(R % 16 == 0 && 5 * R <= 512 && SMEM <= 227 * 1024, "tensor memory: the reference, two times two products");
+    static_assert(R % 16 == 0 && 6 * R <= 512 && SMEM <= 227 * 1024, "tensor memory: the reference, two times two products, its exponentials");
 };
 
 template <int R, int CW, bool MULTI>     // MULTI: a group has more than one chunk of CW columns
@@ -349,35 +372,45 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
             }
         };
         auto fp16_of = [](float v) { return __half2float(__float2half_rn(v)); };
-        float mr = -INFINITY;
+        const uint32_t t_ref = tmem + t_lane + h * C::RH, t_exp = t_ref + 5 * R;              // y and exp(y - m) of the reference
+        double ref_sum = 0.0;
         // sums of candidate c: partial sums of eight outputs in fp32, the rest in fp64
         auto evaluate = [&](int c) {
-            float mq = -INFINITY;
-#pragma unroll
-            for (int i = 0; i < C::RH; ++i)
-                if (i < nv) mq = fmaxf(mq, fp16_of(y[i]));
-            double sum = 0.0, cross = 0.0;
+            float far = 0.f;
+            double f = 0.0, b = 0.0;
 #pragma unroll
             for (int k = 0; k < C::RH / 8; ++k) {
                 if (8 * k >= nv) break;
-                uint32_t e[8];
-                tc::ld8(tmem + t_lane + h * C::RH + 8 * k, e);
+                uint32_t v[8], e[8];
+                tc::ld8(t_ref + 8 * k, v);
+                tc::ld8(t_exp + 8 * k, e);
                 tc::wait_ld();
-                float a = 0.f, b = 0.f;
+                float fs = 0.f, bs = 0.f;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float yq = fp16_of(y[8 * k + i]);
-                    a += expf(yq - mq);
-                    b = fmaf(__uint_as_float(e[i]), yq - mr, b);
+                for (int i = 0; i < 8; i += 2) {
+                    const float2 yq = __half22float2(__floats2half2_rn(y[8 * k + i], y[8 * k + i + 1]));
+                    const float d0 = yq.x - __uint_as_float(v[i]), d1 = yq.y - __uint_as_float(v[i + 1]);
+                    far = fmaxf(far, fmaxf(fabsf(d0), fabsf(d1)));
+                    bs = fmaf(__uint_as_float(e[i]), d0, bs);
+                    bs = fmaf(__uint_as_float(e[i + 1]), d1, bs);
+                    fs = fmaf(__uint_as_float(e[i]), exp_second_order(d0), fs);
+                    fs = fmaf(__uint_as_float(e[i + 1]), exp_second_order(d1), fs);
                 }
-                sum += static_cast<double>(a);
-                cross += static_cast<double>(b);
+                f += static_cast<double>(fs);
+                b += static_cast<double>(bs);
             }
-            if (m < p.M) {
-                const size_t at = (static_cast<size_t>(c) * p.tiles + tile) * p.M + m;
-                p.can_m[at] = mq;
-                p.can_s[at] = make_double2(sum, cross);
+            if (far > kSbaFar || ref_sum + b + f < kSbaLeftOver * ref_sum * far) {
+                float mq = -INFINITY;
+#pragma unroll
+                for (int i = 0; i < C::RH; ++i)
+                    if (i < nv) mq = fmaxf(mq, fp16_of(y[i]));
+                double sum = 0.0;
+#pragma unroll
+                for (int i = 0; i < C::RH; ++i)
+                    if (i < nv) sum += static_cast<double>(expf(fp16_of(y[i]) - mq));
+                f = (static_cast<double>(mq) + log(sum)) - kSbaFarMark;
             }
+            if (m < p.M) p.can[(static_cast<size_t>(c) * p.tiles + tile) * p.M + m] = make_double2(f, b);
         };
         bool ok = true;
         for (int u = 0; u < units && ok; ++u) {
@@ -395,42 +428,40 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
             __syncwarp();
             if (lane == 0) sb::arrive(d_empty(buf));
             if (u == G - 1) {
-                // the reference: e = exp(y - m) takes the place of y
+                // the reference: m, exp(y - m) and its sum
                 if (!tc::warp_wait(ref_full, 0, abort)) break;
                 tc::fence_after();
+                float mr = -INFINITY;
 #pragma unroll
                 for (int k = 0; k < C::RH / 8; ++k) {
                     if (8 * k >= nv) break;
                     uint32_t v[8];
-                    tc::ld8(tmem + t_lane + h * C::RH + 8 * k, v);
+                    tc::ld8(t_ref + 8 * k, v);
                     tc::wait_ld();
 #pragma unroll
                     for (int i = 0; i < 8; ++i) mr = fmaxf(mr, __uint_as_float(v[i]));
                 }
-                double sum = 0.0, cross = 0.0;
 #pragma unroll
                 for (int k = 0; k < C::RH / 8; ++k) {
                     if (8 * k >= nv) break;
                     uint32_t v[8], e[8];
-                    tc::ld8(tmem + t_lane + h * C::RH + 8 * k, v);
+                    tc::ld8(t_ref + 8 * k, v);
                     tc::wait_ld();
-                    float a = 0.f, b = 0.f;
+                    float a = 0.f;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
-                        const float d = __uint_as_float(v[i]) - mr, x = expf(d);
+                        const float x = expf(__uint_as_float(v[i]) - mr);
                         e[i] = __float_as_uint(x);
                         a += x;
-                        b = fmaf(x, d, b);
                     }
-                    sum += static_cast<double>(a);
-                    cross += static_cast<double>(b);
-                    tc::st8(tmem + t_lane + h * C::RH + 8 * k, e);
+                    ref_sum += static_cast<double>(a);
+                    tc::st8(t_exp + 8 * k, e);
                 }
                 tc::wait_st();
                 if (m < p.M) {
                     const size_t at = static_cast<size_t>(tile) * p.M + m;
                     p.ref_m[at] = mr;
-                    p.ref_s[at] = make_double2(sum, cross);
+                    p.ref_s[at] = ref_sum;
                 }
                 if (p.first == 0) evaluate(0);
             } else if (u >= G && ((u - G) & 1)) {
@@ -449,63 +480,75 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
 
 // ------------------------------------------------------------------------------------------ errors
 // kl[c][t] = sum_n p_n (log p_n - log q_n), p the softmax of the reference and q that of candidate c, in fp64 from the tiles'
-// sums.  A block takes 16 tokens of one candidate; its 64 half warps take every 64th tile: the largest outputs first, then
-// the sums relative to them (one exp per sum), added over the half warps by a fixed tree.
+// sums.  A block takes 16 tokens of one candidate; its 64 half warps take every 64th tile: the largest reference output (and the
+// largest L of the tiles that hand it over) first, then the sums relative to them (two exps per tile), added over the half
+// warps by a fixed tree.
 constexpr int kKlTokens = 16, kKlSlices = 64;
 __global__ void __launch_bounds__(kKlTokens * kKlSlices) sba_kl_kernel(SbaParams p, double* kl) {
-    __shared__ float top[2][kKlSlices][kKlTokens + 1];
-    __shared__ double part[3][kKlSlices][kKlTokens + 1];
+    __shared__ float top[kKlSlices][kKlTokens + 1];
+    __shared__ double top_far[kKlSlices][kKlTokens + 1];
+    __shared__ double part[4][kKlSlices][kKlTokens + 1];
     pdl_wait();
     const int tok = threadIdx.x % kKlTokens, slice = threadIdx.x / kKlTokens, c = blockIdx.y, m = blockIdx.x * kKlTokens + tok;
     const float* ref_m = p.ref_m + m;
-    const float* can_m = p.can_m + static_cast<size_t>(c) * p.tiles * p.M + m;
-    const double2* ref_s = p.ref_s + m;
-    const double2* can_s = p.can_s + static_cast<size_t>(c) * p.tiles * p.M + m;
-    float mr = -INFINITY, mq = -INFINITY;
+    const double* ref_s = p.ref_s + m;
+    const double2* can = p.can + static_cast<size_t>(c) * p.tiles * p.M + m;
+    float mr = -INFINITY;
+    double far = -INFINITY;
     if (m < p.M)
         for (int k = slice; k < p.tiles; k += kKlSlices) {
             mr = fmaxf(mr, __ldcg(ref_m + static_cast<size_t>(k) * p.M));
-            mq = fmaxf(mq, __ldcg(can_m + static_cast<size_t>(k) * p.M));
+            const double f = __ldcg(&can[static_cast<size_t>(k) * p.M].x);
+            if (f < 0.0) far = fmax(far, f + kSbaFarMark);
         }
-    top[0][slice][tok] = mr;
-    top[1][slice][tok] = mq;
+    top[slice][tok] = mr;
+    top_far[slice][tok] = far;
     __syncthreads();
 #pragma unroll 8
     for (int w = 0; w < kKlSlices; ++w) {
-        mr = fmaxf(mr, top[0][w][tok]);
-        mq = fmaxf(mq, top[1][w][tok]);
+        mr = fmaxf(mr, top[w][tok]);
+        far = fmax(far, top_far[w][tok]);
     }
-    double v[3] = {0.0, 0.0, 0.0};                 // sum e, sum e (y - y_q), sum e_q
+    // sum e, sum e d, sum e (exp(d) - 1 - d), all relative to the largest reference output, and sum exp(y_q) relative to `base`
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    const double base = fmax(far, static_cast<double>(mr));
     if (m < p.M)
         for (int k = slice; k < p.tiles; k += kKlSlices) {
             const size_t at = static_cast<size_t>(k) * p.M;
-            const double2 r = __ldcg(ref_s + at), q = __ldcg(can_s + at);
-            const double fr = exp(static_cast<double>(__ldcg(ref_m + at)) - static_cast<double>(mr));
-            const double fq = exp(static_cast<double>(__ldcg(can_m + at)) - static_cast<double>(mq));
-            v[0] = fma(r.x, fr, v[0]);
-            v[1] = fma(r.y - q.y, fr, v[1]);
-            v[2] = fma(q.x, fq, v[2]);
+            const double s = __ldcg(ref_s + at), mk = static_cast<double>(__ldcg(ref_m + at));
+            const double2 q = __ldcg(can + at);
+            const double w = exp(mk - static_cast<double>(mr));
+            v[0] = fma(s, w, v[0]);
+            v[1] = fma(q.y, w, v[1]);
+            if (q.x < 0.0) {
+                const double L = q.x + kSbaFarMark;
+                v[2] += exp(L - static_cast<double>(mr)) - (s + q.y) * w;
+                v[3] += exp(L - base);
+            } else {
+                v[2] = fma(q.x, w, v[2]);
+                v[3] = fma(s + q.y + q.x, base == static_cast<double>(mr) ? w : exp(mk - base), v[3]);
+            }
         }
 #pragma unroll
-    for (int i = 0; i < 3; ++i) part[i][slice][tok] = v[i];
+    for (int i = 0; i < 4; ++i) part[i][slice][tok] = v[i];
     __syncthreads();
     // warp w < 16 adds the parts of token w
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = blockIdx.x * kKlTokens + warp;
     if (warp >= kKlTokens || t >= p.M) return;
-    mr = fmaxf(top[0][lane][warp], top[0][lane + 32][warp]);
-    mq = fmaxf(top[1][lane][warp], top[1][lane + 32][warp]);
+    mr = fmaxf(top[lane][warp], top[lane + 32][warp]);
+    far = fmax(top_far[lane][warp], top_far[lane + 32][warp]);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) v[i] = part[i][lane][warp] + part[i][lane + 32][warp];
+    for (int i = 0; i < 4; ++i) v[i] = part[i][lane][warp] + part[i][lane + 32][warp];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
-        mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
+        far = fmax(far, __shfl_xor_sync(0xffffffffu, far, o));
 #pragma unroll
-        for (int i = 0; i < 3; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+        for (int i = 0; i < 4; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
     }
-    // sum p (y - y_q) - log sum exp y + log sum exp y_q
-    if (lane == 0)
-        kl[static_cast<size_t>(c) * p.M + t] = v[1] / v[0] - (static_cast<double>(mr) + log(v[0])) + (static_cast<double>(mq) + log(v[2]));
+    if (lane != 0) return;
+    const double b = v[1] / v[0], f = v[2] / v[0], cc = b + f, top_q = fmax(far, static_cast<double>(mr));
+    kl[static_cast<size_t>(c) * p.M + t] = fabs(cc) < 0.5 ? f - (cc - log1p(cc)) : (top_q - static_cast<double>(mr)) + (log(v[3]) - log(v[0])) - b;
 }
 
 // Mean over the tokens, one warp per candidate, in a fixed order.

@@ -9,10 +9,9 @@ struct SbaParams {
     const __half* W;
     const uint16_t* order;       // groups by salience, the most salient first
     unsigned int* status;
-    float* ref_m;                // [tiles][M]: largest reference output of the tile
-    double2* ref_s;              // [tiles][M]: sum e, sum e (y - m) with e = exp(y - m)
-    float* can_m;                // [candidates][tiles][M]: largest candidate output
-    double2* can_s;              // [candidates][tiles][M]: sum exp(y_q - m_q), sum e (y_q - m)
+    float* ref_m;                // [tiles][M]: m, the largest reference output y of the tile
+    double* ref_s;               // [tiles][M]: sum e with e = exp(y - m)
+    double2* can;                // [candidates][tiles][M]: with d = y_q - y, sum e (exp(d) - 1 - d) or a lowered log sum exp(y_q), and sum e d
     int M, N, K, G;
     int gt;                      // chunks of CW columns in a group
     int avg_bits, first, candidates, tiles;

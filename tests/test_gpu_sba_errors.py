@@ -56,3 +56,33 @@ def test_a_candidate_is_the_layer_it_would_become(N, K, M, g, avg):
     _, _, got = _slim().sba_search(W, x, a, avg, g=g)
     want = _errors(W, x, a, avg, g)
     assert np.linalg.norm(got - want) <= CURVE_RTOL * np.linalg.norm(want), (np.linalg.norm(got - want) / np.linalg.norm(want))
+
+
+@pytest.mark.parametrize("std", [1e-2, 1e-3])
+@pytest.mark.parametrize("N,K,M", [(512, 512, 16), (4096, 1024, 40)])
+def test_errors_of_small_outputs_keep_their_digits(N, K, M, std):
+    """The divergence is second order in the outputs' difference: 1e-7 and less here, with no absolute floor in the comparison."""
+    W, a, x = _inputs(N, K, M, seed=7 + K, scale=std / (0.02 * np.sqrt(2 * K)))
+    _, _, got = _slim().sba_search(W, x, a, 2)
+    want = _errors(W, x, a, 2, 128)
+    assert np.linalg.norm(got - want) <= CURVE_RTOL * np.linalg.norm(want), (np.linalg.norm(got - want) / np.linalg.norm(want))
+
+
+@pytest.mark.parametrize("M", [12, 20])
+def test_errors_of_outputs_that_are_far_apart(M):
+    """One input per token, a power of two: every output is one product, exact before it is rounded to fp16, so the two sides
+    have the same outputs and only the divergence is compared.  It is computed from e = exp(y - m) in fp32, whose argument
+    is off by 2^-24 |y - m|: 1e-5 where |y - m| is 200, beyond which e weighs nothing."""
+    N, K = 320, 1024
+    W, a, _ = _inputs(N, K, M, seed=3)
+    x = torch.zeros((M, K), dtype=torch.float16, device="cuda")
+    for t in range(M):
+        x[t, 37 * t + 5] = 2.0 ** (t if t < 8 else 13 - t % 3)       # outputs from 0.02 to 1000 and more, differences likewise
+    _, _, got = _slim().sba_search(W, x, a, 2)
+    want = _errors(W, x, a, 2, 128)
+    assert want.max() > 10
+    assert np.abs(got - want).max() <= 2e-5 * want.max(), (got, want)
+    for t in (0, 11):                                                # a token of each kind by itself
+        _, _, got = _slim().sba_search(W, x[t:t + 1].contiguous(), a, 2)
+        want = _errors(W, x[t:t + 1], a, 2, 128)
+        assert np.abs(got - want).max() <= 2e-5 * want.max(), (t, got, want)
