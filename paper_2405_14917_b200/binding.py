@@ -3,7 +3,8 @@
 Argument marshalling only: every function checks dtypes/devices, takes raw device
 pointers from torch tensors and the current CUDA stream, and calls the entry point
 of the same name; for the linear layers and the layer sets, which a decode loop calls
-per layer, the host module (csrc/slim_host.cpp) does that without the interpreter.
+per layer, the host module (csrc/slim_host.cpp) does that without the interpreter, where
+it has been built for the running torch.
 There is no fallback: if the CUDA library has not been built the first call raises.
 """
 from __future__ import annotations
@@ -12,6 +13,7 @@ import ctypes
 import importlib.machinery
 import importlib.util
 import os
+import warnings
 
 import numpy as np
 import torch
@@ -22,7 +24,7 @@ GROUP = 128
 GEMV_MAX_M = 16
 
 _lib = None
-_host = None             # the host module, and the addresses of the entry points that it calls
+_host = None             # the host module (or _NoHost), and the addresses of the entry points that it calls
 _entry = {}
 
 
@@ -87,16 +89,30 @@ def lib():
     return _lib
 
 
+class _NoHost:
+    """In place of a host module that cannot be loaded: every call takes the general path."""
+
+    @staticmethod
+    def linear(*_):
+        return None
+
+    @staticmethod
+    def run_set(*_):
+        return None
+
+
 def host():
-    """Loads lib/slim_host.so (built with the CUDA library)."""
+    """Loads the host module (built with the CUDA library); without it calls only take longer on the host."""
     global _host
     if _host is None:
         L = lib()
-        if not os.path.exists(HOST_PATH):
-            raise RuntimeError(f"host module not built: {HOST_PATH} is missing; run `python -m paper_2405_14917_b200.build`")
-        loader = importlib.machinery.ExtensionFileLoader("slim_host", HOST_PATH)
-        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("slim_host", loader))
-        loader.exec_module(module)
+        try:
+            loader = importlib.machinery.ExtensionFileLoader("slim_host", HOST_PATH)
+            module = importlib.util.module_from_spec(importlib.util.spec_from_loader("slim_host", loader))
+            loader.exec_module(module)
+        except ImportError as e:
+            warnings.warn(f"host module not loaded ({e}); `python -m paper_2405_14917_b200.build` builds it for this torch")
+            module = _NoHost
         for name in ("slim_mpq_gemv", "slim_mpq_gemm", "slim_mpq_gemv_set"):
             _entry[name] = ctypes.cast(getattr(L, name), ctypes.c_void_p).value
         _host = module

@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import glob
+import importlib.metadata
 import os
 import subprocess
 import sys
@@ -13,7 +14,9 @@ CSRC = os.path.join(_HERE, "csrc")
 LIB_DIR = os.path.join(_HERE, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libslim_b200.so")
 HOST_SRC = os.path.join(CSRC, "slim_host.cpp")
-HOST_PATH = os.path.join(LIB_DIR, "slim_host.so")
+# an extension serves the interpreter and the torch that it was compiled against, so both are in its name: another torch
+# finds no host module rather than one of the wrong ABI
+HOST_PATH = os.path.join(LIB_DIR, f"slim_host.{sys.implementation.cache_tag}-torch{importlib.metadata.version('torch')}.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xptxas=-v"]
@@ -32,7 +35,7 @@ def _stale() -> bool:
 
 
 def build_host(force: bool = False, verbose: bool = False) -> str:
-    """Compile the host module of the binding (csrc/slim_host.cpp) into lib/slim_host.so.  Returns its path."""
+    """Compile the host module of the binding (csrc/slim_host.cpp) into HOST_PATH.  Returns its path."""
     if not force and os.path.exists(HOST_PATH) and os.path.getmtime(HOST_PATH) >= os.path.getmtime(HOST_SRC):
         return HOST_PATH
     import torch
