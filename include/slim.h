@@ -345,8 +345,10 @@ int slim_dense_linear(const void* x, const void* W, float* y, int M, int N, int 
  * y_ref fp32 [M][N], y_q fp16 [M][N], kl fp64 [M], all device; fp64 arithmetic, fixed reduction order. */
 int slim_softmax_kl(const float* y_ref, const void* y_q, double* kl, int M, int N, void* stream);
 
-/* Host-only: bytes of workspace slim_sba_search needs (the softmax sums of every candidate, token and block of rows;
- * never less than a layer's codes, scales, zeros, packed form and both outputs would take). */
+/* Host-only: bytes of workspace with which slim_sba_search evaluates all candidates in one walk (the softmax sums of every
+ * candidate, token and block of rows; never less than a layer's codes, scales, zeros, packed form and both outputs would
+ * take, N K (1 + (avg_bits + 1) / 8) + 4 N K / g + 6 M N bytes and 8 M for every candidate).  Given less, but no less than
+ * that, it takes several walks; the results are the same. */
 int slim_sba_workspace_bytes(int M, int N, int K, int g, int avg_bits, size_t* out_bytes);
 
 /* The search: groups ranked by salience (slim_group_salience; equal salience: lower index first);

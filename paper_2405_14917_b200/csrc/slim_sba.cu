@@ -125,7 +125,8 @@ struct SbaLayout {
     size_t result, order;                // what the host reads: status word, errors, groups by salience
     size_t result_bytes;
     size_t salience, kl, ref_m, ref_s, can;
-    size_t total;
+    size_t can_bytes;                    // of one candidate
+    size_t total, least;                 // room for every candidate at once, and what a caller has to have
     int candidates, rows, tiles;
 };
 static size_t up256(size_t v) { return (v + 255) / 256 * 256; }
@@ -150,11 +151,15 @@ static int sba_layout(int M, int N, int K, int g, int avg_bits, SbaLayout* lay) 
     lay->kl = o;         o += up256(static_cast<size_t>(lay->candidates) * M * sizeof(double));
     lay->ref_m = o;      o += up256(per_tile * sizeof(float));
     lay->ref_s = o;      o += up256(per_tile * sizeof(double));
-    lay->can = o;        o += up256(per_tile * lay->candidates * sizeof(double2));
-    // callers budget for a layer's codes, scales, zeros, packed form and outputs; a search needs less
+    lay->can = o;        o += up256(per_tile * sizeof(double2) * lay->candidates);
+    lay->can_bytes = per_tile * sizeof(double2);
+    // a caller who sets aside a layer's codes, scales, zeros, packed form and outputs is always served (with groups of 32 columns
+    // and few rows the sums of all candidates can take five times that: then a part of the candidates at a time)
     const size_t budget = static_cast<size_t>(N) * K + 4 * static_cast<size_t>(G) * N + static_cast<size_t>(N) * K / 8 * (avg_bits + 1) +
                           static_cast<size_t>(M) * N * 6 + static_cast<size_t>(lay->candidates) * M * sizeof(double);
     lay->total = o > budget ? o : up256(budget);
+    const size_t one = lay->can + lay->can_bytes;
+    lay->least = one > budget ? one : budget;
     return SLIM_OK;
 }
 
@@ -202,7 +207,7 @@ int slim_sba_search(const void* W, const void* x, const float* act_norm, int M, 
     if (st != SLIM_OK) return st;
     if (W == nullptr || x == nullptr || act_norm == nullptr) return SLIM_ERR_INVALID_ARG;
     if (!slim::aligned16(W) || !slim::aligned16(x)) return SLIM_ERR_ALIGNMENT;
-    if (workspace == nullptr || workspace_bytes < lay.total) return SLIM_ERR_WORKSPACE;
+    if (workspace == nullptr || workspace_bytes < lay.least) return SLIM_ERR_WORKSPACE;
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return SLIM_ERR_ALIGNMENT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
@@ -221,8 +226,6 @@ int slim_sba_search(const void* W, const void* x, const float* act_norm, int M, 
     prm.M = M; prm.N = N; prm.K = K; prm.G = G;
     prm.gt = g <= SLIM_GROUP ? 1 : g / SLIM_GROUP;
     prm.avg_bits = avg_bits;
-    prm.first = first;
-    prm.candidates = lay.candidates - first;
     prm.tiles = lay.tiles;
     prm.half_weights = M > SLIM_GEMV_MAX_M ? 1 : 0;
     double* sal = reinterpret_cast<double*>(ws + lay.salience);
@@ -230,7 +233,19 @@ int slim_sba_search(const void* W, const void* x, const float* act_norm, int M, 
     st = slim_group_salience(W, act_norm, sal, N, K, g, stream);
     if (st != SLIM_OK) return st;
     SLIM_CUDA_TRY(slim::launch_allocate(sal, nullptr, nullptr, const_cast<uint16_t*>(prm.order), G, avg_bits, 0, s));
-    st = slim::sba_search_launch(x, prm, lay.rows, g, reinterpret_cast<double*>(ws + lay.kl), reinterpret_cast<double*>(ws + lay.result + 8), s);
+    // all candidates in one walk, or in as few of equal length as the workspace has room for
+    const int candidates = lay.candidates - first;
+    const size_t fit = (workspace_bytes - lay.can) / lay.can_bytes;
+    const int walks = static_cast<int>((candidates + fit - 1) / fit);
+    double *kl = reinterpret_cast<double*>(ws + lay.kl), *errors_dev = reinterpret_cast<double*>(ws + lay.result + 8);
+    for (int i = 0; i < walks; ++i) {
+        const int c0 = static_cast<int>(static_cast<long long>(candidates) * i / walks), c1 = static_cast<int>(static_cast<long long>(candidates) * (i + 1) / walks);
+        prm.first = first + c0;
+        prm.candidates = c1 - c0;
+        st = slim::sba_search_launch(x, prm, lay.rows, g, kl + static_cast<size_t>(c0) * M, s);
+        if (st != SLIM_OK) return st;
+    }
+    st = slim::sba_mean_launch(kl, errors_dev, candidates, M, s);
     if (st != SLIM_OK) return st;
 
     alignas(16) uint8_t host[8 + (slim::kSbaMaxGroups / 2 + 1) * sizeof(double) + slim::kSbaMaxGroups * sizeof(uint16_t)];
@@ -242,7 +257,7 @@ int slim_sba_search(const void* W, const void* x, const float* act_norm, int M, 
     const double* errors = reinterpret_cast<const double*>(host + 8);
     const uint16_t* order = reinterpret_cast<const uint16_t*>(host + lay.order);
     int best = 0;                                      // the first minimum over p
-    for (int i = 0; i < prm.candidates; ++i) {
+    for (int i = 0; i < candidates; ++i) {
         if (errors_host != nullptr) errors_host[i] = errors[i];
         if (errors[i] < errors[best]) best = i;
     }

@@ -465,7 +465,8 @@ __global__ void __launch_bounds__(32 * kSbaWarps, 1) sba_kernel(const __grid_con
                 }
                 if (p.first == 0) evaluate(0);
             } else if (u >= G && ((u - G) & 1)) {
-                evaluate(((u - G) >> 1) + 1 - p.first);
+                const int c = ((u - G) >> 1) + 1 - p.first;
+                if (c >= 0) evaluate(c);
             }
         }
     }
@@ -601,7 +602,7 @@ int sba_rows(int M, int N) {
     return best;
 }
 
-int sba_search_launch(const void* x, const SbaParams& p, int rows, int g, double* kl, double* errors, cudaStream_t s) {
+int sba_search_launch(const void* x, const SbaParams& p, int rows, int g, double* kl, cudaStream_t s) {
     CUtensorMap map;
     if (!make_x_map(&map, x, p.M, p.K, kSbaTokens)) return SLIM_ERR_CUDA;
     SLIM_CUDA_TRY(rows == 16   ? launch_search_for<16>(g, map, p, s)
@@ -612,8 +613,12 @@ int sba_search_launch(const void* x, const SbaParams& p, int rows, int g, double
     PdlLaunch k(static_cast<unsigned>((p.M + kKlTokens - 1) / kKlTokens), kKlTokens * kKlSlices, 0, s);
     k.cfg.gridDim.y = static_cast<unsigned>(p.candidates);
     SLIM_CUDA_TRY(cudaLaunchKernelEx(&k.cfg, sba_kl_kernel, p, kl));
-    PdlLaunch e(static_cast<unsigned>(p.candidates), 32, 0, s);
-    SLIM_CUDA_TRY(cudaLaunchKernelEx(&e.cfg, sba_mean_kernel, static_cast<const double*>(kl), errors, p.M));
+    return SLIM_OK;
+}
+
+int sba_mean_launch(const double* kl, double* errors, int candidates, int M, cudaStream_t s) {
+    PdlLaunch e(static_cast<unsigned>(candidates), 32, 0, s);
+    SLIM_CUDA_TRY(cudaLaunchKernelEx(&e.cfg, sba_mean_kernel, kl, errors, M));
     return SLIM_OK;
 }
 

@@ -86,3 +86,21 @@ def test_errors_of_outputs_that_are_far_apart(M):
         _, _, got = _slim().sba_search(W, x[t:t + 1].contiguous(), a, 2)
         want = _errors(W, x[t:t + 1], a, 2, 128)
         assert np.abs(got - want).max() <= 2e-5 * want.max(), (t, got, want)
+
+
+@pytest.mark.parametrize("N,K,M,g,avg,include_uniform", [(512, 4096, 256, 32, 2, True), (512, 4096, 130, 32, 3, False), (16, 8192, 250, 32, 2, True)])
+def test_a_small_workspace_means_several_walks_and_the_same_errors(N, K, M, g, avg, include_uniform):
+    slim = _slim()
+    W, a, x = _inputs(N, K, M, seed=11)
+    G = K // g
+    layer = N * K + N * K * (avg + 1) // 8 + 4 * N * G + 6 * M * N + 8 * M * (G // 2 + 1)      # codes, packed, scales, zeros, outputs, errors
+    full = slim.sba_workspace_bytes(M, N, K, avg, g)
+    assert full > 1.3 * layer                                        # the shapes are ones where it matters
+    results = []
+    for size in (full, layer, (full + layer) // 2):
+        ws = torch.full((size,), 0xFF, dtype=torch.uint8, device="cuda")
+        results.append(slim.sba_search(W, x, a, avg, include_uniform, workspace=ws, g=g))
+    for p, bits, errors in results[1:]:
+        assert p == results[0][0] and (bits == results[0][1]).all() and (errors == results[0][2]).all()
+    with pytest.raises(slim.SlimError):
+        slim.sba_search(W, x, a, avg, workspace=torch.empty(layer - 256, dtype=torch.uint8, device="cuda"), g=g)
