@@ -15,6 +15,7 @@
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 namespace {
@@ -25,7 +26,7 @@ using SetFn = int (*)(const void*, const void*, void*, size_t, void*);
 const at::Tensor* plain(PyObject* o, c10::ScalarType dtype) {
     if (!THPVariable_CheckExact(o)) return nullptr;
     const at::Tensor& t = THPVariable_Unpack(o);
-    return t.is_cuda() && t.scalar_type() == dtype && t.is_contiguous() ? &t : nullptr;
+    return t.is_cuda() && t.layout() == c10::kStrided && t.scalar_type() == dtype && t.is_contiguous() ? &t : nullptr;
 }
 
 bool as_int(PyObject* o, int* out) {
@@ -39,8 +40,23 @@ bool as_int(PyObject* o, int* out) {
 
 void* stream_of(const at::Tensor& t) { return c10::cuda::getCurrentCUDAStream(t.get_device()).stream(); }
 
+// The bit map of a layer: a one-dimensional uint8 array that numpy can be asked for without a copy.
+struct Bits {
+    Py_buffer b;
+    bool held = false;
+    bool open(PyObject* o) {
+        if (PyObject_GetBuffer(o, &b, PyBUF_FORMAT | PyBUF_ND | PyBUF_C_CONTIGUOUS) != 0) { PyErr_Clear(); return false; }
+        held = true;
+        return b.ndim == 1 && b.itemsize == 1 && b.format != nullptr && b.format[0] == 'B' && b.format[1] == 0;
+    }
+    ~Bits() { if (held) PyBuffer_Release(&b); }
+};
+
+// What torch throws (a tensor without storage or of a layout that has no strides, no memory left) leaves as the Python
+// exception that the same call in Python raises.
 // linear(address, x, packed, bits, scales, zeros, N, workspace, out or None, g) -> y, or the status of a call that failed, or None (see above)
 PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (n != 10) { PyErr_SetString(PyExc_TypeError, "linear: 10 arguments"); return nullptr; }
     LinearFn fn = reinterpret_cast<LinearFn>(PyLong_AsVoidPtr(a[0]));
     if (fn == nullptr) { if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "linear: no entry point"); return nullptr; }
@@ -52,59 +68,41 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
         Py_RETURN_NONE;
     const at::Tensor* given = nullptr;
     if (a[8] != Py_None && (given = plain(a[8], at::kHalf)) == nullptr) Py_RETURN_NONE;
-    Py_buffer b;
-    if (PyObject_GetBuffer(a[3], &b, PyBUF_FORMAT | PyBUF_ND | PyBUF_C_CONTIGUOUS) != 0) { PyErr_Clear(); Py_RETURN_NONE; }
-    if (b.ndim != 1 || b.itemsize != 1 || b.format == nullptr || b.format[0] != 'B' || b.format[1] != 0) {
-        PyBuffer_Release(&b);
-        Py_RETURN_NONE;
-    }
-    PyObject* result = nullptr;
-    try {
-        const int M = static_cast<int>(x->size(0)), K = static_cast<int>(x->size(1));
-        at::Tensor fresh;
-        if (given == nullptr) fresh = at::empty({M, N}, x->options());
-        const at::Tensor& y = given != nullptr ? *given : fresh;
-        void *xp = x->data_ptr(), *wp = packed->data_ptr(), *sp = scales->data_ptr(), *zp = zeros->data_ptr(), *yp = y.data_ptr();
-        void *wsp = ws->data_ptr(), *stream = stream_of(*x);
-        const size_t wsb = static_cast<size_t>(ws->numel());
-        int status = 0;
-        Py_BEGIN_ALLOW_THREADS                  // the tensors and the bit map are held by the caller's arguments
-        status = fn(xp, wp, static_cast<const uint8_t*>(b.buf), sp, zp, yp, M, N, K, g, wsp, wsb, stream);
-        Py_END_ALLOW_THREADS
-        PyObject* out = given != nullptr ? Py_NewRef(a[8]) : THPVariable_Wrap(fresh);
-        if (out != nullptr && status == 0) {
-            result = out;
-        } else if (out != nullptr) {
-            Py_DECREF(out);
-            result = PyLong_FromLong(status);
-        }
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-    }
-    PyBuffer_Release(&b);
-    return result;
+    Bits bits;
+    if (!bits.open(a[3])) Py_RETURN_NONE;
+    const int M = static_cast<int>(x->size(0)), K = static_cast<int>(x->size(1));
+    at::Tensor fresh;
+    if (given == nullptr) fresh = at::empty({M, N}, x->options());
+    const at::Tensor& y = given != nullptr ? *given : fresh;
+    void *xp = x->data_ptr(), *wp = packed->data_ptr(), *sp = scales->data_ptr(), *zp = zeros->data_ptr(), *yp = y.data_ptr();
+    void *wsp = ws->data_ptr(), *stream = stream_of(*x);
+    const size_t wsb = static_cast<size_t>(ws->numel());
+    int status = 0;
+    Py_BEGIN_ALLOW_THREADS                      // the tensors and the bit map are held by the caller's arguments
+    status = fn(xp, wp, static_cast<const uint8_t*>(bits.b.buf), sp, zp, yp, M, N, K, g, wsp, wsb, stream);
+    Py_END_ALLOW_THREADS
+    if (status != 0) return PyLong_FromLong(status);
+    return given != nullptr ? Py_NewRef(a[8]) : THPVariable_Wrap(fresh);
+    END_HANDLE_TH_ERRORS
 }
 
 // run_set(address, launch record, plan, workspace) -> status, or None
 PyObject* run_set(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (n != 4) { PyErr_SetString(PyExc_TypeError, "run_set: 4 arguments"); return nullptr; }
     SetFn fn = reinterpret_cast<SetFn>(PyLong_AsVoidPtr(a[0]));
     const void* info = fn != nullptr ? PyLong_AsVoidPtr(a[1]) : nullptr;
     if (fn == nullptr || info == nullptr) { if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "run_set: no entry point"); return nullptr; }
     const at::Tensor *plan = plain(a[2], at::kByte), *ws = plain(a[3], at::kByte);
     if (plan == nullptr || ws == nullptr) Py_RETURN_NONE;
-    try {
-        void *pp = plan->data_ptr(), *wp = ws->data_ptr(), *stream = stream_of(*plan);
-        const size_t wsb = static_cast<size_t>(ws->numel());
-        int status = 0;
-        Py_BEGIN_ALLOW_THREADS
-        status = fn(info, pp, wp, wsb, stream);
-        Py_END_ALLOW_THREADS
-        return PyLong_FromLong(status);
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
-    }
+    void *pp = plan->data_ptr(), *wp = ws->data_ptr(), *stream = stream_of(*plan);
+    const size_t wsb = static_cast<size_t>(ws->numel());
+    int status = 0;
+    Py_BEGIN_ALLOW_THREADS
+    status = fn(info, pp, wp, wsb, stream);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(status);
+    END_HANDLE_TH_ERRORS
 }
 
 PyMethodDef methods[] = {

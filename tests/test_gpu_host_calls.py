@@ -60,3 +60,18 @@ def test_calls_that_must_fail():
     with pytest.raises(slim.SlimError):
         slim.mpq_gemm(*ok)                              # one token is not the batched path's
     torch.cuda.synchronize()
+
+
+def test_what_torch_raises_is_what_the_caller_gets():
+    L = _layer(64, 512, 128)
+    x = torch.zeros((1, 512), dtype=torch.float16, device="cuda")
+    ws = slim.new_workspace(1, 64, 512, L.bits)
+    ok = [x, L.packed, L.bits, L.scales, L.zeros, 64, ws]
+    for at in (0, 1, 3, 6):                             # no strides to ask for
+        args = list(ok)
+        args[at] = ok[at].to_sparse()
+        with pytest.raises((TypeError, RuntimeError)):
+            slim.mpq_gemv(*args)
+    many = torch.zeros((200, 512), dtype=torch.float16, device="cuda")
+    with pytest.raises(torch.OutOfMemoryError):         # an output of 800 GB
+        slim.mpq_gemm(many, L.packed, L.bits, L.scales, L.zeros, 2**31 - 16, ws)
