@@ -45,6 +45,7 @@ struct Bits {
     Py_buffer b;
     bool held = false;
     bool open(PyObject* o) {
+        if (PyBytes_Check(o) || PyByteArray_Check(o) || PyMemoryView_Check(o)) return false;      // the general path says what they are
         if (PyObject_GetBuffer(o, &b, PyBUF_FORMAT | PyBUF_ND | PyBUF_C_CONTIGUOUS) != 0) { PyErr_Clear(); return false; }
         held = true;
         return b.ndim == 1 && b.itemsize == 1 && b.format != nullptr && b.format[0] == 'B' && b.format[1] == 0;

@@ -75,3 +75,13 @@ def test_what_torch_raises_is_what_the_caller_gets():
     many = torch.zeros((200, 512), dtype=torch.float16, device="cuda")
     with pytest.raises(torch.OutOfMemoryError):         # an output of 800 GB
         slim.mpq_gemm(many, L.packed, L.bits, L.scales, L.zeros, 2**31 - 16, ws)
+
+
+def test_bytes_are_not_a_bit_map():
+    L = _layer(64, 512, 128)
+    x = torch.randn((1, 512), device="cuda").to(torch.float16)
+    ws = slim.new_workspace(1, 64, 512, L.bits)
+    with pytest.raises(ValueError):
+        slim.mpq_gemv(x, L.packed, L.bits.tobytes(), L.scales, L.zeros, 64, ws)
+    y = slim.mpq_gemv(x, L.packed, L.bits, L.scales, L.zeros, 64, ws)
+    assert torch.equal(slim.mpq_gemv(x, L.packed, bytearray(L.bits), L.scales, L.zeros, 64, ws), y)
