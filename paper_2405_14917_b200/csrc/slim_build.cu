@@ -93,6 +93,46 @@ __device__ __forceinline__ void load_row(const __half* src, bool wide, __half2 (
     }
 }
 
+// What quant_pack_kernel does, for a tile and group with weights that are not finite (the pair arithmetic there is for
+// quotients of less than 2^15): weight by weight, NaN left out of the range as fmin and fmax do.
+template <int T, int GT>
+__device__ __noinline__ void quant_pack_any(const __half* src, int K, int b, uint8_t* dst, size_t tile_step, __half* scale, __half* zero) {
+    constexpr int C = T / 4;
+    const int c = threadIdx.x & 3, levels = (1 << b) - 1;
+    for (int h = 0; h < 2; ++h, src += K) {
+        float lo = 0.f, hi = 0.f;
+        for (int i = 0; i < C * GT; ++i) {
+            const float w = __half2float(src[T * (i / C) + i % C]);
+            lo = fminf(lo, w);
+            hi = fmaxf(hi, w);
+        }
+        for (int o = 1; o < 4; o <<= 1) {
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        const RowQuant q = row_quantizer(lo, hi, levels);
+        if (c == 0) {
+            scale[h] = q.s16;
+            zero[h] = __int2half_rn(q.z);
+        }
+        for (int k = 0; k < GT; ++k)
+            for (int s = 0; s < slice_count(b); ++s) {
+                const int first = slice_lo(b, s), w = slice_w(b, s), nf = C / w;
+                for (int u = 0; u < w; ++u) {
+                    uint32_t item = 0u;
+                    for (int f = 0; f < nf; ++f) {
+                        const int code = clamped_code(__half2float(src[T * k + nf * u + f]), q, static_cast<float>(q.z), static_cast<float>(levels));
+                        item |= ((static_cast<uint32_t>(code) >> first) & ((1u << w) - 1u)) << (w * f);
+                    }
+                    uint8_t* at = dst + tile_step * k + 2 * T * (slice_unit0(b, s) + u) + (C / 8) * h;
+                    if (C == 32) *reinterpret_cast<uint32_t*>(at) = item;
+                    else if (C == 16) *reinterpret_cast<uint16_t*>(at) = static_cast<uint16_t>(item);
+                    else *at = static_cast<uint8_t>(item);
+                }
+            }
+    }
+}
+
 // One warp per (16-row tile, group), lane 4 gq + c = rows 2 gq and 2 gq + 1, quarter c of each of the group's GT tiles of
 // T columns: exactly the words a lane owns in the packed format.
 template <int T, int GT>
@@ -117,11 +157,21 @@ __global__ void __launch_bounds__(256, GT == 1 ? 4 : 3) quant_pack_kernel(const 
         for (int h = 0; h < 2; ++h) {
             load_row<C>(src + static_cast<size_t>(h) * K + T * k, wide, w[h]);
 #pragma unroll
-            for (int i = 0; i < C / 2; ++i) { mn[h] = __hmin2(mn[h], w[h][i]); mx[h] = __hmax2(mx[h], w[h][i]); }
+            for (int i = 0; i < C / 2; ++i) { mn[h] = __hmin2_nan(mn[h], w[h][i]); mx[h] = __hmax2_nan(mx[h], w[h][i]); }
         }
     pdl_wait();                                            // the table; W was complete before the kernels ahead began
     const uint32_t entry = ld_written_ahead(table + j);
     const int b = static_cast<int>(entry & 7u), levels = (1 << b) - 1;
+    uint32_t largest = 0u;                                 // 0x7c00 and more: Inf or NaN
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        largest = __vmaxu2(largest, __vmaxu2(*reinterpret_cast<const uint32_t*>(&mn[h]) & 0x7fff7fffu, *reinterpret_cast<const uint32_t*>(&mx[h]) & 0x7fff7fffu));
+    if (__any_sync(0xffffffffu, max(largest & 0xffffu, largest >> 16) >= 0x7c00u)) {
+        const size_t row0 = static_cast<size_t>(j) * N + 16 * t + 2 * gq, tile_step = static_cast<size_t>(T / 8) * N * b;
+        quant_pack_any<T, GT>(src, K, b, packed + static_cast<size_t>(T / 8) * N * GT * (entry >> 3) + static_cast<size_t>(2 * T) * t * b + (T / 16) * lane,
+                              tile_step, scales + row0, zeros + row0);
+        return;
+    }
     RowQuant rq[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {

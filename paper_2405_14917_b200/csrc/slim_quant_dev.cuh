@@ -21,6 +21,7 @@ __device__ __forceinline__ double ld_written_ahead(const double* p) {
 
 // Scale and zero point of Eq. 1 from the group's range (extended to 0), the values slim_quantize_minmax decides in
 // fp64.
+constexpr float kQuotientMax = 32.f;      // from here on a quotient's code is the last one (z and levels are below 16)
 struct RowQuant {
     float s, inv, inv_lo;    // the fp16 scale, and its reciprocal as a sum of two floats
     int z;
@@ -53,12 +54,13 @@ __device__ __forceinline__ RowQuant row_quantizer(float lo, float hi, int levels
     r.s = __half2float(r.s16);
     r.inv = __frcp_rn(r.s);
     r.inv_lo = fmaf(-r.inv, r.s, 1.f) * r.inv;
-    r.z = min(max(static_cast<int>(0x4B400000u - rounded_bits(lo, r)), 0), levels);
+    r.z = min(max(static_cast<int>(0x4B400000u - rounded_bits(fmaxf(lo, -kQuotientMax * r.s), r)), 0), levels);   // lo may be -Inf
     return r;
 }
 
-// clamp(rint(w / s) + z, 0, levels) for any quotient.
+// clamp(rint(w / s) + z, 0, levels) for any quotient; +-Inf is the last or the first code, and NaN the first.
 __device__ __forceinline__ int clamped_code(float w, const RowQuant& r, float z, float levels) {
+    w = fminf(fmaxf(w, -kQuotientMax * r.s), kQuotientMax * r.s);
     const float t = fminf(fmaxf(fmaf(w, r.inv, w * r.inv_lo), -z), levels - z);
     return static_cast<int>(__float_as_uint(t + 12582912.f) - 0x4B400000u) + static_cast<int>(z);
 }
