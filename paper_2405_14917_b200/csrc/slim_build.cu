@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(256, GT == 1 ? 4 : 3) quant_pack_kernel(const 
         const size_t row0 = static_cast<size_t>(j) * N + 16 * t + 2 * gq, tile_step = static_cast<size_t>(T / 8) * N * b;
         quant_pack_any<T, GT>(src, K, b, packed + static_cast<size_t>(T / 8) * N * GT * (entry >> 3) + static_cast<size_t>(2 * T) * t * b + (T / 16) * lane,
                               tile_step, scales + row0, zeros + row0);
+        publish_weights();
         return;
     }
     RowQuant rq[2];
@@ -266,6 +267,7 @@ __global__ void __launch_bounds__(256, GT == 1 ? 4 : 3) quant_pack_kernel(const 
             store2(2, top);
         }
     }
+    publish_weights();
 }
 
 template <int T, int GT>

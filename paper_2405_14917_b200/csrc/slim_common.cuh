@@ -21,6 +21,17 @@ struct GroupTable {
     uint8_t bits[SLIM_MAX_GROUPS];         // bit-width of every K-tile
 };
 
+#ifdef __CUDACC__
+// What a thread has written of packed, scales or zeros, performed before its block ends.  The kernels of a linear layer request
+// these buffers before griddepcontrol.wait, the only point at which a kernel ahead that did not signal anything is sure to have
+// flushed its writes; without this fence they would rely on when a block's last stores land.  The proxy fence is for the
+// readers that use bulk copies.
+__device__ __forceinline__ void publish_weights() {
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    __threadfence();
+}
+#endif
+
 void set_cuda_error(cudaError_t e);
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

@@ -491,6 +491,7 @@ __global__ void __launch_bounds__(128) gptq_quant_kernel(double* w, uint8_t* cod
     if (lane == 0) {
         scales[n] = r.s16;
         zeros[n] = __float2half_rn(r.z);
+        if (last) publish_weights();
     }
 #pragma unroll
     for (int i = 0; i < CPL; ++i) v[i] = static_cast<double>(r.s) * static_cast<double>(static_cast<float>(r.codes[i]) - r.z) - v[i];

@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const uint8_t* __restrict__ c
         }
     }
     packed[4ull * N * gt.prefix[j] + wi] = word;
+    publish_weights();
 }
 
 // One thread per 8 consecutive columns of one row: reads one word per slice, writes 16 bytes.

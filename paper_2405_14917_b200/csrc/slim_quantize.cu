@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(256) quantize_minmax_kernel(const __half* __re
         if (lane == 0) {
             scales[static_cast<size_t>(j) * N + n] = __ushort_as_half(double_to_half_bits_rn(sum / static_cast<double>(GS / 2)));   // 2 * mean
             zeros[static_cast<size_t>(j) * N + n] = __float2half_rn(0.5f);
+            publish_weights();
         }
         return;
     }
@@ -195,6 +196,7 @@ __global__ void __launch_bounds__(256) quantize_minmax_kernel(const __half* __re
     if (lane == 0) {
         scales[static_cast<size_t>(j) * N + n] = s16;
         zeros[static_cast<size_t>(j) * N + n] = __float2half_rn(static_cast<float>(z));
+        publish_weights();
     }
 }
 
@@ -310,6 +312,7 @@ __global__ void __launch_bounds__(kSqcWarps * 32) quantize_sqc_kernel(const __ha
     if (lane == 0) {
         scales[static_cast<size_t>(j) * N + n] = r.s16;
         zeros[static_cast<size_t>(j) * N + n] = __float2half_rn(r.z);
+        publish_weights();
         if (tau_index != nullptr) tau_index[static_cast<size_t>(j) * N + n] = r.index;
     }
 }

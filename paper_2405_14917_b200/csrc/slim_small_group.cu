@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(256) pack_small_kernel(const uint8_t* __restri
     uint32_t item = 0;
     for (int f = 0; f < nf; ++f) item |= ((static_cast<uint32_t>(src[f]) >> lo) & mask) << (w * f);
     *reinterpret_cast<item_t*>(packed + small_item_offset<T>(N, st, j, t, unit, lane, half)) = static_cast<item_t>(item);
+    publish_weights();
 }
 
 // Code of (row, column kk of group j) from its items.
