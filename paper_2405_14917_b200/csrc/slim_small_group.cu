@@ -296,8 +296,15 @@ template <int T, int NT, int R, int WARPS>
 static cudaError_t launch_small(const __half* x, const uint8_t* packed, const __half* scales, const __half* zeros, __half* y, int M, int N, int K,
                                 const SmallTable& st, cudaStream_t s) {
     PdlLaunch l(static_cast<unsigned>(((N >> 4) + R - 1) / R), 32 * WARPS, 0, s);
-    l.cfg.gridDim.y = static_cast<unsigned>((M + 8 * NT - 1) / (8 * NT));
-    return cudaLaunchKernelEx(&l.cfg, linear_small_kernel<T, NT, R, WARPS>, x, packed, scales, zeros, y, M, N, K, 0x64006400u, st);
+    constexpr int kMost = 65535 * 8 * NT;                  // tokens of a launch: the second grid dimension
+    for (int m0 = 0; m0 < M; m0 += kMost) {
+        const int m = M - m0 < kMost ? M - m0 : kMost;
+        l.cfg.gridDim.y = static_cast<unsigned>((m + 8 * NT - 1) / (8 * NT));
+        const cudaError_t e = cudaLaunchKernelEx(&l.cfg, linear_small_kernel<T, NT, R, WARPS>, x + static_cast<size_t>(m0) * K, packed, scales, zeros,
+                                                 y + static_cast<size_t>(m0) * N, m, N, K, 0x64006400u, st);
+        if (e != cudaSuccess || M - m0 <= kMost) return e;
+    }
+    return cudaSuccess;
 }
 // 16 rows and 16 warps per block up to 16 tokens (blocks are few and the chain of a warp is what counts), 32 rows and 8 warps
 // for more: the loads of x and the ones MMAs serve two row tiles.

@@ -5,6 +5,7 @@ import torch
 
 from oracle import slim_oracle as orc
 from paper_2405_14917_b200 import binding as slim
+from paper_2405_14917_b200 import workloads as wl
 from tests.helpers import check_output
 
 pytestmark = pytest.mark.gpu
@@ -29,3 +30,17 @@ def test_tiles_of_tokens_and_rows(N, K, M, g):
     slim.workspace_status(ws)
     W = np.repeat(scales.astype(np.float64), g, axis=0).T * (codes - np.repeat(zeros.astype(np.float64), g, axis=0).T)
     check_output(y.cpu().numpy(), x.astype(np.float64) @ W.T, f"{N}x{K} M={M} g={g}")
+
+
+def test_more_tokens_than_one_launch_takes():
+    """65535 blocks of 32 tokens are the second grid dimension's limit; a second launch does the rest."""
+    N, K, g, M = 16, 128, 64, 65535 * 32 + 45
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(4)
+    W, norms = wl.make_weight_and_norms_device((5, N, K), N, K, "cuda")
+    L = slim.QuantLinear.from_weight(W, norms, 2, g=g)
+    x = torch.randn((M, K), generator=gen, device="cuda", dtype=torch.float16)
+    y = L.forward(x, slim.new_workspace(M, N, K, L.bits, g=g))
+    for m0 in (0, 65535 * 32 - 100, M - 300):                       # the same tokens by themselves
+        part = x[m0:m0 + 200].contiguous()
+        assert torch.equal(L.forward(part, slim.new_workspace(200, N, K, L.bits, g=g)), y[m0:m0 + 200])
