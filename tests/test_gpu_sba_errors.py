@@ -104,3 +104,17 @@ def test_a_small_workspace_means_several_walks_and_the_same_errors(N, K, M, g, a
         assert p == results[0][0] and (bits == results[0][1]).all() and (errors == results[0][2]).all()
     with pytest.raises(slim.SlimError):
         slim.sba_search(W, x, a, avg, workspace=torch.empty(layer - 256, dtype=torch.uint8, device="cuda"), g=g)
+
+
+# A CTA of the search takes 16, 32, 48, 64 or 80 rows, whatever fills the last wave of 148 CTAs per 128 tokens best.  Below: every one of
+# them at each width of the operand's chunk (groups of 32, 64, 128 columns, and several chunks per group), with a last CTA that
+# is full, ends in its first half, or reaches into the second, and with a second and third block of tokens.
+@pytest.mark.parametrize("rows,N,M", [(16, 1184, 129), (32, 3280, 20), (32, 1200, 200), (48, 4752, 20), (48, 2384, 200), (64, 7120, 20),
+                                      (80, 9488, 20), (80, 3168, 300), (80, 4752, 129)])
+@pytest.mark.parametrize("g", [32, 64, 128, 256])
+def test_every_form_of_the_search_kernel(rows, N, M, g):
+    K = 768
+    W, a, x = _inputs(N, K, M, seed=rows + N + g)
+    _, _, got = _slim().sba_search(W, x, a, 2 + (g >> 6 & 1), g=g)
+    want = _errors(W, x, a, 2 + (g >> 6 & 1), g)
+    assert np.linalg.norm(got - want) <= CURVE_RTOL * np.linalg.norm(want), (np.linalg.norm(got - want) / np.linalg.norm(want))
