@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("N,K,M", [
-    (16, 8192, 17),       # one piece: the other pairs of the tile finish nothing
+    (16, 8192, 17),       # the kernel for a few tokens takes this one
     (272, 4096, 40),      # fewer pieces than pairs; a second row block of one tile
     (512, 8192, 200),     # seven pieces in a tile of 256 tokens
     (256, 2048, 300),     # a second token tile with two pieces, the last one of 12 tokens
@@ -20,6 +20,18 @@ pytestmark = pytest.mark.gpu
     (1296, 512, 700),     # whole tiles of equal width
 ])
 def test_pieces_and_pairs(N, K, M):
+    _check(N, K, M)
+
+
+@pytest.mark.parametrize("N,K,M", [(16, 8320, 17), (272, 8320, 32)])
+def test_one_piece_and_several_pairs(N, K, M):
+    """65 K-tiles are too many for the kernel for a few tokens, so these are tiles of the batched one with a single piece: the
+    pair that has it finishes the tile, the others only hand over theirs."""
+    assert slim.workspace_bytes(M, N, K, np.full(K // 128, 3, dtype=np.uint8)) >= 4 * ((N + 255) // 256) * 128 * 128 * 4     # two pairs per tile at least
+    _check(N, K, M)
+
+
+def _check(N, K, M):
     L = oracle_layer(N, K, 3, M, seed_name="gemm-cuts")
     ref = orc.linear_f64(L["x"], L["codes"], L["scales"], L["zeros"])
     x, packed = torch.from_numpy(L["x"]).cuda(), torch.from_numpy(orc.pack(L["codes"], L["bits"])).cuda()
