@@ -144,10 +144,9 @@ int slim_dequant(const void* packed, const uint8_t* bits_host, const void* scale
  * shared memory with all CTAs resident at once; the others, and M > 1, multiply the fp16 x as it is).
  * The per-layer kernels are launched with programmatic stream serialisation and fetches packed, scales and zeros
  * before it waits for the kernel ahead of it on the stream: those three buffers must be complete when the call is
- * enqueued, or be written by a kernel of this library or by one that does not signal programmatic launch completion early
- * and makes its writes visible to the device itself (__threadfence after the last of them); after any other kernel put
- * something between that is not a kernel, an event for instance (x and y may be produced and consumed by the neighbouring
- * kernels as usual).  At M = 1 the two kernels of the 32 MB route are launched
+ * enqueued, or be written by a call of this library (each of which ends in a kernel that makes them so); between a kernel of
+ * another origin that writes them and the call there has to be one more kernel, launched in plain stream order (x and y
+ * may be produced and consumed by the neighbouring kernels as usual).  At M = 1 the two kernels of the 32 MB route are launched
  * the same way, but touch no buffer before they have waited for the kernel ahead of them. */
 int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host,
                   const void* scales, const void* zeros, void* y,

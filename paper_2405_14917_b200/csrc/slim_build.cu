@@ -170,7 +170,6 @@ __global__ void __launch_bounds__(256, GT == 1 ? 4 : 3) quant_pack_kernel(const 
         const size_t row0 = static_cast<size_t>(j) * N + 16 * t + 2 * gq, tile_step = static_cast<size_t>(T / 8) * N * b;
         quant_pack_any<T, GT>(src, K, b, packed + static_cast<size_t>(T / 8) * N * GT * (entry >> 3) + static_cast<size_t>(2 * T) * t * b + (T / 16) * lane,
                               tile_step, scales + row0, zeros + row0);
-        publish_weights();
         return;
     }
     RowQuant rq[2];
@@ -267,7 +266,6 @@ __global__ void __launch_bounds__(256, GT == 1 ? 4 : 3) quant_pack_kernel(const 
             store2(2, top);
         }
     }
-    publish_weights();
 }
 
 template <int T, int GT>
@@ -331,6 +329,7 @@ int slim_quantize_layer(const void* W, const float* act_norm, int avg_bits, int 
             : g == 128 ? slim::launch_quant_pack<128, 1>(w, table, pk, sc, zp, N, K, G, s)
             : g == 256 ? slim::launch_quant_pack<128, 2>(w, table, pk, sc, zp, N, K, G, s)
                        : slim::launch_quant_pack<128, 4>(w, table, pk, sc, zp, N, K, G, s);
+        if (e == cudaSuccess) e = slim::launch_boundary(s);
     }
     if (e == cudaSuccess) e = cudaEventSynchronize(ready);
     cudaEventDestroy(ready);

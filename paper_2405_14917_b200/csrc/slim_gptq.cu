@@ -491,7 +491,6 @@ __global__ void __launch_bounds__(128) gptq_quant_kernel(double* w, uint8_t* cod
     if (lane == 0) {
         scales[n] = r.s16;
         zeros[n] = __float2half_rn(r.z);
-        if (last) publish_weights();
     }
 #pragma unroll
     for (int i = 0; i < CPL; ++i) v[i] = static_cast<double>(r.s) * static_cast<double>(static_cast<float>(r.codes[i]) - r.z) - v[i];
@@ -676,6 +675,7 @@ int slim_gptq_quantize(const void* W, const void* x, const uint8_t* bits_host, d
             SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, slim::gptq_update_kernel, w, static_cast<const double*>(R), N, K, c0, g));
         }
     }
+    SLIM_CUDA_TRY(slim::launch_boundary(s));
     return SLIM_OK;
 }
 

@@ -38,7 +38,6 @@ __global__ void __launch_bounds__(256) pack_kernel(const uint8_t* __restrict__ c
         }
     }
     packed[4ull * N * gt.prefix[j] + wi] = word;
-    publish_weights();
 }
 
 // One thread per 8 consecutive columns of one row: reads one word per slice, writes 16 bytes.
@@ -74,6 +73,14 @@ __global__ void __launch_bounds__(256) dequant_kernel(const uint32_t* __restrict
     *reinterpret_cast<uint4*>(W + static_cast<size_t>(row) * K + k0) = *reinterpret_cast<const uint4*>(out);
 }
 
+__global__ void boundary_kernel() {}
+cudaError_t launch_boundary(cudaStream_t s) {
+    const cudaError_t e = cudaGetLastError();              // of the launch that this one ends
+    if (e != cudaSuccess) return e;
+    boundary_kernel<<<1, 32, 0, s>>>();
+    return cudaGetLastError();
+}
+
 }  // namespace slim
 
 extern "C" {
@@ -89,7 +96,7 @@ int slim_pack_weights(const uint8_t* codes, const uint8_t* bits_host, void* pack
     const long long max_words = 4ll * N * 4;
     dim3 grid(static_cast<unsigned>((max_words + 255) / 256), static_cast<unsigned>(gt.G));
     slim::pack_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(codes, static_cast<uint32_t*>(packed), N, K, gt);
-    SLIM_CUDA_TRY(cudaGetLastError());
+    SLIM_CUDA_TRY(slim::launch_boundary(static_cast<cudaStream_t>(stream)));
     return SLIM_OK;
 }
 

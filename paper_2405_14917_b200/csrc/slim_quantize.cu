@@ -175,7 +175,6 @@ __global__ void __launch_bounds__(256) quantize_minmax_kernel(const __half* __re
         if (lane == 0) {
             scales[static_cast<size_t>(j) * N + n] = __ushort_as_half(double_to_half_bits_rn(sum / static_cast<double>(GS / 2)));   // 2 * mean
             zeros[static_cast<size_t>(j) * N + n] = __float2half_rn(0.5f);
-            publish_weights();
         }
         return;
     }
@@ -196,7 +195,6 @@ __global__ void __launch_bounds__(256) quantize_minmax_kernel(const __half* __re
     if (lane == 0) {
         scales[static_cast<size_t>(j) * N + n] = s16;
         zeros[static_cast<size_t>(j) * N + n] = __float2half_rn(static_cast<float>(z));
-        publish_weights();
     }
 }
 
@@ -261,7 +259,7 @@ static int quantize_minmax_impl(const void* W, const uint8_t* bits_host, uint8_t
         slim::quantize_minmax_kernel<decltype(tag)::value><<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
             static_cast<const __half*>(W), codes, static_cast<__half*>(scales), static_cast<__half*>(zeros), N, K, sign_alpha, sub, gb);
     });
-    SLIM_CUDA_TRY(cudaGetLastError());
+    SLIM_CUDA_TRY(slim::launch_boundary(static_cast<cudaStream_t>(stream)));
     return SLIM_OK;
 }
 
@@ -312,7 +310,6 @@ __global__ void __launch_bounds__(kSqcWarps * 32) quantize_sqc_kernel(const __ha
     if (lane == 0) {
         scales[static_cast<size_t>(j) * N + n] = r.s16;
         zeros[static_cast<size_t>(j) * N + n] = __float2half_rn(r.z);
-        publish_weights();
         if (tau_index != nullptr) tau_index[static_cast<size_t>(j) * N + n] = r.index;
     }
 }
@@ -337,6 +334,6 @@ extern "C" int slim_quantize_sqc(const void* W, const uint8_t* bits_host, uint8_
             static_cast<const __half*>(W), codes, static_cast<__half*>(scales), static_cast<__half*>(zeros), tau_index, N, K,
             lambda, n, gb);
     });
-    SLIM_CUDA_TRY(cudaGetLastError());
+    SLIM_CUDA_TRY(slim::launch_boundary(static_cast<cudaStream_t>(stream)));
     return SLIM_OK;
 }

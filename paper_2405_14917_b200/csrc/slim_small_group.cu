@@ -74,7 +74,6 @@ __global__ void __launch_bounds__(256) pack_small_kernel(const uint8_t* __restri
     uint32_t item = 0;
     for (int f = 0; f < nf; ++f) item |= ((static_cast<uint32_t>(src[f]) >> lo) & mask) << (w * f);
     *reinterpret_cast<item_t*>(packed + small_item_offset<T>(N, st, j, t, unit, lane, half)) = static_cast<item_t>(item);
-    publish_weights();
 }
 
 // Code of (row, column kk of group j) from its items.
@@ -344,7 +343,7 @@ int small_pack(const uint8_t* codes, const uint8_t* bits_host, void* packed, int
     const dim3 grid(static_cast<unsigned>((4ll * N * 4 + 255) / 256), static_cast<unsigned>(st.G));
     if (g == 32) pack_small_kernel<32><<<grid, 256, 0, s>>>(codes, static_cast<uint8_t*>(packed), N, K, st);
     else pack_small_kernel<64><<<grid, 256, 0, s>>>(codes, static_cast<uint8_t*>(packed), N, K, st);
-    SLIM_CUDA_TRY(cudaGetLastError());
+    SLIM_CUDA_TRY(launch_boundary(s));
     return SLIM_OK;
 }
 
