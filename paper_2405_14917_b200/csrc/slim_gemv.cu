@@ -587,8 +587,8 @@ int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host, c
         const int taken = slim::gemv_one(x, packed, gt, scales, zeros, y, M, N, K, workspace, s);
         if (taken <= 0) return taken;
     }
-    // More tokens, or one whose layer does not fit that kernel: the layer cut over the whole GPU in one launch.  What is
-    // left for the kernel of this file are more than 8 tokens on a K whose fragments do not fit (about 28000 columns).
+    // More tokens, or one whose layer does not fit that kernel: the layer cut over the whole GPU in one launch.  What that leaves
+    // for the kernel of this file (general_is_sooner there): small layers of two or three tokens, and more than 8 on a long K.
     {
         const int taken = slim::gemv_few(x, packed, gt, scales, zeros, y, M, N, K, workspace, s);
         if (taken <= 0) return taken;

@@ -336,7 +336,7 @@ static int few_clusters(int log_cs) {
 }
 
 struct FewPlan {
-    int log_cs, np, pw, npw, kw, n_slots, slot_bytes, sz_off;
+    int log_cs, gc, np, pw, npw, kw, n_slots, slot_bytes, sz_off;
     uint32_t off_x, off_ring;
     size_t smem;
 };
@@ -355,6 +355,7 @@ static bool few_plan(int M, int N, const GroupTable& gt, int log_cs, FewPlan* pl
         gc = gc > b - a ? gc : b - a;
         slices = slices > sl ? slices : sl;
     }
+    pl->gc = gc;
     pl->off_x = kFewOffE + few_sums(nt) * static_cast<uint32_t>(gc);
     pl->off_ring = pl->off_x + static_cast<uint32_t>(slices) * (8 * 8 * nt * 32);
     pl->sz_off = 2 * pl->np * 256 * bmax;
@@ -386,6 +387,19 @@ static bool few_plan(int M, int N, const GroupTable& gt, int log_cs, FewPlan* pl
     return best < 1 << 30;
 }
 
+// Layers of 2 to 16 tokens that are sooner through the kernel of slim_gemv.cu (us, that kernel / this one, average 3 bits):
+//  * two or three tokens and one K-tile or up to 2^18 weights: a launch of fewer steps.  2048 x 128 2.6 / 3.6, 512 x 512 3.2 / 3.4, 128 x
+//    2048 3.2 / 3.5; beyond, 1024 x 512 at 2 tokens 3.4 / 3.4, 512 x 2048 4.1 / 3.7.
+//  * 9 tokens or more, a pair of row tiles per cluster and 64 K-tiles or more: a CTA stages 8 K-tiles of x and more for few
+//    products, where that kernel has x staged once.  256 x 8192 5.7 / 6.4 (9 tokens), 6.3 / 7.7 (16), 512 x 16384 8.0 / 9.9, 9.6 / 8.8 (16:
+//    it can go the other way), 64 x 28672 12.7 / 18.3; two pairs: 1024 x 8192 9.6 / 6.9.
+//  * as many and the longest K, whose fragments leave sums for fewer than six warps: 512 x 32768 13.3 / 36.0 (9), 1024 x 32768 27.5 / 39.7.
+static bool general_is_sooner(int M, int N, int G, const FewPlan& pl) {
+    if (M <= 3) return G == 1 || static_cast<size_t>(N) * G * SLIM_GROUP <= (1u << 18);
+    if (M <= 8) return false;
+    return (pl.np == 1 && G >= 64) || (pl.gc >= 32 && pl.npw * pl.kw < 6);
+}
+
 // Enqueues the layer and returns SLIM_OK, a negative status on failure, or 1 if this shape is not for this kernel.
 int gemv_few(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y,
              int M, int N, int K, void* workspace, cudaStream_t stream) {
@@ -402,6 +416,7 @@ int gemv_few(const void* x, const void* packed, const GroupTable& gt, const void
         for (int log_cs = 3; log_cs >= 1 && !fits; --log_cs) fits = log_cs != first && few_plan(M, N, gt, log_cs, &pl);
         if (!fits) return 1;
     }
+    if (M >= 2 && M <= SLIM_GEMV_MAX_M && general_is_sooner(M, N, gt.G, pl)) return 1;
     FewParams prm;
     memset(&prm, 0, sizeof prm);
     prm.x = static_cast<const __half*>(x);
