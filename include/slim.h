@@ -100,7 +100,8 @@ int slim_workspace_bytes(int M, int N, int K, int g, const uint8_t* bits_host, s
 
 /* Zeroes a workspace (status word, stream-K flags).  Must be enqueued once after allocating a
  * workspace, before its first use; the kernels leave the flags zeroed.  Calls that share a
- * workspace must be ordered on one stream. */
+ * workspace must be ordered on one stream.  slim_mpq_gemv and slim_mpq_gemm may share one of the larger of the two sizes that
+ * slim_workspace_bytes reports; the workspace of a layer set is its own. */
 int slim_workspace_init(void* workspace, size_t workspace_bytes, void* stream);
 
 /* Synchronises `stream`, reads and clears the workspace status word.  Returns SLIM_OK, or

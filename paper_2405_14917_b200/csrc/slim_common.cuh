@@ -30,6 +30,10 @@ cudaError_t launch_boundary(cudaStream_t s);
 
 void set_cuda_error(cudaError_t e);
 
+// Start of a linear layer's workspace: the status word (256 bytes), then the flags of slim_mpq_gemm, which have to be zero
+// between its launches.  The other calls put nothing there (or zeros), so that one workspace serves them all in turn.
+constexpr int kWsFlagsOffset = 256, kWsFlagsBytes = 1024;
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Scratch bytes slim_mpq_gemm wants for (M, N) on the current device (256 when it needs none).

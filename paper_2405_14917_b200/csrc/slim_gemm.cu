@@ -79,9 +79,10 @@ struct GemmParams {
     GroupTable gt;
 };
 
-constexpr int kGemmWsFlags = 256;            // byte offset of the flags in the workspace
+constexpr int kGemmWsFlags = kWsFlagsOffset; // byte offset of the flags in the workspace
 constexpr int kGemmMaxGrid = 256;
 constexpr int kGemmWsPartials = kGemmWsFlags + 4 * kGemmMaxGrid;
+static_assert(4 * kGemmMaxGrid == kWsFlagsBytes, "the other calls leave this much alone");
 
 // ------------------------------------------------------------------------------------------ PTX helpers
 namespace g {

@@ -448,13 +448,13 @@ static bool plan_gemv(int M, int N, const GroupTable& gt, bool pre, GemvPlan* pl
     return false;
 }
 
-// Scratch layout of the pre-staged mode: header, then sums [G][16] float2, then fragments.
-static size_t prestage_sxe_offset() { return kWsHeader; }
-static size_t prestage_xs_offset(int G) { return kWsHeader + static_cast<size_t>(G) * 128; }
-static size_t prestage_bytes(int M, const GroupTable& gt) {
+// Scratch layout of the pre-staged mode, from `base` on: sums [G][16] float2, then fragments.  The base is behind the flags of
+// slim_mpq_gemm, or over them in a workspace without room for both.
+constexpr size_t kPreStageBase = kWsFlagsOffset + kWsFlagsBytes;
+static size_t prestage_bytes(int M, const GroupTable& gt, size_t base = kPreStageBase) {
     int slots = gt.G;
     for (int j = 0; j < gt.G; ++j) slots += gt.bits[j] == 3 ? 1 : 0;
-    return prestage_xs_offset(gt.G) + static_cast<size_t>(slots) * 8 * M * 32;
+    return base + static_cast<size_t>(gt.G) * 128 + static_cast<size_t>(slots) * 8 * M * 32;
 }
 
 static cudaError_t launch_stage_x(const StageParams& sp, cudaStream_t stream) {
@@ -595,7 +595,8 @@ int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host, c
     }
     // From kPreStageMinM tokens on, a small kernel puts x into fragment order once, in the
     // workspace; with a workspace too small for that every CTA stages its own part of x.
-    const bool pre = M >= slim::kPreStageMinM && workspace_bytes >= slim::prestage_bytes(M, gt);
+    const size_t base = workspace_bytes >= slim::prestage_bytes(M, gt) ? slim::kPreStageBase : static_cast<size_t>(slim::kWsHeader);
+    const bool pre = M >= slim::kPreStageMinM && workspace_bytes >= slim::prestage_bytes(M, gt, base);
     slim::GemvPlan pl;
     if (!slim::plan_gemv(M, N, gt, pre, &pl)) return SLIM_ERR_UNSUPPORTED;
 
@@ -626,8 +627,8 @@ int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host, c
         slim::StageParams sp;
         memset(&sp, 0, sizeof sp);
         sp.x = prm.x;
-        sp.sxe_g = reinterpret_cast<float2*>(ws + slim::prestage_sxe_offset());
-        sp.xs_g = ws + slim::prestage_xs_offset(gt.G);
+        sp.sxe_g = reinterpret_cast<float2*>(ws + base);
+        sp.xs_g = ws + base + static_cast<size_t>(gt.G) * 128;
         sp.M = M; sp.K = K; sp.G = gt.G;
         memcpy(sp.pre3, prm.pre3, sizeof sp.pre3);
         memcpy(sp.bits, gt.bits, sizeof sp.bits);

@@ -901,11 +901,13 @@ constexpr size_t kRouteMinBytes = 32u << 20;
 
 struct RouteLayout {
     SetGeometry sg;
-    int n_rb, sp;
+    int n_rb, sp, cnt0;
     size_t plan_off, plan_bytes, x_off, part_off, total;
 };
 
-static bool route_layout(int M, int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt, RouteLayout* r) {
+// keep_flags: the first counters, which stay zero, lie over the flags of slim_mpq_gemm; without, everything is kWsFlagsBytes sooner.
+static bool route_layout(int M, int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt, bool keep_flags, RouteLayout* r) {
+    static_assert(kSetOffCounters == kWsFlagsOffset, "the counters are cleared where the flags are");
     if (M < 1 || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < kRouteMinBytes) return false;
     slim_layer L;
     memset(&L, 0, sizeof L);
@@ -914,7 +916,8 @@ static bool route_layout(int M, int N, int K, int g, const uint8_t* bits_host, c
     const int tpi = kSetConsumers * r->sg.tpw;
     r->n_rb = ((N >> 4) + tpi - 1) / tpi;
     r->sp = layer_split(r->sg.split, gt.G);
-    r->plan_off = kSetOffCounters + r->sg.cnt_bytes;
+    r->cnt0 = keep_flags ? kWsFlagsBytes / static_cast<int>(sizeof(unsigned int)) : 0;
+    r->plan_off = kSetOffCounters + r->cnt0 * sizeof(unsigned int) + r->sg.cnt_bytes;
     r->plan_bytes = set_plan_bytes(1, static_cast<long long>(r->n_rb) * r->sp);
     r->x_off = r->plan_off + align_to(r->plan_bytes, 256);
     r->part_off = r->x_off + layer_ws_bytes(r->sg.mres, gt);
@@ -924,7 +927,7 @@ static bool route_layout(int M, int N, int K, int g, const uint8_t* bits_host, c
 
 size_t gemv_route_workspace_bytes(int M, int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt) {
     RouteLayout r;
-    return route_layout(M, N, K, g, bits_host, gt, &r) ? r.total : 0;
+    return route_layout(M, N, K, g, bits_host, gt, true, &r) ? r.total : 0;
 }
 
 }  // namespace slim
@@ -981,12 +984,13 @@ static int launch_set_for(const slim_gemv_set_info* info, const SetParams& prm, 
 int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, const GroupTable& gt, const void* scales, const void* zeros,
                void* y, int M, int N, int K, int g, void* workspace, size_t workspace_bytes, cudaStream_t stream) {
     RouteLayout r;
-    if (!route_layout(M, N, K, g, bits_host, gt, &r) || workspace_bytes < r.total) return 1;
+    if (!route_layout(M, N, K, g, bits_host, gt, true, &r)) return 1;
+    if (workspace_bytes < r.total && (!route_layout(M, N, K, g, bits_host, gt, false, &r) || workspace_bytes < r.total)) return 1;
     slim_layer L;
     memset(&L, 0, sizeof L);
     L.x = x; L.packed = packed; L.scales = scales; L.zeros = zeros; L.y = y; L.bits_host = bits_host; L.M = M; L.N = N; L.K = K;
     SetLayer d;
-    fill_descriptor(L, gt, r.sg.mpad, 0, r.x_off, r.sp, r.part_off, 0, &d);
+    fill_descriptor(L, gt, r.sg.mpad, 0, r.x_off, r.sp, r.part_off, r.cnt0, &d);
     uint8_t* plan = static_cast<uint8_t*>(workspace) + r.plan_off;
     const long long n_items = static_cast<long long>(r.n_rb) * r.sp;
     const int grid = static_cast<int>(n_items < r.sg.grid ? n_items : r.sg.grid);
@@ -1003,7 +1007,7 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
     info.max_tokens = r.sg.mmax;
     info.tiles_per_warp = r.sg.tpw;
     info.split = r.sg.split;
-    info.n_counters = r.sg.n_counters;
+    info.n_counters = r.cnt0 + r.sg.n_counters;
     info.plan_bytes = r.plan_bytes;
     info.workspace_bytes = r.total;
     SetParams prm;
