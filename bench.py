@@ -951,6 +951,25 @@ def secondary_entries(args, device, timer, primary_layers, clock_gpu):
     return out
 
 
+def short(o):
+    """Floats to seven digits: what is kept of the output is less than 3000 characters, and the line has to fit whole."""
+    if isinstance(o, dict):
+        return {k: short(v) for k, v in o.items()}
+    if isinstance(o, list):
+        return [short(v) for v in o]
+    return float(f"{o:.7g}") if isinstance(o, float) else o
+
+
+def summary(entries):
+    """Name -> rate (GB/s, prefill TFLOP/s) of the secondary entries: in full they make the line 27 kB."""
+    out = {}
+    for e in entries:
+        rate = e.get("value", e.get("rotating_per_layer", {}).get("value"))
+        name = e["name"].replace("llama", "").replace("decode-", "").replace("-blocks8", "")
+        out[name] = e.get("error", "")[:40] if rate is None else round(rate)
+    return out
+
+
 def run_ours(args, spec):
     import torch
     import torch.distributed as dist
@@ -995,10 +1014,11 @@ def run_ours(args, spec):
     elif "traffic" not in line["roofline"]:
         line["roofline"]["traffic"] = None
     if world == 1 and args.workload == "llama7b-decode-avg2" and not args.no_secondary:
-        line["secondary"] = secondary_entries(args, device, timer, layers, clock_gpu)
+        entries = secondary_entries(args, device, timer, layers, clock_gpu)
+        line["secondary"] = entries if args.secondary_full else summary(entries)
     if world == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline_legs(spec) if M <= slim.GEMV_MAX_M else cpu_baseline(spec)
-    print(json.dumps(line), flush=True)
+    print(json.dumps(short(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
@@ -1016,6 +1036,7 @@ def main():
                          "or the calls a decoder can issue (per block: q/k/v as a set, o, gate/up as a set, down)")
     ap.add_argument("--min-seconds", type=float, default=1.0,
                     help="blocks of --steps steps are repeated until this much timed work has run; the median block is reported")
+    ap.add_argument("--secondary-full", action="store_true", help="default workload only: the other configurations with timing, roofline, config and clocks")
     ap.add_argument("--no-secondary", action="store_true", help="default workload only: skip the other configurations of the same JSON line")
     args = ap.parse_args()
     if args.workload == "sqc-llama7b-block" and args.impl != "reference":
