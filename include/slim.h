@@ -33,8 +33,8 @@
  * (slim_quantize_minmax, _groups, _sign1, _sqc; these also take a K that is any multiple of g), the SBA search and
  * the GPTQ loop take every g; the layer-set launch and slim_mpq_gemm_static take 128, 256 and 512
  * (SLIM_ERR_UNSUPPORTED otherwise).  Groups of 256 and 512 columns run on the tensor-core kernels of the 128-column tiles (a group is 2 or 4
- * tiles that share a row of scales and zeros); groups of 32 and 64 columns run on a kernel of their own, and the
- * batched entry point then wants room for the fp16 weights in its workspace (slim_workspace_bytes says how much).
+ * tiles that share a row of scales and zeros); groups of 32 and 64 columns run on a kernel of their own, which
+ * needs no workspace beyond the 256 bytes of the status header, whatever the number of tokens.
  *
  * Packed format ("sliced bit planes", version SLIM_FORMAT_VERSION).  K is cut into K-tiles of T = min(g, 128)
  * columns; a group of more than 128 columns is g/128 consecutive K-tiles of its bit-width.  K-tiles are stored back
@@ -154,9 +154,9 @@ int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host,
                   int M, int N, int K, int g,
                   void* workspace, size_t workspace_bytes, void* stream);
 
-/* Host-only introspection: the launch plan of slim_mpq_gemv's general kernel (M >= 2, and the single-token layers whose
- * K does not fit the single-token kernel) for this shape on the current device
- * (148 SMs assumed when no device is present).  out6 = {16-row tiles per CTA, k-slices =
+/* Host-only introspection: the launch plan that the general kernel of slim_mpq_gemv has for this shape on the current device
+ * (148 SMs assumed when no device is present), whichever kernel runs it.  The general one has what it is soonest at: two or
+ * three tokens on small layers, and 9 and more on few rows or the longest K.  out6 = {16-row tiles per CTA, k-slices =
  * cluster size, row blocks, dynamic shared memory bytes, 8-token MMA tiles, groups per chunk}.
  * grid = k-slices x row blocks, 8 warps per CTA. */
 int slim_gemv_plan(int M, int N, int K, int g, const uint8_t* bits_host, int* out6);

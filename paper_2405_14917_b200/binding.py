@@ -164,7 +164,7 @@ def workspace_bytes(M: int, N: int, K: int, bits, g: int = GROUP) -> int:
 
 
 def gemv_plan(M: int, N: int, K: int, bits, g: int = GROUP) -> dict:
-    """Launch plan of slim_mpq_gemv for this shape (host-only)."""
+    """Launch plan that slim_mpq_gemv's general kernel has for this shape, whichever kernel runs it (host-only)."""
     b = _bits(bits)
     out = (ctypes.c_int * 6)()
     _check("slim_gemv_plan", lib().slim_gemv_plan(M, N, K, g, _bp(b), ctypes.cast(out, ctypes.c_void_p)))

@@ -4,7 +4,7 @@
 // A decode-sized layer is a few megabytes, so the launch is over in a few microseconds and what counts is the
 // length of the dependent chain inside a CTA, not the instruction count.  Hence:
 //
-//  * a CTA owns 2, 4, 6 or 8 tiles of 16 rows and the WHOLE K: no partial sums leave the CTA and there is no second
+//  * a CTA owns 2, 4, 6, 8 or 10 tiles of 16 rows and the WHOLE K: no partial sums leave the CTA and there is no second
 //    pass.  The tile count is the smallest for which all CTAs of the layer are resident at once (else the one that
 //    needs the fewest waves).
 //  * warp w owns the groups w, w + 16, ... of the CTA's tiles: it brings their slices with one cp.async.bulk per
@@ -244,8 +244,8 @@ __global__ void __launch_bounds__(kOneThreads, PAIRS == 1 ? 2 : 1) gemv_one_kern
     one_body<PAIRS>(p, static_cast<int>(blockIdx.x), p.ws, smem);
 }
 
-// Several layers in one launch, every CTA resident at once: layer l owns the CTAs cta0[l] .. cta0[l + 1] (whole
-// clusters).  The descriptors live in the plan buffer of the set; a CTA copies its own into shared memory first.
+// Several layers in one launch, every CTA resident at once: layer l owns the CTAs cta0[l] .. cta0[l + 1] (a multiple of
+// kOneSetPad).  The descriptors live in the plan buffer of the set; a CTA copies its own into shared memory first.
 template <int PAIRS>
 __global__ void __launch_bounds__(kOneThreads, PAIRS == 1 ? 2 : 1) gemv_one_set_kernel(const OneParams* __restrict__ layers,
                                                                                      const int* __restrict__ cta0, int n_layers,

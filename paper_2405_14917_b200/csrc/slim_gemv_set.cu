@@ -66,9 +66,10 @@ struct SetLayer {
     int M, N, K, G;
     uint16_t count[4];     // groups of 1, 2, 3, 4 bits
     int task0;             // first (token, group) staging task of the layer
-    int MP;                // 256-byte pieces per slice in the staged layout: 8 or 16 = tokens of the f16 fragments for the
-                           // whole set (absent tokens are staged as zeros, so the kernel reads without a test); 2 if every
-                           // layer of the set has one token: the 8-bit digit form (stage_groups_i8)
+    int MP;                // 256-byte pieces per slice in the staged layout: a multiple of 8 up to 64 = tokens of the f16 fragments
+                           // for the whole set (what a layer does not have is not staged: the kernel multiplies whatever the
+                           // workspace holds there, in columns of the products that are never stored); 2 if every layer of
+                           // the set has one token: the 8-bit digit form (stage_groups_i8)
     uint16_t prefix[SLIM_MAX_GROUPS + 1];
     uint16_t pre3[SLIM_MAX_GROUPS + 1];   // 3-bit groups (two slices) before group j
     uint8_t bits[SLIM_MAX_GROUPS];
@@ -108,7 +109,7 @@ struct SetParams {
     int one;                               // 1: a multiplier the compiler cannot fold, for selects done as integer multiply-adds
 };
 
-// ------------------------------------------------------e offset kSetOffCounters) start every launch at zero.
+// Arrival counters of the cut row blocks (workspace offset kSetOffCounters) start every launch at zero.
 constexpr uint32_t kSetOffCounters = 256;
 __device__ __forceinline__ void stage_clear_counters(uint8_t* ws, int n_counters) {
     unsigned int* cnt = reinterpret_cast<unsigned int*>(ws + kSetOffCounters);

@@ -10,7 +10,7 @@
 //   errors              sba_kl_kernel, sba_mean_kernel
 // The host waits once, for the ranking and the errors, and takes the minimum of G/2 + 1 numbers.  Evaluating every
 // candidate as a layer of its own (quantise the two groups that change, pack, slim_mpq_gemm, softmax and KL, five launches
-// per candidate) took 2389 us for 11008 x 4096 with 128 tokens at avg 2 bits; this takes 220 us.
+// per candidate) took 2389 us for 11008 x 4096 with 128 tokens at avg 2 bits; this takes 248 us.
 //
 // slim_dense_linear and slim_softmax_kl are the same two steps on their own.
 #include "slim_quant_dev.cuh"
