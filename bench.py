@@ -60,7 +60,7 @@ NCU_TRAFFIC = {
 # DRAM bytes (read + written) of the 14 gemm_kernel launches of one step of llama13b-prefill-avg3-m2048, from one ncu
 # capture of dram__bytes_read.sum and dram__bytes_write.sum; keyed by the SHA-256 of slim_gemm.cu at capture time
 NCU_TRAFFIC_GEMM = {
-    "a9b998b7a42c63bfc7bf8985dc1e3ee6b8be9ec1e3e35774be2538fadf174e9b": {"workload": "llama13b-prefill-avg3-m2048", "launches": 14, "traffic_bytes": 1049365760 + 218744064},
+    "567d7f396a654d6275e04c0c2c7319232189cdccff0160d2be4348d097ede78a": {"workload": "llama13b-prefill-avg3-m2048", "launches": 14, "traffic_bytes": 1083127040 + 228127232},
 }
 
 
