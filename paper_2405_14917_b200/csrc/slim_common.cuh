@@ -55,6 +55,12 @@ int gemv_one(const void* x, const void* packed, const GroupTable& gt, const void
 int gemv_few(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y,
              int M, int N, int K, void* workspace, cudaStream_t stream);
 
+// ... and layers of 2 to 16 tokens, from a workspace of that many bytes on (0: none is enough), to the layer-set kernel on tcgen05
+// without a plan (slim_gemv_set.cu): as above.
+size_t gemv_tc_workspace_bytes(int M, int N, const GroupTable& gt);
+int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y, int M, int N, int K,
+            void* workspace, size_t workspace_bytes, cudaStream_t stream);
+
 // A set of single-token layers as one resident launch of that kernel (small sets: q/k/v, gate/up).  one_set_plan decides
 // (SLIM_OK: taken, descriptors written into the plan buffer; 1: not taken; negative: error), one_set_launch runs it.
 struct OneSetPlan {

@@ -516,6 +516,8 @@ int slim_workspace_bytes(int M, int N, int K, int g, const uint8_t* bits_host, s
     if (M >= 1 && M <= SLIM_GEMV_MAX_M && N > 0 && K > 0) {       // large layers go through the layer-set kernels
         const size_t routed = slim::gemv_route_workspace_bytes(M, N, K, g, bits_host, gt);
         if (routed > *out_bytes) *out_bytes = routed;
+        const size_t tc = slim::gemv_tc_workspace_bytes(M, N, gt);
+        if (tc > *out_bytes) *out_bytes = tc;
     }
     return SLIM_OK;
 }
@@ -585,6 +587,10 @@ int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host, c
     // A single token: the integer form with the whole K of a few tiles per CTA, if the layer fits it.
     {
         const int taken = slim::gemv_one(x, packed, gt, scales, zeros, y, M, N, K, workspace, s);
+        if (taken <= 0) return taken;
+    }
+    {
+        const int taken = slim::gemv_tc(x, packed, gt, scales, zeros, y, M, N, K, workspace, workspace_bytes, s);
         if (taken <= 0) return taken;
     }
     // More tokens, or one whose layer does not fit that kernel: the layer cut over the whole GPU in one launch.  What that leaves

@@ -20,9 +20,14 @@
 //    acc += s * (D * 2^(24-S) - z * sum_k x); after the last group it stores its 16 rows.  A warp
 //    walks the whole K itself: no partial sums, no reduction between warps or CTAs.
 //
+// That is the kernel of single-token sets (on the integer form of slim_gemv_i8.cuh) and of sets with 17 to 64 tokens somewhere.
+// Sets of 2 to 16 tokens, and one large layer of as many, go through gemv_set_tc_kernel: the same ring, blocks of 512 rows, products
+// on tcgen05 (slim_set_tc.cuh), shares of equal cost in place of dealt items.
+//
 // Every wait on an mbarrier is bounded and reports through the workspace status word.
 #include "slim_gemv_dev.cuh"
 #include "slim_gemv_i8.cuh"
+#include "slim_set_tc.cuh"
 
 #include <atomic>
 
@@ -69,7 +74,8 @@ struct SetLayer {
     int MP;                // 256-byte pieces per slice in the staged layout: a multiple of 8 up to 64 = tokens of the f16 fragments
                            // for the whole set (what a layer does not have is not staged: the kernel multiplies whatever the
                            // workspace holds there, in columns of the products that are never stored); 2 if every layer of
-                           // the set has one token: the 8-bit digit form (stage_groups_i8)
+                           // the set has one token: the 8-bit digit form (stage_groups_i8); -mv: the
+                           // form mv of slim_set_tc.cuh
     uint16_t prefix[SLIM_MAX_GROUPS + 1];
     uint16_t pre3[SLIM_MAX_GROUPS + 1];   // 3-bit groups (two slices) before group j
     uint8_t bits[SLIM_MAX_GROUPS];
@@ -90,7 +96,7 @@ struct SetItem {
                            // partial output [M][N] instead
     int M;
     int counts;            // the layer's groups of 1, 2 and 3 bits, 9 bits each (the rest has 4), i.e. where each width
-                           // starts in the streaming order; bit 30: partial item
+                           // starts in the streaming order; bit 30: partial item.  gemv_set_tc_kernel: the item's cut, or -1
 };
 constexpr int kItemPartial = 1 << 30;
 static_assert(sizeof(SetItem) == 32, "items are read as two 16-byte pieces");
@@ -107,6 +113,7 @@ struct SetParams {
     uint8_t* ws;                           // workspace: status word, arrival counters, then the layers' fragments and sums
     int n_layers, n_slots, slot_bytes;
     int one;                               // 1: a multiplier the compiler cannot fold, for selects done as integer multiply-adds
+    int n_items;                           // gemv_set_tc_kernel: the items, after which the cuts come
 };
 
 // Arrival counters of the cut row blocks (workspace offset kSetOffCounters) start every launch at zero.
@@ -128,6 +135,10 @@ __device__ __forceinline__ void stage_task_one(const SetLayer& L, uint8_t* ws, i
 __device__ __forceinline__ void stage_task(const SetLayer& L, uint8_t* ws, int pi, int lane) {
     const int q = pi / L.G, j = pi - q * L.G;
     if (4 * q >= L.M) return;
+    if (L.MP < 0) {                                             // the form of gemv_set_tc_kernel
+        rawtc::stage_tokens(L.x + j * SLIM_GROUP, L.K, L.bits[j], 4 * q, L.M, -L.MP, ws + L.x_off + static_cast<size_t>(j) * rawtc::record_bytes(-L.MP), lane);
+        return;
+    }
     uint8_t* grp = ws + L.x_off + staged_group_offset(j, L.pre3[j], L.MP);
     stage_tokens(L.x + j * SLIM_GROUP, L.K, L.bits[j], 4 * q, L.M, L.MP, grp + staged_header_bytes(L.MP), reinterpret_cast<float2*>(grp), lane);
 }
@@ -652,6 +663,497 @@ __global__ void __launch_bounds__(kSetThreads, NT >= 3 ? 1 : kSetCtasPerSm) gemv
     if (tid == 0 && *abort != 0) atomicOr(reinterpret_cast<unsigned int*>(p.ws), 1u);
 }
 
+// ------------------------------------------------------------------------------------------ the persistent kernel, 2 to 16 tokens
+// Measured against the kernel above, whose mma.sync was its bound (us, all bytes from HBM): two 70B blocks at 2 bits, 16 tokens 241 ->
+// 146 (3.4 TB/s); two 13B blocks at 3 bits, 16 tokens 181 -> 76; eight 7B blocks, 2 and 5 tokens at 2 bits 144 / 145 -> 101 / 112, 8
+// tokens at 3 bits 166 -> 137; one 7B block, 4 tokens 36.9 -> 25.  Bound now: issue slots, 2850 / 3350 / 3800 warp instructions a
+// step at 2 / 8 / 16 tokens (ncu), of which decoding takes 950 and the fold up to 1100, next to 780 cycles of HBM time.
+// What a step of gemv_set_tc_kernel costs in cycles, for the deal: between its bytes (4 + 10 b per row tile) and its instructions.
+__host__ __device__ constexpr unsigned tc_step_cost(int b, int tiles) { return 400u + static_cast<unsigned>(tiles * (4 + 10 * b)); }
+
+// A row block of which several CTAs have a part of the groups.
+struct SetCut {
+    unsigned long long off;       // workspace offset of the parts' fp32 sums, each [M][512 rows]
+    int parts, pad;
+};
+
+// One layer without a plan: the steps of its row blocks, one block after the other, are cut into `grid` shares of equal cost.
+struct TcSingle {
+    SetLayer layer;
+    uint8_t* ws;
+    unsigned long long part_off;  // workspace offset of the parts' fp32 sums: two rooms of [M][512] per CTA
+    int n_slots, slot_bytes, off_rec, n_rb, grid;
+    unsigned per_rb;              // cost of a row block
+};
+struct TcPlace { int rb, p; };    // row block, position in the streaming order
+// Where share c begins.  No part of a single step: such a cut moves to the end of the row block.
+__host__ __device__ inline TcPlace tc_place(const TcSingle& t, int c) {
+    if (c >= t.grid) return TcPlace{t.n_rb, 0};
+    const unsigned long long x = static_cast<unsigned long long>(t.per_rb) * static_cast<unsigned>(t.n_rb) * static_cast<unsigned>(c) / static_cast<unsigned>(t.grid);
+    int rb = static_cast<int>(x / t.per_rb), at = 0;
+    unsigned rem = static_cast<unsigned>(x % t.per_rb);
+    for (int b = 1; b <= 4; ++b) {
+        const unsigned cost = tc_step_cost(b, rawtc::kTiles), has = t.layer.count[b - 1];
+        const unsigned n = rem / cost < has ? rem / cost : has;
+        at += static_cast<int>(n);
+        rem -= n * cost;
+        if (n < has) break;
+    }
+    if (at < 2) at = 0;
+    else if (at > t.layer.G - 2) { at = 0; ++rb; }
+    return TcPlace{rb, at};
+}
+
+// A fold warp has stored its sums of a cut row block (64 of the 512 rows) and counts itself, in its four bits of the block's word; the
+// one that counts last adds the S parts in their order, so the result does not depend on which came last, and leaves the bits
+// at zero.  `place`: the first float of part k.
+constexpr int kTcMaxParts = 15;
+template <int MV, class Place>
+__device__ __forceinline__ void finish_cut(unsigned int* counter, int S, Place place, __half* y, int fw, int lane, int row_block, int M, int N) {
+    __threadfence();                                    // this lane's sums before the count
+    __syncwarp();
+    unsigned int old = 0;
+    if (lane == 0) old = atomicAdd(counter, 1u << (4 * fw));
+    old = __shfl_sync(0xffffffffu, old, 0);
+    if (static_cast<int>((old >> (4 * fw)) & 15u) + 1 != S) return;
+    if (lane == 0) atomicSub(counter, static_cast<unsigned int>(S) << (4 * fw));
+    __threadfence();
+    const int h = fw >> 2, q = fw & 3;
+    // pairs of rows: 16 in each of the warp's two tiles; lane = pair of one tile or the other
+    const int row = 128 * (2 * h + (lane >> 4)) + 32 * q + 2 * (lane & 15);
+    if (rawtc::kRows * row_block + row >= N) return;
+    // all tokens of two parts at a time (of four, up to eight tokens): the loads are in flight together
+    float2 sum[MV];
+#pragma unroll
+    for (int t = 0; t < MV; ++t) sum[t] = make_float2(0.f, 0.f);
+    constexpr int U = MV <= 8 ? 4 : 2;
+    for (int k0 = 0; k0 < S; k0 += U) {
+        float2 v[U][MV];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float* from = place(min(k0 + u, S - 1)) + row;
+#pragma unroll
+            for (int t = 0; t < MV; ++t) v[u][t] = __ldcg(reinterpret_cast<const float2*>(from + (t < M ? t : 0) * rawtc::kRows));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int t = 0; t < MV; ++t) {
+                sum[t].x += k0 + u < S ? v[u][t].x : 0.f;
+                sum[t].y += k0 + u < S ? v[u][t].y : 0.f;
+            }
+    }
+#pragma unroll
+    for (int t = 0; t < MV; ++t)
+        if (t < M) *reinterpret_cast<__half2*>(y + static_cast<size_t>(t) * N + rawtc::kRows * row_block + row) = __floats2half2_rn(sum[t].x, sum[t].y);
+}
+
+// MV: form of the set.  kSet: items from a plan, records from the workspace.  kLocal, kStaged: one layer; its CTAs stage the groups
+// that they multiply themselves, or a kernel ahead has staged all of x.
+enum TcMode { kSet, kLocal, kStaged };
+__device__ __forceinline__ uint32_t p_off_rec(const TcSingle& t) { return static_cast<uint32_t>(t.off_rec); }
+__device__ __forceinline__ uint32_t p_off_rec(const SetParams&) { return 0u; }
+template <int MV, int MODE, class Params>
+__global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const __grid_constant__ Params p) {
+    using namespace rawtc;
+    constexpr uint32_t kOffW = MODE == kLocal ? (kOffE + 127) / 128 * 128 : off_w(MV);
+    extern __shared__ __align__(128) uint8_t smem[];
+    const uint32_t sbase = smem_u32(smem);
+    const int tid = threadIdx.x, lane = tid & 31, warp = static_cast<int>(tc::uniform(tid >> 5));
+    auto full = [&](int s) { return sbase + 8u * s; };
+    auto empty = [&](int s) { return sbase + 8u * (kMaxSlots + s); };
+    const uint32_t bar1 = sbase + 16u * kMaxSlots + 16u;
+    auto a_full = [&](int h, uint32_t k) { return bar1 + 8u * (2 * h + k); };           // k: step parity
+    auto a_empty = [&](int h, uint32_t k) { return bar1 + 32u + 8u * (2 * h + k); };
+    auto d_full = [&](int h, uint32_t k) { return bar1 + 64u + 8u * (2 * h + k); };
+    auto d_empty = [&](int h, uint32_t k) { return bar1 + 96u + 8u * (2 * h + k); };
+    auto drained = [&](int mw) { return bar1 + 128u + 8u * mw; };
+    static_assert(16 * kMaxSlots + 16 + 160 <= static_cast<int>(kSetOffDesc), "barriers end before the ring");
+    volatile int* abort = reinterpret_cast<volatile int*>(smem + 16 * kMaxSlots);
+    const uint32_t tmem_slot = sbase + 16u * kMaxSlots + 4u;
+    const uint32_t ring = sbase + kSetOffDesc;
+
+    if (tid == 0) {
+        for (int s = 0; s < p.n_slots; ++s) { sb::init(full(s), 1); sb::init(empty(s), kFold); }
+        for (int h = 0; h < 2; ++h) {
+            for (uint32_t k = 0; k < 2; ++k) {
+                sb::init(a_full(h, k), 4);
+                sb::init(a_empty(h, k), 1);
+                sb::init(d_full(h, k), 1);
+                sb::init(d_empty(h, k), 4);
+            }
+            sb::init(drained(2 * h), 1);
+            sb::init(drained(2 * h + 1), 1);
+        }
+        *abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == kFirstMma) {
+        tc::alloc(tmem_slot, 512);
+        tc::relinquish();
+    }
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = tc::uniform(*reinterpret_cast<volatile uint32_t*>(smem + 16 * kMaxSlots + 4));
+    pdl_launch_dependents();
+
+    // the CTA's items: (layer, row block, N, first and last position), as in SetItem
+    int i0 = 0, i1 = 0;
+    [[maybe_unused]] TcPlace from = {0, 0}, to = {0, 0};
+    if constexpr (MODE == kSet) {
+        i0 = p.item_begin[blockIdx.x];
+        i1 = p.item_begin[blockIdx.x + 1];
+    } else {
+        from = tc_place(p, static_cast<int>(blockIdx.x));
+        to = tc_place(p, static_cast<int>(blockIdx.x) + 1);
+        i1 = to.rb + (to.p > 0 ? 1 : 0) - from.rb;
+    }
+    auto item = [&](int i) -> int4 {
+        if (i >= i1) return make_int4(0, 0, 0, 0);
+        if constexpr (MODE == kSet) return reinterpret_cast<const int4*>(p.items)[2 * i];
+        else return make_int4(0, from.rb + i, p.layer.N, (i == 0 ? from.p : 0) | ((from.rb + i == to.rb ? to.p : p.layer.G) << 16));
+    };
+    auto layer_of = [&](int l) -> const SetLayer* {
+        if constexpr (MODE == kSet) return p.layers + l;
+        else return &p.layer;
+    };
+    const int n_slots = p.n_slots;
+    const uint32_t slot_bytes = static_cast<uint32_t>(p.slot_bytes);
+    bool ok = true;
+    int s = 0;                               // slot of the step, and the parity of its round
+    uint32_t ph = 0;
+    uint32_t sp = 0, php = 0;                // parity of the step, and of its round of two steps
+    // what a warp needs of an item: its steps, and the 16-row tiles of its block that exist
+    int4 it = item(i0);
+    auto steps_of = [](const int4& v) { return (v.w >> 16) - (v.w & 0xffff); };
+    auto tiles_of = [](const int4& v) { return min(kTiles, (v.z >> 4) - kTiles * v.y); };
+
+    if constexpr (MODE == kLocal) {
+        // the records of the CTA's steps, in their order, by the decoding and the folding warps; the MMAs wait for them
+        if (warp < kFirstMma) {
+            const SetLayer& L = p.layer;
+            const int quads = (L.M + 3) >> 2;
+            int first = 0;                                           // steps of the items so far
+            pdl_wait();                                              // x may be the output of the kernel ahead
+            for (int i = 0; i < i1; ++i) {
+                const int4 v = item(i);
+                const int p0 = v.w & 0xffff, n = (v.w >> 16) - p0;
+                for (int t = warp; t < n * quads; t += kFirstMma) {
+                    const int k = t / quads, m0 = 4 * (t - k * quads), j = L.order[p0 + k];
+                    stage_tokens(L.x + j * SLIM_GROUP, L.K, L.bits[j], m0, L.M, MV, smem + p.off_rec + static_cast<size_t>(first + k) * record_bytes(MV), lane);
+                }
+                first += n;
+            }
+            tc::fence_proxy_async();
+        }
+        if (warp < kFirstProd) asm volatile("bar.sync 1, %0;" ::"n"(32 * kFirstProd) : "memory");
+    }
+
+    if (warp >= kFirstMma) set_registers<kRegMisc>();
+    if (warp >= kFirstProd) {
+        // ------------------------------------------------------------------ producers: slices, scales, zeros, activations
+        // A warp each: three copies per step from one warp took longer than the step lasts.
+        const int what = warp - kFirstProd;
+        const bool is_w = what == 0, is_x = what == 3;
+        if (is_x) pdl_wait();
+        for (int i = i0; i < i1 && ok && !(is_x && MODE == kLocal); ++i) {
+            const int rb = it.y, p0 = it.w & 0xffff, p1 = it.w >> 16, tiles = tiles_of(it);
+            const SetLayer* D = layer_of(it.x);
+            it = item(i + 1);
+            const int N = D->N;
+            const uint8_t* base = is_x ? p.ws + D->x_off
+                                : is_w ? D->packed
+                                : what == 1 ? reinterpret_cast<const uint8_t*>(D->scales + kRows * rb)
+                                            : reinterpret_cast<const uint8_t*>(D->zeros + kRows * rb);
+            constexpr uint32_t xbytes = MODE == kLocal ? 0u : static_cast<uint32_t>(record_bytes(MV));
+            const uint32_t szb = static_cast<uint32_t>(tiles) * 32u;
+            const uint32_t dst0 = is_x ? kOffE : is_w ? kOffW : what == 1 ? kOffS : kOffZ;
+            // lane k knows the k-th of 32 groups: its width, where its bytes are
+            for (int jb = p0; jb < p1 && ok; jb += 32) {
+                const int j = D->order[min(jb + lane, p1 - 1)];
+                const uint32_t b = D->bits[j];
+                const unsigned long long src = reinterpret_cast<unsigned long long>(
+                    base + (is_x ? static_cast<size_t>(j) * xbytes
+                            : is_w ? 16ull * N * D->prefix[j] + static_cast<size_t>(kTiles * rb) * 256 * b
+                                   : 2ull * static_cast<size_t>(j >> D->gshift) * N));
+                const int n = min(32, p1 - jb);
+                for (int k = 0; k < n; ++k) {
+                    const uint32_t bk = __shfl_sync(0xffffffffu, b, k);
+                    const unsigned long long src_k = __shfl_sync(0xffffffffu, src, k);
+                    const uint32_t wbytes = static_cast<uint32_t>(tiles) * 256u * bk;
+                    if (!warp_wait(empty(s), ph ^ 1u, abort)) { ok = false; break; }
+                    const uint32_t slot = ring + static_cast<uint32_t>(s) * slot_bytes;
+                    if (lane == 0) {
+                        if (is_w) {
+                            asm volatile("st.shared.u32 [%0], %1;" ::"r"(slot), "r"(bk) : "memory");
+                            sb::expect_tx(full(s), wbytes + 2 * szb + xbytes);
+                        }
+                        sb::bulk_g2s(slot + dst0, reinterpret_cast<const void*>(src_k), is_x ? xbytes : is_w ? wbytes : szb, full(s));
+                    }
+                    __syncwarp();
+                    if (++s == n_slots) { s = 0; ph ^= 1u; }
+                }
+            }
+        }
+        if (!ok && lane == 0) {
+            // leave no copy in flight: give what was issued a millisecond to land
+            const unsigned long long t0 = sb::timer_ns();
+            while (sb::timer_ns() - t0 < 1000000ull) { }
+        }
+    } else if (warp < kDecode) {
+        // ------------------------------------------------------------------ decode: 32 rows of two tiles, every other step
+        // The steps of an item come sorted by bit-width, so each width has a loop of its own.
+        set_registers<kRegDecode>();
+        const int q = warp & 3, h = (warp >> 2) & 1;
+        const uint32_t set = static_cast<uint32_t>(warp >> 3);
+        const uint32_t a_t = tmem + (static_cast<uint32_t>(32 * q) << 16) + kColA + 128 * h + 64 * set;
+        const int tile0 = 16 * h + 2 * q;                            // my first 16-row tile; those of the other tile are eight on
+        const uint32_t w_t = ring + kOffW + 8u * lane;
+        if (set != 0u) { if (++s == n_slots) { s = 0; ph ^= 1u; } }
+        uint32_t ready = test(full(s), ph);
+        for (int i = i0; i < i1 && ok; ++i) {
+            const int p0 = it.w & 0xffff, p1 = it.w >> 16;
+            const uint2 counts = *reinterpret_cast<const uint2*>(layer_of(it.x)->count);
+            const bool two = tiles_of(it) > tile0 + 8;               // tiles past the end: nothing, or stale bytes that nobody looks at
+            it = item(i + 1);
+            auto run = [&](auto btag, int n) {
+                constexpr int B = decltype(btag)::value;
+                if (n <= 0) return;
+                for (int k = static_cast<int>(set ^ sp); k < n && ok; k += 2) {
+                    ok = warp_wait_after(ready, full(s), ph, abort);
+                    if (!ok) return;
+                    const uint32_t w = w_t + static_cast<uint32_t>(s) * slot_bytes + 256u * B * tile0;
+                    const uint32_t free = test(a_empty(h, set), php ^ 1u);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        if (e == 1 && !two) break;
+                        uint2 x[2][B];
+                        load_words<B>(w + 256u * B * (8 * e), x[0]);
+                        load_words<B>(w + 256u * B * (8 * e + 1), x[1]);
+                        if (e == 0) {
+                            s += 2;
+                            if (s >= n_slots) { s -= n_slots; ph ^= 1u; }
+                            ready = test(full(s), ph);
+                        }
+#pragma unroll
+                        for (int i2 = 0; i2 < 2; ++i2) {
+                            uint32_t r[16];
+                            decode_tile<B>(x[i2], r);
+                            if (e == 0 && i2 == 0) {                 // the MMAs of two steps ago have read the columns
+                                ok = warp_wait_after(free, a_empty(h, set), php ^ 1u, abort);
+                                if (!ok) return;
+                                tc::fence_after();
+                            }
+                            st_16x128b_x8(a_t + 32 * e + ((16u * i2) << 16), r);
+                        }
+                    }
+                    tc::wait_st();
+                    tc::fence_before();
+                    __syncwarp();
+                    if (lane == 0) sb::arrive(a_full(h, set));
+                    php ^= 1u;
+                }
+                sp ^= static_cast<uint32_t>(n) & 1u;
+            };
+            // the widths start at positions 0, e1, e2, e3 of the layer's streaming order; the item covers [p0, p1)
+            const int e1 = counts.x & 0xffff, e2 = e1 + (counts.x >> 16), e3 = e2 + (counts.y & 0xffff);
+            auto part = [&](int from, int to) { return min(p1, to) - max(p0, from); };
+            run(WidthTag<1>{}, part(0, e1));
+            run(WidthTag<2>{}, part(e1, e2));
+            run(WidthTag<3>{}, part(e2, e3));
+            run(WidthTag<4>{}, part(e3, 65535));
+        }
+    } else if (warp < kFirstMma) {
+        // ------------------------------------------------------------------ fold: a row of each of two tiles
+        set_registers<kRegFold>();
+        pdl_wait();                                                  // x, y and the workspace belong to the kernels ahead until here
+        const int fw = warp - kFirstFold, q = fw & 3, h = fw >> 2;
+        const int i16 = lane & 15, r16 = i16 < 8 ? 2 * i16 : 2 * i16 - 15;
+        const uint32_t row2 = 2u * static_cast<uint32_t>(256 * h + 32 * q + (lane & 16) + r16);      // of the block's 512, as bytes
+        const uint32_t d_t = tmem + (static_cast<uint32_t>(32 * q) << 16) + 128 * h;
+        constexpr int P2 = MV / 2, P = MV;
+        uint32_t ready = test(full(0), 0u);
+        // of an item: y, or the workspace offset of its part's sums; M; its cut, or -1
+        auto item_b = [&](int i) -> int4 {
+            if (i >= i1) return make_int4(0, 0, 0, 0);
+            if constexpr (MODE == kSet) return reinterpret_cast<const int4*>(p.items)[2 * i + 1];
+            else {
+                const int rb = from.rb + i;
+                const bool cut = (i == 0 && from.p > 0) || (rb == to.rb && to.p < p.layer.G);
+                const unsigned long long at = cut ? p.part_off + static_cast<unsigned long long>(2 * blockIdx.x + (i == 0 ? 0 : 1)) * (p.layer.M * kRows * 4)
+                                                  : reinterpret_cast<unsigned long long>(p.layer.y);
+                return make_int4(static_cast<int>(at), static_cast<int>(at >> 32), p.layer.M, cut ? rb : -1);
+            }
+        };
+        int4 it_b = item_b(i0);
+        uint32_t rec_l = sbase + (MODE == kLocal ? p_off_rec(p) : 0u);          // kLocal: the step's record
+        for (int i = i0; i < i1 && ok; ++i) {
+            const int layer = it.x, rb = it.y, N = it.z, n = steps_of(it), cut = it_b.w;
+            const uint32_t M = tc::uniform(it_b.z);
+            const unsigned long long yword = (static_cast<unsigned long long>(static_cast<uint32_t>(it_b.y)) << 32) | static_cast<uint32_t>(it_b.x);
+            it = item(i + 1);
+            it_b = item_b(i + 1);
+            f2 acc[2][P2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int k = 0; k < P2; ++k) acc[e][k] = 0ull;
+            for (int k = 0; k < n; ++k) {
+                if (!warp_wait_after(ready, full(s), ph, abort)) { ok = false; break; }
+                const uint32_t slot = ring + static_cast<uint32_t>(s) * slot_bytes;
+                f2 s2[2], z2[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {                        // of rows past the end: stale bytes, not used
+                    uint16_t sh, zh;
+                    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(sh) : "r"(slot + kOffS + 256 * e + row2));
+                    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(zh) : "r"(slot + kOffZ + 256 * e + row2));
+                    const float sf = __half2float(__ushort_as_half(sh)), zf = -__half2float(__ushort_as_half(zh));
+                    s2[e] = pack(sf, sf);
+                    z2[e] = pack(zf, zf);
+                }
+                if (!warp_wait(d_full(h, sp), php, abort)) { ok = false; break; }
+                tc::fence_after();
+                // all columns of a tile; both tiles at once where the registers allow it
+                constexpr int C = MV <= 2 ? 8 : MV <= 4 ? 16 : 32;
+                constexpr bool kBoth = MV <= 8;
+                uint32_t v[2][C];
+                ld_cols<C>(d_t + 64 * sp, v[0]);
+                if (kBoth) ld_cols<C>(d_t + 64 * sp + 32, v[1]);
+                // acc += s (D 2^(9-S) - z sum_x): two tokens at a time, the pieces smallest first
+                auto add = [&](int e) {
+#pragma unroll
+                    for (int k2 = 0; k2 < P2; ++k2) {
+                        f2 sx, sc;
+                        lds_sums((MODE == kLocal ? rec_l : slot + kOffE) + 16u * k2, sx, sc);
+                        const uint32_t* o = v[e] + 2 * k2;
+                        f2 dd = pack(f_of(o[P]), f_of(o[P + 1]));
+                        if (kBoth) dd = add2(pack(f_of(o[2 * P % C]), f_of(o[(2 * P + 1) % C])), dd);
+                        dd = mul2(add2(dd, pack(f_of(o[0]), f_of(o[1]))), sc);
+                        acc[e][k2] = fma2(s2[e], fma2(z2[e], sx, dd), acc[e][k2]);
+                    }
+                };
+                tc::wait_ld();
+                arrived(v[0]);
+                if (!kBoth) {
+                    ld_cols<C>(d_t + 64 * sp + 32, v[1]);
+                    add(0);
+                    tc::wait_ld();
+                }
+                arrived(v[1]);
+                tc::fence_before();
+                __syncwarp();
+                if (lane == 0) sb::arrive(d_empty(h, sp));
+                if (kBoth) add(0);
+                add(1);
+                __syncwarp();
+                if (lane == 0) sb::arrive(empty(s));
+                rec_l += record_bytes(MV);
+                if (++s == n_slots) { s = 0; ph ^= 1u; }
+                ready = test(full(s), ph);
+                php ^= sp;
+                sp ^= 1u;
+            }
+            if (!ok) break;
+            // lanes i and i + 8 of a 16-lane tile hold rows 2 i and 2 i + 1: they trade, so that the first stores both rows of the
+            // even token of a pair and the second those of the odd one
+            const bool odd = (lane & 8) != 0;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int row = 128 * (2 * h + e) + 32 * q + (lane & 16) + 2 * (lane & 7);      // of the block
+                const bool exists = kRows * rb + row < N;
+#pragma unroll
+                for (int k = 0; k < P2; ++k) {
+                    const float2 v = unpack(acc[e][k]);
+                    const float got = __shfl_xor_sync(0xffffffffu, odd ? v.x : v.y, 8);
+                    const float2 out = odd ? make_float2(got, v.y) : make_float2(v.x, got);
+                    const uint32_t m = 2 * k + (odd ? 1 : 0);
+                    if (m >= M || !exists) continue;
+                    if (cut >= 0) *reinterpret_cast<float2*>(p.ws + yword + 4 * (static_cast<size_t>(m) * kRows + row)) = out;
+                    else *reinterpret_cast<__half2*>(reinterpret_cast<__half*>(yword) + static_cast<size_t>(m) * N + kRows * rb + row) = __floats2half2_rn(out.x, out.y);
+                }
+            }
+            if (cut >= 0) {
+                if constexpr (MODE == kSet) {
+                    const SetCut* C = reinterpret_cast<const SetCut*>(p.items + p.n_items) + cut;
+                    const float* part = reinterpret_cast<const float*>(p.ws + C->off);
+                    finish_cut<MV>(reinterpret_cast<unsigned int*>(p.ws + kSetOffCounters) + cut, C->parts, [&](int k) { return part + static_cast<size_t>(k) * M * kRows; },
+                               p.layers[layer].y, fw, lane, rb, static_cast<int>(M), N);
+                } else {
+                    // The CTAs that have a part: those whose shares begin inside the row block, and the one before them.  Lane
+                    // 16 + d looks at the share d after this one (a row block has at most kTcMaxParts).
+                    const int c_lane = static_cast<int>(blockIdx.x) + lane - 16;
+                    const TcPlace pl = tc_place(p, max(c_lane, 0));
+                    const bool here = c_lane >= 0 && c_lane < p.grid && pl.rb == rb;
+                    const uint32_t inside = __ballot_sync(0xffffffffu, here && pl.p > 0), begins = __ballot_sync(0xffffffffu, here);
+                    const int below = __clz(~(inside << 15)), above = __ffs(static_cast<int>(~(inside >> 17))) - 1;
+                    finish_cut<MV>(reinterpret_cast<unsigned int*>(p.ws + kWsFlagsOffset) + cut, below + above + 1, [&](int k) {
+                        const int d = k - below;                     // that share's first row block, or its last
+                        return reinterpret_cast<const float*>(p.ws + p.part_off) +
+                               static_cast<size_t>(2 * (static_cast<int>(blockIdx.x) + d) + (1 ^ static_cast<int>((begins >> (16 + d)) & 1u))) * M * kRows;
+                    }, p.layer.y, fw, lane, rb, static_cast<int>(M), N);
+                }
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ MMAs of a pair of tiles
+        // A batch of MMAs with its waits takes an issuing warp 600 cycles and more from end to end, so two take turns.
+        const int mw = warp - kFirstMma, h = mw >> 1;
+        const uint32_t e = static_cast<uint32_t>(mw & 1);
+        const uint32_t a_t = tmem + kColA + 128 * h + 64 * e, d_t = tmem + 128 * h + 64 * e;
+        constexpr uint32_t rows = 3u * MV;
+        if (e != 0u) { if (++s == n_slots) { s = 0; ph ^= 1u; } }
+        uint32_t ready = test(full(s), ph), free = 1u;
+        [[maybe_unused]] uint32_t rec_l = sbase + e * record_bytes(MV);
+        if constexpr (MODE == kLocal) rec_l += p_off_rec(p);
+        for (int i = i0; i < i1 && ok; ++i) {
+            const int n = steps_of(it);
+            const bool two = tiles_of(it) > 16 * h + 8;
+            it = item(i + 1);
+            for (int k = static_cast<int>(e ^ sp); k < n; k += 2) {
+                ok = warp_wait_after(ready, full(s), ph, abort) && warp_wait_after(free, d_empty(h, e), php ^ 1u, abort) && warp_wait(a_full(h, e), php, abort);
+                if (!ok) break;
+                tc::fence_after();
+                const uint64_t b0 = desc_rows((MODE == kLocal ? rec_l : ring + static_cast<uint32_t>(s) * slot_bytes + kOffE) + sums_bytes(MV), rows);      // + 2 rows per K = 32
+                rec_l += 2 * record_bytes(MV);
+                if (tc::elect()) {
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        if (t == 1 && !two) break;
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks) mma_f8_ts(d_t + 32 * t, a_t + 32 * t + 8 * ks, b0 + 2u * ks * rows, idesc_f8(mma_n(MV)), ks > 0 ? 1u : 0u);
+                        if (MV > 8)
+#pragma unroll
+                            for (int ks = 0; ks < 4; ++ks) mma_f8_ts(d_t + 32 * t, a_t + 32 * t + 8 * ks, b0 + 2u * ks * rows + MV, idesc_f8(mma_n(MV)), 1u);
+                    }
+                    tc::commit(d_full(h, e));
+                    tc::commit(a_empty(h, e));
+                }
+                __syncwarp();
+                s += 2;
+                if (s >= n_slots) { s -= n_slots; ph ^= 1u; }
+                php ^= 1u;
+                ready = test(full(s), ph);
+                free = test(d_empty(h, e), php ^ 1u);
+            }
+            sp ^= static_cast<uint32_t>(n) & 1u;
+        }
+        // no commit of mine is on its way to a barrier when the CTA ends
+        if (tc::elect()) tc::commit(drained(mw));
+        __syncwarp();
+        const unsigned long long t0 = sb::timer_ns();
+        while (!sb::try_wait(drained(mw), 0) && sb::timer_ns() - t0 < kSetWaitNs) { }
+    }
+    tc::fence_before();
+    __syncthreads();
+    if (tid == 0 && *abort != 0) atomicOr(reinterpret_cast<unsigned int*>(p.ws), 1u);
+    if (warp == kFirstMma) {
+        tc::fence_after();
+        tc::dealloc(tmem, 512);
+    }
+}
+
 // ------------------------------------------------------------------------------------------ one-layer sets planned on the device
 // Plan and staging of a one-layer set in one kernel: the descriptor comes by value, every warp stages one (token, group)
 // of x, and block 0 also writes the plan: the items are (row block, part) pairs dealt to the CTAs in turn.  No host
@@ -662,7 +1164,7 @@ __global__ void __launch_bounds__(256) set_single_stage_kernel(const __grid_cons
     pdl_wait();                       // x may be the output of the kernel before; the workspace may still be read by it
     pdl_launch_dependents();
     stage_clear_counters(ws, n_counters);
-    if (blockIdx.x == 0) {
+    if (blockIdx.x == 0 && plan != nullptr) {                    // (null: the kernel after needs no plan)
         int* item_begin = reinterpret_cast<int*>(plan);
         SetLayer* dl = reinterpret_cast<SetLayer*>(plan + kSetPlanHeader);
         SetItem* items = reinterpret_cast<SetItem*>(dl + 1);
@@ -717,7 +1219,7 @@ struct SetGeometry {
     int slot_bytes;
     int n_slots, grid, ctas_per_sm;
     int split;                         // parts the groups of every row block are cut into (fewer for layers with few groups)
-    size_t smem_bytes;
+    int n_cuts;                        // 2 to 16 tokens: row blocks of several parts
     long long n_items, n_tasks;
     int n_counters;                    // arrival counters of the split row blocks: one per (row block, consumer warp)
     size_t cnt_bytes;                  // their room in the workspace, right after the 256-byte header
@@ -739,6 +1241,117 @@ static size_t layer_ws_bytes(int M, const GroupTable& gt) {
     for (int j = 0; j < gt.G; ++j) slots += gt.bits[j] == 3 ? 1 : 0;
     return align_to(static_cast<size_t>(gt.G) * (M == 2 ? 128 : staged_header_bytes(M)) + static_cast<size_t>(slots) * 256 * M, 128);
 }
+// Sets of 2 to 16 tokens go through gemv_set_tc_kernel.
+static bool tc_form(int mmax) { return mmax >= 2 && mmax <= rawtc::kMaxTokens; }
+// Staged activations of a layer, and the staging tasks (token, group) it has.
+static size_t layer_x_bytes(const SetGeometry& sg, int M, const GroupTable& gt) {
+    if (!tc_form(sg.mmax)) return layer_ws_bytes(sg.mres, gt);
+    // no less than a workspace has always had for so many tokens
+    return std::max(align_to(static_cast<size_t>(gt.G) * rawtc::record_bytes(rawtc::form(sg.mmax)), 128), layer_ws_bytes(sg.mres, gt));
+}
+static int layer_tasks(const SetGeometry& sg, int M, int G) {
+    return (tc_form(sg.mmax) ? (M + 3) / 4 * 4 : sg.mpad == 2 ? 1 : sg.mpad) * G;
+}
+// The items of a set of 2 to 16 tokens.  The steps of all row blocks, one after the other, are cut into shares of equal cost, one
+// per CTA: where a share ends inside a row block its sums are added up through the workspace (a deal of whole row blocks left the
+// last CTA of a 7B sweep 15 % over the average).  A row block has at most kTcMaxParts of them.  A set of few steps has its
+// row blocks cut into equal parts instead.
+struct TcDeal {
+    std::vector<SetItem> items;              // y of a cut item: offset in the room of the parts
+    std::vector<SetCut> cuts;                // off: the same
+    std::vector<int> begin;                  // per CTA
+    int grid, split;
+    size_t part_bytes;
+};
+constexpr int kTcMinSteps = 4;               // fewer per CTA: equal parts
+constexpr size_t kTcMaxSmem = 226 * 1024;
+static void tc_deal(const slim_layer* layers, int n_layers, int g, int sms, int uniform_split, TcDeal* out) {
+    struct Block { int layer, rb, G; };
+    std::vector<Block> blocks;
+    std::vector<GroupTable> gt(static_cast<size_t>(n_layers));
+    std::vector<std::vector<uint8_t> > width(static_cast<size_t>(n_layers));       // of the groups in streaming order
+    long long steps = 0;
+    unsigned long long total = 0, widest = 0;                                         // cost of all blocks, of the one that costs most
+    auto tiles_of = [&](const Block& B) { return std::min(rawtc::kTiles, (layers[B.layer].N >> 4) - rawtc::kTiles * B.rb); };
+    for (int l = 0; l < n_layers; ++l) {
+        make_group_table(layers[l].N, layers[l].K, g, layers[l].bits_host, &gt[l]);
+        for (int b = 1; b <= 4; ++b)
+            for (int j = 0; j < gt[l].G; ++j)
+                if (gt[l].bits[j] == b) width[l].push_back(static_cast<uint8_t>(b));
+        for (int rb = 0; rb * rawtc::kRows < layers[l].N; ++rb) {
+            blocks.push_back(Block{l, rb, gt[l].G});
+            steps += gt[l].G;
+            unsigned long long cost = 0;
+            for (int q = 0; q < gt[l].G; ++q) cost += tc_step_cost(width[l][q], tiles_of(blocks.back()));
+            total += cost;
+            widest = std::max(widest, cost);
+        }
+    }
+    out->split = 1;
+    out->part_bytes = 0;
+    out->items.clear();
+    out->cuts.clear();
+    out->begin.clear();
+    // positions [p0, p1) of a block, part `part` of `parts`
+    auto add = [&](const Block& B, int p0, int p1, int part, int parts) {
+        const slim_layer& L = layers[B.layer];
+        SetItem it;
+        memset(&it, 0, sizeof it);
+        it.layer = B.layer; it.rb = B.rb; it.N = L.N; it.M = L.M; it.range = p0 | (p1 << 16);
+        it.y = static_cast<__half*>(L.y);
+        it.counts = -1;
+        if (parts > 1) {
+            if (part == 0) out->cuts.push_back(SetCut{out->part_bytes, parts, 0});
+            it.counts = static_cast<int>(out->cuts.size()) - 1;
+            it.y = reinterpret_cast<__half*>(out->part_bytes);
+            out->part_bytes += static_cast<size_t>(L.M) * rawtc::kRows * sizeof(float);
+            out->split = std::max(out->split, parts);
+        }
+        out->items.push_back(it);
+    };
+    if (steps < static_cast<long long>(kTcMinSteps) * sms) {
+        out->split = 1;
+        for (const Block& B : blocks) {
+            const int parts = layer_split(uniform_split, B.G);
+            for (int k = 0; k < parts; ++k) add(B, B.G * k / parts, B.G * (k + 1) / parts, k, parts);
+        }
+        out->split = uniform_split;
+        const int n = static_cast<int>(out->items.size());
+        out->grid = std::min(n, sms);
+        for (int c = 0; c <= out->grid; ++c) out->begin.push_back(static_cast<int>(static_cast<long long>(n) * c / out->grid));
+        return;
+    }
+    // a block of n shares' cost is cut into n + 2 parts at most
+    out->grid = static_cast<int>(std::min<unsigned long long>(sms, (kTcMaxParts - 2) * total / widest));
+    out->begin.push_back(0);
+    unsigned long long done = 0;
+    int c = 0;                               // the CTA that takes the next step
+    auto share_end = [&](int cta) { return static_cast<unsigned long long>(static_cast<long double>(total) * (cta + 1) / out->grid); };
+    std::vector<int> ends;
+    std::vector<int> owner;
+    for (const Block& B : blocks) {
+        // the positions at which a CTA's share ends inside the block
+        ends.clear();
+        owner.clear();
+        const int tiles = tiles_of(B), edge = std::min(2, B.G / 2);          // no part of a single step
+        int p0 = 0;
+        for (int q = 0; q < B.G; ++q) {
+            done += tc_step_cost(width[B.layer][q], tiles);
+            while (c + 1 < out->grid && done >= share_end(c)) {
+                const int at = q + 1 < edge ? 0 : q + 1 > B.G - edge ? B.G : q + 1;
+                if (at > p0) { ends.push_back(at); owner.push_back(c); p0 = at; }
+                ++c;
+            }
+        }
+        if (p0 < B.G) { ends.push_back(B.G); owner.push_back(c); }
+        for (size_t k = 0; k < ends.size(); ++k) {
+            while (static_cast<int>(out->begin.size()) <= owner[k]) out->begin.push_back(static_cast<int>(out->items.size()));
+            add(B, k == 0 ? 0 : ends[k - 1], ends[k], static_cast<int>(k), static_cast<int>(ends.size()));
+        }
+    }
+    while (static_cast<int>(out->begin.size()) <= out->grid) out->begin.push_back(static_cast<int>(out->items.size()));
+}
+
 // Work of an item for the deal.  The kernel is bound by the instructions it issues, so a (tile, group)
 // weighs what a consumer warp issues for it: about 70 / 73 / 120 / 80 instructions at 1 / 2 / 3 / 4 bits
 // (counted in the kernel's loops: one AND per operand register, one MMA per four, the fragment loads and
@@ -758,12 +1371,14 @@ static int set_sm_count() {
 }
 
 // First pass over the set: validation of the shapes and everything that depends on all layers.
-static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeometry* sg) {
+// `deal`: the items of a set of 2 to 16 tokens, for a caller that writes the plan (may throw); null: the caller makes its own.
+static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeometry* sg, TcDeal* deal) {
     if (layers == nullptr || n_layers < 1 || sg == nullptr) return SLIM_ERR_INVALID_ARG;
     memset(sg, 0, sizeof *sg);
     sg->ws_bytes = 256;
     for (int l = 0; l < n_layers; ++l) sg->mmax = sg->mmax > layers[l].M ? sg->mmax : layers[l].M;
-    sg->tpw = 2;
+    const bool tc = tc_form(sg->mmax);
+    sg->tpw = tc ? rawtc::kTiles / kSetConsumers : 2;
     // one token: the 8-bit digit form, 512 bytes per slice; else the tokens of the widest layer rounded up to 8: the kernel is
     // bound by its MMAs, and with 8, 16, 32 or 64 alone 40 tokens paid for 64 (four LLaMA-7B blocks
     // at 3 bits, 17 / 40 / 56 tokens: 227 / 425 / 428 us -> 181 / 267 / 368; from 17 tokens on one CTA per SM, whose registers
@@ -781,14 +1396,15 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
         for (int j = 0; j < gt.G; ++j) sg->bmax = sg->bmax > gt.bits[j] ? sg->bmax : gt.bits[j];
         const int items = ((L.N >> 4) + tpi - 1) / tpi;
         sg->n_items += items;
-        sg->n_tasks += static_cast<long long>(sg->mpad == 2 ? 1 : sg->mpad) * gt.G;   // staging tasks: (token, group)
-        sg->ws_bytes += layer_ws_bytes(sg->mres, gt);
+        sg->n_tasks += layer_tasks(*sg, L.M, gt.G);
+        sg->ws_bytes += layer_x_bytes(*sg, L.M, gt);
     }
     if (sg->n_items > 0x3fffffff || sg->n_tasks > 0x3fffffff) return SLIM_ERR_UNSUPPORTED;
     sg->nt = sg->mmax <= 1 ? 1 : sg->mpad / 8;
     // A set with fewer row blocks than persistent CTAs cuts the groups of every row block into parts (items of their
     // own, fp32 partial outputs in the workspace, added in part order by the consumer warp whose part lands last).
-    const long long want = static_cast<long long>(set_sm_count()) * (sg->nt >= 3 ? 1 : kSetCtasPerSm);
+    const bool one_cta = sg->nt >= 3 || tc;                      // per SM
+    const long long want = static_cast<long long>(set_sm_count()) * (one_cta ? 1 : kSetCtasPerSm);
     sg->split = 1;
     if (sg->n_items < 2 * want) {
         // the number of parts that fills the last wave of CTAs best (the smallest one within 2 % of the best)
@@ -805,7 +1421,18 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
             if (f > best * 1.02) { best = f; sg->split = split; }
         }
     }
-    if (sg->split > 1) {
+    if (tc) {
+        if (deal != nullptr) {
+            tc_deal(layers, n_layers, g, set_sm_count(), sg->split, deal);
+            sg->n_items = static_cast<long long>(deal->items.size());
+            sg->split = deal->split;
+            sg->n_cuts = static_cast<int>(deal->cuts.size());
+            sg->n_counters = sg->n_cuts;
+            sg->cnt_bytes = align_to(static_cast<size_t>(sg->n_counters) * sizeof(unsigned int), 256);
+            sg->ws_bytes += sg->cnt_bytes + align_to(deal->part_bytes, 128);
+            if (sg->n_counters > 65535) return SLIM_ERR_UNSUPPORTED;
+        }
+    } else if (sg->split > 1) {
         sg->n_items = 0;
         long long counters = 0;
         for (int l = 0; l < n_layers; ++l) {
@@ -823,23 +1450,24 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
         sg->cnt_bytes = align_to(static_cast<size_t>(counters) * sizeof(unsigned int), 256);
         sg->ws_bytes += sg->cnt_bytes;
     }
-    sg->slot_bytes = static_cast<int>(align_to(static_cast<size_t>(slot_off_w(tpi, sg->mpad)) + static_cast<size_t>(tpi) * 256 * sg->bmax, 128));
+    sg->slot_bytes = tc ? rawtc::slot_size(rawtc::form(sg->mmax), sg->bmax)
+                        : static_cast<int>(align_to(static_cast<size_t>(slot_off_w(tpi, sg->mpad)) + static_cast<size_t>(tpi) * 256 * sg->bmax, 128));
     // as many CTAs per SM (kSetCtasPerSm at most) as still leaves each a ring of 4 slots
     const size_t per_sm = 224 * 1024;
     size_t budget = 0;
-    for (sg->ctas_per_sm = sg->nt >= 3 ? 1 : kSetCtasPerSm; sg->ctas_per_sm >= 1; --sg->ctas_per_sm) {
-        budget = per_sm / sg->ctas_per_sm - 1024 - kSetOffRing;   // 1 KB per CTA is reserved by the system
+    for (sg->ctas_per_sm = one_cta ? 1 : kSetCtasPerSm; sg->ctas_per_sm >= 1; --sg->ctas_per_sm) {
+        budget = tc ? kTcMaxSmem - kSetOffDesc : per_sm / sg->ctas_per_sm - 1024 - kSetOffRing;   // 1 KB per CTA is reserved by the system
         if (budget / sg->slot_bytes >= 4 || sg->ctas_per_sm == 1) break;
     }
     size_t slots = budget / sg->slot_bytes;
     if (slots > kSetMaxSlots) slots = kSetMaxSlots;
+    if (tc) slots = static_cast<size_t>(rawtc::even_slots(static_cast<int>(slots)));
     if (slots < 2) return SLIM_ERR_UNSUPPORTED;
     sg->n_slots = static_cast<int>(slots);
-    sg->smem_bytes = kSetOffRing + slots * sg->slot_bytes;
     long long grid = static_cast<long long>(set_sm_count()) * sg->ctas_per_sm;
     if (grid > kSetMaxGrid) grid = kSetMaxGrid;
     if (grid > sg->n_items) grid = sg->n_items;
-    sg->grid = static_cast<int>(grid);
+    sg->grid = tc && deal != nullptr ? deal->grid : static_cast<int>(grid);
     return SLIM_OK;
 }
 
@@ -872,8 +1500,8 @@ static void fill_descriptor(const slim_layer& L, const GroupTable& gt, int mpad,
             if (gt.bits[j] == b) { d.order[n_sorted++] = static_cast<uint8_t>(j); ++d.count[b - 1]; }
 }
 
-static size_t set_plan_bytes(int n_layers, long long n_items) {
-    return kSetPlanHeader + static_cast<size_t>(n_layers) * sizeof(SetLayer) + static_cast<size_t>(n_items) * sizeof(SetItem);
+static size_t set_plan_bytes(int n_layers, long long n_items, long long n_cuts = 0) {
+    return kSetPlanHeader + static_cast<size_t>(n_layers) * sizeof(SetLayer) + static_cast<size_t>(n_items) * sizeof(SetItem) + static_cast<size_t>(n_cuts) * sizeof(SetCut);
 }
 
 template <int NT, bool ONE, int TPW>
@@ -902,26 +1530,27 @@ constexpr size_t kRouteMinBytes = 32u << 20;
 
 struct RouteLayout {
     SetGeometry sg;
-    int n_rb, sp, cnt0;
+    int n_rb, sp, cnt0, n_items;
     size_t plan_off, plan_bytes, x_off, part_off, total;
 };
 
 // keep_flags: the first counters, which stay zero, lie over the flags of slim_mpq_gemm; without, everything is kWsFlagsBytes sooner.
 static bool route_layout(int M, int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt, bool keep_flags, RouteLayout* r) {
     static_assert(kSetOffCounters == kWsFlagsOffset, "the counters are cleared where the flags are");
-    if (M < 1 || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < kRouteMinBytes) return false;
+    if (M != 1 || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < kRouteMinBytes) return false;
     slim_layer L;
     memset(&L, 0, sizeof L);
     L.bits_host = bits_host; L.M = M; L.N = N; L.K = K;
-    if (set_geometry(&L, 1, g, &r->sg) != SLIM_OK) return false;
+    if (set_geometry(&L, 1, g, &r->sg, nullptr) != SLIM_OK) return false;
     const int tpi = kSetConsumers * r->sg.tpw;
     r->n_rb = ((N >> 4) + tpi - 1) / tpi;
     r->sp = layer_split(r->sg.split, gt.G);
+    r->n_items = r->n_rb * r->sp;
     r->cnt0 = keep_flags ? kWsFlagsBytes / static_cast<int>(sizeof(unsigned int)) : 0;
     r->plan_off = kSetOffCounters + r->cnt0 * sizeof(unsigned int) + r->sg.cnt_bytes;
     r->plan_bytes = set_plan_bytes(1, static_cast<long long>(r->n_rb) * r->sp);
     r->x_off = r->plan_off + align_to(r->plan_bytes, 256);
-    r->part_off = r->x_off + layer_ws_bytes(r->sg.mres, gt);
+    r->part_off = r->x_off + layer_x_bytes(r->sg, M, gt);
     r->total = r->part_off + (r->sp > 1 ? align_to(static_cast<size_t>(r->sp) * M * N * sizeof(float), 128) : 0);
     return true;
 }
@@ -941,13 +1570,14 @@ static int set_params(const slim_gemv_set_info* info, const void* plan, void* wo
     if (info->n_layers < 1 || info->grid < 1 || info->grid > kSetMaxGrid || info->n_slots < 2 ||
         info->n_slots > kSetMaxSlots || info->slot_bytes < 128 || info->slot_bytes % 128 != 0 ||
         info->token_tiles < 1 || info->token_tiles > 8 ||
-        info->max_tokens < 1 || info->max_tokens > 8 * info->token_tiles ||
-        info->tiles_per_warp != 2 ||
-        info->max_bits < 1 || info->max_bits > 4 || info->stage_tasks < 1 || info->split < 1 || info->split > kSetMaxSplit ||
+        info->max_tokens < 1 || info->max_tokens > 8 * info->token_tiles || (info->max_tokens > 16 && info->token_tiles < 3) ||
+        info->tiles_per_warp != (tc_form(info->max_tokens) ? rawtc::kTiles / kSetConsumers : 2) ||
+        info->max_bits < 1 || info->max_bits > 4 || info->stage_tasks < 1 || info->split < 1 || info->split > (tc_form(info->max_tokens) ? kTcMaxParts : kSetMaxSplit) ||
         info->n_counters < 0 || info->n_counters > 65535 || info->n_layers > 65535)
         return SLIM_ERR_INVALID_ARG;
-    const size_t smem = kSetOffRing + static_cast<size_t>(info->n_slots) * info->slot_bytes;
-    if (smem > 224 * 1024) return SLIM_ERR_INVALID_ARG;
+    const bool tc = tc_form(info->max_tokens);
+    const size_t smem = (tc ? kSetOffDesc : kSetOffRing) + static_cast<size_t>(info->n_slots) * info->slot_bytes;
+    if (smem > (tc ? kTcMaxSmem : 224 * 1024)) return SLIM_ERR_INVALID_ARG;
     if (!aligned16(plan)) return SLIM_ERR_ALIGNMENT;
     if (workspace == nullptr || workspace_bytes < info->workspace_bytes || workspace_bytes < 256 ||
         workspace_bytes < kSetOffCounters + static_cast<size_t>(info->n_counters) * sizeof(unsigned int))
@@ -964,18 +1594,97 @@ static int set_params(const slim_gemv_set_info* info, const void* plan, void* wo
     prm.slot_bytes = info->slot_bytes;
     prm.one = 1;
     const int tpi = kSetConsumers * info->tiles_per_warp;
+    if (tc) {
+        prm.n_items = info->n_items;
+        if (info->n_slots % 2 != 0 || info->slot_bytes != rawtc::slot_size(rawtc::form(info->max_tokens), info->max_bits)) return SLIM_ERR_INVALID_ARG;
+        *smem_out = smem;
+        return SLIM_OK;
+    }
     const int mp = info->max_tokens == 1 ? 2 : 8 * info->token_tiles;
     if (slot_off_w(tpi, mp) + tpi * 256 * info->max_bits > info->slot_bytes) return SLIM_ERR_INVALID_ARG;
     *smem_out = smem;
     return SLIM_OK;
 }
 
+template <int MV, int MODE, class Params>
+static cudaError_t launch_tc(const Params& prm, int grid, size_t smem, cudaStream_t stream, bool early) {
+    static std::atomic<bool> attr_set[64];    // zero-initialised; set-up is idempotent, so a race repeats it harmlessly
+    const auto kernel = gemv_set_tc_kernel<MV, MODE, Params>;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTcMaxSmem));
+        if (e != cudaSuccess) return e;
+        attr_set[dev] = true;
+    }
+    PdlLaunch l(static_cast<unsigned>(grid), rawtc::kThreads, smem, stream, early);
+    return cudaLaunchKernelEx(&l.cfg, kernel, prm);
+}
+template <int MODE, class Params>
+static cudaError_t launch_tc_form(int M, const Params& prm, int grid, size_t smem, cudaStream_t stream, bool early) {
+    using Launch = cudaError_t (*)(const Params&, int, size_t, cudaStream_t, bool);
+    static const Launch forms[8] = {launch_tc<2, MODE, Params>, launch_tc<4, MODE, Params>, launch_tc<6, MODE, Params>, launch_tc<8, MODE, Params>,
+                                    launch_tc<10, MODE, Params>, launch_tc<12, MODE, Params>, launch_tc<14, MODE, Params>, launch_tc<16, MODE, Params>};
+    return forms[(M - 1) / 2](prm, grid, smem, stream, early);
+}
+
+// ------------------------------------------------------------------------------------------ one layer of 2 to 16 tokens
+constexpr size_t kTcSingleParts = 2048;      // of the workspace: the status word, the flags, whose words count the parts, then the sums
+struct TcSinglePlan {
+    int grid, n_rb, n_slots, slot_bytes, off_rec, smem;
+    bool local;                              // records in shared memory
+    size_t part_off, x_off, total;
+};
+// From 24 MB on up to eight tokens, and from 32 MB on beyond; below, gemv_few, whose clusters exchange their sums through shared memory, is
+// sooner.  us, that kernel / this one: 28672 x 8192 at 2 bits (63 MB) 3 / 8 / 16 tokens 35.8 / 24.8, 37.1 / 29.6, 50.6 / 35.0; 13824 x 5120 at 3
+// bits (27 MB) 2 / 6 / 16 tokens 15.4 / 13.9, 16.2 / 15.8, 21.8 / 21.9; 8192 x 8192 at 2 bits (17 MB) 8 tokens 13.2 / 18.8.
+constexpr size_t kTcSingleMin = 24u << 20, kTcSingleMinMany = 32u << 20;
+static bool tc_single_plan(int M, int N, const GroupTable& gt, TcSinglePlan* pl) {
+    if (!tc_form(M) || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < (M <= 8 ? kTcSingleMin : kTcSingleMinMany)) return false;
+    const int mv = rawtc::form(M);
+    int bmax = 1, bmin = 4;
+    unsigned long long per_rb = 0;
+    for (int j = 0; j < gt.G; ++j) {
+        bmax = std::max<int>(bmax, gt.bits[j]);
+        bmin = std::min<int>(bmin, gt.bits[j]);
+        per_rb += tc_step_cost(gt.bits[j], rawtc::kTiles);
+    }
+    pl->n_rb = (N + rawtc::kRows - 1) / rawtc::kRows;
+    if (pl->n_rb * sizeof(unsigned int) > kWsFlagsBytes) return false;
+    const long long steps = static_cast<long long>(pl->n_rb) * gt.G;
+    const long long most = std::min<long long>((kTcMaxParts - 1) * static_cast<long long>(pl->n_rb), (steps + 1) / 2);
+    pl->grid = static_cast<int>(std::max(1ll, std::min<long long>(set_sm_count(), most)));
+    // (kTcMaxParts - 1 shares to a row block: kTcMaxParts parts)
+    // the most steps of a share: all of the cheapest, and what moves at its ends
+    const int share = static_cast<int>(per_rb * pl->n_rb / pl->grid / tc_step_cost(bmin, rawtc::kTiles)) + 5;
+    const size_t budget = kTcMaxSmem - kSetOffDesc, rec = static_cast<size_t>(rawtc::record_bytes(mv)) * share;
+    const int slot_l = rawtc::kTiles * 256 * bmax + (rawtc::kOffE + 127) / 128 * 128, slot_s = rawtc::slot_size(mv, bmax);
+    // records in shared memory if that leaves a ring of four slots, or of all steps
+    pl->local = rec < budget && (budget - rec) / slot_l >= static_cast<size_t>(std::min(4, share));
+    pl->slot_bytes = pl->local ? slot_l : slot_s;
+    int slots = static_cast<int>((pl->local ? budget - rec : budget) / pl->slot_bytes);
+    slots = rawtc::even_slots(std::min(slots, share + 1));
+    if (slots < 2) return false;
+    pl->n_slots = slots;
+    pl->off_rec = static_cast<int>(kSetOffDesc) + slots * pl->slot_bytes;
+    pl->smem = pl->off_rec + (pl->local ? static_cast<int>(rec) : 0);
+    pl->part_off = kTcSingleParts;
+    pl->x_off = align_to(pl->part_off + static_cast<size_t>(2 * pl->grid) * M * rawtc::kRows * sizeof(float), 256);
+    pl->total = pl->x_off + (pl->local ? 0 : static_cast<size_t>(gt.G) * rawtc::record_bytes(mv));
+    return true;
+}
+
 // The persistent kernel of the set in the form its token count asks for.
 static int launch_set_for(const slim_gemv_set_info* info, const SetParams& prm, size_t smem, cudaStream_t s, bool early) {
+    if (tc_form(info->max_tokens)) {
+        SLIM_CUDA_TRY((launch_tc_form<kSet, SetParams>(info->max_tokens, prm, info->grid, smem, s, early)));
+        return SLIM_OK;
+    }
     using Launch = cudaError_t (*)(const SetParams&, int, size_t, cudaStream_t, bool);
-    static const Launch forms[8] = {launch_set<1, false, 2>, launch_set<2, false, 2>, launch_set<3, false, 2>, launch_set<4, false, 2>,
-                                    launch_set<5, false, 2>, launch_set<6, false, 2>, launch_set<7, false, 2>, launch_set<8, false, 2>};
-    const cudaError_t e = info->max_tokens == 1 ? launch_set<1, true, 2>(prm, info->grid, smem, s, early) : forms[info->token_tiles - 1](prm, info->grid, smem, s, early);
+    static const Launch forms[6] = {launch_set<3, false, 2>, launch_set<4, false, 2>, launch_set<5, false, 2>, launch_set<6, false, 2>,
+                                    launch_set<7, false, 2>, launch_set<8, false, 2>};
+    const cudaError_t e = info->max_tokens == 1 ? launch_set<1, true, 2>(prm, info->grid, smem, s, early) : forms[info->token_tiles - 3](prm, info->grid, smem, s, early);
     SLIM_CUDA_TRY(e);
     return SLIM_OK;
 }
@@ -993,8 +1702,7 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
     SetLayer d;
     fill_descriptor(L, gt, r.sg.mpad, 0, r.x_off, r.sp, r.part_off, r.cnt0, &d);
     uint8_t* plan = static_cast<uint8_t*>(workspace) + r.plan_off;
-    const long long n_items = static_cast<long long>(r.n_rb) * r.sp;
-    const int grid = static_cast<int>(n_items < r.sg.grid ? n_items : r.sg.grid);
+    const int n_items = r.n_items, grid = std::min(n_items, r.sg.grid);
     slim_gemv_set_info info;
     memset(&info, 0, sizeof info);
     info.n_layers = 1;
@@ -1002,8 +1710,8 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
     info.n_slots = r.sg.n_slots;
     info.slot_bytes = r.sg.slot_bytes;
     info.token_tiles = r.sg.nt;
-    info.stage_tasks = (r.sg.mpad == 2 ? 1 : r.sg.mpad) * gt.G;
-    info.n_items = static_cast<int>(n_items);
+    info.stage_tasks = layer_tasks(r.sg, M, gt.G);
+    info.n_items = n_items;
     info.max_bits = r.sg.bmax;
     info.max_tokens = r.sg.mmax;
     info.tiles_per_warp = r.sg.tpw;
@@ -1026,6 +1734,36 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
     return launch_set_for(&info, prm, smem, stream, early);
 }
 
+size_t gemv_tc_workspace_bytes(int M, int N, const GroupTable& gt) {
+    TcSinglePlan pl;
+    // a caller who leaves the flags of slim_mpq_gemm out of the size (they were not always in it) gets the same kernel
+    return tc_single_plan(M, N, gt, &pl) ? pl.total + kWsFlagsBytes : 0;
+}
+int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y, int M, int N, int K,
+            void* workspace, size_t workspace_bytes, cudaStream_t stream) {
+    TcSinglePlan pl;
+    if (!tc_single_plan(M, N, gt, &pl) || workspace_bytes < pl.total) return 1;
+    slim_layer L;
+    memset(&L, 0, sizeof L);
+    L.x = x; L.packed = packed; L.scales = scales; L.zeros = zeros; L.y = y; L.M = M; L.N = N; L.K = K;
+    TcSingle t;
+    memset(&t, 0, sizeof t);
+    fill_descriptor(L, gt, -rawtc::form(M), 0, pl.x_off, 1, 0, 0, &t.layer);
+    t.ws = static_cast<uint8_t*>(workspace);
+    t.part_off = pl.part_off;
+    t.n_slots = pl.n_slots; t.slot_bytes = pl.slot_bytes; t.off_rec = pl.off_rec; t.n_rb = pl.n_rb; t.grid = pl.grid;
+    for (int b = 1; b <= 4; ++b) t.per_rb += t.layer.count[b - 1] * tc_step_cost(b, rawtc::kTiles);
+    if (pl.local) {
+        SLIM_CUDA_TRY((launch_tc_form<kLocal, TcSingle>(M, t, pl.grid, pl.smem, stream, true)));
+        return SLIM_OK;
+    }
+    const int tasks = (M + 3) / 4 * 4 * gt.G;
+    PdlLaunch l(static_cast<unsigned>((tasks + 31) / 32), 256, 0, stream);
+    SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, set_single_stage_kernel, t.layer, static_cast<uint8_t*>(nullptr), t.ws, 1, 1, 1, tasks, 0));
+    SLIM_CUDA_TRY((launch_tc_form<kStaged, TcSingle>(M, t, pl.grid, pl.smem, stream, true)));
+    return SLIM_OK;
+}
+
 }  // namespace slim
 
 extern "C" {
@@ -1033,9 +1771,14 @@ extern "C" {
 int slim_gemv_set_bytes(const slim_layer* layers_host, int n_layers, int g, size_t* plan_bytes, size_t* workspace_bytes) {
     if (plan_bytes == nullptr || workspace_bytes == nullptr) return SLIM_ERR_INVALID_ARG;
     slim::SetGeometry sg;
-    const int st = slim::set_geometry(layers_host, n_layers, g, &sg);
-    if (st != SLIM_OK) return st;
-    *plan_bytes = slim::set_plan_bytes(n_layers, sg.n_items);
+    slim::TcDeal deal;
+    try {
+        const int st = slim::set_geometry(layers_host, n_layers, g, &sg, &deal);
+        if (st != SLIM_OK) return st;
+    } catch (const std::exception&) {
+        return SLIM_ERR_UNSUPPORTED;
+    }
+    *plan_bytes = slim::set_plan_bytes(n_layers, sg.n_items, sg.n_cuts);
     *workspace_bytes = sg.ws_bytes;
     return SLIM_OK;
 }
@@ -1044,10 +1787,15 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
                        slim_gemv_set_info* info, void* stream) {
     if (info == nullptr || plan == nullptr) return SLIM_ERR_INVALID_ARG;
     slim::SetGeometry sg;
-    const int st = slim::set_geometry(layers_host, n_layers, g, &sg);
-    if (st != SLIM_OK) return st;
+    slim::TcDeal deal;
+    try {
+        const int st = slim::set_geometry(layers_host, n_layers, g, &sg, &deal);
+        if (st != SLIM_OK) return st;
+    } catch (const std::exception&) {
+        return SLIM_ERR_UNSUPPORTED;
+    }
     if (!slim::aligned16(plan)) return SLIM_ERR_ALIGNMENT;
-    if (plan_bytes < slim::set_plan_bytes(n_layers, sg.n_items)) return SLIM_ERR_WORKSPACE;
+    if (plan_bytes < slim::set_plan_bytes(n_layers, sg.n_items, sg.n_cuts)) return SLIM_ERR_WORKSPACE;
     for (int l = 0; l < n_layers; ++l) {
         const slim_layer& L = layers_host[l];
         if (L.x == nullptr || L.packed == nullptr || L.scales == nullptr || L.zeros == nullptr || L.y == nullptr)
@@ -1091,6 +1839,7 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
     items.reserve(static_cast<size_t>(sg.n_items));
     cost.reserve(static_cast<size_t>(sg.n_items));
     const int tpi = slim::kSetConsumers * sg.tpw;
+    const bool tc = slim::tc_form(sg.mmax);
     int task = 0, cnt0 = 0;
     size_t ws_off = slim::kSetOffCounters + sg.cnt_bytes;
     // workspace: header, the arrival counters of the split row blocks, the staged activations of all layers, then the
@@ -1101,12 +1850,12 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
         for (int l = 0; l < n_layers; ++l) {
             slim::GroupTable gt;
             slim::make_group_table(layers_host[l].N, layers_host[l].K, g, layers_host[l].bits_host, &gt);
-            off += slim::layer_ws_bytes(sg.mres, gt);
+            off += slim::layer_x_bytes(sg, layers_host[l].M, gt);
         }
         for (int l = 0; l < n_layers; ++l) {
             const slim_layer& L = layers_host[l];
-            const int sp = slim::layer_split(sg.split, L.K / SLIM_GROUP);
-            part_off[l] = off;
+            const int sp = tc ? 1 : slim::layer_split(sg.split, L.K / SLIM_GROUP);
+            part_off[l] = off;                     // (tc: of all layers' parts)
             if (sp > 1) off += slim::align_to(static_cast<size_t>(sp) * L.M * L.N * sizeof(float), 128);
         }
     }
@@ -1115,7 +1864,7 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
         slim::GroupTable gt;
         slim::make_group_table(L.N, L.K, g, L.bits_host, &gt);
         slim::SetLayer d;
-        const int sp = slim::layer_split(sg.split, gt.G);
+        const int sp = tc ? 1 : slim::layer_split(sg.split, gt.G);
         // A layer that reads the activations of an earlier layer through the same bit map (the staged form depends
         // on the group's bit-width) uses that layer's staged copy and has no staging tasks of its own.
         int same = -1;
@@ -1124,13 +1873,13 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
             if (E.x == L.x && E.M == L.M && E.K == L.K && memcmp(E.bits_host, L.bits_host, static_cast<size_t>(L.K / g)) == 0) same = e;
         }
         x_off[l] = same >= 0 ? x_off[same] : ws_off;
-        slim::fill_descriptor(L, gt, sg.mpad, task, x_off[l], sp, part_off[l], cnt0, &d);
-        ws_off += slim::layer_ws_bytes(sg.mres, gt);
+        slim::fill_descriptor(L, gt, tc ? -slim::rawtc::form(sg.mmax) : sg.mpad, task, x_off[l], sp, part_off[l], cnt0, &d);
+        ws_off += slim::layer_x_bytes(sg, L.M, gt);
         SLIM_CUDA_TRY(cudaMemcpyAsync(plan_dev + slim::kSetPlanHeader + static_cast<size_t>(l) * sizeof d, &d, sizeof d,
                                       cudaMemcpyHostToDevice, s));
         const int n_rb = ((L.N >> 4) + tpi - 1) / tpi;
         if (sp > 1) cnt0 += n_rb * slim::kSetConsumers;
-        for (int rb = 0; rb < n_rb; ++rb) {
+        for (int rb = 0; rb < n_rb && !tc; ++rb) {
             const int th = (L.N >> 4) - tpi * rb;
             for (int part = 0; part < sp; ++part) {
                 const int p0 = gt.G * part / sp, p1 = gt.G * (part + 1) / sp;
@@ -1148,11 +1897,23 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
                 cost.push_back(slim::item_cost(th < tpi ? th : tpi, gt, d.order, p0, p1));
             }
         }
-        if (same < 0) task += (sg.mpad == 2 ? 1 : sg.mpad) * gt.G;
+        if (same < 0) task += slim::layer_tasks(sg, L.M, gt.G);
+    }
+    if (tc) {
+        const size_t parts = part_off[0];          // the parts' room begins here
+        for (slim::SetItem& it : deal.items)
+            if (it.counts >= 0) it.y = reinterpret_cast<__half*>(reinterpret_cast<size_t>(it.y) + parts);
+        for (slim::SetCut& cut : deal.cuts) cut.off += parts;
+        uint8_t* at = plan_dev + slim::kSetPlanHeader + static_cast<size_t>(n_layers) * sizeof(slim::SetLayer);
+        SLIM_CUDA_TRY(cudaMemcpyAsync(plan_dev, deal.begin.data(), static_cast<size_t>(deal.grid + 1) * sizeof(int), cudaMemcpyHostToDevice, s));
+        SLIM_CUDA_TRY(cudaMemcpyAsync(at, deal.items.data(), deal.items.size() * sizeof(slim::SetItem), cudaMemcpyHostToDevice, s));
+        if (!deal.cuts.empty())
+            SLIM_CUDA_TRY(cudaMemcpyAsync(at + deal.items.size() * sizeof(slim::SetItem), deal.cuts.data(), deal.cuts.size() * sizeof(slim::SetCut), cudaMemcpyHostToDevice, s));
     }
     // The deal: items by falling cost (equal costs in the set's order), each to the CTA that has the
     // least so far (the lowest-numbered of equals).  Within a CTA the heavy items come first.
-    const int n_items = static_cast<int>(items.size());
+    const int n_items = static_cast<int>(tc ? deal.items.size() : items.size());
+    if (!tc) {
     std::vector<int> by_cost(n_items);
     for (int i = 0; i < n_items; ++i) by_cost[i] = i;
     std::stable_sort(by_cost.begin(), by_cost.end(), [&](int a, int b) { return cost[a] > cost[b]; });
@@ -1176,7 +1937,7 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
     SLIM_CUDA_TRY(cudaMemcpyAsync(plan_dev, item_begin, static_cast<size_t>(sg.grid + 1) * sizeof(int), cudaMemcpyHostToDevice, s));
     SLIM_CUDA_TRY(cudaMemcpyAsync(plan_dev + slim::kSetPlanHeader + static_cast<size_t>(n_layers) * sizeof(slim::SetLayer), dealt.data(),
                                   static_cast<size_t>(n_items) * sizeof(slim::SetItem), cudaMemcpyHostToDevice, s));
-    const int item = n_items;
+    }
 
     memset(info, 0, sizeof *info);
     info->n_layers = n_layers;
@@ -1185,13 +1946,13 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
     info->slot_bytes = sg.slot_bytes;
     info->token_tiles = sg.nt;
     info->stage_tasks = task;
-    info->n_items = item;
+    info->n_items = n_items;
     info->max_bits = sg.bmax;
     info->max_tokens = sg.mmax;
     info->tiles_per_warp = sg.tpw;
     info->split = sg.split;
     info->n_counters = sg.n_counters;
-    info->plan_bytes = slim::set_plan_bytes(n_layers, n_items);
+    info->plan_bytes = slim::set_plan_bytes(n_layers, n_items, sg.n_cuts);
     info->workspace_bytes = sg.ws_bytes;
     } catch (const std::exception&) {
         return SLIM_ERR_UNSUPPORTED;
@@ -1234,7 +1995,8 @@ int slim_mpq_gemv_set(const slim_gemv_set_info* info, const void* plan, void* wo
         slim::PdlLaunch l(static_cast<unsigned>((info->stage_tasks + per_block - 1) / per_block), 256, 0, s, early);
         SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, one ? slim::gemv_set_stage_kernel<true> : slim::gemv_set_stage_kernel<false>, prm.layers, prm.ws, info->n_layers, info->stage_tasks, info->n_counters));
     }
-    return slim::launch_set_for(info, prm, smem, s, early);
+    // The kernel of 2 to 16 tokens asks for its first slices while x is staged; what the staging kernel writes it waits for.
+    return slim::launch_set_for(info, prm, smem, s, early || slim::tc_form(info->max_tokens));
 }
 
 }  // extern "C"

@@ -1,0 +1,121 @@
+"""GPU: the kernel for 2 to 16 tokens on raw codes (tcgen05, 8-bit floats), as a layer set and as one large layer, against the
+oracle or an fp64 product with the dequantised weights."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import slim_oracle as orc
+from paper_2405_14917_b200 import binding as slim
+from paper_2405_14917_b200 import workloads as wl
+from tests.helpers import check_output, oracle_layer
+
+pytestmark = pytest.mark.gpu
+
+
+def _on_device(L):
+    packed = torch.from_numpy(orc.pack(L["codes"], L["bits"])).cuda()
+    return slim.QuantLinear(packed, L["bits"], torch.from_numpy(L["scales"]).cuda(), torch.from_numpy(L["zeros"]).cuda(), L["N"], L["K"])
+
+
+def _quantised(N, K, avg, seed=0):
+    W, a = wl.make_weight_and_norms_device((31, N, K + seed), N, K, "cuda")
+    return slim.QuantLinear.from_weight(W, a, avg)
+
+
+def _fp64(layer, x):
+    What = slim.dequant(layer.packed, layer.bits, layer.scales, layer.zeros, layer.N, layer.K).double()
+    return (x.double() @ What.T).cpu().numpy()
+
+
+def _set(entries):
+    s = slim.LayerSet(entries)
+    s.run()
+    s.check()
+    return s
+
+
+# every form (tokens rounded up to even) with its last column used and not, and row blocks of one row tile, of one less and one more
+# than a row of MMA tiles, and of more than 512 rows
+@pytest.mark.parametrize("M", range(2, 17))
+def test_every_form_on_ragged_row_blocks(M):
+    layers = [oracle_layer(N, K, avg, m, block=i, seed_name="set-tc") for i, (N, K, avg, m) in enumerate(
+        [(16, 128, 2, M), (112, 384, 3, max(1, M - 1)), (272, 256, 2, M), (528, 640, 3, 1), (1040, 128, 2, M)])]
+    entries = [(_on_device(L), torch.from_numpy(L["x"]).cuda(), torch.full((L["M"], L["N"]), float("nan"), dtype=torch.float16, device="cuda")) for L in layers]
+    s = _set(entries)
+    assert s.info["tiles_per_warp"] == 4                              # items of 512 rows
+    for L, (_, _, y) in zip(layers, entries):
+        check_output(y.cpu().numpy(), orc.linear_f64(L["x"], L["codes"], L["scales"], L["zeros"]), f"{L['N']}x{L['K']} M={L['M']} of {M}")
+
+
+@pytest.mark.parametrize("M", [2, 9])
+def test_each_bit_of_a_code_meets_its_activation(M):
+    """One activation at a time: column k of the weights, exact up to the one rounding of the output."""
+    bits = np.array([1, 2, 3, 4], dtype=np.uint8)
+    L = oracle_layer(32, 512, 2, M, bits=bits, seed_name="set-tc-columns")
+    What = orc.dequant_f64(L["codes"], L["scales"], L["zeros"])
+    dl = _on_device(L)
+    entries = []
+    for k0 in range(0, 512, M):
+        x = np.zeros((M, 512), np.float16)
+        for m in range(M):
+            x[m, (k0 + m) % 512] = 1.0
+        entries.append((dl, torch.from_numpy(x).cuda(), torch.empty((M, 32), dtype=torch.float16, device="cuda")))
+    _set(entries)
+    for i, (_, _, y) in enumerate(entries):
+        want = np.stack([What[:, (i * M + m) % 512] for m in range(M)]).astype(np.float16)
+        assert (y.cpu().numpy().view(np.uint16) == want.view(np.uint16)).all(), i
+
+
+def test_activations_of_any_size_are_taken_exactly():
+    """One weight per row and all of x's exponents: x (q - z) s from a group whose largest |x| is 2^15 times the smallest; an infinity and a NaN
+    spoil their token alone."""
+    L = oracle_layer(16, 256, 2, 4, seed_name="set-tc-range")
+    x = np.zeros((4, 256), np.float16)
+    x[0, :128] = [(1 + (37 * i % 1024) / 1024) * 2.0 ** (i % 16 - 13) * (-1) ** i for i in range(128)]
+    x[1, 130:140] = 6e-8 * np.arange(1, 11)                           # subnormals alone
+    x[2, 5], x[3, 200] = np.inf, np.nan
+    L["x"] = x
+    y = torch.empty((4, 16), dtype=torch.float16, device="cuda")
+    _set([(_on_device(L), torch.from_numpy(x).cuda(), y)])
+    y = y.cpu().numpy().astype(np.float64)
+    ref = orc.linear_f64(x[:2], L["codes"], L["scales"], L["zeros"])
+    # one rounding to fp16 (a half unit, or half of the smallest subnormal) and fp32 sums of 128 products
+    bound = 2.0 ** -11 * np.abs(ref) + 2.0 ** -25 + 2.0 ** -20 * np.abs(x[:2].astype(np.float64)).sum(axis=1)[:, None] * np.abs(orc.dequant_f64(L["codes"], L["scales"], L["zeros"])).max()
+    assert (np.abs(y[:2] - ref) <= bound).all()
+    assert np.isnan(y[2:]).all()
+
+
+@pytest.mark.parametrize("M,avg", [(2, 2), (7, 3), (8, 3), (16, 2), (16, 3)])
+def test_shares_that_end_inside_row_blocks_repeat_bit_for_bit(M, avg):
+    """A set of more steps than four per CTA: equal shares, sums of cut row blocks added in the order of their parts.  A step read before it
+    has landed, or sums added before they are written, would show as a run that differs."""
+    entries = []
+    for i, (N, K) in enumerate([(4096, 4096), (1040, 11008), (11008, 1024), (5120, 5120)]):
+        layer = _quantised(N, K, avg, i)
+        entries.append((layer, torch.randn((M, K), device="cuda").half(), torch.empty((M, N), dtype=torch.float16, device="cuda")))
+    s = _set(entries)
+    assert s.info["split"] > 1 and s.info["n_items"] > s.info["grid"]
+    first = [y.clone() for (_, _, y) in entries]
+    for (layer, x, _), y in zip(entries, first):
+        check_output(y.cpu().numpy(), _fp64(layer, x), f"{layer.N}x{layer.K} M={M}")
+    for _ in range(60):
+        s.run()
+        for (_, _, y), want in zip(entries, first):
+            assert torch.equal(y, want)
+    s.check()
+
+
+@pytest.mark.parametrize("N,K,M,avg", [(14336, 8192, 2, 2), (14336, 8192, 8, 2), (26624, 4096, 5, 2), (16, 128, 2, 2), (28672, 8192, 16, 2), (8192, 28672, 13, 2), (14352, 8192, 9, 3)])
+def test_one_large_layer_in_one_or_two_launches(N, K, M, avg):
+    """Records of x in shared memory, or staged by a kernel ahead (many tokens and steps): the layer's own shares, twice into one workspace."""
+    layer = _quantised(N, K, avg)
+    x = torch.randn((M, K), device="cuda").half()
+    ws = slim.new_workspace(M, N, K, layer.bits)
+    y = layer.forward(x, ws)
+    check_output(y.cpu().numpy(), _fp64(layer, x), f"{N}x{K} M={M}")
+    for _ in range(40):
+        assert torch.equal(layer.forward(x, ws), y)
+    assert not ws[256:1280].any()                                     # the words that count the parts are zero again
+    slim.workspace_status(ws)
+    small = torch.zeros(256, dtype=torch.uint8, device="cuda")        # no room for parts: the kernels for a few tokens
+    check_output(layer.forward(x, small).cpu().numpy(), _fp64(layer, x), f"{N}x{K} M={M}, status word alone")
