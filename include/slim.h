@@ -216,13 +216,12 @@ int slim_mpq_gemm_static(const void* x, const void* packed, const uint8_t* bits_
  * fp16 activation within a factor 2^11 of that maximum is taken exactly and a smaller one with an error
  * of at most 2^-22 of the maximum; the sums over the group are then exact.  Per output row n this adds at
  * most  sum over groups of 2^-22 max|x_group| sum_{k in group} |w-hat[n][k]|  to the error of the fp16
- * path at more than one token; x must be finite.  Sets of 2 to 16 tokens multiply
+ * path at more than one token; x must be finite.  Sets of 2 to 64 tokens multiply
  * the codes by x as a sum of three 8-bit floats, exact for an fp16 activation within a factor 2^15 of the group's largest and
  * off by at most 2^-26 of that below, with the sums of a group added up by the tensor cores; their widest layer, rounded up to an
- * even number of tokens, fixes how many columns every layer computes.  Sets of 17 to 64 tokens multiply the fp16 x as it is, in MMA
- * tiles of 8 tokens, as many as the widest layer needs.  A set is fastest when its layers have about the same token count.  (Between
- * 17 and about 100 tokens a layer set streams several times the weights per second that slim_mpq_gemm dequantises,
- * which is built for hundreds of tokens and more.)
+ * even number of tokens (beyond 16 a multiple of 8), fixes how many columns every layer computes, so a set is fastest when its layers have
+ * about the same token count.  (Between 17 and about 100 tokens a layer set streams several times the weights per second that
+ * slim_mpq_gemm dequantises, which is built for hundreds of tokens and more.)
  * N > 0 a multiple of 16, K > 0 a multiple of 128; g in {128, 256, 512}, one value for the whole set (for 256 and
  * 512 "group" in the bound above reads "128 columns of a group"); SLIM_ERR_UNSUPPORTED for 32 and 64. */
 typedef struct slim_layer {
@@ -248,7 +247,7 @@ typedef struct slim_gemv_set_info {
     int max_tokens;        /* largest M of the set */
     int tiles_per_warp;    /* an item is 128 rows times this: 4 for sets of 2 to 16 tokens, else 2 */
     int split;             /* most parts the groups of a row block are cut into: 1 .. 8 when the set has fewer row blocks than
-                              persistent CTAs (layers with few groups get fewer), 1 .. 15 for sets of 2 to 16 tokens, whose CTAs
+                              persistent CTAs (layers with few groups get fewer), 1 .. 15 for sets of 2 to 64 tokens, whose CTAs
                               take equal shares that may end inside a row block; fp32 partial outputs in the workspace, added in
                               part order by the warp whose part lands last */
     int n_counters;        /* arrival counters of the split row blocks (workspace, cleared by every launch) */

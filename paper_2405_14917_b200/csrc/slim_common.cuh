@@ -55,7 +55,7 @@ int gemv_one(const void* x, const void* packed, const GroupTable& gt, const void
 int gemv_few(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y,
              int M, int N, int K, void* workspace, cudaStream_t stream);
 
-// ... and layers of 2 to 16 tokens, from a workspace of that many bytes on (0: none is enough), to the layer-set kernel on tcgen05
+// ... and large layers of 2 to 56 tokens, from a workspace of that many bytes on (0: none is enough), to the layer-set kernel on tcgen05
 // without a plan (slim_gemv_set.cu): as above.
 size_t gemv_tc_workspace_bytes(int M, int N, const GroupTable& gt);
 int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y, int M, int N, int K,

@@ -1117,6 +1117,10 @@ extern "C" int slim_mpq_gemm(const void* x, const void* packed, const uint8_t* b
     if (workspace == nullptr || workspace_bytes < 256) return SLIM_ERR_WORKSPACE;
     if (!slim::aligned16(workspace)) return SLIM_ERR_ALIGNMENT;
 
+    {
+        const int taken = slim::gemv_tc(x, packed, gt, scales, zeros, y, M, N, K, workspace, workspace_bytes, s);
+        if (taken <= 0) return taken;
+    }
     // Up to 24 tokens on a layer of 16 to 64 K-tiles and up to 18 MB, and up to 32 on one of up to 5 MB, are sooner through the
     // kernel for a few tokens (us, that kernel / this one): 2048 x 2048 at 24 and 32 tokens 6.7 / 9.8 and 7.6 / 9.8, 4096 x 4096
     // 10.5 / 13.2 and 12.4 / 13.2, 1024 x 8192 10.7 / 15.7 and 13.1 / 15.8, 8192 x 8192 23.0 / 24.3 and 31.7 / 24.4; beyond: 8192 x

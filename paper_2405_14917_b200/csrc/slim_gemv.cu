@@ -516,6 +516,8 @@ int slim_workspace_bytes(int M, int N, int K, int g, const uint8_t* bits_host, s
     if (M >= 1 && M <= SLIM_GEMV_MAX_M && N > 0 && K > 0) {       // large layers go through the layer-set kernels
         const size_t routed = slim::gemv_route_workspace_bytes(M, N, K, g, bits_host, gt);
         if (routed > *out_bytes) *out_bytes = routed;
+    }
+    if (M >= 2 && N > 0 && K > 0) {
         const size_t tc = slim::gemv_tc_workspace_bytes(M, N, gt);
         if (tc > *out_bytes) *out_bytes = tc;
     }

@@ -20,9 +20,9 @@
 //    acc += s * (D * 2^(24-S) - z * sum_k x); after the last group it stores its 16 rows.  A warp
 //    walks the whole K itself: no partial sums, no reduction between warps or CTAs.
 //
-// That is the kernel of single-token sets (on the integer form of slim_gemv_i8.cuh) and of sets with 17 to 64 tokens somewhere.
-// Sets of 2 to 16 tokens, and one large layer of as many, go through gemv_set_tc_kernel: the same ring, blocks of 512 rows, products
-// on tcgen05 (slim_set_tc.cuh), shares of equal cost in place of dealt items.
+// That is the kernel of single-token sets, on the integer form of slim_gemv_i8.cuh.  Sets of 2 to 64 tokens, and one large layer of as
+// many, go through gemv_set_tc_kernel: the same ring, blocks of 512 or 256 rows, products on tcgen05 (slim_set_tc.cuh), shares of equal
+// cost in place of dealt items.
 //
 // Every wait on an mbarrier is bounded and reports through the workspace status word.
 #include "slim_gemv_dev.cuh"
@@ -45,7 +45,7 @@ constexpr int kSetConsumers = 8;                       // consumer warps; each o
 constexpr int kSetProducers = 2;                       // producer warps: they take the groups in turn
 constexpr int kSetThreads = 32 * (kSetConsumers + kSetProducers);
 constexpr int kSetMaxSlots = 32;
-constexpr int kSetCtasPerSm = 2;                       // resident CTAs per SM the plan aims at (one from 17 tokens on: registers)
+constexpr int kSetCtasPerSm = 2;                       // resident CTAs per SM the plan aims at (single-token sets)
 constexpr int kSetMaxTokens = 64;                      // tokens of a layer in a set: up to eight MMA tiles of 8
 
 // Layout of a ring slot (tpi = 16-row tiles of a work item, mp = 256-byte pieces per slice of the staged
@@ -71,11 +71,8 @@ struct SetLayer {
     int M, N, K, G;
     uint16_t count[4];     // groups of 1, 2, 3, 4 bits
     int task0;             // first (token, group) staging task of the layer
-    int MP;                // 256-byte pieces per slice in the staged layout: a multiple of 8 up to 64 = tokens of the f16 fragments
-                           // for the whole set (what a layer does not have is not staged: the kernel multiplies whatever the
-                           // workspace holds there, in columns of the products that are never stored); 2 if every layer of
-                           // the set has one token: the 8-bit digit form (stage_groups_i8); -mv: the
-                           // form mv of slim_set_tc.cuh
+    int MP;                // form of the staged activations: 2, every layer of the set has one token: 8-bit digits, 512 bytes per slice
+                           // (stage_groups_i8); -mv: the form mv of slim_set_tc.cuh
     uint16_t prefix[SLIM_MAX_GROUPS + 1];
     uint16_t pre3[SLIM_MAX_GROUPS + 1];   // 3-bit groups (two slices) before group j
     uint8_t bits[SLIM_MAX_GROUPS];
@@ -130,17 +127,10 @@ __device__ __forceinline__ void stage_task_one(const SetLayer& L, uint8_t* ws, i
     stage_groups_i8(L.x + pi * SLIM_GROUP, live ? grp : nullptr, L.bits[pi], lane);
 }
 
-// Staging task `pi` of layer L (one warp) of any other set: four tokens from 4 (pi / G) on, group pi % G.  What the workspace
-// holds for tokens that the layer does not have is multiplied like the rest and never stored.
+// Staging task `pi` of layer L (one warp) of any other set: four tokens from 4 (pi / G) on, group pi % G, for gemv_set_tc_kernel.
 __device__ __forceinline__ void stage_task(const SetLayer& L, uint8_t* ws, int pi, int lane) {
     const int q = pi / L.G, j = pi - q * L.G;
-    if (4 * q >= L.M) return;
-    if (L.MP < 0) {                                             // the form of gemv_set_tc_kernel
-        rawtc::stage_tokens(L.x + j * SLIM_GROUP, L.K, L.bits[j], 4 * q, L.M, -L.MP, ws + L.x_off + static_cast<size_t>(j) * rawtc::record_bytes(-L.MP), lane);
-        return;
-    }
-    uint8_t* grp = ws + L.x_off + staged_group_offset(j, L.pre3[j], L.MP);
-    stage_tokens(L.x + j * SLIM_GROUP, L.K, L.bits[j], 4 * q, L.M, L.MP, grp + staged_header_bytes(L.MP), reinterpret_cast<float2*>(grp), lane);
+    if (4 * q < L.M) rawtc::stage_tokens(L.x + j * SLIM_GROUP, L.K, L.bits[j], 4 * q, L.M, -L.MP, ws + L.x_off + static_cast<size_t>(j) * rawtc::record_bytes(-L.MP), lane);
 }
 
 // One warp per (layer, four tokens, group), or eight lanes per (layer, group) if every layer has ONE token: fragments and
@@ -178,21 +168,11 @@ __global__ void __launch_bounds__(256) gemv_set_stage_kernel(const SetLayer* __r
     }
 }
 
-// D = A * B with a zero accumulator input: starts an accumulation chain without clearing registers first.
-__device__ __forceinline__ void mma_f16_first(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint2 b) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
-        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y), "f"(0.f));
-}
-
-
-// A consumer warp that has stored its fp32 partial sums of a split row block (n_act tiles from tile0 on, M tokens)
+// A consumer warp that has stored its fp32 partial sums of a split row block (n_act tiles from tile0 on)
 // counts itself on the row block's counter of this warp.  The warp that counts last sees the other parts and adds all
 // parts in part order, so the result does not depend on which part came last: y = fp16 of that sum.  Out of line: it
 // runs once per item.
-template <int Q>
-__device__ __noinline__ void finish_parts(const SetParams& p, int layer, int rb, int warp, int lane, int tile0, int n_act, int M, int N) {
+__device__ __noinline__ void finish_parts(const SetParams& p, int layer, int rb, int warp, int lane, int tile0, int n_act, int N) {
     const SetLayer* L = p.layers + layer;
     __threadfence();                                    // this lane's partial sums before the count
     __syncwarp();
@@ -204,36 +184,18 @@ __device__ __noinline__ void finish_parts(const SetParams& p, int layer, int rb,
     if (static_cast<int>(old) + 1 != S) return;
     __threadfence();
     const float* part = reinterpret_cast<const float*>(p.ws + L->part_off);
-    const size_t MN = static_cast<size_t>(M) * N;
     __half* y = L->y;
-    // 16 * n_act rows x M tokens as pairs of rows: pair i of token m.  Q pairs of a lane at a time, so that their loads are in
-    // flight together: the warp holds up the ring's slots meanwhile (one 70B block of 16 tokens as a set: 199 us with one pair
-    // at a time, 159 with two).  What is live here costs registers in the loop that calls it, so four only where one CTA has
-    // the SM: with four in the two-CTA forms their loops spilled, 7B sweep of one token 89 -> 93 us.
-    const int pairs = 8 * n_act, total = pairs * M;
-    for (int i0 = lane; i0 < total; i0 += 32 * Q) {
-        float2 sum[Q];
-        unsigned int at[Q];                             // below 64 * N
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const int i = min(i0 + 32 * q, total - 1), m = i / pairs;
-            at[q] = static_cast<unsigned int>(m * N + 16 * tile0 + 2 * (i - m * pairs));
-            sum[q] = __ldcg(reinterpret_cast<const float2*>(part + at[q]));
-        }
-        const float* next = part;
-        for (int k = 1; k < S; ++k) {
-            next += MN;
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const float2 v = __ldcg(reinterpret_cast<const float2*>(next + at[q]));
-                sum[q].x += v.x;
-                sum[q].y += v.y;
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < Q; ++q)
-            if (i0 + 32 * q < total) *reinterpret_cast<__half2*>(y + at[q]) = __floats2half2_rn(sum[q].x, sum[q].y);
+    // 16 * n_act rows as pairs: a lane's
+    if (lane >= 8 * n_act) return;
+    const unsigned int at = static_cast<unsigned int>(16 * tile0 + 2 * lane);
+    float2 sum = __ldcg(reinterpret_cast<const float2*>(part + at));
+    for (int k = 1; k < S; ++k) {
+        part += N;
+        const float2 v = __ldcg(reinterpret_cast<const float2*>(part + at));
+        sum.x += v.x;
+        sum.y += v.y;
     }
+    *reinterpret_cast<__half2*>(y + at) = __floats2half2_rn(sum.x, sum.y);
 }
 
 // Slow path of a consumer's wait, kept out of line so that the loop around it stays small.
@@ -386,181 +348,20 @@ __device__ __forceinline__ void consume_one(const SetParams& p, const uint32_t s
                     else *reinterpret_cast<__half2*>(reinterpret_cast<__half*>(yword) + row) = __floats2half2_rn(acc0, acc2);
                 }
             }
-            if (counts & kItemPartial) finish_parts<1>(p, layer, rb, warp, lane, tile0, n_act, 1, N);
+            if (counts & kItemPartial) finish_parts(p, layer, rb, warp, lane, tile0, n_act, N);
         }
     }
 }
 
-
-// Consumer warp of a set with more than one token somewhere: f16 MMAs on raw code fields (one AND per operand
-// register of two codes, see slim_gemv_dev.cuh), NT tiles of 8 tokens, then the fold
-// acc += s (D 2^(24-S) - z sum_x) per (row, token, group).  Same loop structure as consume_one.
-template <int NT, int TPW>
-__device__ __forceinline__ void consume_f16(const SetParams& p, const uint32_t sbase, const uint32_t ring, volatile int* abort,
-                                            const int i0, const int i1, const int warp, const int lane) {
-    auto full = [&](int s) { return sbase + 8u * s; };
-    auto empty = [&](int s) { return sbase + 8u * (kSetMaxSlots + s); };
-    constexpr int TPI = kSetConsumers * TPW, MPK = 8 * NT;
-    // interleaved accumulation chains per (tile, token tile): with four (tile, token tile) pairs the MMAs of one pair are far
-    // enough apart without a second chain
-    constexpr int CH = NT * TPW >= 4 ? 1 : (NT == 1 ? (TPW == 1 ? 4 : 2) : 2);
-    constexpr uint32_t kOffZ = slot_off_z(TPI), kOffE = slot_off_e(TPI), kOffX = slot_off_x(TPI, MPK), kOffW = slot_off_w(TPI, MPK);
-    const int gq = lane >> 2, c = lane & 3;
-    const uint32_t lane0 = lane == 0 ? 1u : 0u;
-    const uint32_t slot_bytes = static_cast<uint32_t>(p.slot_bytes);
-    const int n_slots = p.n_slots;
-    const uint32_t sz_lane = static_cast<uint32_t>(TPW * warp * 32 + gq * 4);
-    const uint32_t x_lane = kOffX + (gq * 4 + c) * 8;             // fragment of token gq of the first token tile
-    const uint32_t e_lane = kOffE + 16u * c;                      // (sum_x, scale) of tokens 2c, 2c + 1
-    const uint32_t w_lane = kOffW + 8u * lane;
-    int s = 0;
-    uint32_t ph = 0;
-    bool ok = true;
-    const int4* items4 = reinterpret_cast<const int4*>(p.items);
-    int4 it_a = items4[2 * i0], it_b = items4[2 * i0 + 1];       // (layer, rb, N, range), (y, M, counts)
-    for (int i = i0; i < i1 && ok; ++i) {
-        const int layer = it_a.x, rb = it_a.y, N = it_a.z, p0 = it_a.w & 0xffff, p1 = it_a.w >> 16, M = it_b.z, counts = it_b.w;
-        const unsigned long long yword = (static_cast<unsigned long long>(static_cast<uint32_t>(it_b.y)) << 32) | static_cast<uint32_t>(it_b.x);
-        if (i + 1 < i1) {                                        // the next item arrives during this one's groups
-            it_a = items4[2 * i + 2];
-            it_b = items4[2 * i + 3];
-        }
-        const int tile0 = TPI * rb + TPW * warp;                 // this warp's first tile of the layer
-        const int n_act = min(TPW, (N >> 4) - tile0);            // its tiles that exist (<= 0: none)
-        if (n_act <= 0) {
-            for (int j = p0; j < p1; ++j) {                      // only hands the slots back
-                if (!__all_sync(0xffffffffu, sb::try_wait(full(s), ph)) && !wait_full_slow(full(s), ph, abort)) { ok = false; break; }
-                __syncwarp();
-                sb::arrive_if(empty(s), lane0);
-                if (++s == n_slots) { s = 0; ph ^= 1u; }
-            }
-            continue;
-        }
-        float acc[TPW][NT][4];
-#pragma unroll
-        for (int t = 0; t < TPW; ++t)
-#pragma unroll
-            for (int n = 0; n < NT; ++n)
-#pragma unroll
-                for (int r = 0; r < 4; ++r) acc[t][n][r] = 0.f;
-
-        auto run_groups = [&](auto btag, int n_groups) -> bool {
-            constexpr int B = decltype(btag)::value;
-            for (int k = 0; k < n_groups; ++k) {
-                if (!__all_sync(0xffffffffu, sb::try_wait(full(s), ph)) && !wait_full_slow(full(s), ph, abort)) return false;
-                const uint32_t slot = ring + static_cast<uint32_t>(s) * slot_bytes;
-                // tile t of the warp: its slices follow each other.  For a tile past the end of the layer the slot holds
-                // stale bytes: its accumulators are computed and never stored.
-                const uint32_t item0 = slot + w_lane + static_cast<uint32_t>(TPW * warp) * (256u * B);
-                float d[TPW][CH][NT][4];      // every chain is started by an MMA with a zero accumulator
-                // one slice of width WD starting at unit `unit0`, activations in fragment slot `xs`
-                auto run_slice = [&](auto wtag, auto first_tag, int unit0, uint32_t xs) {
-                    constexpr int WD = decltype(wtag)::value;
-                    constexpr int MPU = 8 / WD;                 // MMAs per unit
-                    constexpr bool FIRST = decltype(first_tag)::value != 0;   // the group's first slice
-#pragma unroll
-                    for (int u = 0; u < WD; ++u) {
-                        uint2 wd[TPW];
-                        uint32_t shx[TPW], shy[TPW];
-#pragma unroll
-                        for (int t = 0; t < TPW; ++t) {
-                            wd[t] = lds64(item0 + t * (256u * B) + 256u * (unit0 + u));
-                            shx[t] = wd[t].x >> pair_shift(WD);
-                            shy[t] = wd[t].y >> pair_shift(WD);
-                        }
-#pragma unroll
-                        for (int ii = 0; ii < MPU; ++ii) {
-                            const int mi = u * MPU + ii;
-#pragma unroll
-                            for (int n = 0; n < NT; ++n) {
-                                // fragment of token 8n + gq (tokens the layer lacks are staged as zeros)
-                                const uint2 bv = lds64(xs + ((mi * MPK + 8 * n) * 4) * 8);
-#pragma unroll
-                                for (int t = 0; t < TPW; ++t) {
-                                    const uint32_t a0 = pair<WD>(wd[t].x, shx[t], 2 * ii), a1 = pair<WD>(wd[t].y, shy[t], 2 * ii);
-                                    const uint32_t a2 = pair<WD>(wd[t].x, shx[t], 2 * ii + 1), a3 = pair<WD>(wd[t].y, shy[t], 2 * ii + 1);
-                                    if (FIRST && mi < CH) mma_f16_first(d[t][mi & (CH - 1)][n], a0, a1, a2, a3, bv);
-                                    else mma_f16(d[t][mi & (CH - 1)][n], a0, a1, a2, a3, bv);
-                                }
-                            }
-                        }
-                    }
-                };
-                const uint32_t xs0 = slot + x_lane;
-                if (B == 1) run_slice(W1{}, WidthTag<1>{}, 0, xs0);
-                if (B == 2) run_slice(W2{}, WidthTag<1>{}, 0, xs0);
-                if (B == 3) { run_slice(W2{}, WidthTag<1>{}, 0, xs0); run_slice(W1{}, WidthTag<0>{}, 2, xs0 + 8 * MPK * 32); }
-                if (B == 4) run_slice(W4{}, WidthTag<1>{}, 0, xs0);
-                // fold the group: rows 2gq, 2gq+1, tokens 8n+2c, 8n+2c+1
-#pragma unroll
-                for (int t = 0; t < TPW; ++t) {
-                    const uint32_t s2 = lds32(slot + kSlotOffS + sz_lane + t * 32);
-                    const uint32_t z2 = lds32(slot + kOffZ + sz_lane + t * 32);
-                    const float2 sf = __half22float2(*reinterpret_cast<const __half2*>(&s2));
-                    const float2 zf = __half22float2(*reinterpret_cast<const __half2*>(&z2));
-#pragma unroll
-                    for (int n = 0; n < NT; ++n) {
-                        const uint4 tkw = lds128(slot + e_lane + 64u * n);       // (sx0, e0, sx1, e1)
-                        const float sx0 = __uint_as_float(tkw.x), e0 = __uint_as_float(tkw.y);
-                        const float sx1 = __uint_as_float(tkw.z), e1 = __uint_as_float(tkw.w);
-                        float dd[4];
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            dd[r] = CH == 1 ? d[t][0][n][r] : d[t][0][n][r] + d[t][CH > 1 ? 1 : 0][n][r];
-                            if (CH == 4) dd[r] += d[t][2 % CH][n][r] + d[t][3 % CH][n][r];
-                        }
-                        acc[t][n][0] = fmaf(sf.x, fmaf(-zf.x, sx0, dd[0] * e0), acc[t][n][0]);
-                        acc[t][n][1] = fmaf(sf.x, fmaf(-zf.x, sx1, dd[1] * e1), acc[t][n][1]);
-                        acc[t][n][2] = fmaf(sf.y, fmaf(-zf.y, sx0, dd[2] * e0), acc[t][n][2]);
-                        acc[t][n][3] = fmaf(sf.y, fmaf(-zf.y, sx1, dd[3] * e1), acc[t][n][3]);
-                    }
-                }
-                __syncwarp();
-                sb::arrive_if(empty(s), lane0);
-                if (++s == n_slots) { s = 0; ph ^= 1u; }
-            }
-            return true;
-        };
-        // the widths start at positions 0, e1, e2, e3 of the layer's streaming order; the item covers [p0, p1)
-        const int e1 = counts & 511, e2 = e1 + ((counts >> 9) & 511), e3 = e2 + ((counts >> 18) & 511);
-        auto part = [&](int a, int b) { return max(min(p1, b) - max(p0, a), 0); };
-        ok = run_groups(WidthTag<1>{}, part(0, e1)) && run_groups(WidthTag<2>{}, part(e1, e2)) &&
-             run_groups(WidthTag<3>{}, part(e2, e3)) && run_groups(WidthTag<4>{}, part(e3, 65535));
-        // ---- this warp's rows of the item: rows 2gq, 2gq+1 of tokens 8n+2c, 8n+2c+1 of every tile
-        if (ok) {
-            const bool partial = (counts & kItemPartial) != 0;
-#pragma unroll
-            for (int t = 0; t < TPW; ++t) {
-                if (t >= n_act) break;
-                const int row = 16 * (tile0 + t) + 2 * gq;
-#pragma unroll
-                for (int n = 0; n < NT; ++n) {
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {                    // tokens 8n + 2c and 8n + 2c + 1
-                        const int m = 8 * n + 2 * c + q;
-                        if (m >= M) continue;
-                        const size_t at = static_cast<size_t>(m) * N + row;
-                        if (partial) *reinterpret_cast<float2*>(reinterpret_cast<float*>(p.ws + yword) + at) = make_float2(acc[t][n][q], acc[t][n][2 + q]);
-                        else *reinterpret_cast<__half2*>(reinterpret_cast<__half*>(yword) + at) = __floats2half2_rn(acc[t][n][q], acc[t][n][2 + q]);
-                    }
-                }
-            }
-            if (partial) finish_parts<NT <= 2 ? 2 : 4>(p, layer, rb, warp, lane, tile0, n_act, M, N);
-        }
-    }
-}
 
 // ------------------------------------------------------------------------------------------ the persistent kernel
 constexpr uint32_t kSetOffAbort = 16 * kSetMaxSlots;          // after the full and empty barriers
 constexpr uint32_t kSetOffDesc = 1024;                        // the producer's copy of its layer's descriptor
 constexpr uint32_t kSetOffRing = (kSetOffDesc + kSetProducers * sizeof(SetLayer) + 127) / 128 * 128;
 
-// NT: 8-token MMA tiles, as many as the widest layer needs.  ONE: every layer has a single token; then only
-// column 0 of the MMA results is ever used, so every lane feeds token 0's fragment and folds token 0.
-// TPW: 16-row tiles per consumer warp (an item is 8 * TPW tiles; always 2 today); two tiles share the fragment
-// loads and the per-group bookkeeping.
-template <int NT, bool ONE, int TPW>
-__global__ void __launch_bounds__(kSetThreads, NT >= 3 ? 1 : kSetCtasPerSm) gemv_set_kernel(const __grid_constant__ SetParams p) {
+// Single-token sets.  A consumer warp has two row tiles, which share the fragment loads and the per-group bookkeeping.
+constexpr int kSetTpw = 2;
+__global__ void __launch_bounds__(kSetThreads, kSetCtasPerSm) gemv_set_kernel(const __grid_constant__ SetParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -568,9 +369,8 @@ __global__ void __launch_bounds__(kSetThreads, NT >= 3 ? 1 : kSetCtasPerSm) gemv
     auto empty = [&](int s) { return sbase + 8u * (kSetMaxSlots + s); };
     volatile int* abort = reinterpret_cast<volatile int*>(smem + kSetOffAbort);
     const uint32_t ring = sbase + kSetOffRing;
-    constexpr int TPI = kSetConsumers * TPW;                  // tiles per item
-    constexpr uint32_t kOffZ = slot_off_z(TPI), kOffE = slot_off_e(TPI), kOffX = slot_off_x(TPI, ONE ? 2 : 8 * NT);
-    constexpr uint32_t kOffW = slot_off_w(TPI, ONE ? 2 : 8 * NT);
+    constexpr int TPI = kSetConsumers * kSetTpw;                  // tiles per item
+    constexpr uint32_t kOffZ = slot_off_z(TPI), kOffE = slot_off_e(TPI), kOffW = slot_off_w(TPI, 2);
 
     if (tid == 0) {
         for (int s = 0; s < p.n_slots; ++s) { sb::init(full(s), 1); sb::init(empty(s), kSetConsumers); }
@@ -655,19 +455,20 @@ __global__ void __launch_bounds__(kSetThreads, NT >= 3 ? 1 : kSetCtasPerSm) gemv
             }
         } else {
             // -------------------------------------------------------------- consumer: tile `warp` of every item
-            if constexpr (ONE) consume_one<TPW>(p, sbase, ring, abort, i0, i1, warp, lane);
-            else consume_f16<NT, TPW>(p, sbase, ring, abort, i0, i1, warp, lane);
+            consume_one<kSetTpw>(p, sbase, ring, abort, i0, i1, warp, lane);
         }
     }
     __syncthreads();
     if (tid == 0 && *abort != 0) atomicOr(reinterpret_cast<unsigned int*>(p.ws), 1u);
 }
 
-// ------------------------------------------------------------------------------------------ the persistent kernel, 2 to 16 tokens
-// Measured against the kernel above, whose mma.sync was its bound (us, all bytes from HBM): two 70B blocks at 2 bits, 16 tokens 241 ->
-// 146 (3.4 TB/s); two 13B blocks at 3 bits, 16 tokens 181 -> 76; eight 7B blocks, 2 and 5 tokens at 2 bits 144 / 145 -> 101 / 112, 8
-// tokens at 3 bits 166 -> 137; one 7B block, 4 tokens 36.9 -> 25.  Bound now: issue slots, 2850 / 3350 / 3800 warp instructions a
-// step at 2 / 8 / 16 tokens (ncu), of which decoding takes 950 and the fold up to 1100, next to 780 cycles of HBM time.
+// ------------------------------------------------------------------------------------------ the persistent kernel, 2 to 64 tokens
+// Measured against a kernel on mma.sync m16n8k16 (us, all bytes from HBM): two 70B blocks at 2 bits, 16 and 32 tokens 241 / 391 -> 146 /
+// 209; two 13B blocks at 3 bits, 16 tokens 181 -> 81; eight 7B blocks, 2 and 5 tokens at 2 bits 144 / 145 -> 101 / 112, 8 tokens at 3 bits
+// 166 -> 137; one 7B block, 4 tokens 36.9 -> 25; four 7B blocks, 17 and 40 tokens at 3 bits 181 / 269 -> 104 / 138, 64 at 2 bits 361 -> 174.
+// Bound: issue slots, 2850 / 3350 / 3800 warp instructions a step of 512 rows at 2 / 8 / 16 tokens (ncu), of which decoding takes 950 and
+// the fold up to 1100, next to 780 cycles of HBM time; 256 rows at 40 tokens 3900, most of them the fold's.
+
 // What a step of gemv_set_tc_kernel costs in cycles, for the deal: between its bytes (4 + 10 b per row tile) and its instructions.
 __host__ __device__ constexpr unsigned tc_step_cost(int b, int tiles) { return 400u + static_cast<unsigned>(tiles * (4 + 10 * b)); }
 
@@ -678,31 +479,18 @@ struct SetCut {
 };
 
 // One layer without a plan: the steps of its row blocks, one block after the other, are cut into `grid` shares of equal cost.
+constexpr int kTcMaxGrid = 255;
+struct TcPlace { int rb, p; };    // row block, position in the streaming order
 struct TcSingle {
     SetLayer layer;
     uint8_t* ws;
-    unsigned long long part_off;  // workspace offset of the parts' fp32 sums: two rooms of [M][512] per CTA
-    int n_slots, slot_bytes, off_rec, n_rb, grid;
-    unsigned per_rb;              // cost of a row block
+    unsigned long long part_off;  // workspace offset of the parts' fp32 sums: two rooms of [M][rows] per CTA
+    int n_slots, slot_bytes, off_rec, grid;
+    uint32_t place[kTcMaxGrid + 1];   // where share c begins: row block << 10 | position.  (Worked out by the host: the divisions, in every
+                                      // warp, were half of the instructions of a small layer.)
 };
-struct TcPlace { int rb, p; };    // row block, position in the streaming order
-// Where share c begins.  No part of a single step: such a cut moves to the end of the row block.
-__host__ __device__ inline TcPlace tc_place(const TcSingle& t, int c) {
-    if (c >= t.grid) return TcPlace{t.n_rb, 0};
-    const unsigned long long x = static_cast<unsigned long long>(t.per_rb) * static_cast<unsigned>(t.n_rb) * static_cast<unsigned>(c) / static_cast<unsigned>(t.grid);
-    int rb = static_cast<int>(x / t.per_rb), at = 0;
-    unsigned rem = static_cast<unsigned>(x % t.per_rb);
-    for (int b = 1; b <= 4; ++b) {
-        const unsigned cost = tc_step_cost(b, rawtc::kTiles), has = t.layer.count[b - 1];
-        const unsigned n = rem / cost < has ? rem / cost : has;
-        at += static_cast<int>(n);
-        rem -= n * cost;
-        if (n < has) break;
-    }
-    if (at < 2) at = 0;
-    else if (at > t.layer.G - 2) { at = 0; ++rb; }
-    return TcPlace{rb, at};
-}
+static_assert(SLIM_MAX_GROUPS < 1024 && sizeof(TcSingle) <= 4096, "a place is a word, and the parameters are as many as a kernel takes");
+__device__ __forceinline__ TcPlace tc_place(const TcSingle& t, int c) { return TcPlace{static_cast<int>(t.place[c] >> 10), static_cast<int>(t.place[c] & 1023u)}; }
 
 // A fold warp has stored its sums of a cut row block (64 of the 512 rows) and counts itself, in its four bits of the block's word; the
 // one that counts last adds the S parts in their order, so the result does not depend on which came last, and leaves the bits
@@ -719,33 +507,50 @@ __device__ __forceinline__ void finish_cut(unsigned int* counter, int S, Place p
     if (lane == 0) atomicSub(counter, static_cast<unsigned int>(S) << (4 * fw));
     __threadfence();
     const int h = fw >> 2, q = fw & 3;
-    // pairs of rows: 16 in each of the warp's two tiles; lane = pair of one tile or the other
-    const int row = 128 * (2 * h + (lane >> 4)) + 32 * q + 2 * (lane & 15);
-    if (rawtc::kRows * row_block + row >= N) return;
-    // all tokens of two parts at a time (of four, up to eight tokens): the loads are in flight together
-    float2 sum[MV];
+    // A lane has four rows of each of the warp's tiles and every fourth token: of MB such tokens and U parts it has 16 loads of 16 bytes in
+    // flight, which is what a part costs in time (8 rows' lanes by 4 tokens' lanes).
+    constexpr int kR = rawtc::rows_of(MV), E = kR == 512 ? 2 : 1, MB = MV <= 4 ? 1 : MV <= 8 ? 2 : 4, U = 16 / (E * MB);
+    const int row = 128 * E * h + 32 * q + 4 * (lane & 7);
+    for (int m0 = lane >> 3; m0 < M; m0 += 4 * MB) {
+        float4 sum[E][MB];
 #pragma unroll
-    for (int t = 0; t < MV; ++t) sum[t] = make_float2(0.f, 0.f);
-    constexpr int U = MV <= 8 ? 4 : 2;
-    for (int k0 = 0; k0 < S; k0 += U) {
-        float2 v[U][MV];
+        for (int e = 0; e < E; ++e)
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const float* from = place(min(k0 + u, S - 1)) + row;
+            for (int t = 0; t < MB; ++t) sum[e][t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k0 = 0; k0 < S; k0 += U) {
+            float4 v[U][E][MB];
 #pragma unroll
-            for (int t = 0; t < MV; ++t) v[u][t] = __ldcg(reinterpret_cast<const float2*>(from + (t < M ? t : 0) * rawtc::kRows));
+            for (int u = 0; u < U; ++u) {
+                const float* from = place(min(k0 + u, S - 1)) + row;
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+#pragma unroll
+                    for (int t = 0; t < MB; ++t) v[u][e][t] = __ldcg(reinterpret_cast<const float4*>(from + 128 * e + min(m0 + 4 * t, M - 1) * kR));
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (k0 + u >= S) break;
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+#pragma unroll
+                    for (int t = 0; t < MB; ++t) {
+                        sum[e][t].x += v[u][e][t].x;
+                        sum[e][t].y += v[u][e][t].y;
+                        sum[e][t].z += v[u][e][t].z;
+                        sum[e][t].w += v[u][e][t].w;
+                    }
+            }
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u)
+        for (int e = 0; e < E; ++e)
 #pragma unroll
-            for (int t = 0; t < MV; ++t) {
-                sum[t].x += k0 + u < S ? v[u][t].x : 0.f;
-                sum[t].y += k0 + u < S ? v[u][t].y : 0.f;
+            for (int t = 0; t < MB; ++t) {
+                const int m = m0 + 4 * t, n = kR * row_block + row + 128 * e;
+                if (m >= M || n >= N) continue;                      // (N is a multiple of 16)
+                const __half2 lo = __floats2half2_rn(sum[e][t].x, sum[e][t].y), hi = __floats2half2_rn(sum[e][t].z, sum[e][t].w);
+                *reinterpret_cast<uint2*>(y + static_cast<size_t>(m) * N + n) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
             }
     }
-#pragma unroll
-    for (int t = 0; t < MV; ++t)
-        if (t < M) *reinterpret_cast<__half2*>(y + static_cast<size_t>(t) * N + rawtc::kRows * row_block + row) = __floats2half2_rn(sum[t].x, sum[t].y);
 }
 
 // MV: form of the set.  kSet: items from a plan, records from the workspace.  kLocal, kStaged: one layer; its CTAs stage the groups
@@ -756,7 +561,10 @@ __device__ __forceinline__ uint32_t p_off_rec(const SetParams&) { return 0u; }
 template <int MV, int MODE, class Params>
 __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const __grid_constant__ Params p) {
     using namespace rawtc;
-    constexpr uint32_t kOffW = MODE == kLocal ? (kOffE + 127) / 128 * 128 : off_w(MV);
+    constexpr int kRows = rows_of(MV), kTiles = row_tiles_of(MV);
+    constexpr bool kMany = MV > 16;
+    constexpr int kPer = kMany ? 1 : 2;                                  // MMA tiles of a half h of the rows
+    constexpr uint32_t kOffZ = off_z(MV), kOffE = off_e(MV), kOffW = off_w(MV, MODE != kLocal);
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = static_cast<int>(tc::uniform(tid >> 5));
@@ -905,18 +713,18 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
     } else if (warp < kDecode) {
         // ------------------------------------------------------------------ decode: 32 rows of two tiles, every other step
         // The steps of an item come sorted by bit-width, so each width has a loop of its own.
-        set_registers<kRegDecode>();
+        set_registers<reg_decode(MV)>();
         const int q = warp & 3, h = (warp >> 2) & 1;
         const uint32_t set = static_cast<uint32_t>(warp >> 3);
         const uint32_t a_t = tmem + (static_cast<uint32_t>(32 * q) << 16) + kColA + 128 * h + 64 * set;
-        const int tile0 = 16 * h + 2 * q;                            // my first 16-row tile; those of the other tile are eight on
+        const int tile0 = 8 * kPer * h + 2 * q;                      // my first 16-row tile; those of the other tile are eight on
         const uint32_t w_t = ring + kOffW + 8u * lane;
         if (set != 0u) { if (++s == n_slots) { s = 0; ph ^= 1u; } }
         uint32_t ready = test(full(s), ph);
         for (int i = i0; i < i1 && ok; ++i) {
             const int p0 = it.w & 0xffff, p1 = it.w >> 16;
             const uint2 counts = *reinterpret_cast<const uint2*>(layer_of(it.x)->count);
-            const bool two = tiles_of(it) > tile0 + 8;               // tiles past the end: nothing, or stale bytes that nobody looks at
+            const bool two = !kMany && tiles_of(it) > tile0 + 8;     // tiles past the end: nothing, or stale bytes that nobody looks at
             it = item(i + 1);
             auto run = [&](auto btag, int n) {
                 constexpr int B = decltype(btag)::value;
@@ -967,11 +775,11 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
         }
     } else if (warp < kFirstMma) {
         // ------------------------------------------------------------------ fold: a row of each of two tiles
-        set_registers<kRegFold>();
+        set_registers<reg_fold(MV)>();
         pdl_wait();                                                  // x, y and the workspace belong to the kernels ahead until here
         const int fw = warp - kFirstFold, q = fw & 3, h = fw >> 2;
         const int i16 = lane & 15, r16 = i16 < 8 ? 2 * i16 : 2 * i16 - 15;
-        const uint32_t row2 = 2u * static_cast<uint32_t>(256 * h + 32 * q + (lane & 16) + r16);      // of the block's 512, as bytes
+        const uint32_t row2 = 2u * static_cast<uint32_t>(128 * kPer * h + 32 * q + (lane & 16) + r16);      // of the block, as bytes
         const uint32_t d_t = tmem + (static_cast<uint32_t>(32 * q) << 16) + 128 * h;
         constexpr int P2 = MV / 2, P = MV;
         uint32_t ready = test(full(0), 0u);
@@ -995,17 +803,17 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
             const unsigned long long yword = (static_cast<unsigned long long>(static_cast<uint32_t>(it_b.y)) << 32) | static_cast<uint32_t>(it_b.x);
             it = item(i + 1);
             it_b = item_b(i + 1);
-            f2 acc[2][P2];
+            f2 acc[kPer][P2];
 #pragma unroll
-            for (int e = 0; e < 2; ++e)
+            for (int e = 0; e < kPer; ++e)
 #pragma unroll
                 for (int k = 0; k < P2; ++k) acc[e][k] = 0ull;
             for (int k = 0; k < n; ++k) {
                 if (!warp_wait_after(ready, full(s), ph, abort)) { ok = false; break; }
                 const uint32_t slot = ring + static_cast<uint32_t>(s) * slot_bytes;
-                f2 s2[2], z2[2];
+                f2 s2[kPer], z2[kPer];
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {                        // of rows past the end: stale bytes, not used
+                for (int e = 0; e < kPer; ++e) {                        // of rows past the end: stale bytes, not used
                     uint16_t sh, zh;
                     asm volatile("ld.shared.u16 %0, [%1];" : "=h"(sh) : "r"(slot + kOffS + 256 * e + row2));
                     asm volatile("ld.shared.u16 %0, [%1];" : "=h"(zh) : "r"(slot + kOffZ + 256 * e + row2));
@@ -1015,38 +823,61 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
                 }
                 if (!warp_wait(d_full(h, sp), php, abort)) { ok = false; break; }
                 tc::fence_after();
-                // all columns of a tile; both tiles at once where the registers allow it
-                constexpr int C = MV <= 2 ? 8 : MV <= 4 ? 16 : 32;
-                constexpr bool kBoth = MV <= 8;
-                uint32_t v[2][C];
-                ld_cols<C>(d_t + 64 * sp, v[0]);
-                if (kBoth) ld_cols<C>(d_t + 64 * sp + 32, v[1]);
-                // acc += s (D 2^(9-S) - z sum_x): two tokens at a time, the pieces smallest first
-                auto add = [&](int e) {
-#pragma unroll
-                    for (int k2 = 0; k2 < P2; ++k2) {
-                        f2 sx, sc;
-                        lds_sums((MODE == kLocal ? rec_l : slot + kOffE) + 16u * k2, sx, sc);
-                        const uint32_t* o = v[e] + 2 * k2;
-                        f2 dd = pack(f_of(o[P]), f_of(o[P + 1]));
-                        if (kBoth) dd = add2(pack(f_of(o[2 * P % C]), f_of(o[(2 * P + 1) % C])), dd);
-                        dd = mul2(add2(dd, pack(f_of(o[0]), f_of(o[1]))), sc);
-                        acc[e][k2] = fma2(s2[e], fma2(z2[e], sx, dd), acc[e][k2]);
-                    }
+                // acc += s (D 2^(9-S) - z sum_x) of two tokens
+                auto fold = [&](int e, int k2, f2 dd) {
+                    f2 sx, sc;
+                    lds_sums((MODE == kLocal ? rec_l : slot + kOffE) + 16u * k2, sx, sc);
+                    acc[e][k2] = fma2(s2[e], fma2(z2[e], sx, mul2(dd, sc)), acc[e][k2]);
                 };
-                tc::wait_ld();
-                arrived(v[0]);
-                if (!kBoth) {
-                    ld_cols<C>(d_t + 64 * sp + 32, v[1]);
-                    add(0);
+                if constexpr (!kMany) {
+                    // all columns of a tile; both tiles at once where the registers allow it
+                    constexpr int C = MV <= 2 ? 8 : MV <= 4 ? 16 : 32;
+                    constexpr bool kBoth = MV <= 8;
+                    uint32_t v[2][C];
+                    ld_cols<C>(d_t + 64 * sp, v[0]);
+                    if (kBoth) ld_cols<C>(d_t + 64 * sp + 32, v[1]);
+                    auto add = [&](int e) {                          // the pieces smallest first
+#pragma unroll
+                        for (int k2 = 0; k2 < P2; ++k2) {
+                            const uint32_t* o = v[e] + 2 * k2;
+                            f2 dd = pack(f_of(o[P]), f_of(o[P + 1]));
+                            if (kBoth) dd = add2(pack(f_of(o[2 * P % C]), f_of(o[(2 * P + 1) % C])), dd);
+                            fold(e, k2, add2(dd, pack(f_of(o[0]), f_of(o[1]))));
+                        }
+                    };
                     tc::wait_ld();
+                    arrived(v[0]);
+                    if (!kBoth) {
+                        ld_cols<C>(d_t + 64 * sp + 32, v[1]);
+                        add(0);
+                        tc::wait_ld();
+                    }
+                    arrived(v[1]);
+                    tc::fence_before();
+                    __syncwarp();
+                    if (lane == 0) sb::arrive(d_empty(h, sp));
+                    if (kBoth) add(0);
+                    add(1);
+                } else {
+                    // 16 columns at a time, the next ones in flight
+                    constexpr int NC = (MV + 15) / 16;
+                    uint32_t v[2][16];
+                    ld_cols<16>(d_t + 64 * sp, v[0]);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        tc::wait_ld();
+                        arrived(v[c & 1]);
+                        if (c + 1 < NC) ld_cols<16>(d_t + 64 * sp + 16 * (c + 1), v[(c + 1) & 1]);
+                        else {
+                            tc::fence_before();
+                            __syncwarp();
+                            if (lane == 0) sb::arrive(d_empty(h, sp));
+                        }
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (8 * c + i < P2) fold(0, 8 * c + i, pack(f_of(v[c & 1][2 * i]), f_of(v[c & 1][2 * i + 1])));
+                    }
                 }
-                arrived(v[1]);
-                tc::fence_before();
-                __syncwarp();
-                if (lane == 0) sb::arrive(d_empty(h, sp));
-                if (kBoth) add(0);
-                add(1);
                 __syncwarp();
                 if (lane == 0) sb::arrive(empty(s));
                 rec_l += record_bytes(MV);
@@ -1060,8 +891,8 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
             // even token of a pair and the second those of the odd one
             const bool odd = (lane & 8) != 0;
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int row = 128 * (2 * h + e) + 32 * q + (lane & 16) + 2 * (lane & 7);      // of the block
+            for (int e = 0; e < kPer; ++e) {
+                const int row = 128 * (kPer * h + e) + 32 * q + (lane & 16) + 2 * (lane & 7);      // of the block
                 const bool exists = kRows * rb + row < N;
 #pragma unroll
                 for (int k = 0; k < P2; ++k) {
@@ -1084,7 +915,7 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
                     // The CTAs that have a part: those whose shares begin inside the row block, and the one before them.  Lane
                     // 16 + d looks at the share d after this one (a row block has at most kTcMaxParts).
                     const int c_lane = static_cast<int>(blockIdx.x) + lane - 16;
-                    const TcPlace pl = tc_place(p, max(c_lane, 0));
+                    const TcPlace pl = tc_place(p, min(max(c_lane, 0), p.grid));
                     const bool here = c_lane >= 0 && c_lane < p.grid && pl.rb == rb;
                     const uint32_t inside = __ballot_sync(0xffffffffu, here && pl.p > 0), begins = __ballot_sync(0xffffffffu, here);
                     const int below = __clz(~(inside << 15)), above = __ffs(static_cast<int>(~(inside >> 17))) - 1;
@@ -1109,7 +940,7 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
         if constexpr (MODE == kLocal) rec_l += p_off_rec(p);
         for (int i = i0; i < i1 && ok; ++i) {
             const int n = steps_of(it);
-            const bool two = tiles_of(it) > 16 * h + 8;
+            const bool two = !kMany && tiles_of(it) > 16 * h + 8;
             it = item(i + 1);
             for (int k = static_cast<int>(e ^ sp); k < n; k += 2) {
                 ok = warp_wait_after(ready, full(s), ph, abort) && warp_wait_after(free, d_empty(h, e), php ^ 1u, abort) && warp_wait(a_full(h, e), php, abort);
@@ -1123,9 +954,12 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
                         if (t == 1 && !two) break;
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks) mma_f8_ts(d_t + 32 * t, a_t + 32 * t + 8 * ks, b0 + 2u * ks * rows, idesc_f8(mma_n(MV)), ks > 0 ? 1u : 0u);
-                        if (MV > 8)
+                        // the other pieces
 #pragma unroll
-                            for (int ks = 0; ks < 4; ++ks) mma_f8_ts(d_t + 32 * t, a_t + 32 * t + 8 * ks, b0 + 2u * ks * rows + MV, idesc_f8(mma_n(MV)), 1u);
+                        for (int piece = 1; piece < (MV <= 8 ? 1 : kMany ? 3 : 2); ++piece)
+#pragma unroll
+                            for (int ks = 0; ks < 4; ++ks)
+                                mma_f8_ts(d_t + 32 * t, a_t + 32 * t + 8 * ks, b0 + 2u * ks * rows + static_cast<uint32_t>(piece * MV), idesc_f8(mma_n(MV)), 1u);
                     }
                     tc::commit(d_full(h, e));
                     tc::commit(a_empty(h, e));
@@ -1214,12 +1048,12 @@ __global__ void __launch_bounds__(32) wait_selftest_kernel(uint8_t* ws, unsigned
 // ------------------------------------------------------------------------------------------ host side
 // What the whole set fixes: token tiles, slot geometry, ring depth, grid, sizes.
 struct SetGeometry {
-    int nt, bmax, mmax, tpw, mpad;     // tpw: tiles per consumer warp; mpad: tokens in the staged layout
+    int nt, bmax, mmax, tpw;           // tpw: an item's 16-row tiles, by eight
     int mres;                          // tokens that the workspace has room for: 2 (digit form), 8, 16, 32 or 64
     int slot_bytes;
     int n_slots, grid, ctas_per_sm;
     int split;                         // parts the groups of every row block are cut into (fewer for layers with few groups)
-    int n_cuts;                        // 2 to 16 tokens: row blocks of several parts
+    int n_cuts;                        // 2 to 64 tokens: row blocks of several parts
     long long n_items, n_tasks;
     int n_counters;                    // arrival counters of the split row blocks: one per (row block, consumer warp)
     size_t cnt_bytes;                  // their room in the workspace, right after the 256-byte header
@@ -1241,7 +1075,7 @@ static size_t layer_ws_bytes(int M, const GroupTable& gt) {
     for (int j = 0; j < gt.G; ++j) slots += gt.bits[j] == 3 ? 1 : 0;
     return align_to(static_cast<size_t>(gt.G) * (M == 2 ? 128 : staged_header_bytes(M)) + static_cast<size_t>(slots) * 256 * M, 128);
 }
-// Sets of 2 to 16 tokens go through gemv_set_tc_kernel.
+// Sets of 2 to 64 tokens go through gemv_set_tc_kernel.
 static bool tc_form(int mmax) { return mmax >= 2 && mmax <= rawtc::kMaxTokens; }
 // Staged activations of a layer, and the staging tasks (token, group) it has.
 static size_t layer_x_bytes(const SetGeometry& sg, int M, const GroupTable& gt) {
@@ -1250,9 +1084,9 @@ static size_t layer_x_bytes(const SetGeometry& sg, int M, const GroupTable& gt) 
     return std::max(align_to(static_cast<size_t>(gt.G) * rawtc::record_bytes(rawtc::form(sg.mmax)), 128), layer_ws_bytes(sg.mres, gt));
 }
 static int layer_tasks(const SetGeometry& sg, int M, int G) {
-    return (tc_form(sg.mmax) ? (M + 3) / 4 * 4 : sg.mpad == 2 ? 1 : sg.mpad) * G;
+    return (tc_form(sg.mmax) ? (M + 3) / 4 * 4 : 1) * G;
 }
-// The items of a set of 2 to 16 tokens.  The steps of all row blocks, one after the other, are cut into shares of equal cost, one
+// The items of a set of 2 to 64 tokens.  The steps of all row blocks, one after the other, are cut into shares of equal cost, one
 // per CTA: where a share ends inside a row block its sums are added up through the workspace (a deal of whole row blocks left the
 // last CTA of a 7B sweep 15 % over the average).  A row block has at most kTcMaxParts of them.  A set of few steps has its
 // row blocks cut into equal parts instead.
@@ -1265,20 +1099,21 @@ struct TcDeal {
 };
 constexpr int kTcMinSteps = 4;               // fewer per CTA: equal parts
 constexpr size_t kTcMaxSmem = 226 * 1024;
-static void tc_deal(const slim_layer* layers, int n_layers, int g, int sms, int uniform_split, TcDeal* out) {
+static void tc_deal(const slim_layer* layers, int n_layers, int g, int mv, int sms, int uniform_split, TcDeal* out) {
     struct Block { int layer, rb, G; };
     std::vector<Block> blocks;
     std::vector<GroupTable> gt(static_cast<size_t>(n_layers));
     std::vector<std::vector<uint8_t> > width(static_cast<size_t>(n_layers));       // of the groups in streaming order
     long long steps = 0;
     unsigned long long total = 0, widest = 0;                                         // cost of all blocks, of the one that costs most
-    auto tiles_of = [&](const Block& B) { return std::min(rawtc::kTiles, (layers[B.layer].N >> 4) - rawtc::kTiles * B.rb); };
+    const int rows = rawtc::rows_of(mv), row_tiles = rows / 16;
+    auto tiles_of = [&](const Block& B) { return std::min(row_tiles, (layers[B.layer].N >> 4) - row_tiles * B.rb); };
     for (int l = 0; l < n_layers; ++l) {
         make_group_table(layers[l].N, layers[l].K, g, layers[l].bits_host, &gt[l]);
         for (int b = 1; b <= 4; ++b)
             for (int j = 0; j < gt[l].G; ++j)
                 if (gt[l].bits[j] == b) width[l].push_back(static_cast<uint8_t>(b));
-        for (int rb = 0; rb * rawtc::kRows < layers[l].N; ++rb) {
+        for (int rb = 0; rb * rows < layers[l].N; ++rb) {
             blocks.push_back(Block{l, rb, gt[l].G});
             steps += gt[l].G;
             unsigned long long cost = 0;
@@ -1304,7 +1139,7 @@ static void tc_deal(const slim_layer* layers, int n_layers, int g, int sms, int 
             if (part == 0) out->cuts.push_back(SetCut{out->part_bytes, parts, 0});
             it.counts = static_cast<int>(out->cuts.size()) - 1;
             it.y = reinterpret_cast<__half*>(out->part_bytes);
-            out->part_bytes += static_cast<size_t>(L.M) * rawtc::kRows * sizeof(float);
+            out->part_bytes += static_cast<size_t>(L.M) * rows * sizeof(float);
             out->split = std::max(out->split, parts);
         }
         out->items.push_back(it);
@@ -1327,8 +1162,8 @@ static void tc_deal(const slim_layer* layers, int n_layers, int g, int sms, int 
     unsigned long long done = 0;
     int c = 0;                               // the CTA that takes the next step
     auto share_end = [&](int cta) { return static_cast<unsigned long long>(static_cast<long double>(total) * (cta + 1) / out->grid); };
-    std::vector<int> ends;
-    std::vector<int> owner;
+    std::vector<int> ends, owner;
+    unsigned long long end = share_end(0);
     for (const Block& B : blocks) {
         // the positions at which a CTA's share ends inside the block
         ends.clear();
@@ -1337,10 +1172,10 @@ static void tc_deal(const slim_layer* layers, int n_layers, int g, int sms, int 
         int p0 = 0;
         for (int q = 0; q < B.G; ++q) {
             done += tc_step_cost(width[B.layer][q], tiles);
-            while (c + 1 < out->grid && done >= share_end(c)) {
+            while (c + 1 < out->grid && done >= end) {
                 const int at = q + 1 < edge ? 0 : q + 1 > B.G - edge ? B.G : q + 1;
                 if (at > p0) { ends.push_back(at); owner.push_back(c); p0 = at; }
-                ++c;
+                end = share_end(++c);
             }
         }
         if (p0 < B.G) { ends.push_back(B.G); owner.push_back(c); }
@@ -1371,19 +1206,14 @@ static int set_sm_count() {
 }
 
 // First pass over the set: validation of the shapes and everything that depends on all layers.
-// `deal`: the items of a set of 2 to 16 tokens, for a caller that writes the plan (may throw); null: the caller makes its own.
+// `deal`: the items of a set of 2 to 64 tokens, for a caller that writes the plan (may throw); null: the caller makes its own.
 static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeometry* sg, TcDeal* deal) {
     if (layers == nullptr || n_layers < 1 || sg == nullptr) return SLIM_ERR_INVALID_ARG;
     memset(sg, 0, sizeof *sg);
     sg->ws_bytes = 256;
     for (int l = 0; l < n_layers; ++l) sg->mmax = sg->mmax > layers[l].M ? sg->mmax : layers[l].M;
     const bool tc = tc_form(sg->mmax);
-    sg->tpw = tc ? rawtc::kTiles / kSetConsumers : 2;
-    // one token: the 8-bit digit form, 512 bytes per slice; else the tokens of the widest layer rounded up to 8: the kernel is
-    // bound by its MMAs, and with 8, 16, 32 or 64 alone 40 tokens paid for 64 (four LLaMA-7B blocks
-    // at 3 bits, 17 / 40 / 56 tokens: 227 / 425 / 428 us -> 181 / 267 / 368; from 17 tokens on one CTA per SM, whose registers
-    // hold the accumulators: two gave 197 at 17)
-    sg->mpad = sg->mmax <= 1 ? 2 : (sg->mmax + 7) / 8 * 8;
+    sg->tpw = tc ? rawtc::row_tiles_of(rawtc::form(sg->mmax)) / kSetConsumers : 2;
     sg->mres = sg->mmax <= 1 ? 2 : (sg->mmax <= 8 ? 8 : (sg->mmax <= 16 ? 16 : (sg->mmax <= 32 ? 32 : 64)));
     const int tpi = kSetConsumers * sg->tpw;          // tiles per item
     for (int l = 0; l < n_layers; ++l) {
@@ -1400,11 +1230,10 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
         sg->ws_bytes += layer_x_bytes(*sg, L.M, gt);
     }
     if (sg->n_items > 0x3fffffff || sg->n_tasks > 0x3fffffff) return SLIM_ERR_UNSUPPORTED;
-    sg->nt = sg->mmax <= 1 ? 1 : sg->mpad / 8;
+    sg->nt = (sg->mmax + 7) / 8;
     // A set with fewer row blocks than persistent CTAs cuts the groups of every row block into parts (items of their
     // own, fp32 partial outputs in the workspace, added in part order by the consumer warp whose part lands last).
-    const bool one_cta = sg->nt >= 3 || tc;                      // per SM
-    const long long want = static_cast<long long>(set_sm_count()) * (one_cta ? 1 : kSetCtasPerSm);
+    const long long want = static_cast<long long>(set_sm_count()) * (tc ? 1 : kSetCtasPerSm);
     sg->split = 1;
     if (sg->n_items < 2 * want) {
         // the number of parts that fills the last wave of CTAs best (the smallest one within 2 % of the best)
@@ -1423,7 +1252,7 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
     }
     if (tc) {
         if (deal != nullptr) {
-            tc_deal(layers, n_layers, g, set_sm_count(), sg->split, deal);
+            tc_deal(layers, n_layers, g, rawtc::form(sg->mmax), set_sm_count(), sg->split, deal);
             sg->n_items = static_cast<long long>(deal->items.size());
             sg->split = deal->split;
             sg->n_cuts = static_cast<int>(deal->cuts.size());
@@ -1451,11 +1280,11 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
         sg->ws_bytes += sg->cnt_bytes;
     }
     sg->slot_bytes = tc ? rawtc::slot_size(rawtc::form(sg->mmax), sg->bmax)
-                        : static_cast<int>(align_to(static_cast<size_t>(slot_off_w(tpi, sg->mpad)) + static_cast<size_t>(tpi) * 256 * sg->bmax, 128));
+                        : static_cast<int>(align_to(static_cast<size_t>(slot_off_w(tpi, 2)) + static_cast<size_t>(tpi) * 256 * sg->bmax, 128));
     // as many CTAs per SM (kSetCtasPerSm at most) as still leaves each a ring of 4 slots
     const size_t per_sm = 224 * 1024;
     size_t budget = 0;
-    for (sg->ctas_per_sm = one_cta ? 1 : kSetCtasPerSm; sg->ctas_per_sm >= 1; --sg->ctas_per_sm) {
+    for (sg->ctas_per_sm = tc ? 1 : kSetCtasPerSm; sg->ctas_per_sm >= 1; --sg->ctas_per_sm) {
         budget = tc ? kTcMaxSmem - kSetOffDesc : per_sm / sg->ctas_per_sm - 1024 - kSetOffRing;   // 1 KB per CTA is reserved by the system
         if (budget / sg->slot_bytes >= 4 || sg->ctas_per_sm == 1) break;
     }
@@ -1472,7 +1301,7 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
 }
 
 // Device-side descriptor of one layer.
-static void fill_descriptor(const slim_layer& L, const GroupTable& gt, int mpad, int task0, size_t x_off, int split, size_t part_off,
+static void fill_descriptor(const slim_layer& L, const GroupTable& gt, int form, int task0, size_t x_off, int split, size_t part_off,
                             int cnt0, SetLayer* out) {
     SetLayer& d = *out;
     memset(&d, 0, sizeof d);
@@ -1482,7 +1311,7 @@ static void fill_descriptor(const slim_layer& L, const GroupTable& gt, int mpad,
     d.zeros = static_cast<const __half*>(L.zeros);
     d.y = static_cast<__half*>(L.y);
     d.M = L.M; d.N = L.N; d.K = L.K; d.G = gt.G;
-    d.MP = mpad;
+    d.MP = form;
     d.task0 = task0;
     d.x_off = x_off;
     d.split = static_cast<uint8_t>(split);
@@ -1504,19 +1333,18 @@ static size_t set_plan_bytes(int n_layers, long long n_items, long long n_cuts =
     return kSetPlanHeader + static_cast<size_t>(n_layers) * sizeof(SetLayer) + static_cast<size_t>(n_items) * sizeof(SetItem) + static_cast<size_t>(n_cuts) * sizeof(SetCut);
 }
 
-template <int NT, bool ONE, int TPW>
 static cudaError_t launch_set(const SetParams& prm, int grid, size_t smem, cudaStream_t stream, bool early) {
     static std::atomic<bool> attr_set[64];    // zero-initialised; set-up is idempotent, so a race repeats it harmlessly
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        e = cudaFuncSetAttribute(gemv_set_kernel<NT, ONE, TPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+        e = cudaFuncSetAttribute(gemv_set_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
     PdlLaunch l(static_cast<unsigned>(grid), kSetThreads, smem, stream, early);
-    return cudaLaunchKernelEx(&l.cfg, gemv_set_kernel<NT, ONE, TPW>, prm);
+    return cudaLaunchKernelEx(&l.cfg, gemv_set_kernel, prm);
 }
 
 }  // namespace slim
@@ -1570,8 +1398,8 @@ static int set_params(const slim_gemv_set_info* info, const void* plan, void* wo
     if (info->n_layers < 1 || info->grid < 1 || info->grid > kSetMaxGrid || info->n_slots < 2 ||
         info->n_slots > kSetMaxSlots || info->slot_bytes < 128 || info->slot_bytes % 128 != 0 ||
         info->token_tiles < 1 || info->token_tiles > 8 ||
-        info->max_tokens < 1 || info->max_tokens > 8 * info->token_tiles || (info->max_tokens > 16 && info->token_tiles < 3) ||
-        info->tiles_per_warp != (tc_form(info->max_tokens) ? rawtc::kTiles / kSetConsumers : 2) ||
+        info->max_tokens < 1 || info->max_tokens > 8 * info->token_tiles ||
+        info->tiles_per_warp != (tc_form(info->max_tokens) ? rawtc::row_tiles_of(rawtc::form(info->max_tokens)) / kSetConsumers : 2) ||
         info->max_bits < 1 || info->max_bits > 4 || info->stage_tasks < 1 || info->split < 1 || info->split > (tc_form(info->max_tokens) ? kTcMaxParts : kSetMaxSplit) ||
         info->n_counters < 0 || info->n_counters > 65535 || info->n_layers > 65535)
         return SLIM_ERR_INVALID_ARG;
@@ -1626,42 +1454,51 @@ static cudaError_t launch_tc_form(int M, const Params& prm, int grid, size_t sme
     using Launch = cudaError_t (*)(const Params&, int, size_t, cudaStream_t, bool);
     static const Launch forms[8] = {launch_tc<2, MODE, Params>, launch_tc<4, MODE, Params>, launch_tc<6, MODE, Params>, launch_tc<8, MODE, Params>,
                                     launch_tc<10, MODE, Params>, launch_tc<12, MODE, Params>, launch_tc<14, MODE, Params>, launch_tc<16, MODE, Params>};
-    return forms[(M - 1) / 2](prm, grid, smem, stream, early);
+    if (M <= 16) return forms[(M - 1) / 2](prm, grid, smem, stream, early);
+    if constexpr (MODE != kLocal) {
+        static const Launch many[6] = {launch_tc<24, MODE, Params>, launch_tc<32, MODE, Params>, launch_tc<40, MODE, Params>,
+                                       launch_tc<48, MODE, Params>, launch_tc<56, MODE, Params>, launch_tc<64, MODE, Params>};
+        return many[(M - 17) / 8](prm, grid, smem, stream, early);
+    }
+    return cudaErrorInvalidValue;
 }
 
-// ------------------------------------------------------------------------------------------ one layer of 2 to 16 tokens
+// ------------------------------------------------------------------------------------------ one layer of 2 to 56 tokens
 constexpr size_t kTcSingleParts = 2048;      // of the workspace: the status word, the flags, whose words count the parts, then the sums
 struct TcSinglePlan {
     int grid, n_rb, n_slots, slot_bytes, off_rec, smem;
     bool local;                              // records in shared memory
     size_t part_off, x_off, total;
 };
-// From 24 MB on up to eight tokens, and from 32 MB on beyond; below, gemv_few, whose clusters exchange their sums through shared memory, is
-// sooner.  us, that kernel / this one: 28672 x 8192 at 2 bits (63 MB) 3 / 8 / 16 tokens 35.8 / 24.8, 37.1 / 29.6, 50.6 / 35.0; 13824 x 5120 at 3
-// bits (27 MB) 2 / 6 / 16 tokens 15.4 / 13.9, 16.2 / 15.8, 21.8 / 21.9; 8192 x 8192 at 2 bits (17 MB) 8 tokens 13.2 / 18.8.
-constexpr size_t kTcSingleMin = 24u << 20, kTcSingleMinMany = 32u << 20;
+// Which layers.  Up to 32 tokens from 24 MB on; below, gemv_few (up to 16 tokens), whose clusters exchange their sums through shared memory,
+// and the batched kernel are sooner.  us, those / this one: 28672 x 8192 at 2 bits (63 MB) 3 / 8 / 16 / 24 tokens 35.8 / 24.8, 37.1 / 29.6,
+// 50.6 / 34.8, 59.5 / 38.6; 13824 x 5120 at 3 bits (27 MB) 2 / 6 / 16 / 20 / 32 tokens 15.4 / 13.3, 16.2 / 15.0, 21.8 / 20.6, 26.5 / 20.7, 26.6 /
+// 25.6; 8192 x 8192 at 2 bits (17 MB) 8 tokens 13.2 / 17.1.  33 to 56 tokens from 48 MB on: 28672 x 8192 at 48 tokens 60.3 / 48.8 (64 tokens
+// 60.3 / 59.0: the batched kernel takes the same time up to 128); 13824 x 5120 at 40 tokens 26.9 / 26.1, 5120 x 13824 28.4 / 29.9.
+constexpr size_t kTcSingleMin = 24u << 20, kTcSingleMinMany = 48u << 20;
+constexpr int kTcSingleTokens = 56;
 static bool tc_single_plan(int M, int N, const GroupTable& gt, TcSinglePlan* pl) {
-    if (!tc_form(M) || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < (M <= 8 ? kTcSingleMin : kTcSingleMinMany)) return false;
-    const int mv = rawtc::form(M);
+    if (!tc_form(M) || M > kTcSingleTokens || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < (M <= 32 ? kTcSingleMin : kTcSingleMinMany)) return false;
+    const int mv = rawtc::form(M), rows = rawtc::rows_of(mv), row_tiles = rows / 16;
     int bmax = 1, bmin = 4;
     unsigned long long per_rb = 0;
     for (int j = 0; j < gt.G; ++j) {
         bmax = std::max<int>(bmax, gt.bits[j]);
         bmin = std::min<int>(bmin, gt.bits[j]);
-        per_rb += tc_step_cost(gt.bits[j], rawtc::kTiles);
+        per_rb += tc_step_cost(gt.bits[j], row_tiles);
     }
-    pl->n_rb = (N + rawtc::kRows - 1) / rawtc::kRows;
+    pl->n_rb = (N + rows - 1) / rows;
     if (pl->n_rb * sizeof(unsigned int) > kWsFlagsBytes) return false;
     const long long steps = static_cast<long long>(pl->n_rb) * gt.G;
     const long long most = std::min<long long>((kTcMaxParts - 1) * static_cast<long long>(pl->n_rb), (steps + 1) / 2);
-    pl->grid = static_cast<int>(std::max(1ll, std::min<long long>(set_sm_count(), most)));
+    pl->grid = static_cast<int>(std::max(1ll, std::min<long long>(std::min(set_sm_count(), kTcMaxGrid), most)));
     // (kTcMaxParts - 1 shares to a row block: kTcMaxParts parts)
     // the most steps of a share: all of the cheapest, and what moves at its ends
-    const int share = static_cast<int>(per_rb * pl->n_rb / pl->grid / tc_step_cost(bmin, rawtc::kTiles)) + 5;
+    const int share = static_cast<int>(per_rb * pl->n_rb / pl->grid / tc_step_cost(bmin, row_tiles)) + 5;
     const size_t budget = kTcMaxSmem - kSetOffDesc, rec = static_cast<size_t>(rawtc::record_bytes(mv)) * share;
-    const int slot_l = rawtc::kTiles * 256 * bmax + (rawtc::kOffE + 127) / 128 * 128, slot_s = rawtc::slot_size(mv, bmax);
+    const int slot_l = rawtc::slot_size(mv, bmax, false), slot_s = rawtc::slot_size(mv, bmax);
     // records in shared memory if that leaves a ring of four slots, or of all steps
-    pl->local = rec < budget && (budget - rec) / slot_l >= static_cast<size_t>(std::min(4, share));
+    pl->local = M <= 16 && rec < budget && (budget - rec) / slot_l >= static_cast<size_t>(std::min(4, share));
     pl->slot_bytes = pl->local ? slot_l : slot_s;
     int slots = static_cast<int>((pl->local ? budget - rec : budget) / pl->slot_bytes);
     slots = rawtc::even_slots(std::min(slots, share + 1));
@@ -1670,7 +1507,7 @@ static bool tc_single_plan(int M, int N, const GroupTable& gt, TcSinglePlan* pl)
     pl->off_rec = static_cast<int>(kSetOffDesc) + slots * pl->slot_bytes;
     pl->smem = pl->off_rec + (pl->local ? static_cast<int>(rec) : 0);
     pl->part_off = kTcSingleParts;
-    pl->x_off = align_to(pl->part_off + static_cast<size_t>(2 * pl->grid) * M * rawtc::kRows * sizeof(float), 256);
+    pl->x_off = align_to(pl->part_off + static_cast<size_t>(2 * pl->grid) * M * rows * sizeof(float), 256);
     pl->total = pl->x_off + (pl->local ? 0 : static_cast<size_t>(gt.G) * rawtc::record_bytes(mv));
     return true;
 }
@@ -1681,10 +1518,7 @@ static int launch_set_for(const slim_gemv_set_info* info, const SetParams& prm, 
         SLIM_CUDA_TRY((launch_tc_form<kSet, SetParams>(info->max_tokens, prm, info->grid, smem, s, early)));
         return SLIM_OK;
     }
-    using Launch = cudaError_t (*)(const SetParams&, int, size_t, cudaStream_t, bool);
-    static const Launch forms[6] = {launch_set<3, false, 2>, launch_set<4, false, 2>, launch_set<5, false, 2>, launch_set<6, false, 2>,
-                                    launch_set<7, false, 2>, launch_set<8, false, 2>};
-    const cudaError_t e = info->max_tokens == 1 ? launch_set<1, true, 2>(prm, info->grid, smem, s, early) : forms[info->token_tiles - 3](prm, info->grid, smem, s, early);
+    const cudaError_t e = launch_set(prm, info->grid, smem, s, early);
     SLIM_CUDA_TRY(e);
     return SLIM_OK;
 }
@@ -1700,7 +1534,7 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
     memset(&L, 0, sizeof L);
     L.x = x; L.packed = packed; L.scales = scales; L.zeros = zeros; L.y = y; L.bits_host = bits_host; L.M = M; L.N = N; L.K = K;
     SetLayer d;
-    fill_descriptor(L, gt, r.sg.mpad, 0, r.x_off, r.sp, r.part_off, r.cnt0, &d);
+    fill_descriptor(L, gt, 2, 0, r.x_off, r.sp, r.part_off, r.cnt0, &d);
     uint8_t* plan = static_cast<uint8_t*>(workspace) + r.plan_off;
     const int n_items = r.n_items, grid = std::min(n_items, r.sg.grid);
     slim_gemv_set_info info;
@@ -1751,8 +1585,27 @@ int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void*
     fill_descriptor(L, gt, -rawtc::form(M), 0, pl.x_off, 1, 0, 0, &t.layer);
     t.ws = static_cast<uint8_t*>(workspace);
     t.part_off = pl.part_off;
-    t.n_slots = pl.n_slots; t.slot_bytes = pl.slot_bytes; t.off_rec = pl.off_rec; t.n_rb = pl.n_rb; t.grid = pl.grid;
-    for (int b = 1; b <= 4; ++b) t.per_rb += t.layer.count[b - 1] * tc_step_cost(b, rawtc::kTiles);
+    t.n_slots = pl.n_slots; t.slot_bytes = pl.slot_bytes; t.off_rec = pl.off_rec; t.grid = pl.grid;
+    // Share c ends at cost total c / grid.  No part of a single step: such a cut moves to the end of the row block.
+    unsigned cost[4], per_rb = 0;
+    for (int b = 0; b < 4; ++b) {
+        cost[b] = tc_step_cost(b + 1, rawtc::row_tiles_of(rawtc::form(M)));
+        per_rb += t.layer.count[b] * cost[b];
+    }
+    const double share = static_cast<double>(per_rb) * pl.n_rb / pl.grid;
+    for (int c = 0; c <= pl.grid; ++c) {
+        int rb = c == pl.grid ? pl.n_rb : static_cast<int>(share * c / per_rb), at = 0;
+        double rem = share * c - static_cast<double>(per_rb) * rb;
+        for (int b = 0; b < 4 && rb < pl.n_rb; ++b) {
+            const int has = t.layer.count[b], n = std::min(static_cast<int>(rem / cost[b]), has);
+            at += n;
+            rem -= static_cast<double>(n) * cost[b];
+            if (n < has) break;
+        }
+        if (at < 2) at = 0;
+        else if (at > gt.G - 2) { at = 0; ++rb; }
+        t.place[c] = static_cast<uint32_t>(rb) << 10 | static_cast<uint32_t>(at);
+    }
     if (pl.local) {
         SLIM_CUDA_TRY((launch_tc_form<kLocal, TcSingle>(M, t, pl.grid, pl.smem, stream, true)));
         return SLIM_OK;
@@ -1873,7 +1726,7 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
             if (E.x == L.x && E.M == L.M && E.K == L.K && memcmp(E.bits_host, L.bits_host, static_cast<size_t>(L.K / g)) == 0) same = e;
         }
         x_off[l] = same >= 0 ? x_off[same] : ws_off;
-        slim::fill_descriptor(L, gt, tc ? -slim::rawtc::form(sg.mmax) : sg.mpad, task, x_off[l], sp, part_off[l], cnt0, &d);
+        slim::fill_descriptor(L, gt, tc ? -slim::rawtc::form(sg.mmax) : 2, task, x_off[l], sp, part_off[l], cnt0, &d);
         ws_off += slim::layer_x_bytes(sg, L.M, gt);
         SLIM_CUDA_TRY(cudaMemcpyAsync(plan_dev + slim::kSetPlanHeader + static_cast<size_t>(l) * sizeof d, &d, sizeof d,
                                       cudaMemcpyHostToDevice, s));
@@ -1995,7 +1848,7 @@ int slim_mpq_gemv_set(const slim_gemv_set_info* info, const void* plan, void* wo
         slim::PdlLaunch l(static_cast<unsigned>((info->stage_tasks + per_block - 1) / per_block), 256, 0, s, early);
         SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, one ? slim::gemv_set_stage_kernel<true> : slim::gemv_set_stage_kernel<false>, prm.layers, prm.ws, info->n_layers, info->stage_tasks, info->n_counters));
     }
-    // The kernel of 2 to 16 tokens asks for its first slices while x is staged; what the staging kernel writes it waits for.
+    // The kernel of 2 to 64 tokens asks for its first slices while x is staged; what the staging kernel writes it waits for.
     return slim::launch_set_for(info, prm, smem, s, early || slim::tc_form(info->max_tokens));
 }
 

@@ -1,4 +1,4 @@
-// The layer-set kernel for 2 to 16 tokens: raw codes on tcgen05 (included by slim_gemv_set.cu, whose plan, items and ring it uses).
+// The layer-set kernel for 2 to 64 tokens: raw codes on tcgen05 (included by slim_gemv_set.cu, whose plan, items and ring it uses).
 //
 // The products are formed from the stored codes, not from dequantised weights: acc += s (2^(9-S) sum_k q_k X_k - z sum_k x_k) per
 // (row, token, group).  Both operands are 8-bit floats, and exact:
@@ -16,7 +16,7 @@
 // tcgen05 with A in tensor memory takes 16 / 21 / 26 cycles per 128 x N x 32 at N = 16 / 32 / 48 (fp16 the same per K = 16), where
 // mma.sync takes 128 to 256 per 128 x 16 x 32.
 //
-// A step is one group of 128 columns of a block of 512 rows, four MMA tiles of 128.  The instructions that the warps issue are what
+// A step is one group of 128 columns of a block of 512 rows, four MMA tiles of 128 (beyond 16 tokens 256 rows, two).  The instructions that the warps issue are what
 // bounds the kernel next to HBM, so a step is as large as tensor memory allows: the more rows, the fewer copies, waits and
 // reads of the same sums.
 //
@@ -41,24 +41,32 @@ constexpr int kMaxSlots = 32;
 // phases of.  (With an odd one a slot's last step was another warp's, may not have landed yet, and the parity of its barrier
 // reads as if the next one had.)
 __host__ __device__ constexpr int even_slots(int fit) { return fit > kMaxSlots ? kMaxSlots : fit / 2 * 2; }
-constexpr int kMaxTokens = 16;
-constexpr int kRows = 512, kTiles = kRows / 16;
-// Tensor memory: D in columns [0, 256), A in the rest (pair h, step parity, tile of the pair: 32 columns each).
+constexpr int kMaxTokens = 64;
+// Tensor memory: D in columns [0, 256), A in the rest (half h of the rows, step parity: 64 columns each; two tiles of 32, or beyond 16
+// tokens one tile).
 constexpr int kColA = 256;
-// Registers of a thread: 32 warps are launched with 64 each, which the warpgroups share out as 4 x 56, 2 x 104 and 2 x 40.
-constexpr int kRegLaunch = 64, kRegDecode = 56, kRegFold = 104, kRegMisc = 40;
-static_assert(kDecode == 16 && kFold == 8 && kWarps == 32 && 4 * kRegDecode + 2 * kRegFold + 2 * kRegMisc <= 8 * kRegLaunch, "the launch's registers are all there are");
+// Registers of a thread: 32 warps are launched with 64 each, which the warpgroups (four that decode, two that fold, two others) share out.
+constexpr int kRegLaunch = 64, kRegMisc = 40;
+__host__ __device__ constexpr int reg_decode(int mv) { return mv <= 16 ? 56 : 48; }
+__host__ __device__ constexpr int reg_fold(int mv) { return mv <= 16 ? 104 : 120; }
+static_assert(kDecode == 16 && kFold == 8 && kWarps == 32 && 4 * reg_decode(16) + 2 * reg_fold(16) + 2 * kRegMisc <= 8 * kRegLaunch &&
+              4 * reg_decode(64) + 2 * reg_fold(64) + 2 * kRegMisc <= 8 * kRegLaunch, "the launch's registers are all there are");
 template <int R> __device__ __forceinline__ void set_registers() {
     if constexpr (R > kRegLaunch) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R));
     else if constexpr (R < kRegLaunch) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R));
 }
 
-// A set's form: MV tokens, those of its widest layer rounded up to an even number.  The pieces of a token are MV columns of D (rows
-// of B) apart.  Up to 8 tokens one MMA makes the columns of all three, p1 | p2 | p3.  Beyond, B's rows are p1 | p2 / 2 | p3 and two MMAs add up
-// p1 + p2 / 2 | p2 / 2 + p3, from the first and the last two thirds of the rows: D stays at 32 columns a tile, and the fold is spared a
-// third of its loads.  (Both with one shape and one D: only such MMAs are sure to follow each other without a wait between.)
-__host__ __device__ constexpr int form(int mmax) { return (mmax + 1) / 2 * 2; }
-__host__ __device__ constexpr int mma_n(int mv) { return mv <= 8 ? (3 * mv + 15) / 16 * 16 : 32; }
+// A set's form: MV tokens, those of its widest layer rounded up to an even number, beyond 16 to a multiple of 8.  The pieces p1, p2, p3 of
+// a token are MV rows of B apart.
+//   MV <= 8    one MMA per K = 32 makes columns for all three, p1 | p2 | p3 (N = 3 MV), which the fold adds.
+//   MV <= 16   B's rows are p1 | p2 / 2 | p3, and two MMAs add up p1 + p2 / 2 | p2 / 2 + p3, from the first and the last two thirds of the
+//              rows: D stays at 32 columns a tile, and the fold is spared a third of its loads.
+//   beyond     three MMAs of N = MV add up p1 + p2 + p3; blocks of 256 rows, whose accumulators are what the fold warps' registers hold.
+// (The MMAs that add to one D have one shape: only such are sure to follow each other without a wait between.)
+__host__ __device__ constexpr int form(int mmax) { return mmax <= 16 ? (mmax + 1) / 2 * 2 : (mmax + 7) / 8 * 8; }
+__host__ __device__ constexpr int rows_of(int mv) { return mv <= 16 ? 512 : 256; }
+__host__ __device__ constexpr int row_tiles_of(int mv) { return rows_of(mv) / 16; }
+__host__ __device__ constexpr int mma_n(int mv) { return mv <= 8 ? (3 * mv + 15) / 16 * 16 : mv <= 16 ? 32 : (mv + 15) / 16 * 16; }
 // Staged record of a group: (sum_k x of tokens m, m + 1, then their 2^(9-S)) per pair of tokens, then
 // [8 chunks of 16 k'][piece][mv tokens][16 bytes].  Byte 4 c + bb of chunk j belongs to the code that lane column c decodes
 // into byte bb of its j-th register.
@@ -66,9 +74,11 @@ __host__ __device__ constexpr int sums_bytes(int mv) { return 8 * mv; }
 __host__ __device__ constexpr int record_bytes(int mv) { return sums_bytes(mv) + 8 * 3 * 16 * mv; }
 
 // Ring slot: header (bit-width of the group) | scales | zeros | record | slices.
-constexpr int kOffS = 16, kOffZ = kOffS + 2 * kRows, kOffE = kOffZ + 2 * kRows;
-__host__ __device__ constexpr int off_w(int mv) { return (kOffE + record_bytes(mv) + 127) / 128 * 128; }
-__host__ __device__ constexpr int slot_size(int mv, int bmax) { return off_w(mv) + kTiles * 256 * bmax; }
+constexpr int kOffS = 16;
+__host__ __device__ constexpr int off_z(int mv) { return kOffS + 2 * rows_of(mv); }
+__host__ __device__ constexpr int off_e(int mv) { return kOffS + 4 * rows_of(mv); }
+__host__ __device__ constexpr int off_w(int mv, bool record = true) { return (off_e(mv) + (record ? record_bytes(mv) : 0) + 127) / 128 * 128; }
+__host__ __device__ constexpr int slot_size(int mv, int bmax, bool record = true) { return off_w(mv, record) + row_tiles_of(mv) * 256 * bmax; }
 
 // ------------------------------------------------------------------------------------------ waiting
 // A whole warp waits, bounded: its lanes go on, or give up, together.  The try names a time (1 ms) for which the hardware may keep
@@ -163,7 +173,7 @@ __device__ __forceinline__ void stage_tokens(const __half* x, size_t K, int b, i
         e[0] = sum;
         e[2] = __int_as_float((127 + 9 - S) << 23);
     }
-    const float second = mv <= 8 ? 1.f : 0.5f;                        // the second piece is half of what it stands for
+    const float second = mv > 8 && mv <= 16 ? 0.5f : 1.f;             // the second piece is half of what it stands for
     uint8_t* frag = rec + sums_bytes(mv) + 16 * m + 4 * c;
     // four columns a, b, c, d (bytes 0 to 3) of chunk j, times 2^k
     auto put4 = [&](uint8_t* at, int j, float a0, float a1, float a2, float a3, float k) {

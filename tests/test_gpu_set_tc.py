@@ -1,4 +1,4 @@
-"""GPU: the kernel for 2 to 16 tokens on raw codes (tcgen05, 8-bit floats), as a layer set and as one large layer, against the
+"""GPU: the kernel for 2 to 64 tokens on raw codes (tcgen05, 8-bit floats), as a layer set and as one large layer, against the
 oracle or an fp64 product with the dequantised weights."""
 import numpy as np
 import pytest
@@ -34,20 +34,20 @@ def _set(entries):
     return s
 
 
-# every form (tokens rounded up to even) with its last column used and not, and row blocks of one row tile, of one less and one more
+# every form (tokens rounded up to even, beyond 16 to a multiple of 8) with its last column used and not, and row blocks of one row tile, of one less and one more
 # than a row of MMA tiles, and of more than 512 rows
-@pytest.mark.parametrize("M", range(2, 17))
+@pytest.mark.parametrize("M", list(range(2, 17)) + [17, 24, 25, 32, 33, 40, 41, 48, 49, 56, 57, 64])
 def test_every_form_on_ragged_row_blocks(M):
     layers = [oracle_layer(N, K, avg, m, block=i, seed_name="set-tc") for i, (N, K, avg, m) in enumerate(
         [(16, 128, 2, M), (112, 384, 3, max(1, M - 1)), (272, 256, 2, M), (528, 640, 3, 1), (1040, 128, 2, M)])]
     entries = [(_on_device(L), torch.from_numpy(L["x"]).cuda(), torch.full((L["M"], L["N"]), float("nan"), dtype=torch.float16, device="cuda")) for L in layers]
     s = _set(entries)
-    assert s.info["tiles_per_warp"] == 4                              # items of 512 rows
+    assert s.info["tiles_per_warp"] == (4 if M <= 16 else 2)          # items of 512 or 256 rows
     for L, (_, _, y) in zip(layers, entries):
         check_output(y.cpu().numpy(), orc.linear_f64(L["x"], L["codes"], L["scales"], L["zeros"]), f"{L['N']}x{L['K']} M={L['M']} of {M}")
 
 
-@pytest.mark.parametrize("M", [2, 9])
+@pytest.mark.parametrize("M", [2, 9, 17, 33])
 def test_each_bit_of_a_code_meets_its_activation(M):
     """One activation at a time: column k of the weights, exact up to the one rounding of the output."""
     bits = np.array([1, 2, 3, 4], dtype=np.uint8)
@@ -85,7 +85,7 @@ def test_activations_of_any_size_are_taken_exactly():
     assert np.isnan(y[2:]).all()
 
 
-@pytest.mark.parametrize("M,avg", [(2, 2), (7, 3), (8, 3), (16, 2), (16, 3)])
+@pytest.mark.parametrize("M,avg", [(2, 2), (7, 3), (8, 3), (16, 2), (16, 3), (24, 3), (40, 2), (64, 3)])
 def test_shares_that_end_inside_row_blocks_repeat_bit_for_bit(M, avg):
     """A set of more steps than four per CTA: equal shares, sums of cut row blocks added in the order of their parts.  A step read before it
     has landed, or sums added before they are written, would show as a run that differs."""
@@ -105,7 +105,8 @@ def test_shares_that_end_inside_row_blocks_repeat_bit_for_bit(M, avg):
     s.check()
 
 
-@pytest.mark.parametrize("N,K,M,avg", [(14336, 8192, 2, 2), (14336, 8192, 8, 2), (26624, 4096, 5, 2), (16, 128, 2, 2), (28672, 8192, 16, 2), (8192, 28672, 13, 2), (14352, 8192, 9, 3)])
+@pytest.mark.parametrize("N,K,M,avg", [(14336, 8192, 2, 2), (14336, 8192, 8, 2), (26624, 4096, 5, 2), (16, 128, 2, 2), (28672, 8192, 16, 2), (8192, 28672, 13, 2), (14352, 8192, 9, 3),
+                                       (14336, 8192, 18, 2), (8192, 14336, 32, 3), (28672, 8192, 40, 2), (24592, 8192, 56, 2)])
 def test_one_large_layer_in_one_or_two_launches(N, K, M, avg):
     """Records of x in shared memory, or staged by a kernel ahead (many tokens and steps): the layer's own shares, twice into one workspace."""
     layer = _quantised(N, K, avg)
@@ -117,5 +118,5 @@ def test_one_large_layer_in_one_or_two_launches(N, K, M, avg):
         assert torch.equal(layer.forward(x, ws), y)
     assert not ws[256:1280].any()                                     # the words that count the parts are zero again
     slim.workspace_status(ws)
-    small = torch.zeros(256, dtype=torch.uint8, device="cuda")        # no room for parts: the kernels for a few tokens
+    small = torch.zeros(256, dtype=torch.uint8, device="cuda")        # no room for parts: the other kernels
     check_output(layer.forward(x, small).cpu().numpy(), _fp64(layer, x), f"{N}x{K} M={M}, status word alone")
