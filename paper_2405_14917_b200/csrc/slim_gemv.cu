@@ -361,7 +361,7 @@ struct GemvPlan {
     uint16_t kbegin[kMaxCluster + 1];
 };
 
-static int device_sm_count() {
+int device_sm_count() {
     static std::atomic<int> cached[64];       // zero-initialised; set-up is idempotent, so a race repeats it harmlessly
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;

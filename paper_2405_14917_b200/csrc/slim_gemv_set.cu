@@ -1198,13 +1198,6 @@ static unsigned long long item_cost(int tiles_here, const GroupTable& gt, const 
     return w * static_cast<unsigned long long>(tiles_here);
 }
 
-static int set_sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-    return n;
-}
-
 // First pass over the set: validation of the shapes and everything that depends on all layers.
 // `deal`: the items of a set of 2 to 64 tokens, for a caller that writes the plan (may throw); null: the caller makes its own.
 static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeometry* sg, TcDeal* deal) {
@@ -1233,7 +1226,7 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
     sg->nt = (sg->mmax + 7) / 8;
     // A set with fewer row blocks than persistent CTAs cuts the groups of every row block into parts (items of their
     // own, fp32 partial outputs in the workspace, added in part order by the consumer warp whose part lands last).
-    const long long want = static_cast<long long>(set_sm_count()) * (tc ? 1 : kSetCtasPerSm);
+    const long long want = static_cast<long long>(device_sm_count()) * (tc ? 1 : kSetCtasPerSm);
     sg->split = 1;
     if (sg->n_items < 2 * want) {
         // the number of parts that fills the last wave of CTAs best (the smallest one within 2 % of the best)
@@ -1252,7 +1245,7 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
     }
     if (tc) {
         if (deal != nullptr) {
-            tc_deal(layers, n_layers, g, rawtc::form(sg->mmax), set_sm_count(), sg->split, deal);
+            tc_deal(layers, n_layers, g, rawtc::form(sg->mmax), device_sm_count(), sg->split, deal);
             sg->n_items = static_cast<long long>(deal->items.size());
             sg->split = deal->split;
             sg->n_cuts = static_cast<int>(deal->cuts.size());
@@ -1293,7 +1286,7 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
     if (tc) slots = static_cast<size_t>(rawtc::even_slots(static_cast<int>(slots)));
     if (slots < 2) return SLIM_ERR_UNSUPPORTED;
     sg->n_slots = static_cast<int>(slots);
-    long long grid = static_cast<long long>(set_sm_count()) * sg->ctas_per_sm;
+    long long grid = static_cast<long long>(device_sm_count()) * sg->ctas_per_sm;
     if (grid > kSetMaxGrid) grid = kSetMaxGrid;
     if (grid > sg->n_items) grid = sg->n_items;
     sg->grid = tc && deal != nullptr ? deal->grid : static_cast<int>(grid);
@@ -1491,7 +1484,7 @@ static bool tc_single_plan(int M, int N, const GroupTable& gt, TcSinglePlan* pl)
     if (pl->n_rb * sizeof(unsigned int) > kWsFlagsBytes) return false;
     const long long steps = static_cast<long long>(pl->n_rb) * gt.G;
     const long long most = std::min<long long>((kTcMaxParts - 1) * static_cast<long long>(pl->n_rb), (steps + 1) / 2);
-    pl->grid = static_cast<int>(std::max(1ll, std::min<long long>(std::min(set_sm_count(), kTcMaxGrid), most)));
+    pl->grid = static_cast<int>(std::max(1ll, std::min<long long>(std::min(device_sm_count(), kTcMaxGrid), most)));
     // (kTcMaxParts - 1 shares to a row block: kTcMaxParts parts)
     // the most steps of a share: all of the cheapest, and what moves at its ends
     const int share = static_cast<int>(per_rb * pl->n_rb / pl->grid / tc_step_cost(bmin, row_tiles)) + 5;

@@ -124,8 +124,8 @@ __global__ void __launch_bounds__(256) dequant_small_kernel(const uint8_t* __res
 // acc += s * (sum_k q x - z * sum_k x); the warps' sums are added through shared memory in warp order.
 // A group's codes, scales and zero points are requested one group ahead, the first ones before the kernel ahead is done.
 //
-// Measured (us, 4096 x 4096 at 2 bits, tokens 1 / 8 / 16 / 40 / 128): group size 64 5.9 / 5.9 / 9.0 / 21 / 42, 32 8.2 / 8.1 / 10 /
-// 22 / 42.  An FMA per weight and token took 8.4 / 22 / 43 and 9.5 / 29 / 58 for up to 16 tokens, the weights written out as
+// Measured (us, 4096 x 4096 at 2 bits, tokens 1 / 8 / 16 / 40 / 128): group size 64 5.9 / 5.9 / 8.5 / 17.6 / 33, 32 8.0 / 8.0 / 10 /
+// 22 / 43.  An FMA per weight and token took 8.4 / 22 / 43 and 9.5 / 29 / 58 for up to 16 tokens, the weights written out as
 // fp16 and a product that read its fragments from global memory 280 beyond.  One token is a chain of loads of a few
 // bytes per lane; from 32 tokens on the codes are decoded again for every token tile, and x comes from L2 for every 32 rows.
 template <int T>
@@ -196,8 +196,8 @@ __device__ __forceinline__ void small_codes(const SmallRaw<T>& raw, int b, int h
     }
 }
 
-template <int T, int NT, int R, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS) linear_small_kernel(const __half* x, const uint8_t* packed, const __half* scales, const __half* zeros,
+template <int T, int NT, int R, int WARPS, int BLOCKS>
+__global__ void __launch_bounds__(32 * WARPS, BLOCKS) linear_small_kernel(const __half* x, const uint8_t* packed, const __half* scales, const __half* zeros,
                                                                   __half* __restrict__ y, int M, int N, int K, uint32_t one,
                                                                   const __grid_constant__ SmallTable st) {
     constexpr int STEPS = T / 16, F = T / 8;
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(32 * WARPS) linear_small_kernel(const __half* 
     }
 }
 
-template <int T, int NT, int R, int WARPS>
+template <int T, int NT, int R, int WARPS, int BLOCKS>
 static cudaError_t launch_small(const __half* x, const uint8_t* packed, const __half* scales, const __half* zeros, __half* y, int M, int N, int K,
                                 const SmallTable& st, cudaStream_t s) {
     PdlLaunch l(static_cast<unsigned>(((N >> 4) + R - 1) / R), 32 * WARPS, 0, s);
@@ -299,7 +299,7 @@ static cudaError_t launch_small(const __half* x, const uint8_t* packed, const __
     for (int m0 = 0; m0 < M; m0 += kMost) {
         const int m = M - m0 < kMost ? M - m0 : kMost;
         l.cfg.gridDim.y = static_cast<unsigned>((m + 8 * NT - 1) / (8 * NT));
-        const cudaError_t e = cudaLaunchKernelEx(&l.cfg, linear_small_kernel<T, NT, R, WARPS>, x + static_cast<size_t>(m0) * K, packed, scales, zeros,
+        const cudaError_t e = cudaLaunchKernelEx(&l.cfg, linear_small_kernel<T, NT, R, WARPS, BLOCKS>, x + static_cast<size_t>(m0) * K, packed, scales, zeros,
                                                  y + static_cast<size_t>(m0) * N, m, N, K, 0x64006400u, st);
         if (e != cudaSuccess || M - m0 <= kMost) return e;
     }
@@ -307,12 +307,29 @@ static cudaError_t launch_small(const __half* x, const uint8_t* packed, const __
 }
 // 16 rows and 16 warps per block up to 16 tokens (blocks are few and the chain of a warp is what counts), 32 rows and 8 warps
 // for more: the loads of x and the ones MMAs serve two row tiles.
+//
+// BLOCKS is the number of blocks that an SM's registers are to hold.  Where the grid has at most a block per SM the kernel takes the
+// registers it can use, which keeps a group's loads in flight together; a larger grid is held to two, since every load of a warp is waited
+// for by that warp alone and the second block is what runs meanwhile.  Both forms do the same arithmetic.  Measured (us, one / two, columns
+// of a group in brackets): one block per SM or less, 768 x 12288 at 1 token (64) 9.5 / 15.4, 2048 x 8192 at 12 (32) 12.9 / 19.3, 4096 x 4096
+// at 17 (64) 11.1 / 16.8, at 20 (32) 15.4 / 22.4, 1216 x 12416 at 55 (64) 30.9 / 49; more, 4096 x 4096 at 1 token (64) 7.2 / 5.9, at 40
+// 21 / 17.6, at 128 42 / 33, 17344 x 6016 at 128 216 / 174, 4096 x 4096 at 40 (32) 29 / 23.  The compiler's own choice was one of
+// the two whatever the grid: 15.5, 19.2, 11.3, 22.5, 31 and 5.9, 21, 43, 221, 23.  0 leaves the choice to it, 59 registers where it is
+// given for two blocks as well, 23.2 against 24.0 for 11008 x 4096 at 12 (32).
 template <int T>
 static cudaError_t launch_small_for(const __half* x, const uint8_t* packed, const __half* scales, const __half* zeros, __half* y, int M, int N,
                                     int K, const SmallTable& st, cudaStream_t s) {
-    if (M <= 8) return launch_small<T, 1, 1, 16>(x, packed, scales, zeros, y, M, N, K, st, s);
-    if (M <= 16) return launch_small<T, 2, 1, 16>(x, packed, scales, zeros, y, M, N, K, st, s);
-    return launch_small<T, 4, 2, 8>(x, packed, scales, zeros, y, M, N, K, st, s);
+    const long long tiles = N / 16, alone = device_sm_count();
+    if (M <= 8) {
+        if (tiles <= alone) return launch_small<T, 1, 1, 16, 1>(x, packed, scales, zeros, y, M, N, K, st, s);
+        return launch_small<T, 1, 1, 16, 2>(x, packed, scales, zeros, y, M, N, K, st, s);
+    }
+    if (M <= 16) {
+        if (tiles <= alone) return launch_small<T, 2, 1, 16, 1>(x, packed, scales, zeros, y, M, N, K, st, s);
+        return launch_small<T, 2, 1, 16, T == 64 ? 2 : 0>(x, packed, scales, zeros, y, M, N, K, st, s);
+    }
+    if ((tiles + 1) / 2 * ((M + 31) / 32) <= alone) return launch_small<T, 4, 2, 8, 1>(x, packed, scales, zeros, y, M, N, K, st, s);
+    return launch_small<T, 4, 2, 8, 2>(x, packed, scales, zeros, y, M, N, K, st, s);
 }
 
 // ------------------------------------------------------------------------------------------ host side

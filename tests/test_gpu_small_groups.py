@@ -32,6 +32,33 @@ def test_tiles_of_tokens_and_rows(N, K, M, g):
     check_output(y.cpu().numpy(), x.astype(np.float64) @ W.T, f"{N}x{K} M={M} g={g}")
 
 
+@pytest.mark.parametrize("g", [32, 64])
+@pytest.mark.parametrize("N,M", [(16 * 148, 1), (16 * 149, 8), (16 * 148, 9), (16 * 149, 16), (32 * 148, 32), (32 * 148 + 16, 17), (32 * 49 + 16, 70)])
+def test_blocks_that_share_an_sm_and_blocks_that_do_not(N, M, g):
+    """As many blocks as SMs and one more (148 of them; two row tiles per block from 17 tokens on), every width; the first
+    rows by themselves, which take the form for a block per SM, give the same bits."""
+    K = 384
+    rng = np.random.default_rng(N + M + g)
+    bits = rng.permutation(np.resize(np.array([2, 3, 1, 4], np.uint8), K // g))
+    codes = np.concatenate([rng.integers(0, 1 << b, (N, g)) for b in bits], axis=1).astype(np.uint8)
+    scales = rng.uniform(0.01, 0.1, (K // g, N)).astype(np.float16)
+    zeros = rng.uniform(0, 3, (K // g, N)).astype(np.float16)
+    x = rng.normal(0, 1, (M, K)).astype(np.float16)
+    ws = slim.new_workspace(M, N, K, bits, g=g)
+
+    def run(n):
+        packed = slim.pack_weights(torch.from_numpy(codes[:n]).cuda(), bits, g=g)
+        call = slim.mpq_gemv if M <= slim.GEMV_MAX_M else slim.mpq_gemm
+        s, z = (torch.from_numpy(np.ascontiguousarray(t[:, :n])).cuda() for t in (scales, zeros))
+        return call(torch.from_numpy(x).cuda(), packed, bits, s, z, n, ws, g=g)
+
+    y = run(N)
+    slim.workspace_status(ws)
+    W = np.repeat(scales.astype(np.float64), g, axis=0).T * (codes - np.repeat(zeros.astype(np.float64), g, axis=0).T)
+    check_output(y.cpu().numpy(), x.astype(np.float64) @ W.T, f"{N}x{K} M={M} g={g}")
+    assert torch.equal(run(64), y[:, :64])                          # a few rows: one block per SM
+
+
 def test_more_tokens_than_one_launch_takes():
     """65535 blocks of 32 tokens are the second grid dimension's limit; a second launch does the rest."""
     N, K, g, M = 16, 128, 64, 65535 * 32 + 45
