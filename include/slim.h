@@ -90,9 +90,10 @@ int slim_last_cuda_error(void);
 int slim_packed_bytes(int N, int K, int g, const uint8_t* bits_host, size_t* out_bytes);
 
 /* Scratch size for slim_mpq_gemv / slim_mpq_gemm with these shapes on the current device.
- * Always at least 256 (one status word).  slim_mpq_gemv needs no more up to three tokens; from
+ * Always at least 256 (one status word).  slim_mpq_gemv needs no more up to three tokens on most layers; from
  * four tokens on it asks for room to put x into tensor-core fragment order once (a few bytes
- * per element of x) and, given less, lets every thread block do that for itself.  slim_mpq_gemm asks for
+ * per element of x) and, given less, lets every thread block do that for itself.  Large layers (below) ask for room for
+ * the partial sums of their row blocks too.  slim_mpq_gemm asks for
  * flags and fp32 partial tiles (128 KB per SM) when it would split tiles across CTAs (stream-K:
  * shapes whose tile count leaves the last wave of CTAs mostly idle); given a smaller workspace
  * (at least 256 bytes) it falls back to whole tiles per CTA and uses no scratch. */
@@ -136,8 +137,8 @@ int slim_dequant(const void* packed, const uint8_t* bits_host, const void* scale
  * activation).  Streams the packed slices once; HBM-bound.  Results are deterministic for a
  * given (shape, device, workspace size).  x with Inf/NaN gives unspecified y.  `workspace` must be at least
  * 256 bytes (the kernel itself keeps its partial sums in shared memory).
- * A layer whose packed codes take 32 MB or more is run by the kernels of slim_mpq_gemv_set instead (same result
- * within the rounding of the accumulation order; at M = 1 with the fixed-point x described there) when the
+ * A layer whose packed codes take 32 MB or more (24 MB at M > 1) is run by the kernels of slim_mpq_gemv_set instead (same
+ * result within the rounding of the accumulation order; at M = 1 with the fixed-point x described there) when the
  * workspace has the slim_workspace_bytes() that shape asks for; with a smaller workspace it takes the per-layer
  * kernel.  The call reads no host memory after it returns and can be captured in a CUDA graph either way.
  * At M = 1 every route takes x in the 22-bit fixed-point form described at slim_mpq_gemv_set (the per-layer
@@ -147,8 +148,8 @@ int slim_dequant(const void* packed, const uint8_t* bits_host, const void* scale
  * before it waits for the kernel ahead of it on the stream: those three buffers must be complete when the call is
  * enqueued, or be written by a call of this library (each of which ends in a kernel that makes them so); between a kernel of
  * another origin that writes them and the call there has to be one more kernel, launched in plain stream order (x and y
- * may be produced and consumed by the neighbouring kernels as usual).  At M = 1 the two kernels of the 32 MB route are launched
- * the same way, but touch no buffer before they have waited for the kernel ahead of them. */
+ * may be produced and consumed by the neighbouring kernels as usual).  The kernels of layers of 32 MB or
+ * more are launched the same way, but touch no buffer before they have waited for the kernel ahead of them. */
 int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host,
                   const void* scales, const void* zeros, void* y,
                   int M, int N, int K, int g,

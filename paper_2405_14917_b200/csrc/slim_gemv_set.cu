@@ -1,4 +1,4 @@
-// slim_mpq_gemv_set: the decode path (1 <= M <= 16) over a set of independent layers, sm_100a.
+// slim_mpq_gemv_set: the decode path (1 <= M <= 64) over a set of independent layers, sm_100a.
 //
 // A decode-sized layer holds fewer bytes than HBM must keep in flight, so a launch per layer
 // leaves the memory system idle while kernels start, stage x and reduce.  Here the whole set is
@@ -46,10 +46,10 @@ constexpr int kSetProducers = 2;                       // producer warps: they t
 constexpr int kSetThreads = 32 * (kSetConsumers + kSetProducers);
 constexpr int kSetMaxSlots = 32;
 constexpr int kSetCtasPerSm = 2;                       // resident CTAs per SM the plan aims at (single-token sets)
-constexpr int kSetMaxTokens = 64;                      // tokens of a layer in a set: up to eight MMA tiles of 8
+constexpr int kSetMaxTokens = 64;                      // tokens of a layer in a set
 
-// Layout of a ring slot (tpi = 16-row tiles of a work item, mp = 256-byte pieces per slice of the staged
-// activations: 2 for single-token sets, else the 8 or 16 tokens of the set).  Everything but the packed slices has
+// Layout of a ring slot of single-token sets (tpi = 16-row tiles of a work item, mp = 2, the 256-byte pieces per slice of the
+// staged activations; slim_set_tc.cuh has the other).  Everything but the packed slices has
 // a fixed size, so the slices come last and every other offset is a compile-time constant of the kernel:
 //   header (bit-width of the group) | scales | zeros | (sum_k x, scale) per token | activations of two slices | slices
 constexpr int kSlotOffS = 16;
@@ -486,6 +486,7 @@ struct TcSingle {
     uint8_t* ws;
     unsigned long long part_off;  // workspace offset of the parts' fp32 sums: two rooms of [M][rows] per CTA
     int n_slots, slot_bytes, off_rec, grid;
+    int wait;                         // read nothing before the kernel ahead is done
     uint32_t place[kTcMaxGrid + 1];   // where share c begins: row block << 10 | position.  (Worked out by the host: the divisions, in every
                                       // warp, were half of the instructions of a small layer.)
 };
@@ -666,6 +667,7 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
         const int what = warp - kFirstProd;
         const bool is_w = what == 0, is_x = what == 3;
         if (is_x) pdl_wait();
+        if constexpr (MODE == kLocal) { if (p.wait) pdl_wait(); }
         for (int i = i0; i < i1 && ok && !(is_x && MODE == kLocal); ++i) {
             const int rb = it.y, p0 = it.w & 0xffff, p1 = it.w >> 16, tiles = tiles_of(it);
             const SetLayer* D = layer_of(it.x);
@@ -1578,6 +1580,9 @@ int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void*
     fill_descriptor(L, gt, -rawtc::form(M), 0, pl.x_off, 1, 0, 0, &t.layer);
     t.ws = static_cast<uint8_t*>(workspace);
     t.part_off = pl.part_off;
+    // Layers of that size are never read before the kernel ahead of the call is done, and callers may count on it.  The others gain 1.5 %
+    // (13824 x 5120 at 3 bits, 2 / 6 tokens 13.55 -> 13.3 / 15.1 -> 14.9 us).
+    t.wait = static_cast<size_t>(16) * N * gt.prefix[gt.G] >= kRouteMinBytes;
     t.n_slots = pl.n_slots; t.slot_bytes = pl.slot_bytes; t.off_rec = pl.off_rec; t.grid = pl.grid;
     // Share c ends at cost total c / grid.  No part of a single step: such a cut moves to the end of the row block.
     unsigned cost[4], per_rb = 0;

@@ -20,12 +20,12 @@
 // bounds the kernel next to HBM, so a step is as large as tensor memory allows: the more rows, the fewer copies, waits and
 // reads of the same sums.
 //
-// Warps: 0-7   decode: (tensor-memory lane quarter q, pair of tiles h).  Words of two rows per lane (as the packed format has them
-//              for mma.sync) go to tensor memory by tcgen05.st.16x128b, whose registers are laid out like that: lanes 0-7 of
-//              a 16-lane tile hold its even rows, lanes 8-15 its odd ones.
-//        8-15  fold: (q, h), thread = a row of each tile, accumulators in registers.
-//        16-17 MMAs of pair h.
-//        18-21 producers: slices, scales, zeros, staged activations.  Only the last waits for the kernel ahead.
+// Warps: 0-15  decode: (tensor-memory lane quarter q, half of the tiles h), two sets of eight that take the steps in turn.  Words of two
+//              rows per lane (as the packed format has them for mma.sync) go to tensor memory by tcgen05.st.16x128b, whose registers are
+//              laid out like that: lanes 0-7 of a 16-lane tile hold its even rows, lanes 8-15 its odd ones.
+//        16-23 fold: (q, h), thread = a row of each tile, accumulators in registers.
+//        24-27 MMAs of half h, in the steps of one parity.
+//        28-31 producers: slices, scales, zeros, staged activations.  Only the last waits for the kernel ahead.
 #pragma once
 
 #include "slim_tc.cuh"
