@@ -51,16 +51,16 @@ def set_kernel_hash():
 
 NCU_TRAFFIC = {
     # layer-set kernel, 4 blocks of the LLaMA-7B sweep (28 layers, avg 2-bit, M = 1): 228,564,480 B read +
-    # 3,502,592 B written per launch (algorithmic 228,297,816 B); scaled to the full sweep by the algorithmic bytes
+    # 3,600,640 B written per launch (algorithmic 228,297,816 B); scaled to the full sweep by the algorithmic bytes
     # (the traffic is the packed data read once, so it grows in proportion)
-    "82c2fd441e13745678a562aa06662cc2261718bfbb70d7ee2d8b9a8aa68e09ed": {"layer": "4 blocks", "traffic_bytes": 232067072, "algorithmic_bytes": 228297816},
+    "580f284d4fd032216d895441e0312e39142ce8dca16b15537e9510101dcf10d9": {"layer": "4 blocks", "traffic_bytes": 232165120, "algorithmic_bytes": 228297816},
 }
 
 
 # DRAM bytes (read + written) of the 14 gemm_kernel launches of one step of llama13b-prefill-avg3-m2048, from one ncu
 # capture of dram__bytes_read.sum and dram__bytes_write.sum; keyed by the SHA-256 of slim_gemm.cu at capture time
 NCU_TRAFFIC_GEMM = {
-    "567d7f396a654d6275e04c0c2c7319232189cdccff0160d2be4348d097ede78a": {"workload": "llama13b-prefill-avg3-m2048", "launches": 14, "traffic_bytes": 1083127040 + 228127232},
+    "5ed5b31a15ced45cc8f92a4f71d8a0a0f299d08fafeb769179802466f4465213": {"workload": "llama13b-prefill-avg3-m2048", "launches": 14, "traffic_bytes": 1039438848 + 214971648},
 }
 
 
@@ -599,9 +599,9 @@ def decode_buffers(layers, M, device, seed):
     return x_host, y_host, x_dev, y_dev, xs, ys
 
 
-def _layer_launches(layer):
-    """Kernels of one slim_mpq_gemv call: layers of 32 MB or more go through the layer-set kernels (staging and ring)."""
-    return 2 if layer.packed.numel() >= 32 << 20 else 1
+def _layer_launches(layer, M):
+    """Kernels of one slim_mpq_gemv call, at least: one-token layers of 32 MB or more go through the layer-set kernels (staging and ring)."""
+    return 2 if M == 1 and layer.packed.numel() >= 32 << 20 else 1
 
 
 def decode_sweep(layers, M, device, launch, seed=1234):
@@ -624,7 +624,7 @@ def decode_sweep(layers, M, device, launch, seed=1234):
         def run():
             for L, x, y in zip(layers, xs, ys):
                 L.forward(x, ws, out=y)
-        checks, n_dom, n_kern = [], len(layers), sum(_layer_launches(L) for L in layers)
+        checks, n_dom, n_kern = [], len(layers), sum(_layer_launches(L, M) for L in layers)
     else:
         assert len(layers) % 7 == 0
         calls, checks, n_kern = [], [], 0
@@ -636,7 +636,7 @@ def decode_sweep(layers, M, device, launch, seed=1234):
             checks += [qkv.check, gu.check]
             calls += [qkv.run, (lambda i=o: layers[i].forward(xs[i], ws, out=ys[i])), gu.run,
                       (lambda i=down: layers[i].forward(xs[i], ws, out=ys[i]))]
-            n_kern += sum(1 if st.info["resident_pairs"] > 0 else 2 for st in (qkv, gu)) + _layer_launches(layers[o]) + _layer_launches(layers[down])
+            n_kern += sum(1 if st.info["resident_pairs"] > 0 else 2 for st in (qkv, gu)) + _layer_launches(layers[o], M) + _layer_launches(layers[down], M)
 
         def run():
             for c in calls:
@@ -672,14 +672,16 @@ def decode_entry(name, layers, spec, device, timer, launch, steps, min_total_s, 
     peak, peak_kind = measured_hbm_peak()
     per_launch_us = 1e3 * ms / n_dom
     achieved = alg_bytes / n_dom / (per_launch_us * 1e-6) / 1e9
-    one = "gemv_one_kernel" if M == 1 else "gemv_kernel"      # slim_mpq_gemv's single-token kernel, or the general one
-    kernel = {"set": "gemv_set_kernel", "per-layer": one, "decoder-order": "gemv_set_kernel + " + one}[launch]
+    one = "gemv_one_kernel" if M == 1 else "gemv_few_kernel"  # slim_mpq_gemv's kernel for most layers of one token, or of a few
+    of_set = "gemv_set_kernel" if M == 1 else "gemv_set_tc_kernel"
+    kernel = {"set": of_set, "per-layer": one, "decoder-order": of_set + " + " + one}[launch]
     integer_form = M == 1
     out = {"name": name, "metric": f"mixed-precision dequant GEMV GB/s at M={M} ({spec['model']} layers, avg {spec['avg_bits']}-bit, g=128)",
            "value": value, "unit": UNIT, "ms_per_step": ms, "timing": tm,
            "dtype": ("s32 (mma.sync m16n8k32 u8 x s8: byte-masked code words against base-256 digits of fixed-point x; f32 fold)"
                      if integer_form and launch == "set" else
                      "s32 (mma.sync m16n8k32 u8 x s8 on byte-masked code words, f32 fold) in every call" if integer_form else
+                     "raw codes as e4m3 against x as three e5m2 parts, both exact (tcgen05 kind::f8f6f4, f32 accumulate and fold)" if launch == "set" else
                      "f16 (mma.sync m16n8k16 on raw code fields, f32 accumulate)"),
            "config": {"workload": name, "layers": len(layers), "M": M, "avg_bits": spec["avg_bits"], "g": wl.GROUP,
                       "algorithmic_bytes_per_step": alg_bytes, "l2": f"distinct layers, {alg_bytes / 1e9:.2f} GB per step > L2",
