@@ -316,15 +316,22 @@ static cudaError_t launch_small(const __half* x, const uint8_t* packed, const __
 // 21 / 17.6, at 128 42 / 33, 17344 x 6016 at 128 216 / 174, 4096 x 4096 at 40 (32) 29 / 23.  The compiler's own choice was one of
 // the two whatever the grid: 15.5, 19.2, 11.3, 22.5, 31 and 5.9, 21, 43, 221, 23.  0 leaves the choice to it, 59 registers where it is
 // given for two blocks as well, 23.2 against 24.0 for 11008 x 4096 at 12 (32).
+//
+// A lone block of up to 16 tokens takes 32 warps where each of 16 would have a long chain of groups.  1216 rows, 16 / 32 warps, 1 and 12
+// tokens: groups of 32, K = 3072 5.7 / 6.2, 5.6 / 6.1; 4096 7.8 / 6.2, 7.0 / 6.2; 8192 14.5 / 8.2, 12.6 / 10.2; groups of 64, K = 8192
+// 6.7 / 6.0, 8.1 / 8.3; 12288 9.2 / 8.1, 11.3 / 11.1.
 template <int T>
 static cudaError_t launch_small_for(const __half* x, const uint8_t* packed, const __half* scales, const __half* zeros, __half* y, int M, int N,
                                     int K, const SmallTable& st, cudaStream_t s) {
     const long long tiles = N / 16, alone = device_sm_count();
+    const bool many = st.G >= (T == 32 ? 128 : 160);
     if (M <= 8) {
+        if (tiles <= alone && many) return launch_small<T, 1, 1, 32, 1>(x, packed, scales, zeros, y, M, N, K, st, s);
         if (tiles <= alone) return launch_small<T, 1, 1, 16, 1>(x, packed, scales, zeros, y, M, N, K, st, s);
         return launch_small<T, 1, 1, 16, 2>(x, packed, scales, zeros, y, M, N, K, st, s);
     }
     if (M <= 16) {
+        if (tiles <= alone && many) return launch_small<T, 2, 1, 32, 1>(x, packed, scales, zeros, y, M, N, K, st, s);
         if (tiles <= alone) return launch_small<T, 2, 1, 16, 1>(x, packed, scales, zeros, y, M, N, K, st, s);
         return launch_small<T, 2, 1, 16, T == 64 ? 2 : 0>(x, packed, scales, zeros, y, M, N, K, st, s);
     }

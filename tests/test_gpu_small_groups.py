@@ -12,10 +12,11 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("g", [32, 64])
-@pytest.mark.parametrize("N,K,M", [(16, 128, 1), (48, 640, 8), (48, 1152, 9), (80, 640, 16), (48, 640, 17), (16, 2048, 33), (112, 384, 70)])
+@pytest.mark.parametrize("N,K,M", [(16, 128, 1), (48, 640, 8), (48, 1152, 9), (80, 640, 16), (48, 640, 17), (16, 2048, 33), (112, 384, 70),
+                                   (48, 3968, 3), (48, 4096, 3), (16, 4224, 12), (32, 10112, 1), (16, 10240, 9)])
 def test_tiles_of_tokens_and_rows(N, K, M, g):
-    """Row tiles that are odd in number, token tiles of 8, 16 and 32 with remainders, more and fewer groups than warps, every
-    width, zero points that are no integers."""
+    """Row tiles that are odd in number, token tiles of 8, 16 and 32 with remainders, more and fewer groups than warps, as many
+    groups as 32 warps are taken from and fewer, every width, zero points that are no integers."""
     rng = np.random.default_rng(N + K + M + g)
     G = K // g
     bits = rng.permutation(np.resize(np.array([2, 3, 1, 4], np.uint8), G))
