@@ -99,17 +99,17 @@ int slim_packed_bytes(int N, int K, int g, const uint8_t* bits_host, size_t* out
  * (at least 256 bytes) it falls back to whole tiles per CTA and uses no scratch. */
 int slim_workspace_bytes(int M, int N, int K, int g, const uint8_t* bits_host, size_t* out_bytes);
 
-/* Zeroes a workspace (status word, stream-K flags).  Must be enqueued once after allocating a
+/* Zeroes a workspace (status word, flags).  Must be enqueued once after allocating a
  * workspace, before its first use; the kernels leave the flags zeroed.  Calls that share a
  * workspace must be ordered on one stream.  slim_mpq_gemv and slim_mpq_gemm may share one of the larger of the two sizes that
  * slim_workspace_bytes reports; the workspace of a layer set is its own. */
 int slim_workspace_init(void* workspace, size_t workspace_bytes, void* stream);
 
 /* Synchronises `stream`, reads and clears the workspace status word.  Returns SLIM_OK, or
- * SLIM_ERR_TIMEOUT if a kernel using this workspace abandoned a bounded wait (its output is
- * then undefined), or SLIM_ERR_CUDA.  A kernel that gave up may have left its flags and partial sums
- * behind: after SLIM_ERR_TIMEOUT pass the workspace through slim_workspace_init before the next call
- * that uses more than its status word (slim_mpq_gemm on a shape it cuts across CTAs). */
+ * SLIM_ERR_TIMEOUT if a kernel using this workspace abandoned a bounded wait (its output, and that of
+ * the calls enqueued on this workspace after it, is then undefined), or SLIM_ERR_CUDA.  A kernel that gave
+ * up may have left flags behind: the call that returns SLIM_ERR_TIMEOUT clears those too, so that the workspace
+ * serves the next call as it is. */
 int slim_workspace_status(void* workspace, void* stream);
 
 /* Self-test of the device-side time-out path.  (No counterpart in the paper: it exercises the status-word

@@ -30,9 +30,16 @@ cudaError_t launch_boundary(cudaStream_t s);
 
 void set_cuda_error(cudaError_t e);
 
-// Start of a linear layer's workspace: the status word (256 bytes), then the flags of slim_mpq_gemm, which have to be zero
-// between its launches.  The other calls put nothing there (or zeros), so that one workspace serves them all in turn.
+// Start of a linear layer's workspace: the header (256 bytes), then the flags by which CTAs that share a tile or a row block find each
+// other (slim_mpq_gemm, and large layers of 2 to 56 tokens), which have to be zero between launches.  The other calls put nothing
+// there (or zeros), so that one workspace serves them all in turn.
 constexpr int kWsFlagsOffset = 256, kWsFlagsBytes = 1024;
+// Header: word 0 is not zero after a wait that gave up, nor is word 1 if that kernel uses the flags and may have left some set;
+// slim_workspace_status clears what they name.
+__device__ __forceinline__ void report_timeout(void* header, bool uses_flags) {
+    atomicOr(static_cast<unsigned int*>(header), 1u);
+    if (uses_flags) atomicOr(static_cast<unsigned int*>(header) + 1, 1u);
+}
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

@@ -933,7 +933,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
     // nobody leaves, and the pair's tensor memory stays, until both CTAs are through
     g::tc_fence_before();
     g::cluster_sync_all();
-    if (tid == 0 && *abort != 0) atomicOr(p.status, 1u);
+    if (tid == 0 && *abort != 0) report_timeout(p.status, p.stream_k != 0);
     if (warp == 1) {
         g::tc_fence_after();
         g::tmem_dealloc(tmem, kTmemCols);

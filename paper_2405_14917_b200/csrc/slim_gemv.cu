@@ -546,12 +546,13 @@ int slim_workspace_init(void* workspace, size_t workspace_bytes, void* stream) {
 
 int slim_workspace_status(void* workspace, void* stream) {
     if (workspace == nullptr) return SLIM_ERR_WORKSPACE;
-    unsigned int word = 0;
+    unsigned int word[2] = {0, 0};                                       // see report_timeout
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    SLIM_CUDA_TRY(cudaMemcpyAsync(&word, workspace, sizeof word, cudaMemcpyDeviceToHost, s));
+    SLIM_CUDA_TRY(cudaMemcpyAsync(word, workspace, sizeof word, cudaMemcpyDeviceToHost, s));
     SLIM_CUDA_TRY(cudaStreamSynchronize(s));
-    if (word != 0) {
+    if (word[0] != 0) {
         SLIM_CUDA_TRY(cudaMemsetAsync(workspace, 0, sizeof word, s));
+        if (word[1] != 0) SLIM_CUDA_TRY(cudaMemsetAsync(static_cast<uint8_t*>(workspace) + slim::kWsFlagsOffset, 0, slim::kWsFlagsBytes, s));
         SLIM_CUDA_TRY(cudaStreamSynchronize(s));
         return SLIM_ERR_TIMEOUT;
     }

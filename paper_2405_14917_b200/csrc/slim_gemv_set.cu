@@ -983,7 +983,7 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
     }
     tc::fence_before();
     __syncthreads();
-    if (tid == 0 && *abort != 0) atomicOr(reinterpret_cast<unsigned int*>(p.ws), 1u);
+    if (tid == 0 && *abort != 0) report_timeout(p.ws, MODE != kSet);          // (a set's counters are cleared by every launch)
     if (warp == kFirstMma) {
         tc::fence_after();
         tc::dealloc(tmem, 512);
