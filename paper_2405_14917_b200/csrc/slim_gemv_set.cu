@@ -703,7 +703,13 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
                         sb::bulk_g2s(slot + dst0, reinterpret_cast<const void*>(src_k), is_x ? xbytes : is_w ? wbytes : szb, full(s));
                     }
                     __syncwarp();
-                    if (++s == n_slots) { s = 0; ph ^= 1u; }
+                    if (++s == n_slots) {
+                        s = 0;
+                        ph ^= 1u;
+                        // The ring is full, and the warps that empty it wait for the kernel ahead, for as long as it takes: so do
+                        // these here, for the limit of the waits on a slot to count this kernel's own work alone.
+                        if constexpr (MODE == kLocal) pdl_wait();
+                    }
                 }
             }
         }

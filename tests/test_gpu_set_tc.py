@@ -120,3 +120,30 @@ def test_one_large_layer_in_one_or_two_launches(N, K, M, avg):
     slim.workspace_status(ws)
     small = torch.zeros(256, dtype=torch.uint8, device="cuda")        # no room for parts: the other kernels
     check_output(layer.forward(x, small).cpu().numpy(), _fp64(layer, x), f"{N}x{K} M={M}, status word alone")
+
+
+def test_a_kernel_ahead_that_outlasts_the_limit_of_the_waits():
+    """A neighbour that lets the next kernel start at once and runs for longer than the two seconds that a wait of this library takes
+    at most: its time is not this kernel's, whose ring is full until then."""
+    hold = torch.cuda._compile_kernel("""extern "C" __global__ void hold(unsigned int us) {
+        asm volatile("griddepcontrol.launch_dependents;");
+        unsigned long long t0, t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+        for (int i = 0; i < 10000000; ++i) {
+            __nanosleep(1000);
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+            if (t - t0 >= 1000ull * us) break;
+        }
+    }""", "hold")
+    N, K, M = 26624, 4096, 5
+    layer = _quantised(N, K, 2)
+    assert 24 << 20 <= layer.packed.numel() < 32 << 20                # one launch that reads its slices ahead
+    x = torch.randn((M, K), device="cuda").half()
+    ws = slim.new_workspace(M, N, K, layer.bits)
+    y = layer.forward(x, ws)
+    out = torch.zeros_like(y)
+    torch.cuda.synchronize()
+    hold(grid=(1, 1, 1), block=(32, 1, 1), args=[2_500_000])
+    layer.forward(x, ws, out)
+    slim.workspace_status(ws)
+    assert torch.equal(out, y)
