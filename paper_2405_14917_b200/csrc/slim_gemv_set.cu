@@ -490,7 +490,9 @@ struct TcSingle {
     uint32_t place[kTcMaxGrid + 1];   // where share c begins: row block << 10 | position.  (Worked out by the host: the divisions, in every
                                       // warp, were half of the instructions of a small layer.)
 };
+constexpr int kTcMaxRowBlocks = 1 << 22;
 static_assert(SLIM_MAX_GROUPS < 1024 && sizeof(TcSingle) <= 4096, "a place is a word, and the parameters are as many as a kernel takes");
+static_assert(kTcMaxGrid * sizeof(unsigned int) <= kWsFlagsBytes, "a word per share counts the parts of the row block that is cut where the share ends");
 __device__ __forceinline__ TcPlace tc_place(const TcSingle& t, int c) { return TcPlace{static_cast<int>(t.place[c] >> 10), static_cast<int>(t.place[c] & 1023u)}; }
 
 // A fold warp has stored its sums of a cut row block (64 of the 512 rows) and counts itself, in its four bits of the block's word; the
@@ -800,7 +802,7 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
                 const bool cut = (i == 0 && from.p > 0) || (rb == to.rb && to.p < p.layer.G);
                 const unsigned long long at = cut ? p.part_off + static_cast<unsigned long long>(2 * blockIdx.x + (i == 0 ? 0 : 1)) * (p.layer.M * kRows * 4)
                                                   : reinterpret_cast<unsigned long long>(p.layer.y);
-                return make_int4(static_cast<int>(at), static_cast<int>(at >> 32), p.layer.M, cut ? rb : -1);
+                return make_int4(static_cast<int>(at), static_cast<int>(at >> 32), p.layer.M, cut ? 0 : -1);
             }
         };
         int4 it_b = item_b(i0);
@@ -927,7 +929,8 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
                     const bool here = c_lane >= 0 && c_lane < p.grid && pl.rb == rb;
                     const uint32_t inside = __ballot_sync(0xffffffffu, here && pl.p > 0), begins = __ballot_sync(0xffffffffu, here);
                     const int below = __clz(~(inside << 15)), above = __ffs(static_cast<int>(~(inside >> 17))) - 1;
-                    finish_cut<MV>(reinterpret_cast<unsigned int*>(p.ws + kWsFlagsOffset) + cut, below + above + 1, [&](int k) {
+                    // the word of a row block: the number of the first share that has a part of it, with which no other cut row block begins
+                    finish_cut<MV>(reinterpret_cast<unsigned int*>(p.ws + kWsFlagsOffset) + (blockIdx.x - below), below + above + 1, [&](int k) {
                         const int d = k - below;                     // that share's first row block, or its last
                         return reinterpret_cast<const float*>(p.ws + p.part_off) +
                                static_cast<size_t>(2 * (static_cast<int>(blockIdx.x) + d) + (1 ^ static_cast<int>((begins >> (16 + d)) & 1u))) * M * kRows;
@@ -1489,7 +1492,7 @@ static bool tc_single_plan(int M, int N, const GroupTable& gt, TcSinglePlan* pl)
         per_rb += tc_step_cost(gt.bits[j], row_tiles);
     }
     pl->n_rb = (N + rows - 1) / rows;
-    if (pl->n_rb * sizeof(unsigned int) > kWsFlagsBytes) return false;
+    if (pl->n_rb >= kTcMaxRowBlocks) return false;
     const long long steps = static_cast<long long>(pl->n_rb) * gt.G;
     const long long most = std::min<long long>((kTcMaxParts - 1) * static_cast<long long>(pl->n_rb), (steps + 1) / 2);
     pl->grid = static_cast<int>(std::max(1ll, std::min<long long>(std::min(device_sm_count(), kTcMaxGrid), most)));

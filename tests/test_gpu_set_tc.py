@@ -147,3 +147,17 @@ def test_a_kernel_ahead_that_outlasts_the_limit_of_the_waits():
     layer.forward(x, ws, out)
     slim.workspace_status(ws)
     assert torch.equal(out, y)
+
+
+@pytest.mark.parametrize("N,K,M,avg", [(131088, 1024, 2, 2), (131088, 1024, 9, 2), (152064, 2048, 16, 2), (65552, 2048, 20, 2), (131088, 2048, 40, 2)])
+def test_one_large_layer_of_more_row_blocks_than_flags(N, K, M, avg):
+    """An output head: the row blocks that are cut count their parts, of which there are fewer than shares."""
+    layer = _quantised(N, K, avg)
+    x = torch.randn((M, K), device="cuda").half()
+    ws = slim.new_workspace(M, N, K, layer.bits)
+    y = layer.forward(x, ws)
+    check_output(y.cpu().numpy(), _fp64(layer, x), f"{N}x{K} M={M}")
+    for _ in range(20):
+        assert torch.equal(layer.forward(x, ws), y)
+    assert not ws[256:1280].any()
+    slim.workspace_status(ws)

@@ -194,3 +194,10 @@ def test_gptq_workspace_and_argument_errors(slim):
     assert L.slim_gptq_quantize(*args(0.01, b - 1)) == -4                 # workspace too small
     assert L.slim_gptq_factor(256, 64, 512, ctypes.c_double(0.01), None, None, 256, b, None) == -1   # no output
 
+
+@pytest.mark.parametrize("N,K,M", [(131072, 1024, 8), (131088, 1024, 8), (152064, 4096, 2), (152064, 4096, 16), (65552, 2048, 20), (152064, 4096, 40)])
+def test_large_layers_of_any_number_of_rows_are_cut_over_the_gpu(slim, N, K, M):
+    """Layers of 24 MB and more (48 MB beyond 32 tokens) ask for room for the sums of the row blocks, of 512 rows or 256, that are cut where one
+    of 148 shares ends; there are more row blocks here than flag words."""
+    rows = 512 if M <= 16 else 256
+    assert slim.workspace_bytes(M, N, K, np.full(K // 128, 2, np.uint8)) > 147 * M * rows * 4
