@@ -1474,13 +1474,28 @@ struct TcSinglePlan {
     bool local;                              // records in shared memory
     size_t part_off, x_off, total;
 };
-// Which layers.  Up to 32 tokens from 24 MB on; below, gemv_few (up to 16 tokens), whose clusters exchange their sums through shared memory,
-// and the batched kernel are sooner.  us, those / this one: 28672 x 8192 at 2 bits (63 MB) 3 / 8 / 16 / 24 tokens 35.8 / 24.8, 37.1 / 29.6,
-// 50.6 / 34.8, 59.5 / 38.6; 13824 x 5120 at 3 bits (27 MB) 2 / 6 / 16 / 20 / 32 tokens 15.4 / 13.3, 16.2 / 15.0, 21.8 / 20.6, 26.5 / 20.7, 26.6 /
-// 25.6; 8192 x 8192 at 2 bits (17 MB) 8 tokens 13.2 / 17.1.  33 to 56 tokens from 48 MB on: 28672 x 8192 at 48 tokens 60.3 / 48.8 (64 tokens
-// 60.3 / 59.0: the batched kernel takes the same time up to 128); 13824 x 5120 at 40 tokens 26.9 / 26.1, 5120 x 13824 28.4 / 29.9.
-constexpr size_t kTcSingleMin = 24u << 20, kTcSingleMinMany = 48u << 20;
+// Which layers: up to 32 tokens from 24 MB on, 33 to 56 from 48 MB on, where this kernel is sooner than those that take the layer
+// otherwise: up to 16 tokens gemv_few, whose clusters exchange their sums through shared memory, then the batched kernel.  us,
+// those / this one (one GPU, in turn):
+//  * size: 8192 x 8192 at 2 bits (16 MB) 2 / 8 / 16 tokens 11.1 / 13.9, 12.5 / 16.7, 16.4 / 22.8; 12288 x 8192 (24.0) 15.9 / 15.5, 17.1 / 17.7, 22.4 /
+//    23.1; 7168 x 14336 (24.5) 17.1 / 16.9, 18.3 / 19.6, 23.8 / 26.6; 5120 x 13824 at 3 bits (25.3) 19.7 / 17.3, 20.9 / 19.9, 27.2 / 27.1; 13312 x
+//    8192 (26.0) 18.1 / 16.2, 19.4 / 18.5, 25.4 / 24.0; 28672 x 8192 (56) 16 tokens 49.1 / 34.7.  20 / 32 tokens: 20480 x 4096 (20) 25.6 / 22.0, 25.6 /
+//    23.1; 13312 x 8192 36.1 / 25.1, 36.2 / 26.6.  40 / 56 tokens: 13824 x 5120 at 3 bits (25.3) 27.8 / 27.3, 27.8 / 32.6; 24576 x 8192 (48) 52.7 / 40.3,
+//    52.8 / 49.5 (64 tokens, 28672 x 8192: 60.3 / 59.0, and the batched kernel takes the same time up to 128).
+//  * row blocks: a layer of few has parts for few CTAs (14 to a row block of 512), or many parts to be added up by one warp.  K = 32768, 4
+//    / 8 / 16 tokens: 2560 rows at 4 bits 19.0 / 20.3, 20.9 / 23.8, 27.9 / 30.8; 3072 at 4 bits 21.9 / 20.6, 23.8 / 24.5, 31.4 / 31.8; 3328 at 2 bits 20.3 /
+//    20.1, 22.3 / 24.5, 29.4 / 37.3; 4096 x 24576 at 4 bits 21.0 / 19.0, 22.8 / 23.1, 33.6 / 29.6.  40 / 56 tokens (row blocks of 256): 4096 x
+//    24576 at 4 bits 36.4 / 37.6, 36.6 / 46.3; 4608 x 28672 at 3 bits 43.9 / 41.2, 44.0 / 50.9; 6144 x 32768 at 2 and 3 bits 53.9 / 45.0, 54.1 / 55.9
+//    and 61.3 / 47.7, 61.4 / 58.3.
+// What gemv_few leaves to the general kernel (few rows, the longest K, 9 tokens or more) this one takes from 24 MB on in any shape: 2304 x 29184
+// at 3 bits, 10 / 16 tokens 41.6 / 35.1, 46.7 / 35.9.
+constexpr size_t kTcSingleMin = 24u << 20, kTcSingleMinMany = 48u << 20, kTcSoonerMin = 25u << 20;
 constexpr int kTcSingleTokens = 56;
+static bool tc_sooner(int M, int N, const GroupTable& gt) {
+    const int rows = rawtc::rows_of(rawtc::form(M)), n_rb = (N + rows - 1) / rows;
+    if (M <= 16) return static_cast<size_t>(16) * N * gt.prefix[gt.G] >= kTcSoonerMin && n_rb >= (M <= 4 ? 6 : 8);
+    return M <= 32 || n_rb >= (M <= 48 ? 18 : 24);
+}
 static bool tc_single_plan(int M, int N, const GroupTable& gt, TcSinglePlan* pl) {
     if (!tc_form(M) || M > kTcSingleTokens || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < (M <= 32 ? kTcSingleMin : kTcSingleMinMany)) return false;
     const int mv = rawtc::form(M), rows = rawtc::rows_of(mv), row_tiles = rows / 16;
@@ -1575,12 +1590,12 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
 size_t gemv_tc_workspace_bytes(int M, int N, const GroupTable& gt) {
     TcSinglePlan pl;
     // a caller who leaves the flags of slim_mpq_gemm out of the size (they were not always in it) gets the same kernel
-    return tc_single_plan(M, N, gt, &pl) ? pl.total + kWsFlagsBytes : 0;
+    return (M <= SLIM_GEMV_MAX_M || tc_sooner(M, N, gt)) && tc_single_plan(M, N, gt, &pl) ? pl.total + kWsFlagsBytes : 0;
 }
 int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y, int M, int N, int K,
-            void* workspace, size_t workspace_bytes, cudaStream_t stream) {
+            void* workspace, size_t workspace_bytes, bool only_if_sooner, cudaStream_t stream) {
     TcSinglePlan pl;
-    if (!tc_single_plan(M, N, gt, &pl) || workspace_bytes < pl.total) return 1;
+    if (!tc_single_plan(M, N, gt, &pl) || workspace_bytes < pl.total || (only_if_sooner && !tc_sooner(M, N, gt))) return 1;
     slim_layer L;
     memset(&L, 0, sizeof L);
     L.x = x; L.packed = packed; L.scales = scales; L.zeros = zeros; L.y = y; L.M = M; L.N = N; L.K = K;

@@ -161,3 +161,35 @@ def test_one_large_layer_of_more_row_blocks_than_flags(N, K, M, avg):
         assert torch.equal(layer.forward(x, ws), y)
     assert not ws[256:1280].any()
     slim.workspace_status(ws)
+
+
+# a megabyte less than the rule's 25, one row block of 512 fewer than its 6 and 8, and of 256 fewer than its 18 and 24
+@pytest.mark.parametrize("N,K,M,avg", [(12288, 8192, 2, 2), (12288, 8192, 16, 2), (2560, 32768, 4, 3), (3584, 32768, 5, 2), (3584, 32768, 16, 2),
+                                       (4352, 32768, 33, 3), (5888, 32768, 49, 3)])
+def test_layers_that_other_kernels_are_sooner_at(N, K, M, avg):
+    """Large layers of few row blocks, or little over 24 MB, take the kernels of a workspace without room for parts: the same bits."""
+    layer = _quantised(N, K, avg)
+    x = torch.randn((M, K), device="cuda").half()
+    size = slim.workspace_bytes(M, N, K, layer.bits)
+    ws = slim.new_workspace(M, N, K, layer.bits)
+    y = layer.forward(x, ws)
+    check_output(y.cpu().numpy(), _fp64(layer, x), f"{N}x{K} M={M}")
+    if M <= 16:
+        assert torch.equal(layer.forward(x, torch.zeros(256, dtype=torch.uint8, device="cuda")), y)
+    else:                                                             # no more than the batched kernel's flags and partial tiles
+        assert size <= 1280 + 148 * 128 * 128 * 4
+    slim.workspace_status(ws)
+
+
+@pytest.mark.parametrize("N,K,M,avg", [(3072, 32768, 4, 3), (4096, 32768, 5, 2), (2304, 29184, 16, 3), (4608, 32768, 48, 3), (6144, 32768, 56, 2)])
+def test_layers_of_few_row_blocks(N, K, M, avg):
+    """The fewest row blocks that the rule for large layers takes, and a layer that is left by the kernel for a few tokens: up to 15 parts to a row block."""
+    layer = _quantised(N, K, avg)
+    x = torch.randn((M, K), device="cuda").half()
+    ws = slim.new_workspace(M, N, K, layer.bits)
+    y = layer.forward(x, ws)
+    check_output(y.cpu().numpy(), _fp64(layer, x), f"{N}x{K} M={M}")
+    for _ in range(20):
+        assert torch.equal(layer.forward(x, ws), y)
+    assert ws[2048:].any() and not ws[256:1280].any()                 # parts were added through the workspace
+    slim.workspace_status(ws)
