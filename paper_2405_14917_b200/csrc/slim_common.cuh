@@ -66,10 +66,10 @@ int gemv_few(const void* x, const void* packed, const GroupTable& gt, const void
              int M, int N, int K, void* workspace, cudaStream_t stream);
 
 // ... and large layers of 2 to 56 tokens, from a workspace of that many bytes on (0: none is enough), to the layer-set kernel on tcgen05
-// without a plan (slim_gemv_set.cu): as above.  only_if_sooner: than gemv_few or slim_mpq_gemm's kernel.
+// without a plan (slim_gemv_set.cu): as above.
 size_t gemv_tc_workspace_bytes(int M, int N, const GroupTable& gt);
 int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y, int M, int N, int K,
-            void* workspace, size_t workspace_bytes, bool only_if_sooner, cudaStream_t stream);
+            void* workspace, size_t workspace_bytes, cudaStream_t stream);
 
 // A set of single-token layers as one resident launch of that kernel (small sets: q/k/v, gate/up).  one_set_plan decides
 // (SLIM_OK: taken, descriptors written into the plan buffer; 1: not taken; negative: error), one_set_launch runs it.

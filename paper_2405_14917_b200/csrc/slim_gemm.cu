@@ -1118,7 +1118,7 @@ extern "C" int slim_mpq_gemm(const void* x, const void* packed, const uint8_t* b
     if (!slim::aligned16(workspace)) return SLIM_ERR_ALIGNMENT;
 
     {
-        const int taken = slim::gemv_tc(x, packed, gt, scales, zeros, y, M, N, K, workspace, workspace_bytes, true, s);
+        const int taken = slim::gemv_tc(x, packed, gt, scales, zeros, y, M, N, K, workspace, workspace_bytes, s);
         if (taken <= 0) return taken;
     }
     // Up to 24 tokens on a layer of 16 to 64 K-tiles and up to 18 MB, and up to 32 on one of up to 5 MB, are sooner through the

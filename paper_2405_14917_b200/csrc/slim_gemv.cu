@@ -593,17 +593,13 @@ int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host, c
         if (taken <= 0) return taken;
     }
     {
-        const int taken = slim::gemv_tc(x, packed, gt, scales, zeros, y, M, N, K, workspace, workspace_bytes, true, s);
+        const int taken = slim::gemv_tc(x, packed, gt, scales, zeros, y, M, N, K, workspace, workspace_bytes, s);
         if (taken <= 0) return taken;
     }
     // More tokens, or one whose layer does not fit that kernel: the layer cut over the whole GPU in one launch.  What that leaves
     // for the kernel of this file (general_is_sooner there): small layers of two or three tokens, and more than 8 on a long K.
     {
         const int taken = slim::gemv_few(x, packed, gt, scales, zeros, y, M, N, K, workspace, s);
-        if (taken <= 0) return taken;
-    }
-    {
-        const int taken = slim::gemv_tc(x, packed, gt, scales, zeros, y, M, N, K, workspace, workspace_bytes, false, s);
         if (taken <= 0) return taken;
     }
     // From kPreStageMinM tokens on, a small kernel puts x into fragment order once, in the

@@ -1485,16 +1485,20 @@ struct TcSinglePlan {
 //  * row blocks: a layer of few has parts for few CTAs (14 to a row block of 512), or many parts to be added up by one warp.  K = 32768, 4
 //    / 8 / 16 tokens: 2560 rows at 4 bits 19.0 / 20.3, 20.9 / 23.8, 27.9 / 30.8; 3072 at 4 bits 21.9 / 20.6, 23.8 / 24.5, 31.4 / 31.8; 3328 at 2 bits 20.3 /
 //    20.1, 22.3 / 24.5, 29.4 / 37.3; 4096 x 24576 at 4 bits 21.0 / 19.0, 22.8 / 23.1, 33.6 / 29.6.  40 / 56 tokens (row blocks of 256): 4096 x
-//    24576 at 4 bits 36.4 / 37.6, 36.6 / 46.3; 4608 x 28672 at 3 bits 43.9 / 41.2, 44.0 / 50.9; 6144 x 32768 at 2 and 3 bits 53.9 / 45.0, 54.1 / 55.9
-//    and 61.3 / 47.7, 61.4 / 58.3.
-// What gemv_few leaves to the general kernel (few rows, the longest K, 9 tokens or more) this one takes from 24 MB on in any shape: 2304 x 29184
-// at 3 bits, 10 / 16 tokens 41.6 / 35.1, 46.7 / 35.9.
+//    24576 at 4 bits 36.4 / 37.6, 36.6 / 46.3; 4608 x 28672 at 3 bits 43.9 / 41.2, 44.0 / 50.9; 5120 x 32768 at 3 bits 59.4 / 44.3, 59.7 / 54.1; 6144 x
+//    32768 at 2 and 3 bits 53.9 / 45.0, 54.1 / 55.9 and 61.3 / 47.7, 61.4 / 58.3.
+//  * K-slices: at 9 tokens and more x in gemv_few's fragments leaves little shared memory where they are many (one per K-tile, two at 3 bits),
+//    whatever the rows.  12 tokens, average 3 bits: 3584 x 24576 (288 slices) 32.9 / 29.1, 2560 x 26624 (312) 32.5 / 30.5, 3072 x 28672 (336) 45.0 /
+//    31.5, 2304 x 29184 (342) 45.0 / 34.8; K = 32768 at 2 or 4 bits (256), 3584 and 1536 rows, 27.6 / 29.0, 23.3 / 28.6.
 constexpr size_t kTcSingleMin = 24u << 20, kTcSingleMinMany = 48u << 20, kTcSoonerMin = 25u << 20;
-constexpr int kTcSingleTokens = 56;
+constexpr int kTcSingleTokens = 56, kTcSlices = 272;
 static bool tc_sooner(int M, int N, const GroupTable& gt) {
     const int rows = rawtc::rows_of(rawtc::form(M)), n_rb = (N + rows - 1) / rows;
-    if (M <= 16) return static_cast<size_t>(16) * N * gt.prefix[gt.G] >= kTcSoonerMin && n_rb >= (M <= 4 ? 6 : 8);
-    return M <= 32 || n_rb >= (M <= 48 ? 18 : 24);
+    if (M > 16) return M <= 32 || n_rb >= (M <= 48 ? 18 : 20);
+    int slices = 0;
+    for (int j = 0; j < gt.G; ++j) slices += slice_count(gt.bits[j]);
+    if (M > 8 && slices > kTcSlices) return true;
+    return (M <= 3 || static_cast<size_t>(16) * N * gt.prefix[gt.G] >= kTcSoonerMin) && n_rb >= (M <= 4 ? 6 : 8);
 }
 static bool tc_single_plan(int M, int N, const GroupTable& gt, TcSinglePlan* pl) {
     if (!tc_form(M) || M > kTcSingleTokens || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < (M <= 32 ? kTcSingleMin : kTcSingleMinMany)) return false;
@@ -1590,12 +1594,12 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
 size_t gemv_tc_workspace_bytes(int M, int N, const GroupTable& gt) {
     TcSinglePlan pl;
     // a caller who leaves the flags of slim_mpq_gemm out of the size (they were not always in it) gets the same kernel
-    return (M <= SLIM_GEMV_MAX_M || tc_sooner(M, N, gt)) && tc_single_plan(M, N, gt, &pl) ? pl.total + kWsFlagsBytes : 0;
+    return tc_single_plan(M, N, gt, &pl) && tc_sooner(M, N, gt) ? pl.total + kWsFlagsBytes : 0;
 }
 int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y, int M, int N, int K,
-            void* workspace, size_t workspace_bytes, bool only_if_sooner, cudaStream_t stream) {
+            void* workspace, size_t workspace_bytes, cudaStream_t stream) {
     TcSinglePlan pl;
-    if (!tc_single_plan(M, N, gt, &pl) || workspace_bytes < pl.total || (only_if_sooner && !tc_sooner(M, N, gt))) return 1;
+    if (!tc_single_plan(M, N, gt, &pl) || workspace_bytes < pl.total || !tc_sooner(M, N, gt)) return 1;
     slim_layer L;
     memset(&L, 0, sizeof L);
     L.x = x; L.packed = packed; L.scales = scales; L.zeros = zeros; L.y = y; L.M = M; L.N = N; L.K = K;

@@ -22,6 +22,14 @@ def _quantised(N, K, avg, seed=0):
     return slim.QuantLinear.from_weight(W, a, avg)
 
 
+def _one_width(N, K, b):
+    gen = torch.Generator(device="cuda").manual_seed(N + K + b)
+    bits = np.full(K // 128, b, np.uint8)
+    packed = torch.randint(0, 256, (slim.packed_bytes(N, K, bits),), dtype=torch.uint8, device="cuda", generator=gen)
+    scales = (torch.rand((K // 128, N), device="cuda", generator=gen) * 0.02 + 0.01).half()
+    return slim.QuantLinear(packed, bits, scales, torch.full_like(scales, (1 << b) // 2), N, K)
+
+
 def _fp64(layer, x):
     What = slim.dequant(layer.packed, layer.bits, layer.scales, layer.zeros, layer.N, layer.K).double()
     return (x.double() @ What.T).cpu().numpy()
@@ -163,12 +171,13 @@ def test_one_large_layer_of_more_row_blocks_than_flags(N, K, M, avg):
     slim.workspace_status(ws)
 
 
-# a megabyte less than the rule's 25, one row block of 512 fewer than its 6 and 8, and of 256 fewer than its 18 and 24
-@pytest.mark.parametrize("N,K,M,avg", [(12288, 8192, 2, 2), (12288, 8192, 16, 2), (2560, 32768, 4, 3), (3584, 32768, 5, 2), (3584, 32768, 16, 2),
-                                       (4352, 32768, 33, 3), (5888, 32768, 49, 3)])
+# a megabyte less than the rule's 25, one row block of 512 fewer than its 6 and 8, and of 256 fewer than its 18 and 20; as many K-slices as leave gemv_few its shared memory
+@pytest.mark.parametrize("N,K,M,avg", [(12288, 8192, 4, 2), (12288, 8192, 16, 2), (2560, 32768, 4, 3), (3584, 32768, 5, 2), (3584, 32768, 16, 0),
+                                       (4352, 32768, 33, 3), (4864, 32768, 49, 3)])
 def test_layers_that_other_kernels_are_sooner_at(N, K, M, avg):
-    """Large layers of few row blocks, or little over 24 MB, take the kernels of a workspace without room for parts: the same bits."""
-    layer = _quantised(N, K, avg)
+    """Large layers of few row blocks, or little over 24 MB, take the kernels of a workspace without room for parts: the same bits.
+    (0: two bits throughout, a K-slice per K-tile.)"""
+    layer = _quantised(N, K, avg) if avg else _one_width(N, K, 2)
     x = torch.randn((M, K), device="cuda").half()
     size = slim.workspace_bytes(M, N, K, layer.bits)
     ws = slim.new_workspace(M, N, K, layer.bits)
@@ -181,9 +190,9 @@ def test_layers_that_other_kernels_are_sooner_at(N, K, M, avg):
     slim.workspace_status(ws)
 
 
-@pytest.mark.parametrize("N,K,M,avg", [(3072, 32768, 4, 3), (4096, 32768, 5, 2), (2304, 29184, 16, 3), (4608, 32768, 48, 3), (6144, 32768, 56, 2)])
+@pytest.mark.parametrize("N,K,M,avg", [(3072, 32768, 4, 3), (4096, 32768, 5, 2), (12288, 8192, 3, 2), (2304, 29184, 9, 3), (4608, 32768, 48, 3), (5120, 32768, 56, 3)])
 def test_layers_of_few_row_blocks(N, K, M, avg):
-    """The fewest row blocks that the rule for large layers takes, and a layer that is left by the kernel for a few tokens: up to 15 parts to a row block."""
+    """The smallest layer and the fewest row blocks that the rule for large layers takes, and fewer of more K-slices: up to 15 parts to a row block."""
     layer = _quantised(N, K, avg)
     x = torch.randn((M, K), device="cuda").half()
     ws = slim.new_workspace(M, N, K, layer.bits)
