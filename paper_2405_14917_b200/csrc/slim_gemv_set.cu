@@ -484,8 +484,9 @@ struct TcPlace { int rb, p; };    // row block, position in the streaming order
 struct TcSingle {
     SetLayer layer;
     uint8_t* ws;
-    unsigned long long part_off;  // workspace offset of the parts' fp32 sums: two rooms of [M][rows] per CTA
+    unsigned long long part_off;  // workspace offset of the parts' fp32 sums: a room of [M][rows] each (tc_room)
     int n_slots, slot_bytes, off_rec, grid;
+    int by_row_block;                 // no more row blocks than shares
     int wait;                         // read nothing before the kernel ahead is done
     uint32_t place[kTcMaxGrid + 1];   // where share c begins: row block << 10 | position.  (Worked out by the host: the divisions, in every
                                       // warp, were half of the instructions of a small layer.)
@@ -493,6 +494,11 @@ struct TcSingle {
 constexpr int kTcMaxRowBlocks = 1 << 22;
 static_assert(SLIM_MAX_GROUPS < 1024 && sizeof(TcSingle) <= 4096, "a place is a word, and the parameters are as many as a kernel takes");
 static_assert(kTcMaxGrid * sizeof(unsigned int) <= kWsFlagsBytes, "a word per share counts the parts of the row block that is cut where the share ends");
+// The room of share c's part of a row block.  A part that begins inside has that of its share's number; there are fewer that begin a row block
+// than row blocks, and than shares.
+__device__ __forceinline__ unsigned int tc_room(const TcSingle& t, int c, int rb, bool inside) {
+    return static_cast<unsigned int>(inside ? c : t.grid + (t.by_row_block ? rb : c));
+}
 __device__ __forceinline__ TcPlace tc_place(const TcSingle& t, int c) { return TcPlace{static_cast<int>(t.place[c] >> 10), static_cast<int>(t.place[c] & 1023u)}; }
 
 // A fold warp has stored its sums of a cut row block (64 of the 512 rows) and counts itself, in its four bits of the block's word; the
@@ -800,7 +806,8 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
             else {
                 const int rb = from.rb + i;
                 const bool cut = (i == 0 && from.p > 0) || (rb == to.rb && to.p < p.layer.G);
-                const unsigned long long at = cut ? p.part_off + static_cast<unsigned long long>(2 * blockIdx.x + (i == 0 ? 0 : 1)) * (p.layer.M * kRows * 4)
+                const unsigned int room = tc_room(p, static_cast<int>(blockIdx.x), rb, i == 0 && from.p > 0);
+                const unsigned long long at = cut ? p.part_off + static_cast<unsigned long long>(room) * (p.layer.M * kRows * 4)
                                                   : reinterpret_cast<unsigned long long>(p.layer.y);
                 return make_int4(static_cast<int>(at), static_cast<int>(at >> 32), p.layer.M, cut ? 0 : -1);
             }
@@ -927,13 +934,11 @@ __global__ void __launch_bounds__(rawtc::kThreads, 1) gemv_set_tc_kernel(const _
                     const int c_lane = static_cast<int>(blockIdx.x) + lane - 16;
                     const TcPlace pl = tc_place(p, min(max(c_lane, 0), p.grid));
                     const bool here = c_lane >= 0 && c_lane < p.grid && pl.rb == rb;
-                    const uint32_t inside = __ballot_sync(0xffffffffu, here && pl.p > 0), begins = __ballot_sync(0xffffffffu, here);
-                    const int below = __clz(~(inside << 15)), above = __ffs(static_cast<int>(~(inside >> 17))) - 1;
+                    const uint32_t inside = __ballot_sync(0xffffffffu, here && pl.p > 0);
+                    const int below = __clz(~(inside << 15)), above = __ffs(static_cast<int>(~(inside >> 17))) - 1, c0 = static_cast<int>(blockIdx.x) - below;
                     // the word of a row block: the number of the first share that has a part of it, with which no other cut row block begins
-                    finish_cut<MV>(reinterpret_cast<unsigned int*>(p.ws + kWsFlagsOffset) + (blockIdx.x - below), below + above + 1, [&](int k) {
-                        const int d = k - below;                     // that share's first row block, or its last
-                        return reinterpret_cast<const float*>(p.ws + p.part_off) +
-                               static_cast<size_t>(2 * (static_cast<int>(blockIdx.x) + d) + (1 ^ static_cast<int>((begins >> (16 + d)) & 1u))) * M * kRows;
+                    finish_cut<MV>(reinterpret_cast<unsigned int*>(p.ws + kWsFlagsOffset) + c0, below + above + 1, [&](int k) {
+                        return reinterpret_cast<const float*>(p.ws + p.part_off) + static_cast<size_t>(tc_room(p, c0 + k, rb, k > 0)) * M * kRows;
                     }, p.layer.y, fw, lane, rb, static_cast<int>(M), N);
                 }
             }
@@ -1473,6 +1478,7 @@ struct TcSinglePlan {
     int grid, n_rb, n_slots, slot_bytes, off_rec, smem;
     bool local;                              // records in shared memory
     size_t part_off, x_off, total;
+    uint32_t place[kTcMaxGrid + 1];
 };
 // Which layers: up to 32 tokens from 24 MB on, 33 to 56 from 48 MB on, where this kernel is sooner than those that take the layer
 // otherwise: up to 16 tokens gemv_few, whose clusters exchange their sums through shared memory, then the batched kernel.  us,
@@ -1500,7 +1506,34 @@ static bool tc_sooner(int M, int N, const GroupTable& gt) {
     if (M > 8 && slices > kTcSlices) return true;
     return (M <= 3 || static_cast<size_t>(16) * N * gt.prefix[gt.G] >= kTcSoonerMin) && n_rb >= (M <= 4 ? 6 : 8);
 }
-static bool tc_single_plan(int M, int N, const GroupTable& gt, TcSinglePlan* pl) {
+// Share c of `grid` ends at cost total c / grid.  No part of a single step: such a cut moves to the end of the row block.
+static void tc_places(const GroupTable& gt, int row_tiles, TcSinglePlan* pl) {
+    const int grid = pl->grid;
+    unsigned cost[4], per_rb = 0;
+    int count[4] = {0, 0, 0, 0};
+    for (int j = 0; j < gt.G; ++j) ++count[gt.bits[j] - 1];
+    for (int b = 0; b < 4; ++b) {
+        cost[b] = tc_step_cost(b + 1, row_tiles);
+        per_rb += static_cast<unsigned>(count[b]) * cost[b];
+    }
+    const double share = static_cast<double>(per_rb) * pl->n_rb / grid;
+    for (int c = 0; c <= grid; ++c) {
+        int rb = c == grid ? pl->n_rb : static_cast<int>(share * c / per_rb), at = 0;
+        double rem = share * c - static_cast<double>(per_rb) * rb;
+        for (int b = 0; b < 4 && rb < pl->n_rb; ++b) {
+            const int n = std::min(static_cast<int>(rem / cost[b]), count[b]);
+            at += n;
+            rem -= static_cast<double>(n) * cost[b];
+            if (n < count[b]) break;
+        }
+        if (at < 2) at = 0;
+        else if (at > gt.G - 2) { at = 0; ++rb; }
+        pl->place[c] = static_cast<uint32_t>(rb) << 10 | static_cast<uint32_t>(at);
+    }
+}
+// In a workspace of that many bytes.  One that is short of a few rooms has fewer shares, down to nine tenths: with fewer than that the kernels that
+// take the layer otherwise are as soon (24576 x 8192 at 16 tokens would take 45 us with 105 shares, 32.6 with 148, 44 there).
+static bool tc_single_plan(int M, int N, const GroupTable& gt, size_t bytes, TcSinglePlan* pl) {
     if (!tc_form(M) || M > kTcSingleTokens || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < (M <= 32 ? kTcSingleMin : kTcSingleMinMany)) return false;
     const int mv = rawtc::form(M), rows = rawtc::rows_of(mv), row_tiles = rows / 16;
     int bmax = 1, bmin = 4;
@@ -1514,25 +1547,32 @@ static bool tc_single_plan(int M, int N, const GroupTable& gt, TcSinglePlan* pl)
     if (pl->n_rb >= kTcMaxRowBlocks) return false;
     const long long steps = static_cast<long long>(pl->n_rb) * gt.G;
     const long long most = std::min<long long>((kTcMaxParts - 1) * static_cast<long long>(pl->n_rb), (steps + 1) / 2);
-    pl->grid = static_cast<int>(std::max(1ll, std::min<long long>(std::min(device_sm_count(), kTcMaxGrid), most)));
+    const int widest = static_cast<int>(std::max(1ll, std::min<long long>(std::min(device_sm_count(), kTcMaxGrid), most)));
     // (kTcMaxParts - 1 shares to a row block: kTcMaxParts parts)
-    // the most steps of a share: all of the cheapest, and what moves at its ends
-    const int share = static_cast<int>(per_rb * pl->n_rb / pl->grid / tc_step_cost(bmin, row_tiles)) + 5;
-    const size_t budget = kTcMaxSmem - kSetOffDesc, rec = static_cast<size_t>(rawtc::record_bytes(mv)) * share;
+    const size_t budget = kTcMaxSmem - kSetOffDesc;
     const int slot_l = rawtc::slot_size(mv, bmax, false), slot_s = rawtc::slot_size(mv, bmax);
-    // records in shared memory if that leaves a ring of four slots, or of all steps
-    pl->local = M <= 16 && rec < budget && (budget - rec) / slot_l >= static_cast<size_t>(std::min(4, share));
-    pl->slot_bytes = pl->local ? slot_l : slot_s;
-    int slots = static_cast<int>((pl->local ? budget - rec : budget) / pl->slot_bytes);
-    slots = rawtc::even_slots(std::min(slots, share + 1));
-    if (slots < 2) return false;
-    pl->n_slots = slots;
-    pl->off_rec = static_cast<int>(kSetOffDesc) + slots * pl->slot_bytes;
-    pl->smem = pl->off_rec + (pl->local ? static_cast<int>(rec) : 0);
     pl->part_off = kTcSingleParts;
-    pl->x_off = align_to(pl->part_off + static_cast<size_t>(2 * pl->grid) * M * rows * sizeof(float), 256);
-    pl->total = pl->x_off + (pl->local ? 0 : static_cast<size_t>(gt.G) * rawtc::record_bytes(mv));
-    return true;
+    for (pl->grid = widest; 10 * pl->grid >= 9 * widest && pl->grid > 0; --pl->grid) {
+        // the most steps of a share: all of the cheapest, and what moves at its ends
+        const int share = static_cast<int>(per_rb * pl->n_rb / pl->grid / tc_step_cost(bmin, row_tiles)) + 5;
+        const size_t rec = static_cast<size_t>(rawtc::record_bytes(mv)) * share;
+        // records in shared memory if that leaves a ring of four slots, or of all steps
+        pl->local = M <= 16 && rec < budget && (budget - rec) / slot_l >= static_cast<size_t>(std::min(4, share));
+        pl->slot_bytes = pl->local ? slot_l : slot_s;
+        int slots = static_cast<int>((pl->local ? budget - rec : budget) / pl->slot_bytes);
+        slots = rawtc::even_slots(std::min(slots, share + 1));
+        if (slots < 2) return false;
+        pl->n_slots = slots;
+        pl->off_rec = static_cast<int>(kSetOffDesc) + slots * pl->slot_bytes;
+        pl->smem = pl->off_rec + (pl->local ? static_cast<int>(rec) : 0);
+        pl->x_off = align_to(pl->part_off + static_cast<size_t>(pl->grid + std::min(pl->grid, pl->n_rb)) * M * rows * sizeof(float), 256);
+        pl->total = pl->x_off + (pl->local ? 0 : static_cast<size_t>(gt.G) * rawtc::record_bytes(mv));
+        if (pl->total <= bytes) {
+            tc_places(gt, row_tiles, pl);
+            return true;
+        }
+    }
+    return false;
 }
 
 // The persistent kernel of the set in the form its token count asks for.
@@ -1594,12 +1634,12 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
 size_t gemv_tc_workspace_bytes(int M, int N, const GroupTable& gt) {
     TcSinglePlan pl;
     // a caller who leaves the flags of slim_mpq_gemm out of the size (they were not always in it) gets the same kernel
-    return tc_single_plan(M, N, gt, &pl) && tc_sooner(M, N, gt) ? pl.total + kWsFlagsBytes : 0;
+    return tc_single_plan(M, N, gt, SIZE_MAX, &pl) && tc_sooner(M, N, gt) ? pl.total + kWsFlagsBytes : 0;
 }
 int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void* scales, const void* zeros, void* y, int M, int N, int K,
             void* workspace, size_t workspace_bytes, cudaStream_t stream) {
     TcSinglePlan pl;
-    if (!tc_single_plan(M, N, gt, &pl) || workspace_bytes < pl.total || !tc_sooner(M, N, gt)) return 1;
+    if (!tc_single_plan(M, N, gt, workspace_bytes, &pl) || !tc_sooner(M, N, gt)) return 1;
     slim_layer L;
     memset(&L, 0, sizeof L);
     L.x = x; L.packed = packed; L.scales = scales; L.zeros = zeros; L.y = y; L.M = M; L.N = N; L.K = K;
@@ -1612,26 +1652,8 @@ int gemv_tc(const void* x, const void* packed, const GroupTable& gt, const void*
     // (13824 x 5120 at 3 bits, 2 / 6 tokens 13.55 -> 13.3 / 15.1 -> 14.9 us).
     t.wait = static_cast<size_t>(16) * N * gt.prefix[gt.G] >= kRouteMinBytes;
     t.n_slots = pl.n_slots; t.slot_bytes = pl.slot_bytes; t.off_rec = pl.off_rec; t.grid = pl.grid;
-    // Share c ends at cost total c / grid.  No part of a single step: such a cut moves to the end of the row block.
-    unsigned cost[4], per_rb = 0;
-    for (int b = 0; b < 4; ++b) {
-        cost[b] = tc_step_cost(b + 1, rawtc::row_tiles_of(rawtc::form(M)));
-        per_rb += t.layer.count[b] * cost[b];
-    }
-    const double share = static_cast<double>(per_rb) * pl.n_rb / pl.grid;
-    for (int c = 0; c <= pl.grid; ++c) {
-        int rb = c == pl.grid ? pl.n_rb : static_cast<int>(share * c / per_rb), at = 0;
-        double rem = share * c - static_cast<double>(per_rb) * rb;
-        for (int b = 0; b < 4 && rb < pl.n_rb; ++b) {
-            const int has = t.layer.count[b], n = std::min(static_cast<int>(rem / cost[b]), has);
-            at += n;
-            rem -= static_cast<double>(n) * cost[b];
-            if (n < has) break;
-        }
-        if (at < 2) at = 0;
-        else if (at > gt.G - 2) { at = 0; ++rb; }
-        t.place[c] = static_cast<uint32_t>(rb) << 10 | static_cast<uint32_t>(at);
-    }
+    memcpy(t.place, pl.place, static_cast<size_t>(pl.grid + 1) * sizeof t.place[0]);
+    t.by_row_block = pl.n_rb <= pl.grid;
     if (pl.local) {
         SLIM_CUDA_TRY((launch_tc_form<kLocal, TcSingle>(M, t, pl.grid, pl.smem, stream, true)));
         return SLIM_OK;

@@ -202,3 +202,21 @@ def test_layers_of_few_row_blocks(N, K, M, avg):
         assert torch.equal(layer.forward(x, ws), y)
     assert ws[2048:].any() and not ws[256:1280].any()                 # parts were added through the workspace
     slim.workspace_status(ws)
+
+
+@pytest.mark.parametrize("N,K,M,avg,share", [(28672, 4096, 6, 2, 0.94), (8192, 14336, 16, 3, 0.92), (65552, 2048, 24, 2, 0.95), (28672, 4096, 6, 2, 0.5), (8192, 24576, 56, 2, 0.93)])
+def test_a_workspace_short_of_a_few_parts(N, K, M, avg, share):
+    """Fewer shares as long as that is a few, the other kernels in a workspace that is much smaller; nothing is written past its end."""
+    layer = _quantised(N, K, avg)
+    x = torch.randn((M, K), device="cuda").half()
+    full = slim.workspace_bytes(M, N, K, layer.bits)
+    buffer = torch.zeros(full, dtype=torch.uint8, device="cuda")
+    size = int(share * (full - 1024)) // 16 * 16                      # (a thousand bytes less than asked for are as good)
+    buffer[size:] = 7
+    ws = buffer[:size]
+    y = layer.forward(x, ws)
+    check_output(y.cpu().numpy(), _fp64(layer, x), f"{N}x{K} M={M} in {share}")
+    for _ in range(20):
+        assert torch.equal(layer.forward(x, ws), y)
+    assert (buffer[size:] == 7).all() and not ws[256:1280].any()
+    slim.workspace_status(ws)

@@ -201,3 +201,14 @@ def test_large_layers_of_any_number_of_rows_are_cut_over_the_gpu(slim, N, K, M):
     of 148 shares ends; there are more row blocks here than flag words."""
     rows = 512 if M <= 16 else 256
     assert slim.workspace_bytes(M, N, K, np.full(K // 128, 2, np.uint8)) > 147 * M * rows * 4
+
+
+@pytest.mark.parametrize("N,K,M,b", [(8192, 28672, 16, 2), (28672, 8192, 16, 2), (24576, 8192, 5, 2), (131072, 1024, 8, 2), (8192, 28672, 56, 2), (5120, 13824, 12, 3)])
+def test_large_layers_ask_for_room_for_their_cut_row_blocks_alone(slim, N, K, M, b):
+    """148 shares: each has room for the part that it begins inside a row block, and each row block, or share, for the one that begins it; beside
+    them the header, the flags, and the staged x of layers whose share of it does not fit beside the ring (384 bytes per token and group, and the sums)."""
+    rows = 512 if M <= 16 else 256
+    mv = (M + 1) // 2 * 2 if M <= 16 else (M + 7) // 8 * 8
+    parts = 148 + min(148, (N + rows - 1) // rows)
+    staged = K // 128 * mv * (3 * 128 + 8)
+    assert slim.workspace_bytes(M, N, K, np.full(K // 128, b, np.uint8)) <= 2048 + 1024 + 256 + parts * M * rows * 4 + staged
