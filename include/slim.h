@@ -176,9 +176,10 @@ int slim_mpq_gemm(const void* x, const void* packed, const uint8_t* bits_host,
  * else, and serving loops whose memory budget was handed out at start-up, where a cudaMalloc would
  * stall every stream of the device or fail late.  Such callers have no workspace to pass.
  *
- * Same arithmetic and arguments as slim_mpq_gemm, except that the scratch (status word, stream-K
- * flags and fp32 partial tiles) is a fixed array inside the library: SLIM_STATIC_SCRATCH_MAX bytes
- * of device memory on every GPU that loads the library, held until the process exits.  The call
+ * Same arithmetic and arguments as slim_mpq_gemm, and bit for bit its result with a workspace of
+ * SLIM_STATIC_SCRATCH_MAX bytes: the scratch (status word, flags and fp32 partial sums) is a fixed array of that size
+ * inside the library, in device memory of every GPU that loads the library, held until the process exits.  (Of all shapes only
+ * layers of 49 to 56 tokens with more than 14000 columns and many rows ask slim_workspace_bytes for more, by up to a sixth.)  The call
  * allocates and frees nothing.  A shape that would need more scratch on the current device (only
  * possible on a GPU with more than 148 SMs) returns SLIM_ERR_STATIC_SCRATCH and enqueues nothing.
  *

@@ -220,3 +220,21 @@ def test_a_workspace_short_of_a_few_parts(N, K, M, avg, share):
         assert torch.equal(layer.forward(x, ws), y)
     assert (buffer[size:] == 7).all() and not ws[256:1280].any()
     slim.workspace_status(ws)
+
+
+@pytest.mark.parametrize("N,K,M", [(28672, 8192, 24), (8192, 28672, 56), (38144, 16384, 56)])
+def test_the_built_in_scratch_serves_large_layers_alike(N, K, M):
+    """slim_mpq_gemm_static gives what slim_mpq_gemm gives in a workspace of the built-in scratch's size; all but the last ask for no more."""
+    layer, size = _one_width(N, K, 2), 1280 + 148 * 256 * 128 * 4
+    x = torch.randn((M, K), device="cuda").half()
+    asked = slim.workspace_bytes(M, N, K, layer.bits)
+    assert (asked - 1024 <= size) == (K != 16384)
+    ws = torch.zeros(size, dtype=torch.uint8, device="cuda")
+    y = layer.forward(x, ws)
+    check_output(y[:, :512].cpu().numpy(), _fp64(layer, x)[:, :512], f"{N}x{K} M={M}")
+    if asked <= size:
+        assert torch.equal(layer.forward(x, slim.new_workspace(M, N, K, layer.bits)), y)
+    out, status = torch.empty_like(y), torch.ones(1, dtype=torch.int32, device="cuda")
+    for _ in range(3):
+        slim.mpq_gemm_static(x, layer.packed, layer.bits, layer.scales, layer.zeros, N, out, status)
+        assert torch.equal(out, y) and status.item() == 0
