@@ -1104,8 +1104,15 @@ static int layer_tasks(const SetGeometry& sg, int M, int G) {
 }
 // The items of a set of 2 to 64 tokens.  The steps of all row blocks, one after the other, are cut into shares of equal cost, one
 // per CTA: where a share ends inside a row block its sums are added up through the workspace (a deal of whole row blocks left the
-// last CTA of a 7B sweep 15 % over the average).  A row block has at most kTcMaxParts of them.  A set of few steps has its
-// row blocks cut into equal parts instead.
+// last CTA of a 7B sweep 15 % over the average).  A row block has at most kTcMaxParts of them.
+//
+// A set of few steps has its row blocks cut into equal parts instead, one per CTA: two of the parts that equal shares make are a CTA's, each
+// with its own sums to hand over, and more of them to a row block.  So do sets whose longest part is no more than two steps over the
+// equal share.  us, equal shares / equal parts (2 and 8 tokens, 2 bits, all layers with bit maps of their own): q, k, v of 7B, 24 row blocks of 32 groups in
+// 6 parts, 17.0 / 15.0, 19.0 / 18.2; gate and up of 7B, 44 of 32 in 3, 19.6 / 16.3, 21.7 / 17.6; q, k, v of 13B, 30 of 40 in 4, 18.7 / 17.1, 20.6 / 18.6; 64 layers
+// of 256 x 2048 in 2 19.0 / 15.8, 21.1 / 18.7; q, k, v of 70B, 20 of 64 in 7, 19.5 / 20.1, 22.0 / 21.9; beyond: 70B's at 20 tokens, 40 of 64 in 3, 26.1 / 27.7.
+// A part has four steps at least; more than eight parts are worth their sums from twelve steps on (512 x 28672, 8 / 15 parts 28.3 / 21.1; 1024 x
+// 8192 at 12 tokens, 8 / 15 of four steps 21.3 / 22.7).
 struct TcDeal {
     std::vector<SetItem> items;              // y of a cut item: offset in the room of the parts
     std::vector<SetCut> cuts;                // off: the same
@@ -1114,8 +1121,12 @@ struct TcDeal {
     size_t part_bytes;
 };
 constexpr int kTcMinSteps = 4;               // fewer per CTA: equal parts
+constexpr int kTcSlackSteps = 2;
+static int tc_parts(int split, int G) {
+    return std::max(1, std::min(split, std::max(layer_split(kSetMaxSplit, G), std::min(kTcMaxParts, G / 12))));
+}
 constexpr size_t kTcMaxSmem = 226 * 1024;
-static void tc_deal(const slim_layer* layers, int n_layers, int g, int mv, int sms, int uniform_split, TcDeal* out) {
+static void tc_deal(const slim_layer* layers, int n_layers, int g, int mv, int sms, TcDeal* out) {
     struct Block { int layer, rb, G; };
     std::vector<Block> blocks;
     std::vector<GroupTable> gt(static_cast<size_t>(n_layers));
@@ -1160,13 +1171,20 @@ static void tc_deal(const slim_layer* layers, int n_layers, int g, int mv, int s
         }
         out->items.push_back(it);
     };
-    if (steps < static_cast<long long>(kTcMinSteps) * sms) {
-        out->split = 1;
+    // the most equal parts that one wave of CTAs takes, and the longest of them
+    int split = 1, longest = 0;
+    for (int k = 2; k <= kTcMaxParts; ++k) {
+        long long n = 0;
+        for (const Block& B : blocks) n += tc_parts(k, B.G);
+        if (n <= sms) split = k;
+    }
+    for (const Block& B : blocks) longest = std::max(longest, (B.G + tc_parts(split, B.G) - 1) / tc_parts(split, B.G));
+    const bool one_wave = blocks.size() <= static_cast<size_t>(sms);
+    if (steps < static_cast<long long>(kTcMinSteps) * sms || (one_wave && static_cast<long long>(longest - kTcSlackSteps) * sms <= steps)) {
         for (const Block& B : blocks) {
-            const int parts = layer_split(uniform_split, B.G);
+            const int parts = tc_parts(split, B.G);
             for (int k = 0; k < parts; ++k) add(B, B.G * k / parts, B.G * (k + 1) / parts, k, parts);
         }
-        out->split = uniform_split;
         const int n = static_cast<int>(out->items.size());
         out->grid = std::min(n, sms);
         for (int c = 0; c <= out->grid; ++c) out->begin.push_back(static_cast<int>(static_cast<long long>(n) * c / out->grid));
@@ -1215,7 +1233,7 @@ static unsigned long long item_cost(int tiles_here, const GroupTable& gt, const 
 }
 
 // First pass over the set: validation of the shapes and everything that depends on all layers.
-// `deal`: the items of a set of 2 to 64 tokens, for a caller that writes the plan (may throw); null: the caller makes its own.
+// `deal`: the items of a set of 2 to 64 tokens (may throw); may be null if every layer has one token.
 static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeometry* sg, TcDeal* deal) {
     if (layers == nullptr || n_layers < 1 || sg == nullptr) return SLIM_ERR_INVALID_ARG;
     memset(sg, 0, sizeof *sg);
@@ -1240,11 +1258,21 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
     }
     if (sg->n_items > 0x3fffffff || sg->n_tasks > 0x3fffffff) return SLIM_ERR_UNSUPPORTED;
     sg->nt = (sg->mmax + 7) / 8;
+    sg->split = 1;
+    if (tc) {
+        tc_deal(layers, n_layers, g, rawtc::form(sg->mmax), device_sm_count(), deal);
+        sg->n_items = static_cast<long long>(deal->items.size());
+        sg->split = deal->split;
+        sg->n_cuts = static_cast<int>(deal->cuts.size());
+        sg->n_counters = sg->n_cuts;
+        sg->cnt_bytes = align_to(static_cast<size_t>(sg->n_counters) * sizeof(unsigned int), 256);
+        sg->ws_bytes += sg->cnt_bytes + align_to(deal->part_bytes, 128);
+        if (sg->n_counters > 65535) return SLIM_ERR_UNSUPPORTED;
+    }
     // A set with fewer row blocks than persistent CTAs cuts the groups of every row block into parts (items of their
     // own, fp32 partial outputs in the workspace, added in part order by the consumer warp whose part lands last).
-    const long long want = static_cast<long long>(device_sm_count()) * (tc ? 1 : kSetCtasPerSm);
-    sg->split = 1;
-    if (sg->n_items < 2 * want) {
+    const long long want = static_cast<long long>(device_sm_count()) * kSetCtasPerSm;
+    if (!tc && sg->n_items < 2 * want) {
         // the number of parts that fills the last wave of CTAs best (the smallest one within 2 % of the best)
         auto items_at = [&](int split) {
             long long n = 0;
@@ -1259,18 +1287,7 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
             if (f > best * 1.02) { best = f; sg->split = split; }
         }
     }
-    if (tc) {
-        if (deal != nullptr) {
-            tc_deal(layers, n_layers, g, rawtc::form(sg->mmax), device_sm_count(), sg->split, deal);
-            sg->n_items = static_cast<long long>(deal->items.size());
-            sg->split = deal->split;
-            sg->n_cuts = static_cast<int>(deal->cuts.size());
-            sg->n_counters = sg->n_cuts;
-            sg->cnt_bytes = align_to(static_cast<size_t>(sg->n_counters) * sizeof(unsigned int), 256);
-            sg->ws_bytes += sg->cnt_bytes + align_to(deal->part_bytes, 128);
-            if (sg->n_counters > 65535) return SLIM_ERR_UNSUPPORTED;
-        }
-    } else if (sg->split > 1) {
+    if (!tc && sg->split > 1) {
         sg->n_items = 0;
         long long counters = 0;
         for (int l = 0; l < n_layers; ++l) {
@@ -1305,7 +1322,7 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
     long long grid = static_cast<long long>(device_sm_count()) * sg->ctas_per_sm;
     if (grid > kSetMaxGrid) grid = kSetMaxGrid;
     if (grid > sg->n_items) grid = sg->n_items;
-    sg->grid = tc && deal != nullptr ? deal->grid : static_cast<int>(grid);
+    sg->grid = tc ? deal->grid : static_cast<int>(grid);
     return SLIM_OK;
 }
 

@@ -238,3 +238,24 @@ def test_the_built_in_scratch_serves_large_layers_alike(N, K, M):
     for _ in range(3):
         slim.mpq_gemm_static(x, layer.packed, layer.bits, layer.scales, layer.zeros, N, out, status)
         assert torch.equal(out, y) and status.item() == 0
+
+
+@pytest.mark.parametrize("M", [2, 7, 16, 17, 64])
+@pytest.mark.parametrize("shapes,split", [([(4096, 4096)] * 3, None), ([(512, 28672)], 15), ([(1024, 8192), (16, 8192)], 8), ([(64, 1024)] * 16, 2), ([(1040, 2048)] * 6 + [(512, 128)], None)])
+def test_small_sets_in_equal_parts(shapes, split, M):
+    """A part of a row block per CTA, up to 15 of them: the sums are added in the order of the parts."""
+    entries = []
+    for i, (N, K) in enumerate(shapes):
+        layer = _quantised(N, K, 2 + i % 2, i)
+        entries.append((layer, torch.randn((M, K), device="cuda").half(), torch.empty((M, N), dtype=torch.float16, device="cuda")))
+    s = _set(entries)
+    assert s.info["n_items"] == s.info["grid"] <= torch.cuda.get_device_properties(0).multi_processor_count
+    assert split is None or s.info["split"] == split
+    first = [y.clone() for (_, _, y) in entries]
+    for (layer, x, _), y in zip(entries, first):
+        check_output(y.cpu().numpy(), _fp64(layer, x), f"{layer.N}x{layer.K} M={M}")
+    for _ in range(20):
+        s.run()
+        for (_, _, y), want in zip(entries, first):
+            assert torch.equal(y, want)
+    s.check()
