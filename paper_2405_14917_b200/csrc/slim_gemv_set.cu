@@ -1904,13 +1904,16 @@ int slim_mpq_gemv_set(const slim_gemv_set_info* info, const void* plan, void* wo
     const int st = slim::set_params(info, plan, workspace, workspace_bytes, &prm, &smem);
     if (st != SLIM_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // A small set (its row blocks are cut into parts) of 2 to 8 tokens is launched early, since its launches are a good part of
-    // its time: 7B in decoder order at 5 tokens 229 -> 220 us, at 8 234 -> 225.  Large sets measured 1 to 2 % slower that way, and
-    // with 16 tokens it depends (three 7B blocks 182 -> 163, one 70B block 161 -> 166).
-    const bool one = info->max_tokens == 1, early = !one && info->token_tiles == 1 && info->split > 1;
+    constexpr int per_block = 32;                    // staging tasks
+    const int stage_blocks = (info->stage_tasks + per_block - 1) / per_block;
+    // The staging blocks of a set of 2 to 64 tokens are launched early where there are SMs for them: until the kernel ahead ends, its CTAs leave
+    // a block no room on theirs (a set like this one is taken as that kernel), and blocks that crowd on the other SMs stage more slowly than they
+    // would on all.  us, early / not: no SM free, one and eight 7B blocks at 8 and 2 tokens 29.4 / 28.9, 99.2 / 97.6; 128 blocks for 20 free SMs, 64
+    // layers of 256 x 2048 at 2 and 5 tokens 15.8 / 15.1, 18.5 / 16.5; not / early: 45 for 28, q, k, v of 13B at 12 tokens 23.0 / 21.2, 32 for
+    // 16, gate and up of 7B at 16 tokens 21.9 / 20.3, 24 for 132, 1024 x 8192 at 12 tokens 21.3 / 19.6.
+    const bool one = info->max_tokens == 1, early = !one && stage_blocks <= 4 * (slim::device_sm_count() - info->grid);
     {
-        constexpr int per_block = 32;                // tasks
-        slim::PdlLaunch l(static_cast<unsigned>((info->stage_tasks + per_block - 1) / per_block), 256, 0, s, early);
+        slim::PdlLaunch l(static_cast<unsigned>(stage_blocks), 256, 0, s, early);
         SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, one ? slim::gemv_set_stage_kernel<true> : slim::gemv_set_stage_kernel<false>, prm.layers, prm.ws, info->n_layers, info->stage_tasks, info->n_counters));
     }
     // The kernel of 2 to 64 tokens asks for its first slices while x is staged; what the staging kernel writes it waits for.
