@@ -51,9 +51,9 @@ int device_sm_count();
 
 // slim_mpq_gemv sends large layers of one token through the layer-set kernels: workspace bytes that takes (0: this shape stays on the
 // per-layer kernel), and the call itself (SLIM_OK, a negative status, or 1 if not taken).
-size_t gemv_route_workspace_bytes(int M, int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt);
+size_t gemv_route_workspace_bytes(int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt);
 int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, const GroupTable& gt, const void* scales, const void* zeros,
-               void* y, int M, int N, int K, int g, void* workspace, size_t workspace_bytes, cudaStream_t stream);
+               void* y, int N, int K, int g, void* workspace, size_t workspace_bytes, cudaStream_t stream);
 
 // slim_mpq_gemv sends single-token layers whose K fits a CTA's shared memory to a kernel of their own (slim_gemv_one.cu):
 // SLIM_OK, a negative status, or 1 if not taken.

@@ -513,8 +513,8 @@ int slim_workspace_bytes(int M, int N, int K, int g, const uint8_t* bits_host, s
     if (M > SLIM_GEMV_MAX_M && N > 0) *out_bytes = slim::gemm_workspace_bytes(M, N, gt.G);
     else if (M >= slim::kPreStageMinM && N > 0 && K > 0) *out_bytes = slim::prestage_bytes(M, gt);
     else *out_bytes = slim::kWsHeader;
-    if (M >= 1 && M <= SLIM_GEMV_MAX_M && N > 0 && K > 0) {       // large layers go through the layer-set kernels
-        const size_t routed = slim::gemv_route_workspace_bytes(M, N, K, g, bits_host, gt);
+    if (M == 1 && N > 0 && K > 0) {       // large layers go through the layer-set kernels
+        const size_t routed = slim::gemv_route_workspace_bytes(N, K, g, bits_host, gt);
         if (routed > *out_bytes) *out_bytes = routed;
     }
     if (M >= 2 && N > 0 && K > 0) {
@@ -581,17 +581,16 @@ int slim_mpq_gemv(const void* x, const void* packed, const uint8_t* bits_host, c
     if (workspace == nullptr || workspace_bytes < slim::kWsHeader) return SLIM_ERR_WORKSPACE;
     if (!slim::aligned16(workspace)) return SLIM_ERR_ALIGNMENT;
 
-    // A layer large enough to feed the persistent ring on its own goes through the layer-set kernels, if the workspace
-    // has room for their plan and staged activations (slim_workspace_bytes asks for it).
-    {
-        const int routed = slim::gemv_route(x, packed, bits_host, gt, scales, zeros, y, M, N, K, g, workspace, workspace_bytes, s);
+    if (M == 1) {
+        // A layer large enough to feed the persistent ring on its own goes through the layer-set kernels, if the workspace
+        // has room for their plan and staged activations (slim_workspace_bytes asks for it); others through the integer form with the
+        // whole K of a few tiles per CTA, if they fit it.
+        const int routed = slim::gemv_route(x, packed, bits_host, gt, scales, zeros, y, N, K, g, workspace, workspace_bytes, s);
         if (routed <= 0) return routed;
-    }
-    // A single token: the integer form with the whole K of a few tiles per CTA, if the layer fits it.
-    {
         const int taken = slim::gemv_one(x, packed, gt, scales, zeros, y, M, N, K, workspace, s);
         if (taken <= 0) return taken;
     }
+    // A large one of several tokens: the kernel of layer sets on tcgen05, where that is sooner.
     {
         const int taken = slim::gemv_tc(x, packed, gt, scales, zeros, y, M, N, K, workspace, workspace_bytes, s);
         if (taken <= 0) return taken;

@@ -65,9 +65,8 @@ struct SetLayer {
     const __half* scales;
     const __half* zeros;
     __half* y;
-    size_t x_off;          // workspace offset of the layer's staged activations, group after group:
-                           // (sum_k x, 2^(24-S)) float2[16], then the fragments [slice][8 mma][MP][4 lanes] x 8 B
-    size_t part_off;       // workspace offset of the layer's fp32 partial outputs [split][M][N] (split > 1 only)
+    size_t x_off;          // workspace offset of the layer's staged activations, group after group, in the form that MP names
+    size_t part_off;       // one token: workspace offset of the layer's fp32 partial outputs [split][N] (split > 1 only)
     int M, N, K, G;
     uint16_t count[4];     // groups of 1, 2, 3, 4 bits
     int task0;             // first (token, group) staging task of the layer
@@ -1094,7 +1093,7 @@ static size_t layer_ws_bytes(int M, const GroupTable& gt) {
 // Sets of 2 to 64 tokens go through gemv_set_tc_kernel.
 static bool tc_form(int mmax) { return mmax >= 2 && mmax <= rawtc::kMaxTokens; }
 // Staged activations of a layer, and the staging tasks (token, group) it has.
-static size_t layer_x_bytes(const SetGeometry& sg, int M, const GroupTable& gt) {
+static size_t layer_x_bytes(const SetGeometry& sg, const GroupTable& gt) {
     if (!tc_form(sg.mmax)) return layer_ws_bytes(sg.mres, gt);
     // no less than a workspace has always had for so many tokens
     return std::max(align_to(static_cast<size_t>(gt.G) * rawtc::record_bytes(rawtc::form(sg.mmax)), 128), layer_ws_bytes(sg.mres, gt));
@@ -1254,7 +1253,7 @@ static int set_geometry(const slim_layer* layers, int n_layers, int g, SetGeomet
         const int items = ((L.N >> 4) + tpi - 1) / tpi;
         sg->n_items += items;
         sg->n_tasks += layer_tasks(*sg, L.M, gt.G);
-        sg->ws_bytes += layer_x_bytes(*sg, L.M, gt);
+        sg->ws_bytes += layer_x_bytes(*sg, gt);
     }
     if (sg->n_items > 0x3fffffff || sg->n_tasks > 0x3fffffff) return SLIM_ERR_UNSUPPORTED;
     sg->nt = (sg->mmax + 7) / 8;
@@ -1389,12 +1388,12 @@ struct RouteLayout {
 };
 
 // keep_flags: the first counters, which stay zero, lie over the flags of slim_mpq_gemm; without, everything is kWsFlagsBytes sooner.
-static bool route_layout(int M, int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt, bool keep_flags, RouteLayout* r) {
+static bool route_layout(int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt, bool keep_flags, RouteLayout* r) {
     static_assert(kSetOffCounters == kWsFlagsOffset, "the counters are cleared where the flags are");
-    if (M != 1 || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < kRouteMinBytes) return false;
+    if (N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < kRouteMinBytes) return false;
     slim_layer L;
     memset(&L, 0, sizeof L);
-    L.bits_host = bits_host; L.M = M; L.N = N; L.K = K;
+    L.bits_host = bits_host; L.M = 1; L.N = N; L.K = K;
     if (set_geometry(&L, 1, g, &r->sg, nullptr) != SLIM_OK) return false;
     const int tpi = kSetConsumers * r->sg.tpw;
     r->n_rb = ((N >> 4) + tpi - 1) / tpi;
@@ -1404,14 +1403,14 @@ static bool route_layout(int M, int N, int K, int g, const uint8_t* bits_host, c
     r->plan_off = kSetOffCounters + r->cnt0 * sizeof(unsigned int) + r->sg.cnt_bytes;
     r->plan_bytes = set_plan_bytes(1, static_cast<long long>(r->n_rb) * r->sp);
     r->x_off = r->plan_off + align_to(r->plan_bytes, 256);
-    r->part_off = r->x_off + layer_x_bytes(r->sg, M, gt);
-    r->total = r->part_off + (r->sp > 1 ? align_to(static_cast<size_t>(r->sp) * M * N * sizeof(float), 128) : 0);
+    r->part_off = r->x_off + layer_x_bytes(r->sg, gt);
+    r->total = r->part_off + (r->sp > 1 ? align_to(static_cast<size_t>(r->sp) * N * sizeof(float), 128) : 0);
     return true;
 }
 
-size_t gemv_route_workspace_bytes(int M, int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt) {
+size_t gemv_route_workspace_bytes(int N, int K, int g, const uint8_t* bits_host, const GroupTable& gt) {
     RouteLayout r;
-    return route_layout(M, N, K, g, bits_host, gt, true, &r) ? r.total : 0;
+    return route_layout(N, K, g, bits_host, gt, true, &r) ? r.total : 0;
 }
 
 }  // namespace slim
@@ -1454,8 +1453,7 @@ static int set_params(const slim_gemv_set_info* info, const void* plan, void* wo
         *smem_out = smem;
         return SLIM_OK;
     }
-    const int mp = info->max_tokens == 1 ? 2 : 8 * info->token_tiles;
-    if (slot_off_w(tpi, mp) + tpi * 256 * info->max_bits > info->slot_bytes) return SLIM_ERR_INVALID_ARG;
+    if (slot_off_w(tpi, 2) + tpi * 256 * info->max_bits > info->slot_bytes) return SLIM_ERR_INVALID_ARG;
     *smem_out = smem;
     return SLIM_OK;
 }
@@ -1606,13 +1604,13 @@ static int launch_set_for(const slim_gemv_set_info* info, const SetParams& prm, 
 // Returns SLIM_OK after enqueueing the layer through the layer-set kernels, a negative status on failure, or 1 if this
 // shape or workspace is not routed (the caller then takes the per-layer kernel).
 int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, const GroupTable& gt, const void* scales, const void* zeros,
-               void* y, int M, int N, int K, int g, void* workspace, size_t workspace_bytes, cudaStream_t stream) {
+               void* y, int N, int K, int g, void* workspace, size_t workspace_bytes, cudaStream_t stream) {
     RouteLayout r;
-    if (!route_layout(M, N, K, g, bits_host, gt, true, &r)) return 1;
-    if (workspace_bytes < r.total && (!route_layout(M, N, K, g, bits_host, gt, false, &r) || workspace_bytes < r.total)) return 1;
+    if (!route_layout(N, K, g, bits_host, gt, true, &r)) return 1;
+    if (workspace_bytes < r.total && (!route_layout(N, K, g, bits_host, gt, false, &r) || workspace_bytes < r.total)) return 1;
     slim_layer L;
     memset(&L, 0, sizeof L);
-    L.x = x; L.packed = packed; L.scales = scales; L.zeros = zeros; L.y = y; L.bits_host = bits_host; L.M = M; L.N = N; L.K = K;
+    L.x = x; L.packed = packed; L.scales = scales; L.zeros = zeros; L.y = y; L.bits_host = bits_host; L.M = 1; L.N = N; L.K = K;
     SetLayer d;
     fill_descriptor(L, gt, 2, 0, r.x_off, r.sp, r.part_off, r.cnt0, &d);
     uint8_t* plan = static_cast<uint8_t*>(workspace) + r.plan_off;
@@ -1624,7 +1622,7 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
     info.n_slots = r.sg.n_slots;
     info.slot_bytes = r.sg.slot_bytes;
     info.token_tiles = r.sg.nt;
-    info.stage_tasks = layer_tasks(r.sg, M, gt.G);
+    info.stage_tasks = layer_tasks(r.sg, 1, gt.G);
     info.n_items = n_items;
     info.max_bits = r.sg.bmax;
     info.max_tokens = r.sg.mmax;
@@ -1637,15 +1635,13 @@ int gemv_route(const void* x, const void* packed, const uint8_t* bits_host, cons
     size_t smem = 0;
     const int st = set_params(&info, plan, workspace, workspace_bytes, &prm, &smem);
     if (st != SLIM_OK) return st;
-    // One token: both kernels are launched early (the staging kernel is a handful of blocks).  With more tokens its
-    // blocks are many and early launches measured 1 to 4 % slower, so those keep plain stream order.
-    const bool early = M == 1;
+    // Both kernels are launched early: the staging kernel is a handful of blocks.
     {
         constexpr int per_block = 32;                    // tasks
-        PdlLaunch l(static_cast<unsigned>((info.stage_tasks + per_block - 1) / per_block), 256, 0, stream, early);
+        PdlLaunch l(static_cast<unsigned>((info.stage_tasks + per_block - 1) / per_block), 256, 0, stream, true);
         SLIM_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, set_single_stage_kernel, d, plan, prm.ws, grid, r.n_rb, r.sp, info.stage_tasks, info.n_counters));
     }
-    return launch_set_for(&info, prm, smem, stream, early);
+    return launch_set_for(&info, prm, smem, stream, true);
 }
 
 size_t gemv_tc_workspace_bytes(int M, int N, const GroupTable& gt) {
@@ -1768,7 +1764,7 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
         for (int l = 0; l < n_layers; ++l) {
             slim::GroupTable gt;
             slim::make_group_table(layers_host[l].N, layers_host[l].K, g, layers_host[l].bits_host, &gt);
-            off += slim::layer_x_bytes(sg, layers_host[l].M, gt);
+            off += slim::layer_x_bytes(sg, gt);
         }
         for (int l = 0; l < n_layers; ++l) {
             const slim_layer& L = layers_host[l];
@@ -1792,7 +1788,7 @@ int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g, void*
         }
         x_off[l] = same >= 0 ? x_off[same] : ws_off;
         slim::fill_descriptor(L, gt, tc ? -slim::rawtc::form(sg.mmax) : 2, task, x_off[l], sp, part_off[l], cnt0, &d);
-        ws_off += slim::layer_x_bytes(sg, L.M, gt);
+        ws_off += slim::layer_x_bytes(sg, gt);
         SLIM_CUDA_TRY(cudaMemcpyAsync(plan_dev + slim::kSetPlanHeader + static_cast<size_t>(l) * sizeof d, &d, sizeof d,
                                       cudaMemcpyHostToDevice, s));
         const int n_rb = ((L.N >> 4) + tpi - 1) / tpi;
