@@ -259,3 +259,75 @@ def test_small_sets_in_equal_parts(shapes, split, M):
         for (_, _, y), want in zip(entries, first):
             assert torch.equal(y, want)
     s.check()
+
+
+def _from_codes(codes, bits, scales, zeros):
+    N, K = codes.shape
+    packed = slim.pack_weights(torch.from_numpy(codes).cuda(), bits)
+    return slim.QuantLinear(packed, bits, torch.from_numpy(scales).cuda(), torch.from_numpy(zeros).cuda(), N, K)
+
+
+@pytest.mark.parametrize("M", list(range(2, 17, 2)) + list(range(24, 65, 8)))
+def test_all_bits_of_an_activation_are_multiplied(M):
+    """One activation at a time, of every exponent from -6 to 6 and a full significand of either sign, on every column: s (q - z) x up to the rounding to fp16
+    (2^-11) and those of the two fp32 operations of the fold.  The third piece of x is up to 2^-8 of it, the second 2^-3."""
+    L = oracle_layer(32, 512, 2, M, bits=np.array([1, 2, 3, 4], np.uint8), seed_name="set-tc-bits")
+    What = orc.dequant_f64(L["codes"], L["scales"], L["zeros"])
+    dl = _on_device(L)
+    x = np.zeros((512 // M + 1, M, 512), np.float16)
+    for i in range(x.shape[0]):
+        for m in range(M):
+            k = (i * M + m) % 512
+            x[i, m, k] = (-1) ** (i + k) * (1 + (389 * k + 61 * m) % 1024 / 1024) * 2.0 ** ((i + 5 * m) % 13 - 6)
+    entries = [(dl, torch.from_numpy(xi).cuda(), torch.empty((M, 32), dtype=torch.float16, device="cuda")) for xi in x]
+    _set(entries)
+    for xi, (_, _, y) in zip(x, entries):
+        ref = xi.astype(np.float64) @ What.T
+        assert (np.abs(y.cpu().numpy() - ref) <= 2.0 ** -11 * np.abs(ref) * (1 + 2.0 ** -9) + 2.0 ** -25).all()
+
+
+@pytest.mark.parametrize("M", [4, 8, 12, 16, 24, 64])
+@pytest.mark.parametrize("b", [1, 2, 3, 4])
+def test_small_activations_beside_a_large_one(b, M):
+    """A group whose largest activation meets a weight of exactly zero, and one other: exact down to 2^-(16 + b) of the largest, off by 2^-(27 + b) of it
+    at most below."""
+    rng = np.random.default_rng(10 * b + M)
+    codes = rng.integers(1, 1 << b, (16, 128)).astype(np.uint8)
+    codes[:, 77] = 0
+    scales, zeros = np.full((1, 16), 1.0, np.float16), np.zeros((1, 16), np.float16)
+    layer = _from_codes(codes, np.array([b], np.uint8), scales, zeros)
+    large = 1.9990234375 * 2.0 ** 8
+    entries, xs = [], []
+    for i in range(0, 26 * 32, M):
+        x = np.zeros((M, 128), np.float16)
+        x[:, 77] = large if i % 2 else -1.0 * 2.0 ** 8                # the top and the bottom of a power of two
+        for m in range(M):
+            t, k = (i + m) % 26, (i + m) * 7 % 128
+            if k != 77:
+                x[m, k] = (-1) ** m * (1 + (331 * (i + m)) % 1024 / 1024) * 2.0 ** (8 - t)
+        xs.append(x)
+        entries.append((layer, torch.from_numpy(x).cuda(), torch.empty((M, 16), dtype=torch.float16, device="cuda")))
+    _set(entries)
+    for x, (_, _, y) in zip(xs, entries):
+        small = x.astype(np.float64)
+        top = np.abs(small).max(axis=1)[:, None]
+        small[:, 77] = 0
+        ref = small @ codes.astype(np.float64).T
+        exact = np.abs(small).max(axis=1)[:, None] >= top * 2.0 ** -(16 + b)
+        off = np.where(exact, 0.0, top * 2.0 ** -(27 + b) * codes.max())
+        assert (np.abs(y.cpu().numpy() - ref) <= 2.0 ** -11 * np.abs(ref) * (1 + 2.0 ** -9) + 2.0 ** -25 + off).all()
+
+
+@pytest.mark.parametrize("g,M", [(256, 2), (512, 8), (256, 16), (512, 24), (256, 40)])
+def test_one_large_layer_of_wide_groups(g, M):
+    """Two or four K-tiles that share a row of scales and zero points."""
+    N, K = 24592, 8192
+    W, a = wl.make_weight_and_norms_device((53, g, M), N, K, "cuda")
+    layer = slim.QuantLinear.from_weight(W, a, 3 if M > 32 else 2, g=g)
+    x = torch.randn((M, K), device="cuda").half()
+    ws = slim.new_workspace(M, N, K, layer.bits, g=g)
+    assert ws.numel() > 148 * M * (512 if M <= 16 else 256) * 4       # parts: the kernel for large layers
+    y = layer.forward(x, ws)
+    What = slim.dequant(layer.packed, layer.bits, layer.scales, layer.zeros, N, K, g=g).double()
+    check_output(y.cpu().numpy(), (x.double() @ What.T).cpu().numpy(), f"{N}x{K} M={M} g={g}")
+    slim.workspace_status(ws)
