@@ -462,9 +462,10 @@ __global__ void __launch_bounds__(kSetThreads, kSetCtasPerSm) gemv_set_kernel(co
 }
 
 // ------------------------------------------------------------------------------------------ the persistent kernel, 2 to 64 tokens
-// Measured against a kernel on mma.sync m16n8k16 (us, all bytes from HBM): two 70B blocks at 2 bits, 16 and 32 tokens 241 / 391 -> 146 /
-// 209; two 13B blocks at 3 bits, 16 tokens 181 -> 81; eight 7B blocks, 2 and 5 tokens at 2 bits 144 / 145 -> 101 / 112, 8 tokens at 3 bits
-// 166 -> 137; one 7B block, 4 tokens 36.9 -> 25; four 7B blocks, 17 and 40 tokens at 3 bits 181 / 269 -> 104 / 138, 64 at 2 bits 361 -> 174.
+// Measured against a kernel on mma.sync m16n8k16 (us, all bytes from HBM, in turn on one GPU, short runs at full clocks): two 70B blocks at 2 bits, 16 and
+// 32 tokens 238 / 386 -> 141 / 207; two 13B blocks at 3 bits, 16 tokens 180 -> 75; eight 7B blocks, 2 and 5 tokens at 2 bits 142 / 142 -> 98 /
+// 115, 8 tokens at 3 bits 163 -> 134; one 7B block, 4 tokens 39.0 -> 27.7; four 7B blocks, 17 and 40 tokens at 3 bits 178 / 267 -> 106 / 135, 64 at 2
+// bits 357 -> 170.  Under the power cap of long runs the 70B blocks at 16 tokens take 239 -> 171.
 // Bound: issue slots, 2850 / 3350 / 3800 warp instructions a step of 512 rows at 2 / 8 / 16 tokens (ncu), of which decoding takes 950 and
 // the fold up to 1100, next to 780 cycles of HBM time; 256 rows at 40 tokens 3900, most of them the fold's.
 
@@ -1500,7 +1501,7 @@ struct TcSinglePlan {
 // those / this one (one GPU, in turn):
 //  * size: 8192 x 8192 at 2 bits (16 MB) 2 / 8 / 16 tokens 11.1 / 13.9, 12.5 / 16.7, 16.4 / 22.8; 12288 x 8192 (24.0) 15.9 / 15.5, 17.1 / 17.7, 22.4 /
 //    23.1; 7168 x 14336 (24.5) 17.1 / 16.9, 18.3 / 19.6, 23.8 / 26.6; 5120 x 13824 at 3 bits (25.3) 19.7 / 17.3, 20.9 / 19.9, 27.2 / 27.1; 13312 x
-//    8192 (26.0) 18.1 / 16.2, 19.4 / 18.5, 25.4 / 24.0; 28672 x 8192 (56) 16 tokens 49.1 / 34.7.  20 / 32 tokens: 20480 x 4096 (20) 25.6 / 22.0, 25.6 /
+//    8192 (26.0) 18.1 / 16.2, 19.4 / 18.5, 25.4 / 24.0; 28672 x 8192 (56) 16 tokens 51.7 / 35.0.  20 / 32 tokens: 20480 x 4096 (20) 25.6 / 22.0, 25.6 /
 //    23.1; 13312 x 8192 36.1 / 25.1, 36.2 / 26.6.  40 / 56 tokens: 13824 x 5120 at 3 bits (25.3) 27.8 / 27.3, 27.8 / 32.6; 24576 x 8192 (48) 52.7 / 40.3,
 //    52.8 / 49.5 (64 tokens, 28672 x 8192: 60.3 / 59.0, and the batched kernel takes the same time up to 128).
 //  * row blocks: a layer of few has parts for few CTAs (14 to a row block of 512), or many parts to be added up by one warp.  K = 32768, 4
@@ -1513,12 +1514,15 @@ struct TcSinglePlan {
 //    31.5, 2304 x 29184 (342) 45.0 / 34.8; K = 32768 at 2 or 4 bits (256), 3584 and 1536 rows, 27.6 / 29.0, 23.3 / 28.6.
 constexpr size_t kTcSingleMin = 24u << 20, kTcSingleMinMany = 48u << 20, kTcSoonerMin = 25u << 20;
 constexpr int kTcSingleTokens = 56, kTcSlices = 272;
+static bool many_slices(int M, const GroupTable& gt) {
+    int slices = 0;
+    for (int j = 0; j < gt.G; ++j) slices += slice_count(gt.bits[j]);
+    return M > 8 && slices > kTcSlices;
+}
 static bool tc_sooner(int M, int N, const GroupTable& gt) {
     const int rows = rawtc::rows_of(rawtc::form(M)), n_rb = (N + rows - 1) / rows;
     if (M > 16) return M <= 32 || n_rb >= (M <= 48 ? 18 : 20);
-    int slices = 0;
-    for (int j = 0; j < gt.G; ++j) slices += slice_count(gt.bits[j]);
-    if (M > 8 && slices > kTcSlices) return true;
+    if (many_slices(M, gt)) return true;
     return (M <= 3 || static_cast<size_t>(16) * N * gt.prefix[gt.G] >= kTcSoonerMin) && n_rb >= (M <= 4 ? 6 : 8);
 }
 // Share c of `grid` ends at cost total c / grid.  No part of a single step: such a cut moves to the end of the row block.
@@ -1546,8 +1550,9 @@ static void tc_places(const GroupTable& gt, int row_tiles, TcSinglePlan* pl) {
         pl->place[c] = static_cast<uint32_t>(rb) << 10 | static_cast<uint32_t>(at);
     }
 }
-// In a workspace of that many bytes.  One that is short of a few rooms has fewer shares, down to nine tenths: with fewer than that the kernels that
-// take the layer otherwise are as soon (24576 x 8192 at 16 tokens would take 45 us with 105 shares, 32.6 with 148, 44 there).
+// In a workspace of that many bytes.  One that is short of rooms has fewer shares as long as that is sooner than the kernels that take the layer
+// otherwise: down to nine tenths, where those are near (24576 x 8192 at 2 / 8 / 16 tokens 27.1 / 28.7 / 38.5 us there, 22.1 / 27.0 / 32.6 here with all
+// shares), and to a half of them at many K-slices (8192 x 28672 at 2 bits and 16 tokens 85.8 there, 39.6 here).
 static bool tc_single_plan(int M, int N, const GroupTable& gt, size_t bytes, TcSinglePlan* pl) {
     if (!tc_form(M) || M > kTcSingleTokens || N <= 0 || static_cast<size_t>(16) * N * gt.prefix[gt.G] < (M <= 32 ? kTcSingleMin : kTcSingleMinMany)) return false;
     const int mv = rawtc::form(M), rows = rawtc::rows_of(mv), row_tiles = rows / 16;
@@ -1567,7 +1572,8 @@ static bool tc_single_plan(int M, int N, const GroupTable& gt, size_t bytes, TcS
     const size_t budget = kTcMaxSmem - kSetOffDesc;
     const int slot_l = rawtc::slot_size(mv, bmax, false), slot_s = rawtc::slot_size(mv, bmax);
     pl->part_off = kTcSingleParts;
-    for (pl->grid = widest; 10 * pl->grid >= 9 * widest && pl->grid > 0; --pl->grid) {
+    const int least = std::max(1, many_slices(M, gt) ? widest / 2 : (9 * widest + 9) / 10);
+    for (pl->grid = widest; pl->grid >= least; --pl->grid) {
         // the most steps of a share: all of the cheapest, and what moves at its ends
         const int share = static_cast<int>(per_rb * pl->n_rb / pl->grid / tc_step_cost(bmin, row_tiles)) + 5;
         const size_t rec = static_cast<size_t>(rawtc::record_bytes(mv)) * share;

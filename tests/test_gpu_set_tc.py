@@ -204,7 +204,7 @@ def test_layers_of_few_row_blocks(N, K, M, avg):
     slim.workspace_status(ws)
 
 
-@pytest.mark.parametrize("N,K,M,avg,share", [(28672, 4096, 6, 2, 0.94), (8192, 14336, 16, 3, 0.92), (65552, 2048, 24, 2, 0.95), (28672, 4096, 6, 2, 0.5), (8192, 24576, 56, 2, 0.93)])
+@pytest.mark.parametrize("N,K,M,avg,share", [(28672, 4096, 6, 2, 0.94), (8192, 14336, 16, 3, 0.92), (65552, 2048, 24, 2, 0.95), (28672, 4096, 6, 2, 0.5), (8192, 24576, 56, 2, 0.93), (8192, 28672, 16, 2, 0.7)])
 def test_a_workspace_short_of_a_few_parts(N, K, M, avg, share):
     """Fewer shares as long as that is a few, the other kernels in a workspace that is much smaller; nothing is written past its end."""
     layer = _quantised(N, K, avg)
