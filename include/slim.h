@@ -136,14 +136,14 @@ int slim_dequant(const void* packed, const uint8_t* bits_host, const void* scale
  * inference kernel, App. B.2: group-by-group dequantisation and dot product with the shared
  * activation).  Streams the packed slices once; HBM-bound.  Results are deterministic for a
  * given (shape, device, workspace size).  x with Inf/NaN gives unspecified y.  `workspace` must be at least
- * 256 bytes (the kernel itself keeps its partial sums in shared memory).
- * A layer whose packed codes take 32 MB or more (24 MB at M > 1) is run by the kernels of slim_mpq_gemv_set instead (same
- * result within the rounding of the accumulation order; at M = 1 with the fixed-point x described there) when the
- * workspace has the slim_workspace_bytes() that shape asks for; with a smaller workspace it takes the per-layer
- * kernel.  The call reads no host memory after it returns and can be captured in a CUDA graph either way.
- * At M = 1 every route takes x in the 22-bit fixed-point form described at slim_mpq_gemv_set (the per-layer
+ * 256 bytes (the per-layer kernels keep their partial sums in shared memory).
+ * A layer whose packed codes take 32 MB or more is run by the kernels of slim_mpq_gemv_set instead, at M > 1 most layers from 24 MB
+ * on (same result within the rounding of the accumulation order, with x in the form described there for that many tokens), when the
+ * workspace has the slim_workspace_bytes() that shape asks for (at M > 1 somewhat less may do); with a smaller workspace it takes the
+ * per-layer kernel.  The call reads no host memory after it returns and can be captured in a CUDA graph either way.
+ * The per-layer kernels take x at M = 1 in the 22-bit fixed-point form described at slim_mpq_gemv_set (the
  * single-token kernel, CTAs that hold the whole K of a few 16-row tiles, serves the layers whose K fits a CTA's
- * shared memory with all CTAs resident at once; the others, and M > 1, multiply the fp16 x as it is).
+ * shared memory with all CTAs resident at once); the others, and M > 1, multiply the fp16 x as it is.
  * The per-layer kernels are launched with programmatic stream serialisation and fetches packed, scales and zeros
  * before it waits for the kernel ahead of it on the stream: those three buffers must be complete when the call is
  * enqueued, or be written by a call of this library (each of which ends in a kernel that makes them so); between a kernel of
@@ -164,7 +164,9 @@ int slim_gemv_plan(int M, int N, int K, int g, const uint8_t* bits_host, int* ou
 
 /* Batched / prefill path, M > 16: same contract, tensor-core (tcgen05) kernel.  Zero points that
  * are multiples of 1/16 in [-16, 16) (every zero point Eq. 1 or Eq. 2 produces) are applied exactly,
- * others are rounded (to the nearest 1/16 at worst).  Deterministic for a given (shape, device, workspace size). */
+ * others are rounded (to the nearest 1/16 at worst).  Most layers of 24 MB and more at up to 32 tokens, and of 48 MB and more at up to 56, are
+ * run by the kernel of slim_mpq_gemv_set, with exact codes, fp32 zero points and x in the form described there, when the workspace has
+ * the slim_workspace_bytes() that shape asks for.  Deterministic for a given (shape, device, workspace size). */
 int slim_mpq_gemm(const void* x, const void* packed, const uint8_t* bits_host,
                   const void* scales, const void* zeros, void* y,
                   int M, int N, int K, int g,
@@ -205,13 +207,13 @@ int slim_mpq_gemm_static(const void* x, const void* packed, const uint8_t* bits_
 /* Several INDEPENDENT layers of the decode path (1 <= M <= SLIM_GEMV_SET_MAX_M = 64 tokens each) in one launch: the q/k/v or
  * gate/up projections that share an input, or a sweep over a model's layers.  (The paper launches
  * its kernel per layer, App. B.2; a decode-sized layer is too small to keep HBM busy on its own,
- * so the set is walked by persistent CTAs that stream the packed slices of one 128-row block after
+ * so the set is walked by persistent CTAs that stream the packed slices of one row block (256 or 512 rows) after
  * another through a ring of shared-memory slots, with no pause between layers.)  No layer of a set
  * may read what another layer of the same set writes.
  *
  * Every layer gets the y = x * W-hat^T of slim_mpq_gemv (same products, fp32 accumulation in a
- * different order: the groups of a layer are added sorted by bit-width, and a set with fewer row blocks
- * than persistent CTAs adds them in up to 8 parts; fp16 output); the results are deterministic for a
+ * different order: the groups of a layer are added sorted by bit-width, those of a row block in several parts
+ * where it is cut (slim_gemv_set_info.split); fp16 output); the results are deterministic for a
  * given (set, device).
  * A set in which EVERY layer has M = 1 runs on integer tensor-core instructions: per group of 128
  * columns x is first rounded to fixed point with 22 bits relative to the group's largest |x_k|, so an
@@ -219,8 +221,9 @@ int slim_mpq_gemm_static(const void* x, const void* packed, const uint8_t* bits_
  * of at most 2^-22 of the maximum; the sums over the group are then exact.  Per output row n this adds at
  * most  sum over groups of 2^-22 max|x_group| sum_{k in group} |w-hat[n][k]|  to the error of the fp16
  * path at more than one token; x must be finite.  Sets of 2 to 64 tokens multiply
- * the codes by x as a sum of three 8-bit floats, exact for an fp16 activation within a factor 2^15 of the group's largest and
- * off by at most 2^-26 of that below, with the sums of a group added up by the tensor cores; their widest layer, rounded up to an
+ * the codes by x as a sum of three 8-bit floats: in a group of b bits exact for an fp16 activation within a factor 2^(16+b) of
+ * the largest of its 128 columns, and off by at most 2^-(27+b) of that largest below; the products of a group are added up
+ * in fp32 by the tensor cores; their widest layer, rounded up to an
  * even number of tokens (beyond 16 a multiple of 8), fixes how many columns every layer computes, so a set is fastest when its layers have
  * about the same token count.  (Between 17 and about 100 tokens a layer set streams several times the weights per second that
  * slim_mpq_gemm dequantises, which is built for hundreds of tokens and more.)
@@ -243,15 +246,16 @@ typedef struct slim_gemv_set_info {
     int n_slots;           /* ring slots per CTA */
     int slot_bytes;
     int token_tiles;       /* 8-token MMA tiles: 1 to 8 */
-    int stage_tasks;       /* (layer, token, group) triples staged; layers with one x and one bit map count once */
-    int n_items;           /* row blocks (work items) of the set */
+    int stage_tasks;       /* (layer, token, group) triples staged, tokens rounded up to four in sets of several; layers with one x and one bit
+                              map count once */
+    int n_items;           /* row blocks of the set, and parts of those that are cut (work items) */
     int max_bits;          /* widest group of the set */
     int max_tokens;        /* largest M of the set */
     int tiles_per_warp;    /* an item is 128 rows times this: 4 for sets of 2 to 16 tokens, else 2 */
-    int split;             /* most parts the groups of a row block are cut into: 1 .. 8 when the set has fewer row blocks than
-                              persistent CTAs (layers with few groups get fewer), 1 .. 15 for sets of 2 to 64 tokens, whose CTAs
-                              take equal shares that may end inside a row block; fp32 partial outputs in the workspace, added in
-                              part order by the warp whose part lands last */
+    int split;             /* most parts the groups of a row block are cut into: single-token sets 1 .. 8, more than one where they have
+                              fewer row blocks than persistent CTAs (layers with few groups get fewer); sets of 2 to 64 tokens 1 .. 15:
+                              equal parts in small sets, in others what equal shares of the CTAs that end inside a row block make of it.
+                              fp32 partial outputs in the workspace, added in part order by the warp whose part lands last */
     int n_counters;        /* arrival counters of the split row blocks (workspace, cleared by every launch) */
     int resident_pairs;    /* > 0: a small single-token set that runs as ONE launch with every CTA resident at once (the
                               whole K of 2 x resident_pairs row tiles per CTA, no ring, no staging kernel); the ring
@@ -263,13 +267,14 @@ typedef struct slim_gemv_set_info {
 } slim_gemv_set_info;
 
 /* Host-only.  Sizes of the device plan buffer and of the workspace a set needs on the current
- * device.  The workspace holds the status word and, per layer, its activations in tensor-core
- * fragment order. */
+ * device.  The workspace holds the status word, the arrival counters and partial sums of cut row blocks and, per layer, its
+ * activations in the form that the tensor cores read. */
 int slim_gemv_set_bytes(const slim_layer* layers_host, int n_layers, int g,
                         size_t* plan_bytes, size_t* workspace_bytes);
 
-/* Validates the set, deals the work items to the persistent CTAs (heaviest item first, each to the
- * CTA with the least work so far, so the CTAs finish together) and writes the plan (layer
+/* Validates the set, deals the work items to the persistent CTAs (single-token sets: heaviest item first, each to the
+ * CTA with the least work so far; sets of 2 to 64 tokens: shares of equal cost in the set's order, or one part each in a small set; either way the
+ * CTAs finish together) and writes the plan (layer
  * descriptors, every CTA's list of items) into `plan` (device, 16-byte aligned, plan_bytes from
  * slim_gemv_set_bytes) with copies enqueued on `stream`; fills *info.  layers_host and the bit
  * maps are read during the call only.  The plan stays valid while the layers' pointers do.
@@ -277,7 +282,7 @@ int slim_gemv_set_bytes(const slim_layer* layers_host, int n_layers, int g,
 int slim_gemv_set_plan(const slim_layer* layers_host, int n_layers, int g,
                        void* plan, size_t plan_bytes, slim_gemv_set_info* info, void* stream);
 
-/* Runs the set: one small kernel puts every layer's activations into fragment order in the
+/* Runs the set: one small kernel puts every layer's activations into the form that the tensor cores read in the
  * workspace, one persistent kernel computes all layers (a small single-token set whose CTAs are all resident at
  * once runs as one launch instead: slim_gemv_set_info.resident_pairs; that launch uses programmatic stream
  * serialisation and requests packed, scales and zeros before it waits for the kernel ahead of it on the stream, under

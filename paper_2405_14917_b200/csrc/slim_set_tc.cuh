@@ -8,10 +8,11 @@
 //    e4m3 is linear.  So a register of four operand bytes costs one logic instruction (five per 16 codes of two bits with
 //    the shift), half of what pairs of fp16 cost, and half of their bytes go through tensor memory.
 //  * B = activations, x 2^(S + lo - pp) as the sum of three e5m2 numbers (three significant bits each take the 11 of an
-//    fp16 with the signs' help).  S lifts the group's largest |x| to the top of e5m2's range, so a value down to 2^-15 of that is
-//    taken exactly, and smaller ones are off by 2^-26 of the largest.  The pieces are columns of their own (N = 3 M rounded up to
-//    16), which the fold adds.  tcgen05 adds the products of a group without loss (measured: 128 products of random codes and
-//    normal x, no difference from fp64).
+//    fp16 with the signs' help).  S lifts the group's largest |x| to [2^14, 2^15), e5m2's smallest step is 2^-16, and pp is up to 4 - b at b
+//    bits: the eleventh bit of a value is no less than that step down to 2^-(16 + b) of the largest, so to there x is taken exactly, and below it is off
+//    by half of the step, 2^-(27 + b) of the largest.  The pieces are columns of their own (N = 3 M rounded up to
+//    16), which the fold adds, or rows that further MMAs add (form).  D is fp32 (128 products of random codes and normal x differed in no bit from
+//    fp64; sums that span more than 24 bits are rounded).
 //
 // tcgen05 with A in tensor memory takes 16 / 21 / 26 cycles per 128 x N x 32 at N = 16 / 32 / 48 (fp16 the same per K = 16), where
 // mma.sync takes 128 to 256 per 128 x 16 x 32.
