@@ -75,8 +75,8 @@ def test_each_bit_of_a_code_meets_its_activation(M):
 
 
 def test_activations_of_any_size_are_taken_exactly():
-    """One weight per row and all of x's exponents: x (q - z) s from a group whose largest |x| is 2^15 times the smallest; an infinity and a NaN
-    spoil their token alone."""
+    """Groups of x with sixteen exponents and of subnormals alone stay within the rounding of sums of 128 products (which x is taken exactly is tested
+    above one activation at a time, and below); an infinity and a NaN spoil their token alone."""
     L = oracle_layer(16, 256, 2, 4, seed_name="set-tc-range")
     x = np.zeros((4, 256), np.float16)
     x[0, :128] = [(1 + (37 * i % 1024) / 1024) * 2.0 ** (i % 16 - 13) * (-1) ** i for i in range(128)]
