@@ -1106,7 +1106,7 @@ static int layer_tasks(const SetGeometry& sg, int M, int G) {
 // per CTA: where a share ends inside a row block its sums are added up through the workspace (a deal of whole row blocks left the
 // last CTA of a 7B sweep 15 % over the average).  A row block has at most kTcMaxParts of them.
 //
-// A set of few steps has its row blocks cut into equal parts instead, one per CTA: two of the parts that equal shares make are a CTA's, each
+// A set of few steps has its row blocks cut into parts of about one length instead, one per CTA: two of the parts that equal shares make are a CTA's, each
 // with its own sums to hand over, and more of them to a row block.  So do sets whose longest part is no more than two steps over the
 // equal share.  us, equal shares / equal parts (2 and 8 tokens, 2 bits, all layers with bit maps of their own): q, k, v of 7B, 24 row blocks of 32 groups in
 // 6 parts, 17.0 / 15.0, 19.0 / 18.2; gate and up of 7B, 44 of 32 in 3, 19.6 / 16.3, 21.7 / 17.6; q, k, v of 13B, 30 of 40 in 4, 18.7 / 17.1, 20.6 / 18.6; 64 layers
@@ -1122,8 +1122,9 @@ struct TcDeal {
 };
 constexpr int kTcMinSteps = 4;               // fewer per CTA: equal parts
 constexpr int kTcSlackSteps = 2;
-static int tc_parts(int split, int G) {
-    return std::max(1, std::min(split, std::max(layer_split(kSetMaxSplit, G), std::min(kTcMaxParts, G / 12))));
+// Parts of no more than that many groups, as far as so many are worth it.
+static int tc_parts(int length, int G) {
+    return std::max(1, std::min((G + length - 1) / length, std::max(layer_split(kSetMaxSplit, G), std::min(kTcMaxParts, G / 12))));
 }
 constexpr size_t kTcMaxSmem = 226 * 1024;
 static void tc_deal(const slim_layer* layers, int n_layers, int g, int mv, int sms, TcDeal* out) {
@@ -1171,18 +1172,19 @@ static void tc_deal(const slim_layer* layers, int n_layers, int g, int mv, int s
         }
         out->items.push_back(it);
     };
-    // the most equal parts that one wave of CTAs takes, and the longest of them
-    int split = 1, longest = 0;
-    for (int k = 2; k <= kTcMaxParts; ++k) {
+    // the shortest parts that one wave of CTAs takes, and the longest of them
+    int length = SLIM_MAX_GROUPS, longest = 0;
+    for (int len = SLIM_MAX_GROUPS; len >= 1; --len) {
         long long n = 0;
-        for (const Block& B : blocks) n += tc_parts(k, B.G);
-        if (n <= sms) split = k;
+        for (const Block& B : blocks) n += tc_parts(len, B.G);
+        if (n > sms) break;
+        length = len;
     }
-    for (const Block& B : blocks) longest = std::max(longest, (B.G + tc_parts(split, B.G) - 1) / tc_parts(split, B.G));
+    for (const Block& B : blocks) longest = std::max(longest, (B.G + tc_parts(length, B.G) - 1) / tc_parts(length, B.G));
     const bool one_wave = blocks.size() <= static_cast<size_t>(sms);
     if (steps < static_cast<long long>(kTcMinSteps) * sms || (one_wave && static_cast<long long>(longest - kTcSlackSteps) * sms <= steps)) {
         for (const Block& B : blocks) {
-            const int parts = tc_parts(split, B.G);
+            const int parts = tc_parts(length, B.G);
             for (int k = 0; k < parts; ++k) add(B, B.G * k / parts, B.G * (k + 1) / parts, k, parts);
         }
         const int n = static_cast<int>(out->items.size());
